@@ -143,6 +143,10 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 template <int THREADS> __device__ __forceinline__ void consumer_bar_sync() { asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory"); }
 
+// Everything the kernel before wrote (queries) is read behind this; keys, values, row counts and context lengths are
+// older, so the producer streams ahead of it.
+__device__ __forceinline__ void x_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Byte offset of (row, 16-byte chunk) inside a 128-byte-swizzled tile whose rows are 128 bytes.
 __device__ __forceinline__ uint32_t swz(int row, int chunk) { return (uint32_t)(row * 128 + ((chunk ^ (row & 7)) << 4)); }
 
@@ -227,6 +231,7 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
   __shared__ int pfx_s[XMAXB + 1];
   __shared__ int aseq_s[XMAXB];             // the a-th sequence that has an active row
   __shared__ int n_aseq_s;
+  __shared__ int row0_s[XMAXB];             // first query row of every sequence
   __shared__ unsigned char nact_s[XMAXB];   // active rows of every sequence (at most 32 here)
   const Dims &dm = a.dm;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -270,14 +275,27 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
       n += __popc(m);
     }
     if (lane == 0) n_aseq_s = n;
+  } else if (warp == 2) {   // first query row of every sequence
+    int carry = 0;
+    for (int c0 = 0; c0 < batch; c0 += 32) {
+      const int b = c0 + lane;
+      const int own = b < batch ? nact_s[b] : 0;
+      int v = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { int u = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += u; }
+      if (b < batch) row0_s[b] = a.row_base != nullptr ? a.row_base[b] : a.packed ? carry + v - own : b * dm.C;
+      carry += __shfl_sync(0xffffffffu, v, 31);
+    }
   }
   // rows of a sequence beyond its active ones come back as zeros (all heads)
-  for (int b = cta; b < batch && a.row_base == nullptr; b += G) {
+  // (packed rows: there are none)
+  for (int b = cta; b < batch && a.row_base == nullptr && !a.packed; b += G) {
     const int S = nact_s[b];
     uint4 *z = reinterpret_cast<uint4 *>(out + (size_t)(b * dm.C + S) * dm.d);      // rows are d * 2 bytes, d a multiple of 64
     for (int idx = tid; idx < (dm.C - S) * dm.d / 8; idx += XTHREADS) z[idx] = make_uint4(0u, 0u, 0u, 0u);
   }
   __syncthreads();
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const long long T = (long long)H * pfx_s[batch];
   // CTAs that get work: every one of them at least XMIN_TILES tiles (when there are that many), so
   // that few tiles do not turn into many one-tile CTAs whose records one CTA then merges serially
@@ -296,7 +314,7 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
   if (two_per_segment && 2 * n_seg < Ge) Ge = 2 * n_seg;
   if (whole_segments) {
     Ge = (n_seg + seg_per_cta - 1) / seg_per_cta;
-    if (cta >= Ge) return;
+    if (cta >= Ge) { x_dependency_wait(); return; }
     auto seg_tile = [&](int sidx) {    // first tile of segment sidx in the flat list
       if (sidx >= n_seg) return (int)T;
       const int bb = aseq_s[sidx / H], hh = sidx % H;
@@ -305,7 +323,7 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
     lo = seg_tile(cta * seg_per_cta);
     hi = seg_tile((cta + 1) * seg_per_cta);
   } else {
-    if (cta >= Ge) return;
+    if (cta >= Ge) { x_dependency_wait(); return; }
     lo = (int)(cta * T / Ge); hi = (int)((cta + 1) * T / Ge);
   }
 
@@ -338,6 +356,7 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
   }
 
   // -------------------------------------------------------------------- consumers
+  x_dependency_wait();
   const int g = lane >> 2, tig = lane & 3;
   const __nv_bfloat16 *qbuf = (const __nv_bfloat16 *)a.q;
   const int kb = warp * KPW;         // this warp's keys inside every tile
@@ -351,7 +370,7 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
     const int seg_start = H * pfx_s[b] + h * cur.nt, seg_end = seg_start + cur.nt;
     const int my_end = min(hi, seg_end);
     const int S = nact_s[b], ctx_len = min(max(a.st.ctx_len[b], 1), dm.ctx);
-    const int row0 = a.row_base != nullptr ? a.row_base[b] : b * dm.C;
+    const int row0 = row0_s[b];
     float seg_sl2 = sl2, seg_vscale = 1.f;          // 8-bit: the key scale joins the score scale, the value scale the final 1 / l
     if (FP8) {
       const int kv_b = a.kv_seq != nullptr ? a.kv_seq[b] : b;
@@ -368,8 +387,8 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
         const __nv_bfloat16 *q_hi = qbuf + (size_t)(row0 + r_hi) * dm.d + h * kDh + 4 * tig;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          const uint2 lo = r_lo < S ? *reinterpret_cast<const uint2 *>(q_lo + kk * 16) : make_uint2(0u, 0u);
-          const uint2 hi = r_hi < S ? *reinterpret_cast<const uint2 *>(q_hi + kk * 16) : make_uint2(0u, 0u);
+          const uint2 lo = r_lo < S ? __ldcg(reinterpret_cast<const uint2 *>(q_lo + kk * 16)) : make_uint2(0u, 0u);
+          const uint2 hi = r_hi < S ? __ldcg(reinterpret_cast<const uint2 *>(q_hi + kk * 16)) : make_uint2(0u, 0u);
           qf[mt][kk][0] = bf16x2_to_f16x2(lo.x); qf[mt][kk][2] = bf16x2_to_f16x2(lo.y);
           qf[mt][kk][1] = bf16x2_to_f16x2(hi.x); qf[mt][kk][3] = bf16x2_to_f16x2(hi.y);
         }
@@ -378,10 +397,10 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
         const __nv_bfloat16 *q_hi = qbuf + (size_t)(row0 + r_hi) * dm.d + h * kDh + 2 * tig;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          qf[mt][kk][0] = r_lo < S ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16) : 0u;
-          qf[mt][kk][1] = r_hi < S ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16) : 0u;
-          qf[mt][kk][2] = r_lo < S ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8) : 0u;
-          qf[mt][kk][3] = r_hi < S ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8) : 0u;
+          qf[mt][kk][0] = r_lo < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_lo + kk * 16)) : 0u;
+          qf[mt][kk][1] = r_hi < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_hi + kk * 16)) : 0u;
+          qf[mt][kk][2] = r_lo < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8)) : 0u;
+          qf[mt][kk][3] = r_hi < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8)) : 0u;
         }
       }
     }
@@ -676,15 +695,25 @@ cudaError_t cross_attn_tma_prepare() {
 // n_ctas persistent CTAs (two per SM); a.part_o holds cross_attn_tma_partial_bytes(n_ctas, C),
 // a.tickets one zeroed int32 per (sequence, head) (the kernel leaves them zeroed).
 // 8-bit keys/values (a.kv_scale set): tmap = the keys' lines, tmap_v = the transposed values; else tmap alone.
+// Packed rows (a.packed): launched as a programmatic dependent of the query projection before it, which writes none of the keys,
+// values, row counts and context lengths, so the first tiles travel while that kernel runs.
 cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, int n_ctas, cudaStream_t s) {
-  int mt = (a.dm.C + 15) / 16;
+  const int mt = (a.dm.C + 15) / 16;
   const bool fp8 = a.kv_scale != nullptr;
-  if (mt == 1 && !fp8) cross_attn_tma_kernel<1, false><<<n_ctas, xthreads(false), xsmem(false), s>>>(tmap, tmap_v, a);
-  else if (mt == 2 && !fp8) cross_attn_tma_kernel<2, false><<<n_ctas, xthreads(false), xsmem(false), s>>>(tmap, tmap_v, a);
-  else if (mt == 1) cross_attn_tma_kernel<1, true><<<n_ctas, xthreads(true), xsmem(true), s>>>(tmap, tmap_v, a);
-  else if (mt == 2) cross_attn_tma_kernel<2, true><<<n_ctas, xthreads(true), xsmem(true), s>>>(tmap, tmap_v, a);
-  else return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  if (mt < 1 || mt > 2) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_ctas, 1, 1);
+  cfg.blockDim = dim3(xthreads(fp8), 1, 1);
+  cfg.dynamicSmemBytes = xsmem(fp8);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = a.packed ? 1 : 0;
+  if (mt == 1 && !fp8) return cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, false>, tmap, tmap_v, a);
+  if (mt == 2 && !fp8) return cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, false>, tmap, tmap_v, a);
+  if (mt == 1) return cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, true>, tmap, tmap_v, a);
+  return cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, true>, tmap, tmap_v, a);
 }
 
 }  // namespace pd

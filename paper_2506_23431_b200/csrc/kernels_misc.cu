@@ -160,6 +160,59 @@ cudaError_t launch_embed(const Dims &dm, const DecState &st, int batch, int dtyp
   return cudaGetLastError();
 }
 
+// The same over the step's active rows packed back to back: row (b, c) goes to m = (active rows of the sequences before b) + c.
+// Leaves what the packed products (proj_mma.cu) read: x, bf16 x * gain and the row's sum of squares (they apply the norm's
+// scale behind the product), where each packed row's cache entry goes, the sequence's first packed row, and each row's packed
+// place (-1: none).
+__global__ void __launch_bounds__(128) embed_packed_kernel(Dims dm, DecState st, const __nv_bfloat16 *__restrict__ embed, float *__restrict__ x,
+                                                           const __nv_bfloat16 *__restrict__ gain, __nv_bfloat16 *__restrict__ xg,
+                                                           float *__restrict__ ssq, int ssq_stride, int4 *__restrict__ row_meta_packed,
+                                                           int32_t *__restrict__ row_at) {
+  __shared__ float red[4];
+  __shared__ int redi[4];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int r = blockIdx.x, b = r / dm.C, c = r % dm.C, tid = threadIdx.x;
+  const int i = st.row_sub[r];
+  const int S = st.n_active[b];
+  int before = 0;
+  for (int bb = tid; bb < b; bb += 128) before += st.n_active[bb];
+  const int tok = i > 0 ? st.last_tok[b * dm.SM + i - 1] : 0;
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  if ((tid & 31) == 0) redi[tid >> 5] = before;
+  __syncthreads();
+  before = redi[0] + redi[1] + redi[2] + redi[3];
+  if (tid == 0) {
+    if (c == 0) st.crow[b] = before;
+    row_at[r] = c < S ? before + c : -1;
+  }
+  if (c >= S) return;
+  const size_t m = (size_t)(before + c);
+  if (tid == 0) row_meta_packed[m] = st.row_meta[r];
+  const uint2 *e = reinterpret_cast<const uint2 *>(embed + (size_t)tok * dm.d);       // four columns per thread; d is a multiple of 64
+  const uint2 *g = reinterpret_cast<const uint2 *>(gain);
+  float ss = 0.f;
+  for (int q = tid; q < dm.d / 4; q += 128) {
+    const uint2 ev = e[q], gv = g[q];
+    const __nv_bfloat162 *e2 = reinterpret_cast<const __nv_bfloat162 *>(&ev), *g2 = reinterpret_cast<const __nv_bfloat162 *>(&gv);
+    const float2 a = __bfloat1622float2(e2[0]), bb = __bfloat1622float2(e2[1]), ga = __bfloat1622float2(g2[0]), gb = __bfloat1622float2(g2[1]);
+    *reinterpret_cast<float4 *>(x + m * dm.d + 4 * q) = make_float4(a.x, a.y, bb.x, bb.y);
+    const __nv_bfloat162 o0 = __floats2bfloat162_rn(a.x * ga.x, a.y * ga.y), o1 = __floats2bfloat162_rn(bb.x * gb.x, bb.y * gb.y);
+    *reinterpret_cast<uint2 *>(xg + m * dm.d + 4 * q) = make_uint2(*reinterpret_cast<const uint32_t *>(&o0), *reinterpret_cast<const uint32_t *>(&o1));
+    ss += a.x * a.x + a.y * a.y + bb.x * bb.x + bb.y * bb.y;
+  }
+  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+  if ((tid & 31) == 0) red[tid >> 5] = ss;
+  __syncthreads();
+  if (tid == 0) ssq[m * ssq_stride] = red[0] + red[1] + red[2] + red[3];
+}
+
+cudaError_t launch_embed_packed(const Dims &dm, const DecState &st, int batch, const void *embed, float *x, const void *gain, void *xg,
+                                float *ssq, int ssq_stride, int4 *row_meta_packed, int32_t *row_at, cudaStream_t s) {
+  embed_packed_kernel<<<batch * dm.C, 128, 0, s>>>(dm, st, (const __nv_bfloat16 *)embed, x, (const __nv_bfloat16 *)gain, (__nv_bfloat16 *)xg, ssq,
+                                                   ssq_stride, row_meta_packed, row_at);
+  return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------------------------------------
 // RMSNorm of the fp32 residual stream, output in the GEMM input type.  One CTA per row; a thread
 // keeps its part of the row in registers (one pass over memory) when the row fits RN_REGS values

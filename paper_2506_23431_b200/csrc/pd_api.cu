@@ -25,7 +25,7 @@ struct Layout {
   // integer state (offsets in int32 words from the start of the state block)
   size_t w_hdr, w_stats, w_k, w_done, w_steps, w_nact, w_ctx, w_ticket, w_start, w_len, w_state, w_flag, w_last,
       w_forced, w_row, w_prow, w_rtok, w_ptab, w_tokens, w_chosen, w_trace, w_plist_n, w_xtick, w_crow, w_t0, w_plan, state_words;
-  Region state, plist, row_meta, bias_tab, ctx_len_in, forced_in, teacher, dist_bucket, rope_tab, x, hbuf, qkv, qbuf, self_out, cq, cross_out,
+  Region state, plist, row_meta, row_meta_packed, row_at, ssq, bias_tab, ctx_len_in, forced_in, teacher, dist_bucket, rope_tab, x, hbuf, qkv, qbuf, self_out, cq, cross_out,
       ffn, logits, vpart_val, vpart_idx, vterm, part_o, part_ml, kv_c, kv_scale, kv_pool, enc_stage, proj_stage, cublas_ws;
   size_t total = 0;
 };
@@ -107,6 +107,9 @@ void make_layout(const pd_config &c, const Dims &dm, int max_splits, Layout &L) 
   reg(L.state, L.state_words * 4);
   reg(L.plist, B * SM * dm.PPS * sizeof(int4));
   reg(L.row_meta, B * C * sizeof(int4));
+  reg(L.row_meta_packed, B * C * sizeof(int4));
+  reg(L.row_at, B * C * 4);
+  reg(L.ssq, M * (size_t)(dm.d / 32) * 4);
   reg(L.bias_tab, (size_t)dm.H * dm.n_dist * 4);
   reg(L.ctx_len_in, B * 4);
   reg(L.forced_in, B * SM * 4);
@@ -173,6 +176,8 @@ struct pd_handle {
   bool kv8 = false;
   VocabMaps vmaps;                 // hidden rows and lm_head for the tcgen05 vocabulary projection
   bool vocab_tc = false;
+  bool packed_ok = false;          // bf16, and every kernel of the packed path takes this configuration
+  bool rows_packed = false;        // the last step left the activation buffers packed (pd_debug_read)
   // pd_generate_host: host-to-device copies of the encoder memory run on a stream of their own, in
   // chunks of sequences, so that the context projection of one chunk overlaps the copy of the next
   static constexpr int kMaxChunks = 8;
@@ -312,6 +317,17 @@ int fused_append(const pd_handle *h) {
   return h->dm.PPS >= 2 ? 2 : 0;
 }
 
+// The packed decode path: every active row of a step in one packed row list, the layers' products on proj_mma.cu, every launch a
+// programmatic dependent of the one before it.  For few rows, where a step is a chain of launch and load latencies: the products
+// take less than cuBLAS with its norm kernels up to about 128 allocated rows (per layer, 90 active rows of 128 at width 768: 30 us
+// against 31 us, 6 of 8: 16 us against 31 us), and the dependent launches give the attentions a head start.  With more rows
+// the products are bound by the bytes their 32-column slices read again for every row group (190 of 512 at width 1024:
+// 58 us against 40 us): there the unpacked path below, with cuBLAS over the allocated rows, stays.
+constexpr int kPackedMaxRows = 128;
+bool packed_path(const pd_handle *h) {
+  return h->packed_ok && h->batch * h->dm.C <= kPackedMaxRows && cross_attn_tma_supported(h->dm, h->batch);
+}
+
 AttnArgs attn_args(pd_handle *h, int layer, bool self) {
   AttnArgs a;
   a.dm = h->dm; a.st = h->st; a.layer = layer; a.batch = h->batch;
@@ -328,6 +344,7 @@ AttnArgs attn_args(pd_handle *h, int layer, bool self) {
   a.bias_tab = h->cfg.pos_mode == PD_POS_T5_BIAS ? h->ptr<float>(h->lay.bias_tab) : nullptr;
   a.qkv = h->ptr<void>(h->lay.qkv);
   a.fused_append = self ? fused_append(h) : 0;
+  a.packed = packed_path(h) ? 1 : 0;
   a.rope_tab = h->ptr<float2>(h->lay.rope_tab);
   a.kv_scale = (!self && h->kv8) ? h->ptr<float>(h->lay.kv_scale) : nullptr;
   a.kv_seq = nullptr; a.row_base = nullptr;
@@ -366,8 +383,77 @@ pd_status enqueue_cross_attention(pd_handle *h, int layer) {
   return PD_OK;
 }
 
-// The launch sequence of one decode step (one pass of Eq. 3 for all active rows + Algorithm 1's bookkeeping).
+// Vocabulary projection, greedy choice and scheduler on packed rows.  ssq null: hb holds normalised rows; else x * gain,
+// and the rows' scales come from the sums of squares.
+pd_status enqueue_vocab(pd_handle *h, const float *ssq) {
+  const Dims &dm = h->dm;
+  const Layout &L = h->lay;
+  VocabArgs va;                                       // logits stay in tensor memory unless they were asked for
+  va.n_active = h->st.n_active; va.batch = h->batch; va.m_fixed = 0; va.V = dm.V; va.K = dm.d; va.rows_cap = h->batch * dm.C;
+  va.eos = dm.eos; va.sep = dm.sep;
+  va.part_val = h->ptr<float>(L.vpart_val); va.part_idx = h->ptr<int32_t>(L.vpart_idx); va.term_val = h->ptr<float>(L.vterm);
+  va.logits = h->cfg.store_logits ? h->ptr<float>(L.logits) : nullptr;
+  va.ssq = ssq; va.parts = proj_mma_parts(dm.d); va.ssq_stride = dm.d / 32; va.inv_width = 1.f / (float)dm.d; va.eps = dm.eps;
+  va.status = h->st.hdr + HDR_STATUS;
+  OWN(h, PD_PROF_VOCAB, launch_vocab_tc(h->vmaps, va, h->stream));
+  OWN(h, PD_PROF_ARGMAX_SCHED, launch_pick_sched(dm, h->st, h->batch, vocab_tc_tiles(dm.V), va.part_val, va.part_idx, va.term_val,
+                                                 h->ptr<int32_t>(L.teacher), h->stream));
+  return PD_OK;
+}
+
+// The launch sequence of one decode step (one pass of Eq. 3 for all active rows + Algorithm 1's bookkeeping) on packed
+// rows: embed, eight launches per layer, vocabulary projection, pick + scheduler.
+pd_status enqueue_step_packed(pd_handle *h) {
+  const Dims &dm = h->dm;
+  const Layout &L = h->lay;
+  cudaStream_t s = h->stream;
+  __nv_bfloat16 *hb = h->ptr<__nv_bfloat16>(L.hbuf);
+  float *ssq = h->ptr<float>(L.ssq);
+  const bool rope = dm.pos_mode == PD_POS_ROPE;
+  ProjArgs p;
+  memset(&p, 0, sizeof(p));
+  p.n_active = h->st.n_active; p.batch = h->batch; p.rows_cap = h->batch * dm.C;
+  p.ssq_in = ssq; p.parts_in = proj_mma_parts(dm.d); p.ssq_stride = dm.d / 32; p.inv_width = 1.f / (float)dm.d; p.eps = dm.eps;
+  p.x = h->ptr<float>(L.x); p.ssq_out = ssq;
+  p.row_meta = h->ptr<int4>(L.row_meta_packed); p.rope_tab = rope ? h->ptr<float2>(L.rope_tab) : nullptr;
+  p.kv_pool = h->ptr<__nv_bfloat16>(L.kv_pool); p.pool = dm.pool; p.P = dm.P; p.raw_f32 = rope ? 1 : 0;
+  auto bf = [](const void *q) { return static_cast<const __nv_bfloat16 *>(q); };
+  OWN(h, PD_PROF_OTHER, launch_embed_packed(dm, h->st, h->batch, h->w.embed, p.x, h->layer_w[0], hb, ssq, p.ssq_stride,
+                                            h->ptr<int4>(L.row_meta_packed), h->ptr<int32_t>(L.row_at), s));
+  for (int l = 0; l < dm.L; ++l) {
+    const void *const *lw = &h->layer_w[(size_t)l * kLayerTensors];
+    ProjArgs a = p;                                   // queries, keys, values; the cache append
+    a.act = hb; a.w = bf(lw[1]); a.K = dm.d; a.N = 3 * dm.d; a.layer = l;
+    if (l == 0) a.parts_in = 1;                       // the embedding kernel leaves whole sums
+    a.out = h->ptr<__nv_bfloat16>(L.qbuf); a.raw = l == dm.L - 1 ? h->ptr<void>(L.qkv) : nullptr;
+    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_QKV, a, s));
+    {
+      ProfScope ps(h, PD_PROF_SELF_ATTN);
+      PD_TRY(enqueue_self_attention(h, l));
+    }
+    a = p; a.act = h->ptr<__nv_bfloat16>(L.self_out); a.w = bf(lw[2]); a.K = dm.d; a.N = dm.d; a.out = hb; a.gain_next = bf(lw[3]);
+    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_RESID, a, s));
+    a = p; a.act = hb; a.w = bf(lw[4]); a.K = dm.d; a.N = dm.d; a.out = h->ptr<__nv_bfloat16>(L.cq);
+    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_STORE, a, s));
+    {
+      ProfScope ps(h, PD_PROF_CROSS_ATTN);
+      PD_TRY(enqueue_cross_attention(h, l));
+    }
+    a = p; a.act = h->ptr<__nv_bfloat16>(L.cross_out); a.w = bf(lw[6]); a.K = dm.d; a.N = dm.d; a.out = hb; a.gain_next = bf(lw[7]);
+    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_RESID, a, s));
+    a = p; a.act = hb; a.w = bf(lw[8]); a.K = dm.d; a.N = dm.ff; a.out = h->ptr<__nv_bfloat16>(L.ffn);
+    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_RELU, a, s));
+    a = p; a.act = h->ptr<__nv_bfloat16>(L.ffn); a.w = bf(lw[9]); a.K = dm.ff; a.N = dm.d; a.out = hb;
+    a.gain_next = bf(l + 1 < dm.L ? h->layer_w[(size_t)(l + 1) * kLayerTensors] : h->w.final_norm);
+    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_RESID, a, s));
+  }
+  return enqueue_vocab(h, ssq);
+}
+
+// The same on unpacked rows (row c of sequence b at b * C + c).
 pd_status enqueue_step(pd_handle *h) {
+  h->rows_packed = packed_path(h);
+  if (h->rows_packed) return enqueue_step_packed(h);
   const Dims &dm = h->dm;
   const int dt = h->cfg.dtype;
   const int M = h->batch * dm.C;
@@ -423,19 +509,8 @@ pd_status enqueue_step(pd_handle *h) {
     PD_TRY(gemm(h, false, M, dm.d, dm.ff, ffn, lw[9], x, true, 1.f));
   }
   if (h->vocab_tc) {
-    // active rows only, packed; logits stay in tensor memory unless they were asked for
-    VocabArgs va;
-    va.n_active = h->st.n_active; va.batch = h->batch; va.m_fixed = 0; va.V = dm.V; va.K = dm.d; va.rows_cap = M;
-    va.eos = dm.eos; va.sep = dm.sep;
-    va.part_val = h->ptr<float>(h->lay.vpart_val); va.part_idx = h->ptr<int32_t>(h->lay.vpart_idx);
-    va.term_val = h->ptr<float>(h->lay.vterm);
-    va.logits = h->cfg.store_logits ? logits : nullptr;
-    va.status = h->st.hdr + HDR_STATUS;
     OWN(h, PD_PROF_OTHER, launch_rmsnorm_packed(dm, h->st, h->batch, dt, x, h->w.final_norm, hb, s));
-    OWN(h, PD_PROF_VOCAB, launch_vocab_tc(h->vmaps, va, s));
-    OWN(h, PD_PROF_ARGMAX_SCHED, launch_pick_sched(dm, h->st, h->batch, vocab_tc_tiles(dm.V), va.part_val, va.part_idx, va.term_val,
-                                                   h->ptr<int32_t>(h->lay.teacher), s));
-    return PD_OK;
+    return enqueue_vocab(h, nullptr);
   }
   OWN(h, PD_PROF_OTHER, launch_rmsnorm(dm, M, dt, x, h->w.final_norm, hb, s));
   PD_TRY(gemm(h, true, M, dm.V, dm.d, hb, h->w.lm_head, logits, true, 0.f));
@@ -593,6 +668,17 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
       return bail(PD_ERR_CUDA);
     if (vocab_tc_prepare() != cudaSuccess) return bail(PD_ERR_CUDA);
     h->vocab_tc = true;
+  }
+  if (h->vocab_tc && h->have_tmap && self_attn_tc_supported(dm)) {
+    h->packed_ok = true;
+    const int spec[6][3] = {{1, dm.d, 3 * dm.d}, {2, dm.d, dm.d}, {4, dm.d, dm.d}, {6, dm.d, dm.d}, {8, dm.d, dm.ff}, {9, dm.ff, dm.d}};
+    for (int l = 0; l < dm.L; ++l)
+      for (const auto &sp : spec)
+        h->packed_ok = h->packed_ok && proj_mma_supported(sp[1], sp[2], h->layer_w[(size_t)l * kLayerTensors + sp[0]]);
+    if (h->packed_ok && (proj_mma_prepare() != cudaSuccess ||
+                         cudaMemsetAsync(h->ptr<void>(L.row_at), 0xFF, L.row_at.bytes, h->stream) != cudaSuccess ||
+                         cudaStreamSynchronize(h->stream) != cudaSuccess))
+      return bail(PD_ERR_CUDA);
   }
   *out = h;
   return PD_OK;
@@ -965,6 +1051,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
       a.batch = (int)std::min<size_t>(kTfCrossBatch, G - g0);
       a.q = cq; a.out = co;
       a.st.n_active = d_gn + g0; a.st.ctx_len = d_gctx + g0;
+      a.packed = 0;
       a.kv_seq = d_gseq + g0; a.row_base = d_grow0 + g0;
       a.part_o = reinterpret_cast<float *>(base + L.part);
       a.tickets = reinterpret_cast<int32_t *>(base + L.tickets);
@@ -1095,6 +1182,32 @@ pd_status pd_debug_read(pd_handle *h, int32_t which, void *dst_host, size_t max_
     default: return fail(h, PD_ERR_ARG, "pd_debug_read: unknown buffer");
   }
   size_t n = r->bytes < max_bytes ? r->bytes : max_bytes;
+  if (h->rows_packed && which != PD_BUF_STATE) {
+    // The step left its active rows packed in (sequence, row) order: bring them over and spread them to row c of
+    // sequence b at b * C + c, from the last one down (a row never moves to a lower place); other rows are zero.
+    const size_t rows = (size_t)h->batch * h->dm.C, row_bytes = r->bytes / ((size_t)h->dm.B * h->dm.C);
+    const size_t width = which == PD_BUF_QKV && h->dm.pos_mode != PD_POS_ROPE ? row_bytes / 2 : row_bytes;   // bf16 rows in a buffer sized for fp32
+    std::vector<int32_t> at(rows);
+    CU_TRY(h, cudaMemcpyAsync(at.data(), h->ptr<void>(L.row_at), rows * 4, cudaMemcpyDeviceToHost, h->stream));
+    CU_TRY(h, cudaStreamSynchronize(h->stream));
+    size_t packed = 0;
+    for (size_t i = 0; i < rows; ++i) packed += at[i] >= 0;
+    const bool whole = max_bytes >= rows * width;
+    std::vector<uint8_t> tmp(whole ? 0 : rows * width);
+    uint8_t *dst = whole ? static_cast<uint8_t *>(dst_host) : tmp.data();
+    if (packed > 0) {
+      CU_TRY(h, cudaMemcpyAsync(dst, h->ws + r->off, packed * width, cudaMemcpyDeviceToHost, h->stream));
+      CU_TRY(h, cudaStreamSynchronize(h->stream));
+    }
+    for (size_t i = rows; i-- > 0;) {
+      if (at[i] >= 0) { if ((size_t)at[i] != i) memcpy(dst + i * width, dst + at[i] * width, width); }
+      else memset(dst + i * width, 0, width);
+    }
+    if (!whole) memcpy(dst_host, tmp.data(), n);
+    else if (n > rows * width) memset(dst + rows * width, 0, n - rows * width);
+    if (bytes_out) *bytes_out = n;
+    return PD_OK;
+  }
   CU_TRY(h, cudaMemcpyAsync(dst_host, h->ws + r->off, n, cudaMemcpyDeviceToHost, h->stream));
   CU_TRY(h, cudaStreamSynchronize(h->stream));
   if (bytes_out) *bytes_out = n;

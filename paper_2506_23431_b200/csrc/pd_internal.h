@@ -104,6 +104,9 @@ struct AttnArgs {
   const void *qkv;
   int fused_append;
   const float2 *rope_tab;
+  // rows of q and out: 1 = the step's active rows packed back to back in (sequence, row) order, the step's keys/values are in the
+  // cache, and the launch is a programmatic dependent of the one before it; 0 = row c of sequence b at b * C + c
+  int packed;
   // cross-attention over 8-bit keys/values: [layer][sequence][head][keys | values] fp32 scales (else null)
   const float *kv_scale;
   // cross-attention over row groups that are not one per sequence (the teacher-forced forward: many rows per
@@ -135,6 +138,8 @@ cudaError_t launch_reset_state(const Dims &dm, const DecState &st, int batch, co
 cudaError_t launch_admit_row(const Dims &dm, const DecState &st, int row, int ctx_len, const int32_t *forced_len_dev, cudaStream_t s);
 cudaError_t launch_embed(const Dims &dm, const DecState &st, int batch, int dtype, const void *embed, float *x, const void *gain,
                          void *h, cudaStream_t s);
+cudaError_t launch_embed_packed(const Dims &dm, const DecState &st, int batch, const void *embed, float *x, const void *gain, void *xg,
+                                float *ssq, int ssq_stride, int4 *row_meta_packed, int32_t *row_at, cudaStream_t s);
 cudaError_t launch_rmsnorm(const Dims &dm, int rows, int dtype, const float *x, const void *gain, void *out,
                            cudaStream_t s);
 cudaError_t launch_rmsnorm_packed(const Dims &dm, const DecState &st, int batch, int dtype, const float *x, const void *gain,
@@ -185,6 +190,8 @@ struct VocabArgs {
   int32_t *part_idx;         // [tiles][rows_cap] the id that holds it (lowest on ties; INT_MAX = none)
   float *term_val;           // [rows_cap][2] logits of eos and sep
   float *logits;             // [rows][V] fp32, or null when nobody reads them
+  // scale of the RMSNorm in front of the projection, rsqrt(sum_p ssq[m][p] * inv_width + eps) (null: none)
+  const float *ssq; int parts, ssq_stride; float inv_width, eps;
   int32_t *status;           // error word (PD_ERR_TIMEOUT on an expired wait)
 };
 struct VocabMaps { CUtensorMap a, a32, b; };   // hidden rows (128-row and 32-row boxes), lm_head (one slice per box)
@@ -195,6 +202,33 @@ cudaError_t vocab_tc_prepare();          // once per device, outside any stream 
 cudaError_t encode_vocab_maps(VocabMaps *m, const void *hidden, uint64_t rows, const void *lm_head, uint64_t vocab, uint64_t K,
                               int *driver_code);
 cudaError_t launch_vocab_tc(const VocabMaps &m, const VocabArgs &a, cudaStream_t s);
+
+// ---- the linear layers of a decode step over its packed active rows (proj_mma.cu) -----------------------
+enum { PROJ_STORE = 0,   // out = bf16(acc * row scale)
+       PROJ_RELU = 1,    // out = bf16(max(acc * row scale, 0))
+       PROJ_RESID = 2,   // x += acc; out = bf16(x * gain_next); partial sums of x^2 per row
+       PROJ_QKV = 3 };   // queries (rotated) to out, keys (rotated) and values to the cache
+struct ProjArgs {
+  const __nv_bfloat16 *act, *w;     // [rows][K] packed; [K][N]
+  int K, N;
+  const int32_t *n_active;   // [batch] active rows per sequence: their sum is the number of packed rows
+  int batch, rows_cap;       // rows the row-indexed buffers are allocated for
+  // scale of the RMSNorm in front of the layer: rsqrt(sum_p ssq_in[m][p] * inv_width + eps)
+  const float *ssq_in; int parts_in, ssq_stride; float inv_width, eps;
+  __nv_bfloat16 *out;        // [rows][N] (PROJ_QKV: the queries, [rows][N / 3])
+  float *x;                  // PROJ_RESID: fp32 residual stream [rows][N]
+  const __nv_bfloat16 *gain_next;   // PROJ_RESID: gain of the norm in front of the next layer
+  float *ssq_out;            // PROJ_RESID: [rows][ssq_stride], one part per column tile
+  // PROJ_QKV: where each packed row's entry goes (page, slot, position, subsequence), rotary table or null, the cache;
+  // raw: the unrotated product [rows][N] as well (fp32 or bf16), or null
+  const int4 *row_meta; const float2 *rope_tab;
+  __nv_bfloat16 *kv_pool; int layer, pool, P;
+  void *raw; int raw_f32;
+};
+bool proj_mma_supported(int K, int N, const void *w);
+int proj_mma_parts(int N);               // column tiles = parts of ssq_out
+cudaError_t proj_mma_prepare();          // once per device, outside any stream capture
+cudaError_t launch_proj_mma(int epi, const ProjArgs &a, cudaStream_t s);
 
 // ---- skinny-M linear layers on tcgen05 (linear_tc.cu) --------------------------------------------
 enum { LIN_EPI_STORE = 0,   // out = bf16(acc * row_scale)

@@ -369,13 +369,14 @@ __global__ void __launch_bounds__(PT) pick_sched_kernel(Dims dm, DecState st, in
   // first round of loads: the row's subsequence, the sequence's place among the packed rows, and the
   // sequence's state for the scheduler
   const int i = st.row_sub[r];
-  const int m = st.crow[b] + r % dm.C;                 // the row's place among the packed rows (meaningful when i > 0)
   const SeqStage stage = seq_stage_views(dm, sched_smem);
-  const SeqScalars sc = stage_in(dm, st, b, teacher, stage);
+  const SeqScalars sc = stage_in(dm, st, b, teacher, stage);      // ahead of the dependency wait: only schedulers write this state
+  const int sidx0 = i > 0 ? b * dm.SM + i - 1 : 0;
+  const int fl = st.forced_len[sidx0], len = st.len[sidx0];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int m = __ldcg(st.crow + b) + r % dm.C;        // the row's place among the packed rows (meaningful when i > 0)
   if (i > 0) {
-    const int sidx = b * dm.SM + i - 1;
-    // second round: the forced-length rule's inputs and the row's candidates
-    const int fl = st.forced_len[sidx], len = st.len[sidx];
+    // second round: the row's candidates
     float bv = -INFINITY;
     int bi = INT_MAX;
     for (int t = tid; t < tiles; t += PT) better(bv, bi, __ldcg(part_val + (size_t)t * rows_cap + m), __ldcg(part_idx + (size_t)t * rows_cap + m));
@@ -401,8 +402,17 @@ __global__ void __launch_bounds__(PT) pick_sched_kernel(Dims dm, DecState st, in
 
 cudaError_t launch_pick_sched(const Dims &dm, const DecState &st, int batch, int tiles, const float *part_val,
                               const int32_t *part_idx, const float *term_val, const int32_t *teacher, cudaStream_t s) {
-  pick_sched_kernel<<<batch * dm.C, PT, seq_stage_bytes(dm), s>>>(dm, st, batch, tiles, batch * dm.C, part_val, part_idx, term_val, teacher);
-  return cudaGetLastError();
+  // a programmatic dependent of the vocabulary projection: the sequences' state is staged while that kernel still runs
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(batch * dm.C, 1, 1);
+  cfg.blockDim = dim3(PT, 1, 1);
+  cfg.dynamicSmemBytes = seq_stage_bytes(dm);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, pick_sched_kernel, dm, st, batch, tiles, batch * dm.C, part_val, part_idx, term_val, teacher);
 }
 
 }  // namespace pd

@@ -28,6 +28,11 @@
 // known.  After the CTA's barrier they are cache entries like any other.  Queries come from the same
 // projection output (rotated likewise).  Split CTAs of one (sequence, head) write the same bits.
 //
+// Packed form (MODE 3): the launch is a programmatic dependent of the self-attention projection (proj_mma.cu), which rotates
+// queries and keys and appends the step's entries itself.  Everything but the queries and those new entries is older, so the
+// page list, the key list and the first tiles of old keys are read ahead of the dependency wait, while the projection is
+// still running; the new entries, one per active row, come last in the key list, in tiles of their own.
+//
 // Splits: the number of splits in use follows the key list's length (a CTA whose split is not needed
 // leaves at once).  Warps merge through shared memory; split CTAs leave a partial record, take a
 // ticket, and the last one to arrive merges the records in split order (deterministic) and writes
@@ -54,6 +59,7 @@ __device__ __forceinline__ uint32_t s_smem_u32(const void *p) { return (uint32_t
 __device__ __forceinline__ void s_cp_async16(uint32_t dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
+__device__ __forceinline__ void s_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void s_cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void s_cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void s_st_shared_u32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
@@ -93,7 +99,7 @@ __host__ __device__ constexpr int self_attn_tc_ring_bytes(int mt) {
 
 // MT = 16-row query tiles (rows per sequence <= 16 * MT); P = page_tokens; MODE 0 = the launch follows the append
 // kernel (queries in a.q); 1 = it appends the step's keys/values itself from the projection's bf16 output a.qkv;
-// 2 = the same from an fp32 output that it rotates by the rows' positions first (rotary mode)
+// 2 = the same from an fp32 output that it rotates by the rows' positions first (rotary mode); 3 = the packed form
 // OCC = CTAs per SM the register budget is set for: four leave the compiler 128 registers (nothing spills),
 // five 96 (more CTAs resident, which wins when there are more (sequence, head) pairs than four per SM)
 template <int MT, int P, int MODE, int OCC>
@@ -103,24 +109,88 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
   // this head's bias row
   extern __shared__ __align__(128) uint8_t s_ring_raw[];
   __shared__ int rsub_s[16 * MT];          // subsequence of row r
+  __shared__ int4 meta_s[16 * MT];         // MODE 3: (page, slot, position, subsequence) of the entry row r appends at this step
+  __shared__ int before_s[SW];
   __shared__ int last_s, n_keys_s;
 
   const Dims &dm = a.dm;
   const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int row0 = b * dm.C;
+  int row0 = b * dm.C;
   __nv_bfloat16 *out = (__nv_bfloat16 *)a.out;
   const int g = lane >> 2, tig = lane & 3;
   const int list_cap = dm.SM * dm.PPS;
   int4 *plist_s = reinterpret_cast<int4 *>(s_ring_raw + self_attn_tc_ring_bytes(MT));
   int *off_s = reinterpret_cast<int *>(plist_s + list_cap);                  // [list_cap + 1]
-  int2 *key_s = reinterpret_cast<int2 *>(off_s + ((list_cap + 1 + 1) & ~1));   // [list_cap * P]: (page * 32 + slot, subsequence | (distance base + 1024) << 8)
-  float *bias_s = reinterpret_cast<float *>(key_s + (size_t)list_cap * P);
+  int2 *key_s = reinterpret_cast<int2 *>(off_s + ((list_cap + 1 + 1) & ~1));   // [list_cap * P + STK]: (page * 32 + slot, subsequence | (distance base + 1024) << 8)
+  float *bias_s = reinterpret_cast<float *>(key_s + (size_t)list_cap * P + STK);
 
+  const __nv_bfloat16 *pool_lh = (const __nv_bfloat16 *)a.kv + kv_block_offset(a.layer, dm.pool, 0, dm.H, h, P);
+  const size_t page_stride = (size_t)dm.H * 2 * P * kDh;      // elements from one page's block of this head to the next page's
+  const bool use_bias = a.bias_tab != nullptr;
+  uint32_t qf[MT][4][4];
+  int S, n_keys, n_old;                    // active rows; keys of the list; keys ahead of the new entries' own tiles (all, but in MODE 3)
+  if constexpr (MODE == 3) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // ---- ahead of the dependency wait: what the previous step's scheduler left
+  S = a.st.n_active[b];
+  const int n_list = a.st.plist_n[b];
+  if (S == 0) { s_dependency_wait(); return; }
+  const int4 *pl = a.st.plist + (size_t)b * list_cap;
+  for (int j = tid; j < n_list; j += STHREADS) plist_s[j] = pl[j];
+  if (tid < 16 * MT) {
+    meta_s[tid] = a.st.row_meta[b * dm.C + min(tid, S - 1)];
+    rsub_s[tid] = meta_s[tid].w;
+  }
+  if (use_bias)
+    for (int dd = tid; dd < dm.n_dist; dd += STHREADS) bias_s[dd] = a.bias_tab[h * dm.n_dist + dd];
+  int before = 0;                          // packed rows of the sequences before this one
+  for (int bb = tid; bb < b; bb += STHREADS) before += a.st.n_active[bb];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(0xffffffffu, before, o);
+  if (lane == 0) before_s[warp] = before;
+  __syncthreads();
+  row0 = 0;
+#pragma unroll
+  for (int w = 0; w < SW; ++w) row0 += before_s[w];
+  // the key list: every page's entries but the one this step appends, then those, from the next tile boundary on
+  for (int j = tid; j < n_list; j += STHREADS) {
+    const int4 e = plist_s[j];
+    int fresh = 0;
+    for (int r = 0; r < S; ++r) fresh |= (meta_s[r].x == e.x && meta_s[r].y == e.y - 1) ? 1 : 0;
+    plist_s[j].y = e.y - fresh;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int carry = 0;
+    for (int j0 = 0; j0 < n_list; j0 += 32) {
+      const int nv = j0 + lane < n_list ? plist_s[j0 + lane].y : 0;
+      int incl = nv;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) { const int u = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += u; }
+      if (j0 + lane < n_list) off_s[j0 + lane] = carry + incl - nv;
+      carry += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) n_keys_s = carry;
+  }
+  __syncthreads();
+  n_old = n_keys_s;
+  const int new0 = (n_old + STK - 1) / STK * STK;
+  n_keys = new0 + S;
+  for (int j = tid; j < n_list; j += STHREADS) {
+    const int4 e = plist_s[j];
+    const int o0 = off_s[j];
+    for (int k = 0; k < e.y; ++k)      // entry k of the page: its distance base is the page's minus its offset
+      key_s[o0 + k] = make_int2(e.x * 32 + k, e.z | ((e.w - k + 1024) << 8));
+  }
+  // a new entry sits at its row's own query position, so its distance base is minus its subsequence
+  if (tid < S) key_s[new0 + tid] = make_int2(meta_s[tid].x * 32 + meta_s[tid].y, meta_s[tid].w | ((1024 - meta_s[tid].w) << 8));
+  __syncthreads();
+  } else {
   // ---- ONE round of independent global loads, none waiting for another: active-row count, page list, row ->
   // subsequence, where every row's new entry goes, bias row of this head, query fragments, and (fused modes) the
   // new keys/values of the rows this warp appends.  What turns out to be unused is masked afterwards.
-  const int S = a.st.n_active[b];
+  S = a.st.n_active[b];
   const int n_list = a.st.plist_n[b];
   const int4 *pl = a.st.plist + (size_t)b * list_cap;
   int4 my_entry[(SMAXLIST + STHREADS - 1) / STHREADS];
@@ -131,14 +201,12 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
   if (tid < dm.C) my_rsub = a.st.row_sub[row0 + tid];
   // (page, slot, position tau + i, subsequence) of the entry row `lane` of this sequence appends at this step
   const int4 meta = (MODE != 0 && lane < dm.C) ? a.st.row_meta[row0 + lane] : make_int4(-1, 0, 0, 0);
-  const bool use_bias = a.bias_tab != nullptr;
   float my_bias[SBIAS_PER_THREAD];
 #pragma unroll
   for (int k = 0; k < SBIAS_PER_THREAD; ++k) {
     const int dd = k * STHREADS + tid;
     my_bias[k] = (use_bias && dd < dm.n_dist) ? a.bias_tab[h * dm.n_dist + dd] : 0.f;
   }
-  uint32_t qf[MT][4][4];
   if (MODE != 2) {
     const __nv_bfloat16 *qsrc = MODE == 1 ? (const __nv_bfloat16 *)a.qkv : (const __nv_bfloat16 *)a.q;
     const size_t qstride = MODE == 1 ? 3 * (size_t)dm.d : (size_t)dm.d;
@@ -190,8 +258,6 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
         out[(size_t)(row0 + idx / kDh) * dm.d + h * kDh + idx % kDh] = __float2bfloat16_rn(0.f);
     return;
   }
-  const __nv_bfloat16 *pool_lh = (const __nv_bfloat16 *)a.kv + kv_block_offset(a.layer, dm.pool, 0, dm.H, h, P);
-  const size_t page_stride = (size_t)dm.H * 2 * P * kDh;      // elements from one page's block of this head to the next page's
 
   // ---- append (every CTA of the (sequence, head) pair writes the same bits) and, in rotary mode, the queries
   if (MODE == 2) {
@@ -270,12 +336,18 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
       key_s[o0 + k] = make_int2(e.x * 32 + k, e.z | ((e.w - k + 1024) << 8));
   }
   __syncthreads();
-  const int n_keys = n_keys_s;
+  n_keys = n_old = n_keys_s;
+  }
 
   // splits in use: enough that a warp gets about STILES_PER_WARP tiles, at most the launched ones
   const int n_tiles = (n_keys + STK - 1) / STK;
   const int n_eff = min(a.splits, max(1, (n_tiles + SW * STILES_PER_WARP - 1) / (SW * STILES_PER_WARP)));
-  if (split >= n_eff) return;
+  if (split >= n_eff) {
+    if (MODE == 3) s_dependency_wait();
+    return;
+  }
+  // keys that exist of the tile that starts at key `first`
+  auto keys_of = [&](int first) { return min(STK, (MODE == 3 && first < n_old ? n_old : n_keys) - first); };
   const int W = n_eff * SW, g0 = split * SW + warp;
   const int n_mine = n_tiles > g0 ? (n_tiles - g0 + W - 1) / W : 0;
   const uint32_t my_ring = s_smem_u32(s_ring_raw) + warp * SDEPTH * SSLOT;
@@ -284,12 +356,12 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
   // each: round k covers keys 2 k and 2 k + 1, chunks 0-7 = the key row, 8-15 = the value row.  A cache row's chunk c
   // lies at place c ^ (slot & 7) of its row; in the tile it goes to place c ^ (row in tile & 7).
   auto fetch = [&](int n) {
-    const int first = STK * (g0 + n * W);
+    const int first = STK * (g0 + n * W), nv = keys_of(first);
     const uint32_t dst = my_ring + (n % SDEPTH) * SSLOT;
 #pragma unroll
     for (int k = 0; k < STK / 2; ++k) {
       const int r = 2 * k + (lane >> 4), p = lane & 15;
-      if (first + r < n_keys) {
+      if (r < nv) {
         const int src = key_s[first + r].x;
         const int page = src >> 5, slot = src & 31;
         const uint8_t *from = reinterpret_cast<const uint8_t *>(pool_lh + page * page_stride) + slot * 256 + p * 16;
@@ -300,10 +372,33 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
   };
   // Nothing is ever cleared: what a slot holds beyond the list's last key (anything) gets score -inf, and the value
   // fragments of those keys are zeroed in registers after ldmatrix.
+  int n_ahead = 0;                   // MODE 3: this warp's first tiles, as far as they hold old keys, go ahead of the wait
+  if (MODE == 3) {
 #pragma unroll
-  for (int n = 0; n < SDEPTH; ++n) {
-    if (n < n_mine) fetch(n);
-    s_cp_async_commit();
+    for (int n = 0; n < SDEPTH; ++n)
+      if (n < n_mine && STK * (g0 + n * W) < n_old) { fetch(n); s_cp_async_commit(); n_ahead = n + 1; }
+    s_dependency_wait();
+  }
+#pragma unroll
+  for (int n = 0; n < SDEPTH; ++n)
+    if (MODE != 3 || n >= n_ahead) {
+      if (n < n_mine) fetch(n);
+      s_cp_async_commit();
+    }
+  if (MODE == 3) {
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) {
+      const int r_lo = mt * 16 + g, r_hi = r_lo + 8;
+      const __nv_bfloat16 *q_lo = (const __nv_bfloat16 *)a.q + (size_t)(row0 + r_lo) * dm.d + h * kDh + 2 * tig;
+      const __nv_bfloat16 *q_hi = (const __nv_bfloat16 *)a.q + (size_t)(row0 + r_hi) * dm.d + h * kDh + 2 * tig;
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        qf[mt][kk][0] = r_lo < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_lo + kk * 16)) : 0u;
+        qf[mt][kk][1] = r_hi < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_hi + kk * 16)) : 0u;
+        qf[mt][kk][2] = r_lo < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8)) : 0u;
+        qf[mt][kk][3] = r_hi < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8)) : 0u;
+      }
+    }
   }
 
   int rs[MT][2];                     // subsequence of rows g and g + 8 of every query tile
@@ -330,7 +425,7 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
     s_cp_async_wait<SDEPTH - 1>();     // everything but the newest group has landed: tile n is in its slot
     __syncwarp();
     const int first = STK * (g0 + n * W);
-    const int nv = min(STK, n_keys - first);           // keys of this tile that exist
+    const int nv = keys_of(first);                     // keys of this tile that exist
     // this thread's four keys of the tile (two per 8-key score tile): subsequence and distance base
     int ksub[2][2], kd[2][2];
 #pragma unroll
@@ -501,7 +596,7 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
     ml[ROWS + r] = M;              // ... and warp 1's the merged maxima
   }
   __syncthreads();
-  for (int idx = tid; idx < dm.C * (kDh / 2); idx += STHREADS) {          // two columns per thread
+  for (int idx = tid; idx < (MODE == 3 ? S : dm.C) * (kDh / 2); idx += STHREADS) {      // two columns per thread (packed: no unused rows)
     const int r = idx / (kDh / 2), col = 2 * (idx % (kDh / 2));
     const size_t orow = (size_t)(row0 + r) * dm.d + h * kDh + col;
     if (r >= S) {
@@ -559,7 +654,7 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
 
 static int self_attn_tc_smem(const Dims &dm) {
   const int mt = (dm.C + 15) / 16, list_cap = dm.SM * dm.PPS;
-  return self_attn_tc_ring_bytes(mt) + list_cap * (int)sizeof(int4) + ((list_cap + 2) & ~1) * 4 + list_cap * dm.P * (int)sizeof(int2) +
+  return self_attn_tc_ring_bytes(mt) + list_cap * (int)sizeof(int4) + ((list_cap + 2) & ~1) * 4 + (list_cap * dm.P + STK) * (int)sizeof(int2) +
          (dm.pos_mode == PD_POS_T5_BIAS ? dm.n_dist * 4 : 0);
 }
 
@@ -592,6 +687,8 @@ static cudaError_t prepare_one() {
   if (e == cudaSuccess) e = cudaFuncSetAttribute(self_attn_tc_kernel<MT, P, 0, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(self_attn_tc_kernel<MT, P, 1, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(self_attn_tc_kernel<MT, P, 2, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(self_attn_tc_kernel<MT, P, 3, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(self_attn_tc_kernel<MT, P, 3, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   return e;
 }
 
@@ -603,6 +700,7 @@ cudaError_t self_attn_tc_prepare() {
   return e;
 }
 
+// a.packed: a.q = the queries of the packed rows, the step's new keys/values are in the cache.  Else
 // a.fused_append 1: a.qkv = the projection's output [rows][3 d] in bf16; 2: in fp32, rotated here with a.rope_tab;
 // 0: a.q = the queries the append kernel left.  a.tickets one zeroed int32 per (sequence, head) (the kernel leaves them zeroed), a.part_o /
 // a.part_ml sized for a.splits records per (row, head).
@@ -613,8 +711,19 @@ cudaError_t launch_self_attn_tc(const AttnArgs &a, cudaStream_t s) {
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const bool roomy = (long long)a.splits * a.dm.H * a.batch <= 4LL * sms;      // all CTAs resident at four per SM
+  cudaLaunchConfig_t cfg = {};             // packed form: a programmatic dependent of the projection
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(STHREADS, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr; cfg.numAttrs = 1;
 #define PD_SELF_LAUNCH(MT_, P_)                                                                            \
   do {                                                                                                   \
+    if (a.packed && roomy) return cudaLaunchKernelEx(&cfg, self_attn_tc_kernel<MT_, P_, 3, 4>, a);             \
+    if (a.packed) return cudaLaunchKernelEx(&cfg, self_attn_tc_kernel<MT_, P_, 3, 5>, a);                      \
     if (a.fused_append == 1 && roomy) self_attn_tc_kernel<MT_, P_, 1, 4><<<grid, STHREADS, smem, s>>>(a);        \
     else if (a.fused_append == 1) self_attn_tc_kernel<MT_, P_, 1, 5><<<grid, STHREADS, smem, s>>>(a);            \
     else if (a.fused_append == 2 && roomy) self_attn_tc_kernel<MT_, P_, 2, 4><<<grid, STHREADS, smem, s>>>(a);   \

@@ -82,6 +82,7 @@ pd_status pd_vocab_argmax(int32_t rows, int32_t d_model, int32_t vocab, const vo
   a.part_idx = reinterpret_cast<int32_t *>(base + L.off_part_idx);
   a.term_val = reinterpret_cast<float *>(base + L.off_term);
   a.logits = logits;
+  a.ssq = nullptr; a.parts = 0; a.ssq_stride = 0; a.inv_width = 0.f; a.eps = 0.f;
   a.status = reinterpret_cast<int32_t *>(base) + HDR_STATUS;
   if (launch_vocab_tc(maps, a, s) != cudaSuccess) return PD_ERR_CUDA;
   const int warps = 8;

@@ -136,6 +136,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   extern __shared__ uint8_t v_smem_raw[];
   __shared__ uint32_t tmem_base_s;
   __shared__ int red_s[VT_THREADS / 32];
+  __shared__ float inv_s[2 * VT_M];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int vt = blockIdx.x;
 
@@ -181,6 +182,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   __syncthreads();
   v_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   bool ok = true;
   const uint32_t b_bytes = (uint32_t)(wn * VT_BK * 2);
   // bytes of the hidden-row tiles of pass p that travel: whole 128-row tiles, 32-row boxes of the ragged last one
@@ -261,6 +263,17 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const int v_tile0 = vt * wn;
     for (int p = 0; p < n_pass; ++p) {
       const int tiles = min(2, n_tt - 2 * p);
+      for (int j = 0; j < tiles; ++j) {                  // the rows' norm scales, while the product runs (each lane reads back its own)
+        const int m = (2 * p + j) * VT_M + quarter * 32 + lane;
+        float s0 = 0.f, s1 = 0.f;
+        if (a.ssq != nullptr && m < Mc) {
+          const float *q = a.ssq + (size_t)m * a.ssq_stride;
+          int pp = 0;
+          for (; pp + 1 < a.parts; pp += 2) { s0 += __ldcg(q + pp); s1 += __ldcg(q + pp + 1); }
+          if (pp < a.parts) s0 += __ldcg(q + pp);
+        }
+        inv_s[j * VT_M + quarter * 32 + lane] = a.ssq != nullptr ? rsqrtf((s0 + s1) * a.inv_width + a.eps) : 1.f;
+      }
       if (ok && !v_mbar_wait(bar_acc_full, (uint32_t)p & 1u)) ok = false;
       if (!ok) break;
       v_fence_after();
@@ -268,6 +281,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         const int m = (2 * p + j) * VT_M + quarter * 32 + lane;
         float bv = -INFINITY, te = -INFINITY, ts = -INFINITY;
         int bi = INT_MAX;
+        const float inv = inv_s[j * VT_M + quarter * 32 + lane];
 #pragma unroll 1
         for (int c = 0; c * 32 < wn; ++c) {              // 32 columns at a time; a slice of an odd number of 16s ends with 16
           uint32_t r[32];
@@ -284,13 +298,13 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           if (!special) {
 #pragma unroll
             for (int i = 0; i < 32; ++i) {               // ascending ids and a strict compare: ties keep the lowest id
-              const float x = __uint_as_float(r[i]);
+              const float x = __uint_as_float(r[i]) * inv;
               if (x > bv) { bv = x; bi = v0 + i; }
             }
           } else {
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
-              const float x = __uint_as_float(r[i]);
+              const float x = __uint_as_float(r[i]) * inv;
               const int v = v0 + i;
               if (v >= a.V || i >= ncol) continue;
               if (v == a.eos) te = x;
@@ -302,7 +316,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             float *row = a.logits + (size_t)m * a.V + v0;
 #pragma unroll
             for (int i = 0; i < 32; ++i)
-              if (v0 + i < a.V && i < ncol) row[i] = __uint_as_float(r[i]);
+              if (v0 + i < a.V && i < ncol) row[i] = __uint_as_float(r[i]) * inv;
           }
         }
         if (m < Mc) {
@@ -365,8 +379,8 @@ cudaError_t vocab_tc_prepare() {
   return cudaFuncSetAttribute(vocab_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, VT_SMEM);
 }
 
-// Launched as a programmatic dependent of the kernel before it in the stream (the packed final norm, which lets its
-// dependents start early): set-up and the first lm_head blocks overlap that kernel's tail.
+// Launched as a programmatic dependent of the kernel before it in the stream (the packed final norm or the last
+// feed-forward product, which let their dependents start early): set-up and the first lm_head blocks overlap that kernel's tail.
 cudaError_t launch_vocab_tc(const VocabMaps &m, const VocabArgs &a_in, cudaStream_t s) {
   VocabArgs a = a_in;
   a.wn = vocab_tc_slice(a.V);
