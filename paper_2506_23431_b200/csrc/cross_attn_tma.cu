@@ -619,24 +619,9 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
 // keys or values of one tile, 16 KB contiguous), 128-byte swizzle.  *driver_code gets the CUresult
 // when the encode itself fails.
 cudaError_t encode_ctx_kv_tensor_map(CUtensorMap *out, const void *base, uint64_t rows, int *driver_code) {
-  typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                               const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  if (driver_code) *driver_code = 0;
-  void *fn = nullptr;
-  cudaDriverEntryPointQueryResult qres;
-  cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
-  if (e != cudaSuccess) return e;
-  if (fn == nullptr || qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
-  cuuint64_t gdim[2] = {(cuuint64_t)kDh, (cuuint64_t)rows};
-  cuuint64_t gstride[1] = {(cuuint64_t)kDh * 2};
-  cuuint32_t box[2] = {(cuuint32_t)kDh, (cuuint32_t)XK};
-  cuuint32_t estr[2] = {1u, 1u};
-  CUresult r = ((EncodeFn)fn)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), gdim, gstride, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) { if (driver_code) *driver_code = (int)r; return cudaErrorInvalidValue; }
-  return cudaSuccess;
+  const uint64_t gdim[2] = {kDh, rows}, gstride[1] = {kDh * 2};
+  const uint32_t box[2] = {kDh, XK};
+  return encode_tensor_map(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, gdim, gstride, box, driver_code);
 }
 
 int cross_attn_ctas() {
@@ -652,44 +637,21 @@ int cross_attn_ctas() {
 // 128 keys x 64 dims.  Both with the 128-byte swizzle; reads beyond max_ctx are filled with zeros.
 cudaError_t encode_ctx_kv8_tensor_maps(CUtensorMap *map_k, CUtensorMap *map_v, const void *base, uint64_t n_blocks, uint64_t ctx,
                                        int *driver_code) {
-  typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                               const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  if (driver_code) *driver_code = 0;
-  void *fn = nullptr;
-  cudaDriverEntryPointQueryResult qres;
-  cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
+  const uint64_t kdim[2] = {128, n_blocks * 2 * ctx * kDh / 128}, kstride[1] = {128};
+  const uint32_t kbox[2] = {128, XK / 2};
+  cudaError_t e = encode_tensor_map(map_k, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, base, kdim, kstride, kbox, driver_code);
   if (e != cudaSuccess) return e;
-  if (fn == nullptr || qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
-  {
-    cuuint64_t gdim[2] = {128, (cuuint64_t)(n_blocks * 2 * ctx * kDh / 128)};
-    cuuint64_t gstride[1] = {128};
-    cuuint32_t box[2] = {128, (cuuint32_t)(XK / 2)};
-    cuuint32_t estr[2] = {1u, 1u};
-    CUresult r = ((EncodeFn)fn)(map_k, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void *>(base), gdim, gstride, box, estr,
-                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) { if (driver_code) *driver_code = (int)r; return cudaErrorInvalidValue; }
-  }
-  {
-    cuuint64_t gdim[3] = {(cuuint64_t)ctx, (cuuint64_t)kDh, (cuuint64_t)(n_blocks * 2)};
-    cuuint64_t gstride[2] = {(cuuint64_t)ctx, (cuuint64_t)ctx * kDh};
-    cuuint32_t box[3] = {(cuuint32_t)XK, (cuuint32_t)kDh, 1u};
-    cuuint32_t estr[3] = {1u, 1u, 1u};
-    CUresult r = ((EncodeFn)fn)(map_v, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<void *>(base), gdim, gstride, box, estr,
-                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) { if (driver_code) *driver_code = (int)r; return cudaErrorInvalidValue; }
-  }
-  return cudaSuccess;
+  const uint64_t vdim[3] = {ctx, kDh, n_blocks * 2}, vstride[2] = {ctx, ctx * kDh};
+  const uint32_t vbox[3] = {XK, kDh, 1u};
+  return encode_tensor_map(map_v, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, base, vdim, vstride, vbox, driver_code);
 }
 
-cudaError_t cross_attn_tma_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(cross_attn_tma_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, xsmem(false));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(cross_attn_tma_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, xsmem(false));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(cross_attn_tma_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, xsmem(true));
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(cross_attn_tma_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, xsmem(true));
-  return e;
+// rows_per_seq, fp8: the variant to prepare
+cudaError_t cross_attn_tma_prepare(int rows_per_seq, bool fp8) {
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if (rows_per_seq <= 16)
+    return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<1, true>, attr, xsmem(true)) : cudaFuncSetAttribute(cross_attn_tma_kernel<1, false>, attr, xsmem(false));
+  return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<2, true>, attr, xsmem(true)) : cudaFuncSetAttribute(cross_attn_tma_kernel<2, false>, attr, xsmem(false));
 }
 
 // n_ctas persistent CTAs (two per SM); a.part_o holds cross_attn_tma_partial_bytes(n_ctas, C),

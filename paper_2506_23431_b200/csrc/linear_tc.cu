@@ -408,24 +408,9 @@ linear_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
 // Tensor map of a row-major bf16 matrix [rows, cols] (cols a multiple of 64): boxes of box_rows rows x
 // 64 columns, 128-byte swizzle, rows beyond the matrix read as zeros.
 cudaError_t encode_linear_map(CUtensorMap *out, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows, int *driver_code) {
-  typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                               const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  if (driver_code) *driver_code = 0;
-  void *fn = nullptr;
-  cudaDriverEntryPointQueryResult qres;
-  cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
-  if (e != cudaSuccess) return e;
-  if (fn == nullptr || qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
-  cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t gstride[1] = {(cuuint64_t)cols * 2};
-  cuuint32_t box[2] = {(cuuint32_t)LT_BK, box_rows};
-  cuuint32_t estr[2] = {1u, 1u};
-  CUresult r = ((EncodeFn)fn)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), gdim, gstride, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) { if (driver_code) *driver_code = (int)r; return cudaErrorInvalidValue; }
-  return cudaSuccess;
+  const uint64_t gdim[2] = {cols, rows}, gstride[1] = {cols * 2};
+  const uint32_t box[2] = {LT_BK, box_rows};
+  return encode_tensor_map(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, gdim, gstride, box, driver_code);
 }
 // activations: one map with 128-row boxes (full row tiles), one with 32-row boxes (the ragged last tile)
 cudaError_t encode_linear_act_maps(LinearActMaps *out, const void *act, uint64_t rows, uint64_t K, int *driver_code) {

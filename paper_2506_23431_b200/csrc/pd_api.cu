@@ -18,6 +18,7 @@ namespace {
 
 constexpr size_t kAlign = 256;
 constexpr size_t kCublasWs = 64u << 20;
+constexpr int kTfGroup = 32;          // teacher-forced forward: query rows per attention group
 
 struct Region { size_t off = 0, bytes = 0; };
 
@@ -657,7 +658,7 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
   if (cfg->dtype == PD_DTYPE_BF16 && dm.C <= 32) {
     pd_status s = make_tensor_map(h);
     if (s != PD_OK) return bail(s);
-    if (cross_attn_tma_prepare() != cudaSuccess) return bail(PD_ERR_CUDA);
+    if (cross_attn_tma_prepare(dm.C, h->kv8) != cudaSuccess || cross_attn_tma_prepare(kTfGroup, h->kv8) != cudaSuccess) return bail(PD_ERR_CUDA);   // decode, teacher-forced groups
     h->cross_ctas = cross_attn_ctas();
   }
   if (cfg->dtype == PD_DTYPE_BF16 && self_attn_tc_supported(dm) && self_attn_tc_prepare() != cudaSuccess) return bail(PD_ERR_CUDA);
@@ -666,7 +667,7 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
     if (encode_vocab_maps(&h->vmaps, h->ptr<void>(L.hbuf), (uint64_t)dm.B * dm.C, weights->lm_head, (uint64_t)dm.V,
                           (uint64_t)dm.d, &code) != cudaSuccess)
       return bail(PD_ERR_CUDA);
-    if (vocab_tc_prepare() != cudaSuccess) return bail(PD_ERR_CUDA);
+    if (vocab_tc_prepare(1) != cudaSuccess || vocab_tc_prepare(dm.B * dm.C) != cudaSuccess) return bail(PD_ERR_CUDA);   // (a smaller batch may take the other variant)
     h->vocab_tc = true;
   }
   if (h->vocab_tc && h->have_tmap && self_attn_tc_supported(dm)) {
@@ -930,7 +931,6 @@ pd_status pd_collect_row(pd_handle *h, int32_t row, int32_t *tokens, int32_t *le
 
 // ---- the teacher-forced forward of Eq. 6 -----------------------------------------------------------------
 namespace {
-constexpr int kTfGroup = 32;          // query rows per attention group
 constexpr int kTfCrossBatch = 256;    // groups per cross-attention launch
 struct TfLayout { size_t tables, x, hb, qkv, att, cq, co, ffn, logprob, part, tickets, logits, total; int logit_rows; };
 

@@ -132,6 +132,9 @@ cudaError_t launch_dense_self_attn(const DenseAttnArgs &a, cudaStream_t s);
 cudaError_t launch_gather_rows(int rows, int d, const int32_t *row_tok, const void *embed, float *x, cudaStream_t s);
 cudaError_t launch_target_logprob(int rows, int V, const float *logits, const int32_t *targets, float *logprob, cudaStream_t s);
 
+cudaError_t encode_tensor_map(CUtensorMap *out, CUtensorMapDataType type, int rank, const void *base, const uint64_t *gdim,
+                              const uint64_t *gstride, const uint32_t *box, int *driver_code);      // tensor_map.cu
+
 // ---- launchers (each enqueues on `s`; returns cudaGetLastError()) ------------------------
 cudaError_t launch_reset_state(const Dims &dm, const DecState &st, int batch, const int32_t *ctx_len_dev,
                                const int32_t *forced_len_dev, size_t state_words, int32_t *state_base, cudaStream_t s);
@@ -174,7 +177,7 @@ cudaError_t launch_pick_sched(const Dims &dm, const DecState &st, int batch, int
                               const int32_t *part_idx, const float *term_val, const int32_t *teacher, cudaStream_t s);
 cudaError_t encode_ctx_kv_tensor_map(CUtensorMap *out, const void *base, uint64_t rows, int *driver_code);
 int cross_attn_tma_smem_bytes();
-cudaError_t cross_attn_tma_prepare();   // once per device, outside any stream capture
+cudaError_t cross_attn_tma_prepare(int rows_per_seq, bool fp8);   // once per device, outside any stream capture
 
 
 // ---- vocabulary projection + per-slice maxima on tcgen05 (vocab_tc.cu) -------------------------
@@ -198,7 +201,7 @@ struct VocabMaps { CUtensorMap a, a32, b; };   // hidden rows (128-row and 32-ro
 int vocab_tc_slice(int V);
 int vocab_tc_tiles(int V);
 bool vocab_tc_supported(int K, int V);
-cudaError_t vocab_tc_prepare();          // once per device, outside any stream capture
+cudaError_t vocab_tc_prepare(int rows_cap);   // the variant for this many rows: once per device, outside any stream capture
 cudaError_t encode_vocab_maps(VocabMaps *m, const void *hidden, uint64_t rows, const void *lm_head, uint64_t vocab, uint64_t K,
                               int *driver_code);
 cudaError_t launch_vocab_tc(const VocabMaps &m, const VocabArgs &a, cudaStream_t s);

@@ -6,11 +6,11 @@
 // One CTA per slice of the vocabulary; the slice width (a multiple of 16, at most 224) is chosen so that the
 // slices fill whole waves of 148 SMs (224 ids for 32128: 144 CTAs, one wave; 176 for 50265: 286 CTAs, two
 // balanced rounds instead of one and a half of 224).  Rows are the M dimension of
-// tcgen05.mma (128 per accumulator, two accumulators = up to 256 rows per pass over the CTA's slice
+// tcgen05.mma (128 per accumulator, one or two accumulators = up to 256 rows per pass over the CTA's slice
 // of lm_head; more rows take more passes, which re-read the slice from L2).  The number of rows is
 // read on the device (the sum of the sequences' active rows), so work follows the rows that exist,
 // not the allocated maximum.  Warp 0 streams 64-column blocks of hidden and lm_head into a
-// three-stage shared-memory ring with TMA (128-byte swizzle, mbarrier completion; of a ragged last row
+// shared-memory ring of two or three stages with TMA (128-byte swizzle, mbarrier completion; of a ragged last row
 // tile only the 32-row boxes that hold rows travel; the first lm_head blocks, which do not depend on the
 // kernel before, are requested ahead of the programmatic-dependency wait); one lane of
 // warp 1 issues tcgen05.mma (M 128, N 224, K 16, bf16 in, fp32 accumulators in tensor memory) and
@@ -28,15 +28,21 @@ constexpr int VT_N = 224;                       // most vocabulary ids per CTA (
 constexpr int VT_SMS = 148;                     // SMs the slice width is balanced for
 constexpr int VT_M = 128;                       // rows per accumulator
 constexpr int VT_BK = 64;                       // columns of K per stage (128 bytes: one swizzle span)
-constexpr int VT_STAGES = 3;
 constexpr int VT_THREADS = 192;                 // producer warp, MMA warp, four epilogue warps
 constexpr int VT_A_BYTES = VT_M * VT_BK * 2;    // 16 KB
 constexpr int VT_B_BYTES = VT_N * VT_BK * 2;    // 28 KB: room for the widest slice
 constexpr int VT_BOX_M = 32;                    // rows per box of a ragged row tile
 constexpr int VT_BOX_BYTES = VT_BOX_M * VT_BK * 2;
-constexpr int VT_STAGE_BYTES = 2 * VT_A_BYTES + VT_B_BYTES;
-constexpr int VT_SMEM = VT_STAGES * VT_STAGE_BYTES + 128 /*barriers*/ + 1024 /*alignment slack*/;
-constexpr int VT_TMEM_COLS = 512;               // two accumulators at columns 0 and 256
+constexpr int VT_LPITCH = 33;                   // floats per row of a warp's 32 x 32 block of logits on its way out
+constexpr int VT_LOGIT_BYTES = 4 * 32 * VT_LPITCH * 4;
+// TILES = row tiles (accumulators) per pass.  Up to 128 rows one is enough, and half the stage and half of tensor memory let two
+// CTAs share an SM: all slices of a vocabulary of 50265 are then resident at once, and one CTA's epilogue runs under the
+// other's copies.  100 rows x 50265 ids of width 768, logits stored, per launch: 23.6 us, against 34.4 us with the two-tile form
+// (one CTA per SM, two rounds).
+__host__ __device__ constexpr int vt_stages(int tiles) { return tiles == 1 ? 2 : 3; }
+__host__ __device__ constexpr int vt_stage_bytes(int tiles) { return tiles * VT_A_BYTES + VT_B_BYTES; }
+__host__ __device__ constexpr int vt_tmem_cols(int tiles) { return 256 * tiles; }      // accumulator j at column 256 j
+constexpr int vt_smem(int tiles) { return vt_stages(tiles) * vt_stage_bytes(tiles) + 128 /*barriers*/ + VT_LOGIT_BYTES + 1024 /*alignment slack*/; }
 constexpr uint32_t VT_SPIN_LIMIT = 1u << 24;
 // instruction descriptor of kind::f16: D fp32, A and B bf16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24
 __device__ __forceinline__ uint32_t v_idesc(int n) {
@@ -130,13 +136,15 @@ __device__ __forceinline__ void v_tmem_ld16(uint32_t taddr, uint32_t (&r)[32]) {
 __device__ __forceinline__ void v_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void v_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-__global__ void __launch_bounds__(VT_THREADS, 1)
+template <int TILES>
+__global__ void __launch_bounds__(VT_THREADS, TILES == 1 ? 2 : 1)
 vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_a32,
                 const __grid_constant__ CUtensorMap map_b, VocabArgs a) {
+  constexpr int VT_STAGES = vt_stages(TILES), VT_STAGE_BYTES = vt_stage_bytes(TILES), VT_TMEM_COLS = vt_tmem_cols(TILES);
   extern __shared__ uint8_t v_smem_raw[];
   __shared__ uint32_t tmem_base_s;
   __shared__ int red_s[VT_THREADS / 32];
-  __shared__ float inv_s[2 * VT_M];
+  __shared__ float inv_s[TILES * VT_M];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int vt = blockIdx.x;
 
@@ -160,7 +168,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     return;
   }
   const int n_tt = (Mc + VT_M - 1) / VT_M;               // 128-row tiles
-  const int n_pass = (n_tt + 1) / 2;                     // two tiles (accumulators) per pass
+  const int n_pass = (n_tt + TILES - 1) / TILES;
   const int nkb = a.K / VT_BK;
 
   const uint32_t base = (v_smem_u32(v_smem_raw) + 1023u) & ~1023u;
@@ -188,8 +196,8 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
   // bytes of the hidden-row tiles of pass p that travel: whole 128-row tiles, 32-row boxes of the ragged last one
   auto a_bytes = [&](int p) {
     uint32_t n = 0;
-    for (int j = 0; j < min(2, n_tt - 2 * p); ++j) {
-      const int rows_here = min(VT_M, Mc - (2 * p + j) * VT_M);
+    for (int j = 0; j < min(TILES, n_tt - TILES * p); ++j) {
+      const int rows_here = min(VT_M, Mc - (TILES * p + j) * VT_M);
       n += rows_here == VT_M ? (uint32_t)VT_A_BYTES : (uint32_t)((rows_here + VT_BOX_M - 1) / VT_BOX_M * VT_BOX_BYTES);
     }
     return n;
@@ -202,12 +210,12 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       const int ahead = min(VT_STAGES, nkb);
       for (int kb = 0; kb < ahead; ++kb) {
         v_mbar_expect_tx(bar_full + 8 * kb, b_bytes + a_bytes(0));
-        v_tma_load_2d(base + kb * VT_STAGE_BYTES + 2 * VT_A_BYTES, &map_b, bar_full + 8 * kb, kb * VT_BK, vt * wn);
+        v_tma_load_2d(base + kb * VT_STAGE_BYTES + TILES * VT_A_BYTES, &map_b, bar_full + 8 * kb, kb * VT_BK, vt * wn);
       }
       asm volatile("griddepcontrol.wait;" ::: "memory");
       int it = 0;
       for (int p = 0; p < n_pass && ok; ++p) {
-        const int tiles = min(2, n_tt - 2 * p);
+        const int tiles = min(TILES, n_tt - TILES * p);
         for (int kb = 0; kb < nkb; ++kb, ++it) {
           const int s = it % VT_STAGES;
           const uint32_t dst = base + s * VT_STAGE_BYTES;
@@ -215,10 +223,10 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             const uint32_t u = (uint32_t)(it / VT_STAGES);
             if (!v_mbar_wait(bar_empty + 8 * s, (u & 1u) ^ 1u)) { ok = false; break; }
             v_mbar_expect_tx(bar_full + 8 * s, b_bytes + a_bytes(p));
-            v_tma_load_2d(dst + 2 * VT_A_BYTES, &map_b, bar_full + 8 * s, kb * VT_BK, vt * wn);
+            v_tma_load_2d(dst + TILES * VT_A_BYTES, &map_b, bar_full + 8 * s, kb * VT_BK, vt * wn);
           }
           for (int j = 0; j < tiles; ++j) {
-            const int row0 = (2 * p + j) * VT_M, rows_here = min(VT_M, Mc - row0);
+            const int row0 = (TILES * p + j) * VT_M, rows_here = min(VT_M, Mc - row0);
             if (rows_here == VT_M) {
               v_tma_load_2d(dst + j * VT_A_BYTES, &map_a, bar_full + 8 * s, kb * VT_BK, row0);
             } else {
@@ -236,7 +244,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       int it = 0;
       const uint32_t idesc = v_idesc(wn);
       for (int p = 0; p < n_pass && ok; ++p) {
-        const int tiles = min(2, n_tt - 2 * p);
+        const int tiles = min(TILES, n_tt - TILES * p);
         // the epilogue must be done with the previous pass's accumulators
         if (!v_mbar_wait(bar_acc_empty, ((uint32_t)p & 1u) ^ 1u)) { ok = false; break; }
         v_fence_after();
@@ -245,7 +253,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
           const uint32_t u = (uint32_t)(it / VT_STAGES);
           if (!v_mbar_wait(bar_full + 8 * s, u & 1u)) { ok = false; break; }
           v_fence_after();
-          const uint32_t sa = base + s * VT_STAGE_BYTES, sb = sa + 2 * VT_A_BYTES;
+          const uint32_t sa = base + s * VT_STAGE_BYTES, sb = sa + TILES * VT_A_BYTES;
           for (int j = 0; j < tiles; ++j)
 #pragma unroll
             for (int k4 = 0; k4 < VT_BK / 16; ++k4)      // 16 columns of K = 32 bytes further inside the swizzle span
@@ -261,10 +269,11 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     asm volatile("griddepcontrol.wait;" ::: "memory");
     const int quarter = warp & 3;                        // tensor-memory lanes 32 * quarter .. + 31 belong to this warp
     const int v_tile0 = vt * wn;
+    float *lblk = reinterpret_cast<float *>(v_smem_raw + (base - v_smem_u32(v_smem_raw)) + VT_STAGES * VT_STAGE_BYTES + 128) + quarter * 32 * VT_LPITCH;
     for (int p = 0; p < n_pass; ++p) {
-      const int tiles = min(2, n_tt - 2 * p);
+      const int tiles = min(TILES, n_tt - TILES * p);
       for (int j = 0; j < tiles; ++j) {                  // the rows' norm scales, while the product runs (each lane reads back its own)
-        const int m = (2 * p + j) * VT_M + quarter * 32 + lane;
+        const int m = (TILES * p + j) * VT_M + quarter * 32 + lane;
         float s0 = 0.f, s1 = 0.f;
         if (a.ssq != nullptr && m < Mc) {
           const float *q = a.ssq + (size_t)m * a.ssq_stride;
@@ -278,7 +287,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       if (!ok) break;
       v_fence_after();
       for (int j = 0; j < tiles; ++j) {
-        const int m = (2 * p + j) * VT_M + quarter * 32 + lane;
+        const int m = (TILES * p + j) * VT_M + quarter * 32 + lane;
         float bv = -INFINITY, te = -INFINITY, ts = -INFINITY;
         int bi = INT_MAX;
         const float inv = inv_s[j * VT_M + quarter * 32 + lane];
@@ -312,11 +321,20 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
               else if (x > bv) { bv = x; bi = v; }
             }
           }
-          if (a.logits != nullptr && m < Mc) {
-            float *row = a.logits + (size_t)m * a.V + v0;
+          if (a.logits != nullptr) {
+            // a thread holds 32 columns of its row: turned in shared memory, so that a warp stores 32 columns of one row at a
+            // time (stored from the registers, every lane of a store touched another line: 48.8 us per launch at 100 rows
+            // x 50265 ids of width 768, against 34.4 us)
+            float *blk = lblk + lane * VT_LPITCH;
 #pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (v0 + i < a.V && i < ncol) row[i] = __uint_as_float(r[i]) * inv;
+            for (int i = 0; i < 32; ++i) blk[i] = __uint_as_float(r[i]) * inv;
+            __syncwarp();
+            const int m0 = (TILES * p + j) * VT_M + quarter * 32, mr = min(32, Mc - m0);
+            if (lane < ncol && v0 + lane < a.V) {
+              float *col = a.logits + (size_t)m0 * a.V + v0 + lane;
+              for (int i = 0; i < mr; ++i) __stcs(col + (size_t)i * a.V, lblk[i * VT_LPITCH + lane]);
+            }
+            __syncwarp();
           }
         }
         if (m < Mc) {
@@ -344,24 +362,9 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 // one swizzle span), 128-byte swizzle, out-of-range rows read as zeros.
 cudaError_t encode_rowmajor_bf16_map(CUtensorMap *out, const void *base, uint64_t rows, uint64_t cols, uint32_t box_rows,
                                      int *driver_code) {
-  typedef CUresult (*EncodeFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
-                               const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                               CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  if (driver_code) *driver_code = 0;
-  void *fn = nullptr;
-  cudaDriverEntryPointQueryResult qres;
-  cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
-  if (e != cudaSuccess) return e;
-  if (fn == nullptr || qres != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
-  cuuint64_t gdim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-  cuuint64_t gstride[1] = {(cuuint64_t)cols * 2};
-  cuuint32_t box[2] = {(cuuint32_t)VT_BK, box_rows};
-  cuuint32_t estr[2] = {1u, 1u};
-  CUresult r = ((EncodeFn)fn)(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), gdim, gstride, box, estr,
-                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) { if (driver_code) *driver_code = (int)r; return cudaErrorInvalidValue; }
-  return cudaSuccess;
+  const uint64_t gdim[2] = {cols, rows}, gstride[1] = {cols * 2};
+  const uint32_t box[2] = {VT_BK, box_rows};
+  return encode_tensor_map(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, base, gdim, gstride, box, driver_code);
 }
 
 // hidden rows: boxes of 128 rows (whole row tiles) and of 32 rows (the ragged last tile); lm_head: boxes of one slice
@@ -375,8 +378,9 @@ cudaError_t encode_vocab_maps(VocabMaps *m, const void *hidden, uint64_t rows, c
 
 bool vocab_tc_supported(int K, int V) { return K >= VT_BK && K % VT_BK == 0 && V >= 1; }
 
-cudaError_t vocab_tc_prepare() {
-  return cudaFuncSetAttribute(vocab_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, VT_SMEM);
+cudaError_t vocab_tc_prepare(int rows_cap) {
+  return rows_cap <= VT_M ? cudaFuncSetAttribute(vocab_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, vt_smem(1))
+                          : cudaFuncSetAttribute(vocab_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, vt_smem(2));
 }
 
 // Launched as a programmatic dependent of the kernel before it in the stream (the packed final norm or the last
@@ -387,13 +391,14 @@ cudaError_t launch_vocab_tc(const VocabMaps &m, const VocabArgs &a_in, cudaStrea
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(vocab_tc_tiles(a.V), 1, 1);
   cfg.blockDim = dim3(VT_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = VT_SMEM;
+  cfg.dynamicSmemBytes = a.rows_cap <= VT_M ? vt_smem(1) : vt_smem(2);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, vocab_tc_kernel, m.a, m.a32, m.b, a);
+  return a.rows_cap <= VT_M ? cudaLaunchKernelEx(&cfg, vocab_tc_kernel<1>, m.a, m.a32, m.b, a)
+                            : cudaLaunchKernelEx(&cfg, vocab_tc_kernel<2>, m.a, m.a32, m.b, a);
 }
 
 }  // namespace pd
