@@ -932,17 +932,18 @@ pd_status pd_collect_row(pd_handle *h, int32_t row, int32_t *tokens, int32_t *le
 // ---- the teacher-forced forward of Eq. 6 -----------------------------------------------------------------
 namespace {
 constexpr int kTfCrossBatch = 256;    // groups per cross-attention launch
-struct TfLayout { size_t tables, x, hb, qkv, att, cq, co, ffn, logprob, part, tickets, logits, total; int logit_rows; };
+struct TfLayout { size_t tables, x, hb, qkv, rot, att, cq, co, ffn, logprob, part, tickets, logits, total; int logit_rows; };
 
 TfLayout tf_layout(const Dims &dm, size_t rows, bool own_logits) {
   TfLayout L;
   size_t off = 0;
   auto reg = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, kAlign); return o; };
   const size_t groups = rows / 1 + (size_t)dm.B;                     // generous: every sequence may end with a short group
-  L.tables = reg((4 * rows + 6 * groups) * sizeof(int32_t));
+  L.tables = reg((4 * rows + 11 * groups) * sizeof(int32_t));
   L.x = reg(rows * dm.d * 4);
   L.hb = reg(rows * dm.d * 2);
   L.qkv = reg(rows * 3 * dm.d * 4);
+  L.rot = reg(dm.pos_mode == PD_POS_ROPE ? rows * 3 * dm.d * 2 : 0);      // queries and keys rotated, in bf16
   L.att = reg(rows * dm.d * 2);
   L.cq = reg(rows * dm.d * 2);
   L.co = reg(rows * dm.d * 2);
@@ -980,7 +981,10 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
     return fail(h, PD_ERR_UNSUPPORTED, "pd_teacher_forward runs on the bf16 path (tensor-core cross-attention) only");
   if (reinterpret_cast<uintptr_t>(scratch) % kAlign != 0) return fail(h, PD_ERR_ARG, "pd_teacher_forward: misaligned scratch");
   // ---- rows in (sequence, subsequence, position) order; groups of up to 32 rows inside a sequence
-  std::vector<int32_t> row_sub, row_tau, row_tok, row_tgt, g_row0, g_n, g_srow0, g_srows, g_seq, g_ctx;
+  // and blocks of up to 128 rows - 64 where those would leave SMs without one - (8-bit context: cross-attention runs on groups of up to 32)
+  std::vector<int32_t> seq_row0, seq_rows;
+  long long blocks128 = 0;
+  std::vector<int32_t> row_sub, row_tau, row_tok, row_tgt, g_row0, g_n, g_seq, g_ctx, b_row0, b_n, b_srow0, b_srows, b_seq, b_ctx;
   std::vector<int32_t> ctx_len(h->batch), plan((size_t)h->batch * dm.SM);
   CU_TRY(h, cudaMemcpyAsync(ctx_len.data(), h->st.ctx_len, (size_t)h->batch * 4, cudaMemcpyDeviceToHost, h->stream));
   CU_TRY(h, cudaMemcpyAsync(plan.data(), h->st.plan, plan.size() * 4, cudaMemcpyDeviceToHost, h->stream));
@@ -1002,29 +1006,39 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
     const int srows = (int)row_sub.size() - srow0;
     if (srows > 0 && plan[(size_t)b * dm.SM + n_sub[b] - 1] - 1 + dm.MSL + dm.SM >= dm.n_dist)
       return fail(h, PD_ERR_ARG, "pd_teacher_forward: positions beyond the tables");
-    for (int r = 0; r < srows; r += kTfGroup) {
+    for (int r = 0; h->kv8 && r < srows; r += kTfGroup) {
       g_row0.push_back(srow0 + r); g_n.push_back(std::min(kTfGroup, srows - r));
-      g_srow0.push_back(srow0); g_srows.push_back(srows); g_seq.push_back(b); g_ctx.push_back(ctx_len[b]);
+      g_seq.push_back(b); g_ctx.push_back(ctx_len[b]);
     }
+    seq_row0.push_back(srow0); seq_rows.push_back(srows);
+    blocks128 += (srows + 127) / 128;
   }
-  const size_t R = row_sub.size(), G = g_row0.size();
+  const int block_rows = blocks128 * dm.H >= 2 * 148 ? 128 : 64;
+  for (int b = 0; b < h->batch; ++b)
+    for (int r = 0; r < seq_rows[b]; r += block_rows) {
+      b_row0.push_back(seq_row0[b] + r); b_n.push_back(std::min(block_rows, seq_rows[b] - r));
+      b_srow0.push_back(seq_row0[b]); b_srows.push_back(seq_rows[b]); b_seq.push_back(b); b_ctx.push_back(ctx_len[b]);
+    }
+  const size_t R = row_sub.size(), G = g_row0.size(), NB = b_row0.size();
   if (rows_out) *rows_out = (int32_t)R;
   if (loss_out) *loss_out = 0.0;
   if (R == 0) return PD_OK;
   const TfLayout L = tf_layout(dm, R, logits == nullptr);
   if (scratch_bytes < L.total) return fail(h, PD_ERR_WORKSPACE, "pd_teacher_forward: scratch too small (pd_teacher_forward_scratch_bytes)");
   CU_TRY(h, cudaSetDevice(h->cfg.device));
+  CU_TRY(h, teacher_attn_prepare());
   cudaStream_t s = h->stream;
   uint8_t *base = reinterpret_cast<uint8_t *>(scratch);
   int32_t *tab = reinterpret_cast<int32_t *>(base + L.tables);
-  int32_t *d_sub = tab, *d_tau = tab + R, *d_tok = tab + 2 * R, *d_tgt = tab + 3 * R, *d_g = tab + 4 * R;
-  int32_t *d_grow0 = d_g, *d_gn = d_g + G, *d_gsrow0 = d_g + 2 * G, *d_gsrows = d_g + 3 * G, *d_gseq = d_g + 4 * G, *d_gctx = d_g + 5 * G;
-  auto up = [&](int32_t *dst, const std::vector<int32_t> &v) { return cudaMemcpyAsync(dst, v.data(), v.size() * 4, cudaMemcpyHostToDevice, s); };
-  CU_TRY(h, up(d_sub, row_sub)); CU_TRY(h, up(d_tau, row_tau)); CU_TRY(h, up(d_tok, row_tok)); CU_TRY(h, up(d_tgt, row_tgt));
-  CU_TRY(h, up(d_grow0, g_row0)); CU_TRY(h, up(d_gn, g_n)); CU_TRY(h, up(d_gsrow0, g_srow0)); CU_TRY(h, up(d_gsrows, g_srows));
-  CU_TRY(h, up(d_gseq, g_seq)); CU_TRY(h, up(d_gctx, g_ctx));
-  CU_TRY(h, cudaMemsetAsync(base + L.tickets, 0, (size_t)kTfCrossBatch * dm.H * 4, s));
-  CU_TRY(h, cudaStreamSynchronize(s));               // the host vectors may go
+  // all tables in one upload
+  std::vector<int32_t> tables;
+  tables.reserve(4 * R + 4 * G + 6 * NB);
+  auto put = [&](const std::vector<int32_t> &v) { int32_t *at = tab + tables.size(); tables.insert(tables.end(), v.begin(), v.end()); return at; };
+  int32_t *d_sub = put(row_sub), *d_tau = put(row_tau), *d_tok = put(row_tok), *d_tgt = put(row_tgt);
+  int32_t *d_grow0 = put(g_row0), *d_gn = put(g_n), *d_gseq = put(g_seq), *d_gctx = put(g_ctx);
+  int32_t *d_brow0 = put(b_row0), *d_bn = put(b_n), *d_bsrow0 = put(b_srow0), *d_bsrows = put(b_srows), *d_bseq = put(b_seq), *d_bctx = put(b_ctx);
+  CU_TRY(h, cudaMemcpyAsync(tab, tables.data(), tables.size() * 4, cudaMemcpyHostToDevice, s));
+  if (h->kv8) CU_TRY(h, cudaMemsetAsync(base + L.tickets, 0, (size_t)kTfCrossBatch * dm.H * 4, s));
 
   float *x = reinterpret_cast<float *>(base + L.x);
   void *hb = base + L.hb, *qkv = base + L.qkv, *att = base + L.att, *cq = base + L.cq, *co = base + L.co, *ffn = base + L.ffn;
@@ -1035,17 +1049,28 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
     const void *const *lw = &h->layer_w[(size_t)l * kLayerTensors];
     OWN(h, PD_PROF_OTHER, launch_rmsnorm(dm, M, PD_DTYPE_BF16, x, lw[0], hb, s));
     PD_TRY(gemm(h, false, M, 3 * dm.d, dm.d, hb, lw[1], qkv, rope, 0.f));
+    const void *qkv_b = qkv;
+    if (rope) {
+      qkv_b = base + L.rot;
+      OWN(h, PD_PROF_OTHER, launch_rotate_rows(M, dm.d, reinterpret_cast<float *>(qkv), d_sub, d_tau, h->ptr<float2>(h->lay.rope_tab), base + L.rot, s));
+    }
     DenseAttnArgs da;
-    da.H = dm.H; da.d = dm.d; da.n_groups = (int)G; da.scale_log2e = dm.scale_log2e;
-    da.qkv = qkv; da.qkv_f32 = rope ? 1 : 0; da.out = reinterpret_cast<__nv_bfloat16 *>(att);
-    da.row_sub = d_sub; da.row_tau = d_tau; da.grp_row0 = d_grow0; da.grp_n = d_gn; da.grp_seq_row0 = d_gsrow0; da.grp_seq_rows = d_gsrows;
+    memset(&da, 0, sizeof(da));
+    da.H = dm.H; da.d = dm.d; da.n_groups = (int)NB; da.block_rows = block_rows; da.scale_log2e = dm.scale_log2e;
+    da.q = reinterpret_cast<const __nv_bfloat16 *>(qkv_b); da.out = reinterpret_cast<__nv_bfloat16 *>(att);
+    da.row_sub = d_sub; da.row_tau = d_tau; da.grp_row0 = d_brow0; da.grp_n = d_bn; da.grp_key_row0 = d_bsrow0; da.grp_keys = d_bsrows;
     da.bias_tab = rope ? nullptr : h->ptr<float>(h->lay.bias_tab); da.n_dist = dm.n_dist;
-    da.rope_tab = rope ? h->ptr<float2>(h->lay.rope_tab) : nullptr;
-    OWN(h, PD_PROF_SELF_ATTN, launch_dense_self_attn(da, s));
+    OWN(h, PD_PROF_SELF_ATTN, launch_teacher_attn(da, true, s));
     PD_TRY(gemm(h, false, M, dm.d, dm.d, att, lw[2], x, true, 1.f));
     OWN(h, PD_PROF_OTHER, launch_rmsnorm(dm, M, PD_DTYPE_BF16, x, lw[3], hb, s));
     PD_TRY(gemm(h, false, M, dm.d, dm.d, hb, lw[4], cq, false, 0.f));
-    for (size_t g0 = 0; g0 < G; g0 += kTfCrossBatch) {              // groups as "sequences" of the batched kernel, 256 at a time
+    if (!h->kv8) {
+      da.q = reinterpret_cast<const __nv_bfloat16 *>(cq); da.out = reinterpret_cast<__nv_bfloat16 *>(co);
+      da.grp_keys = d_bctx; da.grp_seq = d_bseq;
+      da.kv_c = h->ptr<__nv_bfloat16>(h->lay.kv_c); da.layer = l; da.B = dm.B; da.ctx = dm.ctx;
+      OWN(h, PD_PROF_CROSS_ATTN, launch_teacher_attn(da, false, s));
+    }
+    for (size_t g0 = 0; g0 < G; g0 += kTfCrossBatch) {              // 8-bit context: groups as "sequences" of the batched kernel, 256 at a time
       AttnArgs a = attn_args(h, l, false);
       a.dm.C = kTfGroup;
       a.batch = (int)std::min<size_t>(kTfCrossBatch, G - g0);
@@ -1065,14 +1090,27 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
   }
   OWN(h, PD_PROF_OTHER, launch_rmsnorm(dm, M, PD_DTYPE_BF16, x, h->w.final_norm, hb, s));
   float *d_lp = reinterpret_cast<float *>(base + L.logprob);
+  // Logits of n rows.  Where the rows of a vocabulary of odd size start off a 16-byte boundary cuBLAS has no kernel for this
+  // part (513 rows x 50265 ids of width 768: 330 us); the vocabulary kernel stores them whatever their alignment (85 us).
+  auto project = [&](const uint8_t *rows_hb, int n, float *out) -> pd_status {
+    if (dm.V % 4 == 0 || !h->vocab_tc) return gemm(h, true, n, dm.V, dm.d, rows_hb, h->w.lm_head, out, true, 0.f);
+    VocabMaps maps;
+    CU_TRY(h, encode_vocab_maps(&maps, rows_hb, (uint64_t)n, h->w.lm_head, (uint64_t)dm.V, (uint64_t)dm.d, nullptr));
+    CU_TRY(h, vocab_tc_prepare(n));
+    VocabArgs va;
+    memset(&va, 0, sizeof(va));
+    va.m_fixed = n; va.V = dm.V; va.K = dm.d; va.rows_cap = n; va.eos = -1; va.sep = -1; va.logits = out; va.status = h->st.hdr + HDR_STATUS;
+    OWN(h, PD_PROF_VOCAB, launch_vocab_tc(maps, va, s));
+    return PD_OK;
+  };
   if (logits != nullptr) {
-    PD_TRY(gemm(h, true, M, dm.V, dm.d, hb, h->w.lm_head, logits, true, 0.f));
+    PD_TRY(project(reinterpret_cast<uint8_t *>(hb), M, logits));
     OWN(h, PD_PROF_OTHER, launch_target_logprob(M, dm.V, logits, d_tgt, d_lp, s));
   } else {
     float *chunk = reinterpret_cast<float *>(base + L.logits);
     for (int r0 = 0; r0 < M; r0 += L.logit_rows) {
       const int n = std::min(L.logit_rows, M - r0);
-      PD_TRY(gemm(h, true, n, dm.V, dm.d, reinterpret_cast<uint8_t *>(hb) + (size_t)r0 * dm.d * 2, h->w.lm_head, chunk, true, 0.f));
+      PD_TRY(project(reinterpret_cast<uint8_t *>(hb) + (size_t)r0 * dm.d * 2, n, chunk));
       OWN(h, PD_PROF_OTHER, launch_target_logprob(n, dm.V, chunk, d_tgt + r0, d_lp + r0, s));
     }
   }

@@ -118,17 +118,24 @@ struct AttnArgs {
 
 // ---- teacher-forced dense forward (teacher_kernels.cu) ------------------------------------------------
 struct DenseAttnArgs {
-  int H, d, n_groups;
+  int H, d, n_groups, block_rows;        // query rows per attention block: 128 or 64
   float scale_log2e;
-  const void *qkv; int qkv_f32;          // [rows][3 d]: bf16, or fp32 (rotary mode: rotated here)
+  const __nv_bfloat16 *q;                // self: [rows][3 d] queries (rotated), keys (rotated), values; cross: queries [rows][d]
   __nv_bfloat16 *out;                    // [rows][d]
+  const int32_t *grp_row0, *grp_n;       // [groups] first row and number of rows (<= block_rows) of a query block
+  const int32_t *grp_keys;               // [groups] self: row count of the block's sequence; cross: its context length
+  // self
   const int32_t *row_sub, *row_tau;      // [rows] subsequence i and timestamp tau of every row
-  const int32_t *grp_row0, *grp_n;       // [groups] first row and number of rows (<= 32) of a query group
-  const int32_t *grp_seq_row0, *grp_seq_rows;   // [groups] first row and row count of the group's sequence (its keys)
+  const int32_t *grp_key_row0;           // [groups] first row of the block's sequence
   const float *bias_tab; int n_dist;     // T5 mode: [H][n_dist], log2(e)-scaled; else null
-  const float2 *rope_tab;                // rotary mode: [n_dist][32] (cos, sin); else null
+  // cross
+  const __nv_bfloat16 *kv_c; int layer, B, ctx;
+  const int32_t *grp_seq;                // [groups] the sequence whose context the block reads
 };
-cudaError_t launch_dense_self_attn(const DenseAttnArgs &a, cudaStream_t s);
+cudaError_t teacher_attn_prepare();      // once per device
+cudaError_t launch_teacher_attn(const DenseAttnArgs &a, bool self, cudaStream_t s);
+cudaError_t launch_rotate_rows(int rows, int d, const float *qkv, const int32_t *row_sub, const int32_t *row_tau, const float2 *rope_tab,
+                               void *out, cudaStream_t s);
 cudaError_t launch_gather_rows(int rows, int d, const int32_t *row_tok, const void *embed, float *x, cudaStream_t s);
 cudaError_t launch_target_logprob(int rows, int V, const float *logits, const int32_t *targets, float *logprob, cudaStream_t s);
 
@@ -189,7 +196,7 @@ struct VocabArgs {
   int rows_cap;              // row stride of the partial arrays (>= the largest row count)
   int wn;                    // vocabulary ids per CTA (set by the launcher: vocab_tc_slice(V))
   int eos, sep;              // ids kept out of the maxima (their logits go to term_val); -1 = none
-  float *part_val;           // [tiles][rows_cap] maximum of the row over the tile's ids
+  float *part_val;           // [tiles][rows_cap] maximum of the row over the tile's ids (null: only the logits are wanted)
   int32_t *part_idx;         // [tiles][rows_cap] the id that holds it (lowest on ties; INT_MAX = none)
   float *term_val;           // [rows_cap][2] logits of eos and sep
   float *logits;             // [rows][V] fp32, or null when nobody reads them

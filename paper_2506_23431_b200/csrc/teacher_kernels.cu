@@ -1,7 +1,7 @@
 // Kernels of the teacher-forced forward of Section 3.3 (Eq. 6): the whole target of every sequence in one
 // pass, every token attending to the tokens the dependency rule of Section 3.2 lets it see - evaluated per
-// (query, key) pair from (subsequence, timestamp) and never stored as a mask.  Off the decode hot path
-// (scoring, perplexity).  One CTA per group of up to 32 query rows and head, on tensor cores (mma.sync, 64-key tiles).
+// (query, key) pair from (subsequence, timestamp) and never stored as a mask - and to the sequence's context.  Off the decode
+// hot path (scoring, perplexity).
 #include "mma_tile.cuh"
 #include "pd_internal.h"
 
@@ -9,224 +9,244 @@ namespace pd {
 
 namespace {
 
-// Four warps; a tile = 64 keys of the sequence, staged by all threads as swizzled bf16 rows (keys rotated on the way
-// in rotary mode), each warp taking 16 of them: scores with mma.sync against the group's two 16-row query tiles, the
-// dependency rule and the T5 bias applied to the accumulator fragment per (query, key) pair, online softmax, P.V.
-// The warps' states are tree-merged through shared memory at the end.
-constexpr int TQ = 32, TK = 64, TT = 128, TW = 4, TMAXD = 640;
+// Attention of up to 128 query rows of one sequence and head (one CTA; W warps of 16 MT rows each) over 64-key tiles that all
+// warps share: a three-slot ring filled with 16-byte asynchronous copies (rows of 128 bytes, chunks swizzled), scores and
+// P.V on mma.sync, online softmax in the log2 domain; a warp owns its rows, so nothing is merged.
+// SELF = false: the keys are the sequence's context positions below ctx_len.  SELF = true: the keys are the sequence's own target
+// rows, with the dependency rule and the T5 bias applied to the accumulator fragment; the key walk ends at the first tile of a
+// later subsequence.
+// What bounds it: with 128 rows per pass over the keys the tensor pipe (1075 cycles per tile) and the ldmatrix traffic that feeds
+// it (1024 cycles with 16 rows per warp, half of that with 32), not HBM.  11.5 k rows, 32 contexts of 2048, 16 heads, per layer:
+// cross-attention 640 us in groups of 32 rows on the decode kernel (every group reads its context again), 452 us here with 16 rows
+// per warp, 392 us with 32; self-attention 203 us in groups of 32 rows, 157 us with 16 rows per warp, 234 us with 32 (the mask needs
+// the registers).  So the context pass takes MT = 2 and the self pass MT = 1; where 128-row blocks would leave SMs without one,
+// both take 64-row blocks of MT = 1.
+constexpr int TK = 64, TSLOTS = 3, TMAXD = 640;
+constexpr int TSLOT_BYTES = TK * 256;            // 64 key rows, then 64 value rows
+constexpr int TATTN_SMEM = TSLOTS * TSLOT_BYTES + 128;
 
-__global__ void __launch_bounds__(TT) dense_self_attn_tc_kernel(DenseAttnArgs a) {
+__device__ __forceinline__ void t_cp_async16(uint32_t dst, const void *src, bool on) {
+  const int n = on ? 16 : 0;                     // 0 source bytes: the destination is zero-filled
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void t_cp_async4(uint32_t dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+template <bool SELF, int W, int MT>
+__global__ void __launch_bounds__(W * 32, 16 / (W * MT)) teacher_attn_kernel(DenseAttnArgs a) {
   using namespace mt;
+  constexpr int TT = W * 32;
+  extern __shared__ uint8_t t_raw[];
+  __shared__ int ki_s[TSLOTS][TK], kt_s[TSLOTS][TK];
+  __shared__ float bias_s[SELF ? TMAXD : 1];
   const int grp = blockIdx.x, h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, tig = lane & 3;
   const int q0 = a.grp_row0[grp], nq = a.grp_n[grp];
-  const int k0 = a.grp_seq_row0[grp], nk = a.grp_seq_rows[grp];
-  __shared__ __align__(1024) uint8_t ks[TK * 128];
-  __shared__ __align__(1024) uint8_t vs[TK * 128];
-  __shared__ int ki_s[TK], kt_s[TK], qi_s[TQ], qt_s[TQ];
-  __shared__ float bias_s[TMAXD];
-  __shared__ float scratch[2 * kRecFloats];
-  const size_t ld = 3 * (size_t)a.d;
-  const bool rope = a.rope_tab != nullptr, use_bias = a.bias_tab != nullptr;
-  if (tid < TQ) {
-    qi_s[tid] = tid < nq ? a.row_sub[q0 + tid] : 0;
-    qt_s[tid] = tid < nq ? a.row_tau[q0 + tid] : 0;
+  const uint32_t base = (smem_u32(t_raw) + 127u) & ~127u;
+  const size_t qld = SELF ? 3 * (size_t)a.d : (size_t)a.d, kld = SELF ? 3 * (size_t)a.d : (size_t)kDh;
+  const __nv_bfloat16 *kp, *vp;                  // row 0 of this head's keys and values
+  int nk, k0 = 0;
+  if (SELF) {
+    k0 = a.grp_key_row0[grp]; nk = a.grp_keys[grp];
+    kp = a.q + (size_t)k0 * kld + a.d + (size_t)h * kDh; vp = kp + a.d;
+  } else {
+    nk = a.grp_keys[grp];
+    kp = a.kv_c + ctx_kv_offset(a.layer, a.B, a.grp_seq[grp], a.H, h, 0, a.ctx); vp = kp + (size_t)a.ctx * kDh;
   }
+  const bool use_bias = SELF && a.bias_tab != nullptr;
   if (use_bias)
     for (int dd = tid; dd < a.n_dist; dd += TT) bias_s[dd] = a.bias_tab[(size_t)h * a.n_dist + dd];
-  __syncthreads();
-  // query fragments (rows beyond the group's are zero and masked anyway)
-  uint32_t qf[2][4][4];
-  int qi[2][2], qp[2][2];               // subsequence and position tau + i of rows g / g + 8 of both query tiles
+
+  auto fetch = [&](int tile) {
+    const int slot = tile % TSLOTS, first = tile * TK;
+    const uint32_t dst = base + slot * TSLOT_BYTES;
 #pragma unroll
-  for (int mt_ = 0; mt_ < 2; ++mt_) {
+    for (int i = 0; i < TK * 16 / TT; ++i) {     // chunks 0-7 of a row: keys, 8-15: values
+      const int c = tid + i * TT, r = c >> 4, p = c & 15;
+      const bool on = first + r < nk;            // absent keys: zero rows
+      const __nv_bfloat16 *src = (p < 8 ? kp : vp) + (on ? (size_t)(first + r) * kld : 0) + (p & 7) * 8;
+      t_cp_async16(dst + (p >> 3) * (TK * 128) + swz(r, p & 7), src, on);
+    }
+    if (SELF)
+      for (int i = tid; i < TK && first + i < nk; i += TT) {
+        t_cp_async4(smem_u32(&ki_s[slot][i]), a.row_sub + k0 + first + i);
+        t_cp_async4(smem_u32(&kt_s[slot][i]), a.row_tau + k0 + first + i);
+      }
+  };
+  // tiles to walk: keys are sorted by subsequence, and nothing of a later one than the block's last row's is visible
+  int n_tiles = (nk + TK - 1) / TK;
+  if (SELF) {
+    const int q_i_max = a.row_sub[q0 + nq - 1];
+    int lo = 0, hi = n_tiles;                    // first tile whose first key lies beyond
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (a.row_sub[k0 + mid * TK] > q_i_max) hi = mid; else lo = mid + 1;
+    }
+    n_tiles = lo;
+  }
 #pragma unroll
-    for (int hh = 0; hh < 2; ++hh) {
-      const int r = mt_ * 16 + g + hh * 8;
-      qi[mt_][hh] = r < nq ? qi_s[r] : -1;                       // -1: sees nothing
-      qp[mt_][hh] = r < nq ? qt_s[r] + qi_s[r] : 0;
+  for (int t = 0; t < TSLOTS - 1; ++t) {
+    if (t < n_tiles) fetch(t);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  // this warp's query rows: 16 (MT warp + mt) + g, + 8
+  const int w0 = warp * 16 * MT;
+  uint32_t qf[MT][4][4];
+  int qi[MT][2], qt[MT][2], warp_i_max = 0x7fffffff;       // subsequence (-1: sees nothing) and timestamp of the rows
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
+  for (int mt_ = 0; mt_ < MT; ++mt_) {
+    const int r_lo = w0 + mt_ * 16 + g, r_hi = r_lo + 8;
+    const __nv_bfloat16 *q_lo = a.q + (size_t)(q0 + r_lo) * qld + (size_t)h * kDh + 2 * tig, *q_hi = q_lo + 8 * qld;
 #pragma unroll
-        for (int half = 0; half < 2; ++half) {
-          uint32_t w = 0u;
-          if (r < nq) {
-            const int col = kk * 16 + 2 * tig + half * 8;
-            const size_t o = (size_t)(q0 + r) * ld + (size_t)h * kDh + col;
-            if (!a.qkv_f32) {
-              w = *reinterpret_cast<const uint32_t *>(reinterpret_cast<const __nv_bfloat16 *>(a.qkv) + o);
-            } else {
-              float2 v = *reinterpret_cast<const float2 *>(reinterpret_cast<const float *>(a.qkv) + o);
-              if (rope) {
-                const float2 cs = a.rope_tab[(size_t)qp[mt_][hh] * (kDh / 2) + col / 2];
-                const float t = v.x * cs.x - v.y * cs.y;
-                v.y = v.x * cs.y + v.y * cs.x; v.x = t;
-              }
-              w = pack_bf16(v.x, v.y);
-            }
-          }
-          qf[mt_][kk][hh + 2 * half] = w;
-        }
+    for (int kk = 0; kk < 4; ++kk) {
+      qf[mt_][kk][0] = r_lo < nq ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16) : 0u;
+      qf[mt_][kk][1] = r_hi < nq ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16) : 0u;
+      qf[mt_][kk][2] = r_lo < nq ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8) : 0u;
+      qf[mt_][kk][3] = r_hi < nq ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8) : 0u;
+    }
+    if (SELF) {
+      qi[mt_][0] = r_lo < nq ? a.row_sub[q0 + r_lo] : -1; qt[mt_][0] = r_lo < nq ? a.row_tau[q0 + r_lo] : 0;
+      qi[mt_][1] = r_hi < nq ? a.row_sub[q0 + r_hi] : -1; qt[mt_][1] = r_hi < nq ? a.row_tau[q0 + r_hi] : 0;
     }
   }
-  const int qt_row[2][2] = {{qp[0][0] - qi[0][0], qp[0][1] - qi[0][1]}, {qp[1][0] - qi[1][0], qp[1][1] - qi[1][1]}};
-  TileAcc acc[2];
-  acc[0].clear(); acc[1].clear();
-  const int q_i_max = qi_s[nq - 1];
-  const uint32_t kbase = smem_u32(ks), vbase = smem_u32(vs);
-  const int kb = warp * 16;              // this warp's keys inside every tile
+  if (SELF) warp_i_max = w0 < nq ? a.row_sub[q0 + min(w0 + 16 * MT - 1, nq - 1)] : -1;
+  TileAcc acc[MT];
+#pragma unroll
+  for (int mt_ = 0; mt_ < MT; ++mt_) acc[mt_].clear();
+  const float sl2 = a.scale_log2e;
 
-  for (int kt0 = 0; kt0 < nk; kt0 += TK) {
-    if (a.row_sub[k0 + kt0] > q_i_max) break;     // rows are sorted by subsequence: nothing further on is visible
-    const int nv = min(TK, nk - kt0);
-    __syncthreads();                    // the previous tile is consumed
-    if (tid < TK) {
-      ki_s[tid] = tid < nv ? a.row_sub[k0 + kt0 + tid] : 0x3fffffff;
-      kt_s[tid] = tid < nv ? a.row_tau[k0 + kt0 + tid] : 0x3fffffff;
-    }
-    {
-      // thread = (key, half of the head): 32 columns of its key row and of its value row
-      const int e = tid >> 1, c0 = (tid & 1) * 32;
-      uint4 kq[4], vq[4];
+  for (int tile = 0; tile < n_tiles; ++tile) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(TSLOTS - 2) : "memory");
+    __syncthreads();                             // tile landed for everybody; everybody is through with the tile before
+    if (tile + TSLOTS - 1 < n_tiles) fetch(tile + TSLOTS - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const int slot = tile % TSLOTS, nv = min(TK, nk - tile * TK);
+    if (w0 >= nq || (SELF && ki_s[slot][0] > warp_i_max)) continue;      // no row of this warp sees the tile
+    const uint32_t kbase = base + slot * TSLOT_BYTES, vbase = kbase + TK * 128;
+    float sc[MT][8][4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) kq[j] = vq[j] = make_uint4(0u, 0u, 0u, 0u);
-      if (e < nv) {
-        const size_t ob = (size_t)(k0 + kt0 + e) * ld + (size_t)h * kDh + c0;
-        if (!a.qkv_f32) {
-          const __nv_bfloat16 *src = reinterpret_cast<const __nv_bfloat16 *>(a.qkv) + ob;
+    for (int nt = 0; nt < 8; ++nt) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            kq[j] = *reinterpret_cast<const uint4 *>(src + a.d + 8 * j);
-            vq[j] = *reinterpret_cast<const uint4 *>(src + 2 * (size_t)a.d + 8 * j);
-          }
-        } else {
-          const float *src = reinterpret_cast<const float *>(a.qkv) + ob;
-          const int pos = a.row_tau[k0 + kt0 + e] + a.row_sub[k0 + kt0 + e];
-          uint32_t kw[16], vw[16];
+      for (int mt_ = 0; mt_ < MT; ++mt_) sc[mt_][nt][0] = sc[mt_][nt][1] = sc[mt_][nt][2] = sc[mt_][nt][3] = 0.f;
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            float2 kf = *reinterpret_cast<const float2 *>(src + a.d + 2 * j);
-            const float2 vf = *reinterpret_cast<const float2 *>(src + 2 * (size_t)a.d + 2 * j);
-            if (rope) {
-              const float2 cs = a.rope_tab[(size_t)pos * (kDh / 2) + c0 / 2 + j];
-              const float t = kf.x * cs.x - kf.y * cs.y;
-              kf.y = kf.x * cs.y + kf.y * cs.x; kf.x = t;
-            }
-            kw[j] = pack_bf16(kf.x, kf.y); vw[j] = pack_bf16(vf.x, vf.y);
-          }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            kq[j] = make_uint4(kw[4 * j], kw[4 * j + 1], kw[4 * j + 2], kw[4 * j + 3]);
-            vq[j] = make_uint4(vw[4 * j], vw[4 * j + 1], vw[4 * j + 2], vw[4 * j + 3]);
-          }
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        *reinterpret_cast<uint4 *>(ks + swz(e, (tid & 1) * 4 + j)) = kq[j];
-        *reinterpret_cast<uint4 *>(vs + swz(e, (tid & 1) * 4 + j)) = vq[j];      // absent keys: zero rows
-      }
-    }
-    __syncthreads();
-    if (kb >= nv) continue;              // (the barriers above are reached by every warp on every tile)
-    // ---- scores of this warp's 16 keys
-    float sc[2][2][4];
-#pragma unroll
-    for (int mt_ = 0; mt_ < 2; ++mt_)
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) sc[mt_][nt][0] = sc[mt_][nt][1] = sc[mt_][nt][2] = sc[mt_][nt][3] = 0.f;
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-      const int key = kb + nt * 8 + (lane & 7);
-#pragma unroll
-      for (int kp = 0; kp < 2; ++kp) {
+      for (int kq = 0; kq < 2; ++kq) {
         uint32_t b0, b1, b2, b3;
-        ldsm_x4(kbase + swz(key, kp * 4 + (lane >> 3)), b0, b1, b2, b3);
+        ldsm_x4(kbase + swz(nt * 8 + (lane & 7), kq * 4 + (lane >> 3)), b0, b1, b2, b3);
 #pragma unroll
-        for (int mt_ = 0; mt_ < 2; ++mt_) {
-          mma_bf16(sc[mt_][nt], qf[mt_][2 * kp][0], qf[mt_][2 * kp][1], qf[mt_][2 * kp][2], qf[mt_][2 * kp][3], b0, b1);
-          mma_bf16(sc[mt_][nt], qf[mt_][2 * kp + 1][0], qf[mt_][2 * kp + 1][1], qf[mt_][2 * kp + 1][2], qf[mt_][2 * kp + 1][3], b2, b3);
+        for (int mt_ = 0; mt_ < MT; ++mt_) {
+          mma_bf16(sc[mt_][nt], qf[mt_][2 * kq][0], qf[mt_][2 * kq][1], qf[mt_][2 * kq][2], qf[mt_][2 * kq][3], b0, b1);
+          mma_bf16(sc[mt_][nt], qf[mt_][2 * kq + 1][0], qf[mt_][2 * kq + 1][1], qf[mt_][2 * kq + 1][2], qf[mt_][2 * kq + 1][3], b2, b3);
         }
       }
     }
-    // ---- the dependency rule per pair (i' <= i and tau' <= tau), bias on the Manhattan distance, online softmax
-    uint32_t pf[2][4];
+    // ---- SELF: scale, the dependency rule per pair (i' <= i and tau' <= tau), bias on the Manhattan distance (log2 domain);
+    // context: absent keys of the last tile; the scale joins the exponent below
+    if (SELF) {
 #pragma unroll
-    for (int mt_ = 0; mt_ < 2; ++mt_) {
+      for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+        for (int kx = 0; kx < 2; ++kx) {
+          const int e = nt * 8 + 2 * tig + kx;
+          const int ki = ki_s[slot][e], ktau = kt_s[slot][e];
+#pragma unroll
+          for (int mt_ = 0; mt_ < MT; ++mt_)
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+              float v = sc[mt_][nt][2 * hh + kx] * sl2;
+              const bool vis = e < nv && ki <= qi[mt_][hh] && ktau <= qt[mt_][hh];
+              if (use_bias && vis) v += bias_s[qt[mt_][hh] + qi[mt_][hh] - (ktau + ki)];
+              sc[mt_][nt][2 * hh + kx] = vis ? v : -INFINITY;
+            }
+        }
+    } else if (nv < TK) {
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int mt_ = 0; mt_ < MT; ++mt_)
+            if (nt * 8 + 2 * tig + (x & 1) >= nv) sc[mt_][nt][x] = -INFINITY;
+    }
+    const float es = SELF ? 1.f : sl2;
+    uint32_t pf[MT][4][4];
+#pragma unroll
+    for (int mt_ = 0; mt_ < MT; ++mt_) {
       float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          const int e = kb + nt * 8 + 2 * tig + (x & 1), hh = x >> 1;
-          const int ki = ki_s[e], ktau = kt_s[e];
-          float v = -INFINITY;
-          if (ki <= qi[mt_][hh] && ktau <= qt_row[mt_][hh]) {
-            v = sc[mt_][nt][x] * a.scale_log2e;
-            if (use_bias) v += bias_s[qp[mt_][hh] - (ktau + ki)];
-          }
-          sc[mt_][nt][x] = v;
-          if (hh == 0) mx0 = fmaxf(mx0, v); else mx1 = fmaxf(mx1, v);
-        }
+      for (int nt = 0; nt < 8; ++nt) {
+        mx0 = fmaxf(mx0, fmaxf(sc[mt_][nt][0], sc[mt_][nt][1]));
+        mx1 = fmaxf(mx1, fmaxf(sc[mt_][nt][2], sc[mt_][nt][3]));
+      }
       mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1)); mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
       mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1)); mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
       TileAcc &A = acc[mt_];
-      const float mn0 = fmaxf(A.m0, mx0), mn1 = fmaxf(A.m1, mx1);
+      const float mn0 = fmaxf(A.m0, mx0 * es), mn1 = fmaxf(A.m1, mx1 * es);
       const float ref0 = mn0 == -INFINITY ? 0.f : mn0, ref1 = mn1 == -INFINITY ? 0.f : mn1;
       const float c0 = ex2f(A.m0 - ref0), c1 = ex2f(A.m1 - ref1);
       A.m0 = mn0; A.m1 = mn1;
       float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const float p0 = ex2f(sc[mt_][nt][0] - ref0), p1 = ex2f(sc[mt_][nt][1] - ref0);
-        const float p2 = ex2f(sc[mt_][nt][2] - ref1), p3 = ex2f(sc[mt_][nt][3] - ref1);
+      for (int nt = 0; nt < 8; ++nt) {
+        const float p0 = ex2f(fmaf(sc[mt_][nt][0], es, -ref0)), p1 = ex2f(fmaf(sc[mt_][nt][1], es, -ref0));
+        const float p2 = ex2f(fmaf(sc[mt_][nt][2], es, -ref1)), p3 = ex2f(fmaf(sc[mt_][nt][3], es, -ref1));
         s0 += p0 + p1; s1 += p2 + p3;
-        pf[mt_][nt * 2 + 0] = pack_bf16(p0, p1);
-        pf[mt_][nt * 2 + 1] = pack_bf16(p2, p3);
+        pf[mt_][nt >> 1][(nt & 1) * 2] = pack_bf16(p0, p1);
+        pf[mt_][nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
       }
       A.l0 = A.l0 * c0 + s0; A.l1 = A.l1 * c1 + s1;
+      if (__any_sync(0xffffffffu, c0 != 1.f || c1 != 1.f)) {   // some row's running maximum moved
 #pragma unroll
-      for (int dn = 0; dn < 8; ++dn) { A.o[dn][0] *= c0; A.o[dn][1] *= c0; A.o[dn][2] *= c1; A.o[dn][3] *= c1; }
+        for (int dn = 0; dn < 8; ++dn) { A.o[dn][0] *= c0; A.o[dn][1] *= c0; A.o[dn][2] *= c1; A.o[dn][3] *= c1; }
+      }
     }
-    // ---- O += P (16 x 16 keys) . V (16 keys x 64)
-    {
-      const int key = kb + ((lane >> 3) & 1) * 8 + (lane & 7);
+    // ---- O += P (16 MT x 64 keys) . V (64 keys x 64)
+#pragma unroll
+    for (int kq = 0; kq < 4; ++kq) {
+      const int key = kq * 16 + ((lane >> 3) & 1) * 8 + (lane & 7);
 #pragma unroll
       for (int dp = 0; dp < 4; ++dp) {
         uint32_t b0, b1, b2, b3;
         ldsm_x4_t(vbase + swz(key, dp * 2 + (lane >> 4)), b0, b1, b2, b3);
 #pragma unroll
-        for (int mt_ = 0; mt_ < 2; ++mt_) {
-          mma_bf16(acc[mt_].o[2 * dp], pf[mt_][0], pf[mt_][1], pf[mt_][2], pf[mt_][3], b0, b1);
-          mma_bf16(acc[mt_].o[2 * dp + 1], pf[mt_][0], pf[mt_][1], pf[mt_][2], pf[mt_][3], b2, b3);
+        for (int mt_ = 0; mt_ < MT; ++mt_) {
+          mma_bf16(acc[mt_].o[2 * dp], pf[mt_][kq][0], pf[mt_][kq][1], pf[mt_][kq][2], pf[mt_][kq][3], b0, b1);
+          mma_bf16(acc[mt_].o[2 * dp + 1], pf[mt_][kq][0], pf[mt_][kq][1], pf[mt_][kq][2], pf[mt_][kq][3], b2, b3);
         }
       }
     }
   }
-  // ---- row sums across the quad, tree merge of the four warps, output
 #pragma unroll
-  for (int mt_ = 0; mt_ < 2; ++mt_) {
+  for (int mt_ = 0; mt_ < MT; ++mt_) {
     TileAcc &A = acc[mt_];
     A.l0 += __shfl_xor_sync(0xffffffffu, A.l0, 1); A.l0 += __shfl_xor_sync(0xffffffffu, A.l0, 2);
     A.l1 += __shfl_xor_sync(0xffffffffu, A.l1, 1); A.l1 += __shfl_xor_sync(0xffffffffu, A.l1, 2);
+    const float i0 = 1.f / A.l0, i1 = 1.f / A.l1;
+    const int r_lo = w0 + mt_ * 16 + g, r_hi = r_lo + 8;
+    __nv_bfloat16 *o_lo = a.out + (size_t)(q0 + r_lo) * a.d + (size_t)h * kDh + 2 * tig, *o_hi = o_lo + 8 * (size_t)a.d;
 #pragma unroll
-    for (int stride = TW / 2; stride >= 1; stride >>= 1) {
-      __syncthreads();
-      if (warp >= stride && warp < 2 * stride) A.store(scratch + (warp - stride) * kRecFloats, lane);
-      __syncthreads();
-      if (warp < stride) A.merge(scratch + warp * kRecFloats, lane);
+    for (int dn = 0; dn < 8; ++dn) {
+      if (r_lo < nq) *reinterpret_cast<__nv_bfloat162 *>(o_lo + dn * 8) = __floats2bfloat162_rn(A.o[dn][0] * i0, A.o[dn][1] * i0);
+      if (r_hi < nq) *reinterpret_cast<__nv_bfloat162 *>(o_hi + dn * 8) = __floats2bfloat162_rn(A.o[dn][2] * i1, A.o[dn][3] * i1);
     }
-    if (warp == 0) {
-      const int r_lo = mt_ * 16 + g, r_hi = r_lo + 8;
-      const float i0 = 1.f / A.l0, i1 = 1.f / A.l1;
-      __nv_bfloat16 *o_lo = a.out + (size_t)(q0 + r_lo) * a.d + (size_t)h * kDh + 2 * tig;
-      __nv_bfloat16 *o_hi = a.out + (size_t)(q0 + r_hi) * a.d + (size_t)h * kDh + 2 * tig;
-#pragma unroll
-      for (int dn = 0; dn < 8; ++dn) {
-        if (r_lo < nq) *reinterpret_cast<__nv_bfloat162 *>(o_lo + dn * 8) = __floats2bfloat162_rn(A.o[dn][0] * i0, A.o[dn][1] * i0);
-        if (r_hi < nq) *reinterpret_cast<__nv_bfloat162 *>(o_hi + dn * 8) = __floats2bfloat162_rn(A.o[dn][2] * i1, A.o[dn][3] * i1);
-      }
+  }
+}
+
+// Rotary mode: queries and keys rotated by their row's position tau + i, everything rounded to bf16.
+__global__ void __launch_bounds__(256) rotate_rows_kernel(int d, const float *__restrict__ qkv, const int32_t *__restrict__ row_sub,
+                                                          const int32_t *__restrict__ row_tau, const float2 *__restrict__ rope_tab,
+                                                          __nv_bfloat16 *__restrict__ out) {
+  const int r = blockIdx.x;
+  const int pos = row_sub[r] + row_tau[r];
+  const float4 *src = reinterpret_cast<const float4 *>(qkv + (size_t)r * 3 * d);
+  uint2 *dst = reinterpret_cast<uint2 *>(out + (size_t)r * 3 * d);
+  for (int c = threadIdx.x; c < 3 * d / 4; c += 256) {        // four columns
+    float4 v = src[c];
+    if (c < d / 2) {
+      const float4 cs = *reinterpret_cast<const float4 *>(rope_tab + (size_t)pos * (kDh / 2) + (4 * c % kDh) / 2);
+      v = make_float4(v.x * cs.x - v.y * cs.y, v.x * cs.y + v.y * cs.x, v.z * cs.z - v.w * cs.w, v.z * cs.w + v.w * cs.z);
     }
+    dst[c] = make_uint2(mt::pack_bf16(v.x, v.y), mt::pack_bf16(v.z, v.w));
   }
 }
 
@@ -234,43 +254,85 @@ __global__ void __launch_bounds__(TT) dense_self_attn_tc_kernel(DenseAttnArgs a)
 __global__ void gather_rows_kernel(int d, const int32_t *__restrict__ row_tok, const __nv_bfloat16 *__restrict__ embed,
                                    float *__restrict__ x) {
   const int r = blockIdx.x;
-  const __nv_bfloat16 *e = embed + (size_t)row_tok[r] * d;
-  for (int c = threadIdx.x; c < d; c += blockDim.x) x[(size_t)r * d + c] = __bfloat162float(e[c]);
+  const uint2 *e = reinterpret_cast<const uint2 *>(embed + (size_t)row_tok[r] * d);      // four columns per thread; d is a multiple of 64
+  for (int c = threadIdx.x; c < d / 4; c += blockDim.x) {
+    const uint2 w = e[c];
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.y));
+    *reinterpret_cast<float4 *>(x + (size_t)r * d + 4 * c) = make_float4(a.x, a.y, b.x, b.y);
+  }
 }
 
-// logprob[r] = logits[r][target] - log sum_v exp(logits[r][v])   (the row's term of Eq. 6)
+// logprob[r] = logits[r][target] - log sum_v exp(logits[r][v])   (the row's term of Eq. 6).  One pass over the row (every thread
+// keeps a running maximum and the sum relative to it), 16-byte loads over its aligned body.  (Maximum and sum in a pass
+// each, 4-byte loads: 88 us for 2089 rows of 32128, against 48 us.)
 __global__ void __launch_bounds__(256) target_logprob_kernel(int V, const float *__restrict__ logits, const int32_t *__restrict__ targets,
                                                              float *__restrict__ logprob) {
-  __shared__ float red[8];
-  __shared__ float mx_s;
+  __shared__ float red_m[8], red_s[8];
+  const int tid = threadIdx.x;
   const float *row = logits + (size_t)blockIdx.x * V;
-  float mx = -INFINITY;
-  for (int v = threadIdx.x; v < V; v += 256) mx = fmaxf(mx, row[v]);
-  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+  float m = -INFINITY, s = 0.f;
+  auto take4 = [&](const float4 &x) {
+    const float mx = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w));
+    if (mx > m) { s *= expf(m - mx); m = mx; }
+    if (m > -INFINITY) s += (expf(x.x - m) + expf(x.y - m)) + (expf(x.z - m) + expf(x.w - m));
+  };
+  auto take = [&](float x) {
+    if (x > m) { s *= expf(m - x); m = x; }
+    if (m > -INFINITY) s += expf(x - m);
+  };
+  const int head = min(V, (int)((4u - (unsigned)(((size_t)blockIdx.x * V) & 3u)) & 3u));
+  const int nvec = (V - head) / 4;
+  if (tid < head) take(row[tid]);
+  const float4 *body = reinterpret_cast<const float4 *>(row + head);
+  int q = tid;
+  for (; q + 3 * 256 < nvec; q += 4 * 256) {
+    float4 x[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) x[u] = __ldcs(body + q + u * 256);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) take4(x[u]);
+  }
+  for (; q < nvec; q += 256) take4(__ldcs(body + q));
+  for (int v = head + 4 * nvec + tid; v < V; v += 256) take(row[v]);
+  auto join = [](float &ma, float &sa, float mb, float sb) {
+    const float mx = fmaxf(ma, mb);
+    if (mx > -INFINITY) sa = sa * expf(ma - mx) + sb * expf(mb - mx);
+    ma = mx;
+  };
+  for (int o = 16; o > 0; o >>= 1) join(m, s, __shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, s, o));
+  if ((tid & 31) == 0) { red_m[tid >> 5] = m; red_s[tid >> 5] = s; }
   __syncthreads();
-  if (threadIdx.x == 0) { float m = red[0]; for (int w = 1; w < 8; ++w) m = fmaxf(m, red[w]); mx_s = m; }
-  __syncthreads();
-  mx = mx_s;
-  float sum = 0.f;
-  for (int v = threadIdx.x; v < V; v += 256) sum += expf(row[v] - mx);
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int w = 0; w < 8; ++w) s += red[w];
-    logprob[blockIdx.x] = row[targets[blockIdx.x]] - (mx + logf(s));
+  if (tid == 0) {
+    for (int w = 1; w < 8; ++w) join(m, s, red_m[w], red_s[w]);
+    logprob[blockIdx.x] = row[targets[blockIdx.x]] - (m + logf(s));
   }
 }
 
 }  // namespace
 
-cudaError_t launch_dense_self_attn(const DenseAttnArgs &a, cudaStream_t s) {
+cudaError_t teacher_attn_prepare() {
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(teacher_attn_kernel<false, 4, 2>, attr, TATTN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_attn_kernel<true, 8, 1>, attr, TATTN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_attn_kernel<false, 4, 1>, attr, TATTN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_attn_kernel<true, 4, 1>, attr, TATTN_SMEM);
+  return e;
+}
+
+cudaError_t launch_teacher_attn(const DenseAttnArgs &a, bool self, cudaStream_t s) {
   if (a.n_groups < 1) return cudaSuccess;
-  if (a.bias_tab != nullptr && a.n_dist > TMAXD) return cudaErrorInvalidValue;      // the head's bias row is held in shared memory
-  dense_self_attn_tc_kernel<<<dim3(a.n_groups, a.H), TT, 0, s>>>(a);
+  if (self && a.bias_tab != nullptr && a.n_dist > TMAXD) return cudaErrorInvalidValue;      // the head's bias row is held in shared memory
+  const dim3 grid(a.n_groups, a.H);
+  if (self && a.block_rows == 128) teacher_attn_kernel<true, 8, 1><<<grid, 256, TATTN_SMEM, s>>>(a);
+  else if (self) teacher_attn_kernel<true, 4, 1><<<grid, 128, TATTN_SMEM, s>>>(a);
+  else if (a.block_rows == 128) teacher_attn_kernel<false, 4, 2><<<grid, 128, TATTN_SMEM, s>>>(a);
+  else teacher_attn_kernel<false, 4, 1><<<grid, 128, TATTN_SMEM, s>>>(a);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_rotate_rows(int rows, int d, const float *qkv, const int32_t *row_sub, const int32_t *row_tau, const float2 *rope_tab,
+                               void *out, cudaStream_t s) {
+  rotate_rows_kernel<<<rows, 256, 0, s>>>(d, qkv, row_sub, row_tau, rope_tab, (__nv_bfloat16 *)out);
   return cudaGetLastError();
 }
 

@@ -337,7 +337,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             __syncwarp();
           }
         }
-        if (m < Mc) {
+        if (m < Mc && a.part_val != nullptr) {
           a.part_val[(size_t)vt * a.rows_cap + m] = bv;
           a.part_idx[(size_t)vt * a.rows_cap + m] = bi;
           if (a.eos >= v_tile0 && a.eos < v_tile0 + wn) a.term_val[2 * m] = te;
