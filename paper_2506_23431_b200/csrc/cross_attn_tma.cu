@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
       n += __popc(m);
     }
     if (lane == 0) n_aseq_s = n;
-  } else if (warp == 2) {   // first query row of every sequence
+  } else if (warp == 2 && a.packed) {   // first query row of every sequence
     int carry = 0;
     for (int c0 = 0; c0 < batch; c0 += 32) {
       const int b = c0 + lane;
@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
       int v = own;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) { int u = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += u; }
-      if (b < batch) row0_s[b] = a.row_base != nullptr ? a.row_base[b] : a.packed ? carry + v - own : b * dm.C;
+      if (b < batch) row0_s[b] = carry + v - own;
       carry += __shfl_sync(0xffffffffu, v, 31);
     }
   }
@@ -370,14 +370,14 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
     const int seg_start = H * pfx_s[b] + h * cur.nt, seg_end = seg_start + cur.nt;
     const int my_end = min(hi, seg_end);
     const int S = nact_s[b], ctx_len = min(max(a.st.ctx_len[b], 1), dm.ctx);
-    const int row0 = row0_s[b];
+    const int row0 = a.packed ? row0_s[b] : a.row_base != nullptr ? a.row_base[b] : b * dm.C;
     float seg_sl2 = sl2, seg_vscale = 1.f;          // 8-bit: the key scale joins the score scale, the value scale the final 1 / l
     if (FP8) {
       const int kv_b = a.kv_seq != nullptr ? a.kv_seq[b] : b;
       const float2 sc2 = *reinterpret_cast<const float2 *>(a.kv_scale + ((((size_t)a.layer * dm.B + kv_b) * H + h) << 1));
       seg_sl2 = sl2 * sc2.x; seg_vscale = sc2.y;
     }
-    uint32_t qf[MT][4][4];
+    uint32_t qf[MT][4][4];             // (plain loads: neighbouring lanes share sectors, and loads past L1 made a launch 1 us slower)
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
       int r_lo = mt * 16 + g, r_hi = r_lo + 8;
@@ -387,8 +387,8 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
         const __nv_bfloat16 *q_hi = qbuf + (size_t)(row0 + r_hi) * dm.d + h * kDh + 4 * tig;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          const uint2 lo = r_lo < S ? __ldcg(reinterpret_cast<const uint2 *>(q_lo + kk * 16)) : make_uint2(0u, 0u);
-          const uint2 hi = r_hi < S ? __ldcg(reinterpret_cast<const uint2 *>(q_hi + kk * 16)) : make_uint2(0u, 0u);
+          const uint2 lo = r_lo < S ? *reinterpret_cast<const uint2 *>(q_lo + kk * 16) : make_uint2(0u, 0u);
+          const uint2 hi = r_hi < S ? *reinterpret_cast<const uint2 *>(q_hi + kk * 16) : make_uint2(0u, 0u);
           qf[mt][kk][0] = bf16x2_to_f16x2(lo.x); qf[mt][kk][2] = bf16x2_to_f16x2(lo.y);
           qf[mt][kk][1] = bf16x2_to_f16x2(hi.x); qf[mt][kk][3] = bf16x2_to_f16x2(hi.y);
         }
@@ -397,10 +397,10 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
         const __nv_bfloat16 *q_hi = qbuf + (size_t)(row0 + r_hi) * dm.d + h * kDh + 2 * tig;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {
-          qf[mt][kk][0] = r_lo < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_lo + kk * 16)) : 0u;
-          qf[mt][kk][1] = r_hi < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_hi + kk * 16)) : 0u;
-          qf[mt][kk][2] = r_lo < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8)) : 0u;
-          qf[mt][kk][3] = r_hi < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8)) : 0u;
+          qf[mt][kk][0] = r_lo < S ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16) : 0u;
+          qf[mt][kk][1] = r_hi < S ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16) : 0u;
+          qf[mt][kk][2] = r_lo < S ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8) : 0u;
+          qf[mt][kk][3] = r_hi < S ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8) : 0u;
         }
       }
     }

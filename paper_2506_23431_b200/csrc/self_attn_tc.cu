@@ -393,10 +393,10 @@ __global__ void __launch_bounds__(STHREADS, MT == 1 ? OCC : 2) self_attn_tc_kern
       const __nv_bfloat16 *q_hi = (const __nv_bfloat16 *)a.q + (size_t)(row0 + r_hi) * dm.d + h * kDh + 2 * tig;
 #pragma unroll
       for (int kk = 0; kk < 4; ++kk) {
-        qf[mt][kk][0] = r_lo < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_lo + kk * 16)) : 0u;
-        qf[mt][kk][1] = r_hi < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_hi + kk * 16)) : 0u;
-        qf[mt][kk][2] = r_lo < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8)) : 0u;
-        qf[mt][kk][3] = r_hi < S ? __ldcg(reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8)) : 0u;
+        qf[mt][kk][0] = r_lo < S ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16) : 0u;
+        qf[mt][kk][1] = r_hi < S ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16) : 0u;
+        qf[mt][kk][2] = r_lo < S ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8) : 0u;
+        qf[mt][kk][3] = r_hi < S ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8) : 0u;
       }
     }
   }
