@@ -68,7 +68,8 @@ pd_status cross_attention_enqueue(int dtype, int batch, int rows_per_seq, int n_
     if (cross_attn_tma_prepare(rows_per_seq, false) != cudaSuccess) return PD_ERR_CUDA;
     return launch_cross_attn_tma(a, tmap, tmap, cross_attn_ctas(), s) == cudaSuccess ? PD_OK : PD_ERR_CUDA;
   }
-  e = launch_attn_core(a, dtype, false, s);
+  if (attn_core_prepare(dtype, false) != cudaSuccess) return PD_ERR_CUDA;
+  e = launch_attn_core(a, dtype, false, false, s);
   if (e != cudaSuccess) return PD_ERR_CUDA;
   if (splits > 1 && launch_attn_merge(a, dtype, s) != cudaSuccess) return PD_ERR_CUDA;
   return PD_OK;

@@ -178,6 +178,7 @@ struct pd_handle {
   VocabMaps vmaps;                 // hidden rows and lm_head for the tcgen05 vocabulary projection
   bool vocab_tc = false;
   bool packed_ok = false;          // bf16, and every kernel of the packed path takes this configuration
+  bool f32_own = false;            // fp32: the layers' products on proj_f32 (at most 32 allocated rows)
   bool rows_packed = false;        // the last step left the activation buffers packed (pd_debug_read)
   // pd_generate_host: host-to-device copies of the encoder memory run on a stream of their own, in
   // chunks of sequences, so that the context projection of one chunk overlaps the copy of the next
@@ -363,7 +364,7 @@ pd_status enqueue_self_attention(pd_handle *h, int layer) {
     h->own_launches++;
     return PD_OK;
   }
-  CU_TRY(h, launch_attn_core(a, dt, true, h->stream));
+  CU_TRY(h, launch_attn_core(a, dt, true, h->f32_own, h->stream));
   h->own_launches++;
   if (a.splits > 1) { CU_TRY(h, launch_attn_merge(a, dt, h->stream)); h->own_launches++; }
   return PD_OK;
@@ -378,7 +379,7 @@ pd_status enqueue_cross_attention(pd_handle *h, int layer) {
     h->own_launches++;
     return PD_OK;
   }
-  CU_TRY(h, launch_attn_core(a, dt, false, h->stream));
+  CU_TRY(h, launch_attn_core(a, dt, false, h->f32_own, h->stream));
   h->own_launches++;
   if (a.splits > 1) { CU_TRY(h, launch_attn_merge(a, dt, h->stream)); h->own_launches++; }
   return PD_OK;
@@ -451,6 +452,52 @@ pd_status enqueue_step_packed(pd_handle *h) {
   return enqueue_vocab(h, ssq);
 }
 
+// The layers of a step in fp32 on the own products (unpacked rows): eight launches per layer, programmatic dependents of one
+// another.  Leaves x and, normalised for the vocabulary projection, hb.
+pd_status enqueue_layers_f32(pd_handle *h) {
+  const Dims &dm = h->dm;
+  const Layout &L = h->lay;
+  cudaStream_t s = h->stream;
+  float *hb = h->ptr<float>(L.hbuf);
+  const bool rope = dm.pos_mode == PD_POS_ROPE;
+  ProjF32Args p;
+  memset(&p, 0, sizeof(p));
+  p.rows = h->batch * dm.C;
+  p.ssq_in = h->ptr<float>(L.ssq); p.parts_in = dm.d / 32; p.ssq_stride = dm.d / 32; p.inv_width = 1.f / (float)dm.d; p.eps = dm.eps;
+  p.x = h->ptr<float>(L.x); p.ssq_out = h->ptr<float>(L.ssq);
+  p.row_meta = h->st.row_meta; p.rope_tab = rope ? h->ptr<float2>(L.rope_tab) : nullptr;
+  p.kv_pool = h->ptr<float>(L.kv_pool); p.pool = dm.pool; p.P = dm.P;
+  auto f = [](const void *q) { return static_cast<const float *>(q); };
+  for (int l = 0; l < dm.L; ++l) {
+    const void *const *lw = &h->layer_w[(size_t)l * kLayerTensors];
+    ProjF32Args a = p;
+    a.act = hb; a.w = f(lw[1]); a.K = dm.d; a.N = 3 * dm.d; a.layer = l; a.out = h->ptr<float>(L.qbuf);
+    if (l == 0) a.ssq_in = nullptr;                   // the embedding kernel leaves normalised rows
+    a.raw = l == dm.L - 1 ? h->ptr<float>(L.qkv) : nullptr;
+    OWN(h, PD_PROF_GEMM, launch_proj_f32(PROJ_QKV, a, s));
+    {
+      ProfScope ps(h, PD_PROF_SELF_ATTN);
+      PD_TRY(enqueue_self_attention(h, l));
+    }
+    a = p; a.act = h->ptr<float>(L.self_out); a.w = f(lw[2]); a.K = dm.d; a.N = dm.d; a.out = hb; a.gain_next = f(lw[3]);
+    OWN(h, PD_PROF_GEMM, launch_proj_f32(PROJ_RESID, a, s));
+    a = p; a.act = hb; a.w = f(lw[4]); a.K = dm.d; a.N = dm.d; a.out = h->ptr<float>(L.cq);
+    OWN(h, PD_PROF_GEMM, launch_proj_f32(PROJ_STORE, a, s));
+    {
+      ProfScope ps(h, PD_PROF_CROSS_ATTN);
+      PD_TRY(enqueue_cross_attention(h, l));
+    }
+    a = p; a.act = h->ptr<float>(L.cross_out); a.w = f(lw[6]); a.K = dm.d; a.N = dm.d; a.out = hb; a.gain_next = f(lw[7]);
+    OWN(h, PD_PROF_GEMM, launch_proj_f32(PROJ_RESID, a, s));
+    a = p; a.act = hb; a.w = f(lw[8]); a.K = dm.d; a.N = dm.ff; a.out = h->ptr<float>(L.ffn);
+    OWN(h, PD_PROF_GEMM, launch_proj_f32(PROJ_RELU, a, s));
+    a = p; a.act = h->ptr<float>(L.ffn); a.w = f(lw[9]); a.K = dm.ff; a.N = dm.d; a.out = hb;
+    a.gain_next = f(l + 1 < dm.L ? h->layer_w[(size_t)(l + 1) * kLayerTensors] : h->w.final_norm);
+    OWN(h, PD_PROF_GEMM, launch_proj_f32(PROJ_RESID, a, s));
+  }
+  return PD_OK;
+}
+
 // The same on unpacked rows (row c of sequence b at b * C + c).
 pd_status enqueue_step(pd_handle *h) {
   h->rows_packed = packed_path(h);
@@ -466,7 +513,8 @@ pd_status enqueue_step(pd_handle *h) {
   float *logits = h->ptr<float>(h->lay.logits);
 
   OWN(h, PD_PROF_OTHER, launch_embed(dm, h->st, h->batch, dt, h->w.embed, x, h->layer_w[0], hb, s));   // with the first layer's norm
-  for (int l = 0; l < dm.L; ++l) {
+  if (h->f32_own) PD_TRY(enqueue_layers_f32(h));
+  for (int l = 0; l < dm.L && !h->f32_own; ++l) {
     const void *const *lw = &h->layer_w[(size_t)l * kLayerTensors];
     if (l > 0) OWN(h, PD_PROF_OTHER, launch_rmsnorm(dm, M, dt, x, lw[0], hb, s));
     if (fused_append(h) != 0) {
@@ -654,6 +702,7 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
       (launch_build_bias_table(dm, weights->rel_bias, cfg->rel_buckets, h->ptr<int32_t>(L.dist_bucket), h->ptr<float>(L.bias_tab),
                                h->stream) != cudaSuccess || cudaStreamSynchronize(h->stream) != cudaSuccess))
     return bail(PD_ERR_CUDA);
+  if (attn_core_prepare(cfg->dtype, true) != cudaSuccess || attn_core_prepare(cfg->dtype, false) != cudaSuccess) return bail(PD_ERR_CUDA);
   h->kv8 = cfg->kv_c_dtype == PD_KV_E4M3;
   if (cfg->dtype == PD_DTYPE_BF16 && dm.C <= 32) {
     pd_status s = make_tensor_map(h);
@@ -680,6 +729,15 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
                          cudaMemsetAsync(h->ptr<void>(L.row_at), 0xFF, L.row_at.bytes, h->stream) != cudaSuccess ||
                          cudaStreamSynchronize(h->stream) != cudaSuccess))
       return bail(PD_ERR_CUDA);
+  }
+  if (cfg->dtype == PD_DTYPE_FP32) {
+    // own products while the step is a chain of launches: at most 32 allocated rows
+    const int spec[6][3] = {{1, dm.d, 3 * dm.d}, {2, dm.d, dm.d}, {4, dm.d, dm.d}, {6, dm.d, dm.d}, {8, dm.d, dm.ff}, {9, dm.ff, dm.d}};
+    h->f32_own = true;
+    for (int l = 0; l < dm.L; ++l)
+      for (const auto &sp : spec)
+        h->f32_own = h->f32_own && proj_f32_supported(sp[1], sp[2], dm.B * dm.C, h->layer_w[(size_t)l * kLayerTensors + sp[0]]);
+    if (h->f32_own && proj_f32_prepare() != cudaSuccess) return bail(PD_ERR_CUDA);
   }
   *out = h;
   return PD_OK;
@@ -727,19 +785,17 @@ pd_status encode_prepare(pd_handle *h, const int32_t *ctx_len, int32_t batch, co
   if (batch != h->batch) drop_graph(h);
   h->batch = batch;
   make_ff_plan(h, batch * dm.C, dm.ff, dm.d);   // host-side planning, kept out of any stream capture
-  // split-K factors
+  // Split-K factors.  Plain-ALU kernel: a CTA takes eight tiles (pages, 32 context positions) at a time and a tile round costs
+  // about a microsecond, a split the merge launch and its round trip (about 4 us): a split once it saves four rounds.
   auto cdiv = [](int a, int b) { return (a + b - 1) / b; };
-  const int bh = batch * dm.H;
-  int ss = h->cfg.self_splits > 0 ? h->cfg.self_splits : cdiv(2 * 148, bh);
-  if (ss > 8 && h->cfg.self_splits == 0) ss = 8;
+  const int bh = batch * dm.H, ctas = bh * cdiv(dm.C, kCoreRows);
+  auto core_splits = [&](int tiles) {
+    const int by_gpu = cdiv(2 * 148, ctas), by_work = tiles / (4 * 8);
+    return std::max(1, std::min(std::min(by_gpu, by_work), 8));
+  };
+  int ss = h->cfg.self_splits > 0 ? h->cfg.self_splits : core_splits(dm.SM * dm.PPS);
   if (h->cfg.self_splits == 0 && self_tc(h)) ss = self_attn_tc_splits(dm, bh, h->cross_ctas / 2);   // the kernel uses as many of them as the lists need
-  int cs = h->cfg.cross_splits;
-  if (cs == 0) {
-    int tiles = cdiv(dm.ctx, 128);
-    cs = cdiv(4 * 148, bh);
-    int cap = tiles / 2 > 1 ? tiles / 2 : 1;
-    if (cs > cap) cs = cap;
-  }
+  int cs = h->cfg.cross_splits > 0 ? h->cfg.cross_splits : core_splits(cdiv(dm.ctx, 32));
   if (ss > h->max_splits) ss = h->max_splits;
   if (cs > h->max_splits) cs = h->max_splits;
   if (ss != h->self_splits || cs != h->cross_splits) drop_graph(h);

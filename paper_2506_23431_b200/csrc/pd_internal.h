@@ -161,7 +161,9 @@ cudaError_t launch_append_copy_bf16(const Dims &dm, const DecState &st, int batc
                                     void *kv_pool, cudaStream_t s);
 cudaError_t launch_ctx_kv_relayout(const Dims &dm, int b0, int batch, int layer, int dtype, const void *proj, void *kv_c,
                                    cudaStream_t s);
-cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, cudaStream_t s);
+constexpr int kCoreRows = 16;            // rows per CTA of the plain-ALU attention kernel
+cudaError_t attn_core_prepare(int dtype, bool self);      // once per device, outside any stream capture
+cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, bool pdl, cudaStream_t s);
 cudaError_t launch_attn_merge(const AttnArgs &a, int dtype, cudaStream_t s);
 constexpr int kMaxCrossCtas = 320;      // persistent cross-attention CTAs (two per SM) the scratch is sized for
 cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, int n_ctas, cudaStream_t s);
@@ -239,6 +241,24 @@ bool proj_mma_supported(int K, int N, const void *w);
 int proj_mma_parts(int N);               // column tiles = parts of ssq_out
 cudaError_t proj_mma_prepare();          // once per device, outside any stream capture
 cudaError_t launch_proj_mma(int epi, const ProjArgs &a, cudaStream_t s);
+
+// ---- the same layers in fp32 over few unpacked rows (proj_f32.cu) ---------------------------------------
+struct ProjF32Args {
+  const float *act, *w;      // [rows][K]; [K][N]
+  int K, N, rows;            // at most 32 rows
+  // scale of the RMSNorm in front of the layer: rsqrt(sum_p ssq_in[m][p] * inv_width + eps); ssq_in null: none
+  const float *ssq_in; int parts_in, ssq_stride; float inv_width, eps;
+  float *out;                // [rows][N] (PROJ_QKV: the queries, [rows][N / 3])
+  float *x;                  // PROJ_RESID: residual stream [rows][N]; out = x * gain_next
+  const float *gain_next;
+  float *ssq_out;            // PROJ_RESID: [rows][ssq_stride], one part per 32 columns
+  const int4 *row_meta; const float2 *rope_tab;      // PROJ_QKV: as in ProjArgs
+  float *kv_pool; int layer, pool, P;
+  float *raw;                // PROJ_QKV: the unrotated product [rows][N] as well, or null
+};
+bool proj_f32_supported(int K, int N, int rows, const void *w);
+cudaError_t proj_f32_prepare();          // once per device, outside any stream capture
+cudaError_t launch_proj_f32(int epi, const ProjF32Args &a, cudaStream_t s);
 
 // ---- skinny-M linear layers on tcgen05 (linear_tc.cu) --------------------------------------------
 enum { LIN_EPI_STORE = 0,   // out = bf16(acc * row_scale)
