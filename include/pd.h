@@ -308,12 +308,10 @@ PD_API pd_status pd_get_stats(pd_handle *h, int64_t *stats);
  *                result for that sequence, never an access outside the tensors)
  *   splits       1..32: split-K factor over the context of the plain-ALU kernel (fp32, or more
  *                than 32 rows per sequence; partials are merged by a second kernel).  The bf16
- *                tensor-core kernel divides the context tiles of all sequences evenly over the
- *                GPU by itself and merges its partials in the same launch.
+ *                tensor-core kernel spreads the context tiles over the GPU by itself.
  *   scratch      device, 256-byte aligned, at least pd_cross_attention_scratch_bytes(...): a
  *                256-byte header (int32 word 2 receives PD_ERR_TIMEOUT if a bounded wait inside
- *                the kernel expired) and per-(sequence, head) arrival counters, both cleared by
- *                the call, then the partial results
+ *                the kernel expired, else 0), then the partial results
  * rows_per_seq <= 64.  Enqueues on cuda_stream (a cudaStream_t) and returns; allocates nothing on
  * the device.  The caller owns every buffer and keeps it alive until the stream has passed the
  * call.  PD_ERR_ARG for null pointers or sizes out of range, PD_ERR_WORKSPACE for a scratch
@@ -385,11 +383,8 @@ PD_API pd_status pd_linear(int32_t rows, int32_t d_in, int32_t d_out, int32_t mo
  * out exactly as for pd_cross_attention; results are the same.
  *  - Sizes whose partials would not fit are refused with PD_ERR_WORKSPACE and a message in
  *    pd_static_last_error(); use fewer splits, fewer sequences or rows per call, or
- *    pd_cross_attention with a buffer of your own.  What is needed depends on the kernel that
- *    runs: the bf16 tensor-core kernel (at most 32 rows per sequence) keeps per-CTA records
- *    (2.9 MiB up to 16 rows, 5.9 MiB up to 32, whatever the batch), the plain-ALU kernel (fp32,
- *    or 33..64 rows) batch*rows*heads*splits*264 bytes; pd_cross_attention_scratch_bytes() is
- *    the larger of the two.
+ *    pd_cross_attention with a buffer of your own.  What is needed is what
+ *    pd_cross_attention_scratch_bytes() says: batch*rows*heads*splits*264 bytes and the header.
  *  - Calls no cudaMalloc, cudaFree or any other allocating routine.  The first call on a device
  *    looks up the array's device address (cudaGetSymbolAddress, with the current device, which
  *    must be the device of the stream and of the buffers); make that first call before any

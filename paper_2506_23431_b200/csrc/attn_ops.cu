@@ -8,20 +8,13 @@ using namespace pd;
 
 namespace pd {
 
-// Scratch of the stand-alone op: header, arrival counters, partial results.  The flat partial records
-// of the tensor-core kernel are only reserved where that kernel can run (bf16, at most 32 rows per
-// sequence); the plain-ALU kernel needs the split-K records alone.
-size_t cross_attention_scratch_layout(int dtype, int batch, int rows_per_seq, int n_heads, int splits, size_t *off_tickets,
-                                      size_t *off_part_o, size_t *off_part_ml) {
+// Scratch of the stand-alone op: header, split-K records of the plain-ALU kernel.
+size_t cross_attention_scratch_layout(int batch, int rows_per_seq, int n_heads, int splits, size_t *off_part_o,
+                                      size_t *off_part_ml) {
   const size_t rows = (size_t)batch * rows_per_seq;
   size_t off = kOpHeaderBytes;
-  if (off_tickets) *off_tickets = off;
-  off += ((size_t)batch * n_heads * sizeof(int32_t) + 255) / 256 * 256;      // cleared with the header
   if (off_part_o) *off_part_o = off;
-  const size_t split_bytes = rows * n_heads * splits * kDh * sizeof(float);
-  const bool tensor_core = dtype == PD_DTYPE_BF16 && rows_per_seq <= 32;
-  const size_t flat_bytes = tensor_core ? cross_attn_tma_partial_bytes(kMaxCrossCtas, rows_per_seq) : 0;
-  off += ((split_bytes > flat_bytes ? split_bytes : flat_bytes) + 255) / 256 * 256;
+  off += (rows * n_heads * splits * kDh * sizeof(float) + 255) / 256 * 256;
   if (off_part_ml) *off_part_ml = off;
   off += (rows * n_heads * splits * 2 * sizeof(float) + 255) / 256 * 256;
   return off;
@@ -41,10 +34,9 @@ bool cross_attention_args_ok(int dtype, int batch, int rows_per_seq, int n_heads
 pd_status cross_attention_enqueue(int dtype, int batch, int rows_per_seq, int n_heads, int max_ctx, float attn_scale,
                                   int splits, const void *q, const void *kv, const int32_t *n_rows,
                                   const int32_t *ctx_len, void *out, void *scratch, cudaStream_t s) {
-  size_t off_t = 0, off_o = 0, off_ml = 0;
-  cross_attention_scratch_layout(dtype, batch, rows_per_seq, n_heads, splits, &off_t, &off_o, &off_ml);
+  size_t off_o = 0, off_ml = 0;
+  cross_attention_scratch_layout(batch, rows_per_seq, n_heads, splits, &off_o, &off_ml);
   uint8_t *base = reinterpret_cast<uint8_t *>(scratch);
-  if (cudaMemsetAsync(base, 0, off_o, s) != cudaSuccess) return PD_ERR_CUDA;      // header and arrival counters
 
   AttnArgs a;
   memset(&a, 0, sizeof(a));
@@ -59,18 +51,17 @@ pd_status cross_attention_enqueue(int dtype, int batch, int rows_per_seq, int n_
   a.q = q; a.kv = kv; a.out = out;
   a.part_o = reinterpret_cast<float *>(base + off_o);
   a.part_ml = reinterpret_cast<float *>(base + off_ml);
-  a.tickets = reinterpret_cast<int32_t *>(base + off_t);
 
-  cudaError_t e;
-  if (dtype == PD_DTYPE_BF16 && cross_attn_tma_supported(dm, batch)) {
+  if (dtype == PD_DTYPE_BF16 && cross_attn_tma_supported(dm)) {
     CUtensorMap tmap;
     if (encode_ctx_kv_tensor_map(&tmap, kv, (uint64_t)batch * n_heads * 2 * max_ctx, nullptr) != cudaSuccess) return PD_ERR_CUDA;
     if (cross_attn_tma_prepare(rows_per_seq, false) != cudaSuccess) return PD_ERR_CUDA;
-    return launch_cross_attn_tma(a, tmap, tmap, cross_attn_ctas(), s) == cudaSuccess ? PD_OK : PD_ERR_CUDA;
+    a.clear_status = 1;      // one launch is the whole call: a separate clear of the header cost 2 us
+    return launch_cross_attn_tma(a, tmap, tmap, s) == cudaSuccess ? PD_OK : PD_ERR_CUDA;
   }
+  if (cudaMemsetAsync(base, 0, kOpHeaderBytes, s) != cudaSuccess) return PD_ERR_CUDA;
   if (attn_core_prepare(dtype, false) != cudaSuccess) return PD_ERR_CUDA;
-  e = launch_attn_core(a, dtype, false, false, s);
-  if (e != cudaSuccess) return PD_ERR_CUDA;
+  if (launch_attn_core(a, dtype, false, false, s) != cudaSuccess) return PD_ERR_CUDA;
   if (splits > 1 && launch_attn_merge(a, dtype, s) != cudaSuccess) return PD_ERR_CUDA;
   return PD_OK;
 }
@@ -81,7 +72,7 @@ extern "C" {
 
 size_t pd_cross_attention_scratch_bytes(int32_t batch, int32_t rows_per_seq, int32_t n_heads, int32_t splits) {
   if (!cross_attention_args_ok(PD_DTYPE_BF16, batch, rows_per_seq, n_heads, 1, 1.f, splits)) return 0;
-  return cross_attention_scratch_layout(PD_DTYPE_BF16, batch, rows_per_seq, n_heads, splits, nullptr, nullptr, nullptr);   // the larger of the two types
+  return cross_attention_scratch_layout(batch, rows_per_seq, n_heads, splits, nullptr, nullptr);
 }
 
 pd_status pd_cross_attention(int32_t dtype, int32_t batch, int32_t rows_per_seq, int32_t n_heads, int32_t max_ctx,
@@ -91,7 +82,7 @@ pd_status pd_cross_attention(int32_t dtype, int32_t batch, int32_t rows_per_seq,
   if (!cross_attention_args_ok(dtype, batch, rows_per_seq, n_heads, max_ctx, attn_scale, splits)) return PD_ERR_ARG;
   if (reinterpret_cast<uintptr_t>(kv) % 16 != 0 || reinterpret_cast<uintptr_t>(q) % 16 != 0 ||
       reinterpret_cast<uintptr_t>(out) % 16 != 0 || reinterpret_cast<uintptr_t>(scratch) % 256 != 0) return PD_ERR_ARG;
-  if (scratch_bytes < cross_attention_scratch_layout(dtype, batch, rows_per_seq, n_heads, splits, nullptr, nullptr, nullptr))
+  if (scratch_bytes < cross_attention_scratch_layout(batch, rows_per_seq, n_heads, splits, nullptr, nullptr))
     return PD_ERR_WORKSPACE;
   return cross_attention_enqueue(dtype, batch, rows_per_seq, n_heads, max_ctx, attn_scale, splits, q, kv, n_rows, ctx_len,
                                  out, scratch, reinterpret_cast<cudaStream_t>(cuda_stream));

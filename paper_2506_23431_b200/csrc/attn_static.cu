@@ -60,7 +60,7 @@ pd_status pd_cross_attention_static(int32_t dtype, int32_t batch, int32_t rows_p
     return fail(PD_ERR_ARG, "a size or parameter is out of range");
   if (reinterpret_cast<uintptr_t>(kv) % 16 != 0 || reinterpret_cast<uintptr_t>(q) % 16 != 0 || reinterpret_cast<uintptr_t>(out) % 16 != 0)
     return fail(PD_ERR_ARG, "q, kv and out must be 16-byte aligned");
-  const size_t need = cross_attention_scratch_layout(dtype, batch, rows_per_seq, n_heads, splits, nullptr, nullptr, nullptr);
+  const size_t need = cross_attention_scratch_layout(batch, rows_per_seq, n_heads, splits, nullptr, nullptr);
   if (need > kStaticScratchBytes)
     return fail(PD_ERR_WORKSPACE, "these sizes need %lld bytes of scratch; the built-in scratch holds %lld "
                                   "(fewer splits, fewer sequences or rows per call, or pd_cross_attention with a buffer of your own)",

@@ -132,10 +132,7 @@ void make_layout(const pd_config &c, const Dims &dm, int max_splits, Layout &L) 
     reg(L.vpart_idx, tiles * M * 4);
     reg(L.vterm, M * 2 * 4);
   }
-  {
-    size_t split_bytes = M * dm.H * max_splits * kDh * 4, flat_bytes = cross_attn_tma_partial_bytes(kMaxCrossCtas, dm.C);
-    reg(L.part_o, split_bytes > flat_bytes ? split_bytes : flat_bytes);
-  }
+  reg(L.part_o, M * dm.H * max_splits * kDh * 4);
   reg(L.part_ml, M * dm.H * max_splits * 2 * 4);
   if (c.kv_c_dtype == PD_KV_E4M3) {
     reg(L.kv_c, (size_t)dm.L * B * dm.ctx * 2 * dm.d);                       // one byte per value
@@ -192,7 +189,7 @@ struct pd_handle {
   int batch = 0;
   bool encoded = false;
   int self_splits = 1, cross_splits = 1;
-  int cross_ctas = 296;
+  int sms = 148;
   int steps_enqueued = 0;
   bool teacher_clear = false;
   // graph
@@ -327,7 +324,7 @@ int fused_append(const pd_handle *h) {
 // 58 us against 40 us): there the unpacked path below, with cuBLAS over the allocated rows, stays.
 constexpr int kPackedMaxRows = 128;
 bool packed_path(const pd_handle *h) {
-  return h->packed_ok && h->batch * h->dm.C <= kPackedMaxRows && cross_attn_tma_supported(h->dm, h->batch);
+  return h->packed_ok && h->batch * h->dm.C <= kPackedMaxRows && cross_attn_tma_supported(h->dm);
 }
 
 AttnArgs attn_args(pd_handle *h, int layer, bool self) {
@@ -347,6 +344,7 @@ AttnArgs attn_args(pd_handle *h, int layer, bool self) {
   a.qkv = h->ptr<void>(h->lay.qkv);
   a.fused_append = self ? fused_append(h) : 0;
   a.packed = packed_path(h) ? 1 : 0;
+  a.clear_status = 0;
   a.rope_tab = h->ptr<float2>(h->lay.rope_tab);
   a.kv_scale = (!self && h->kv8) ? h->ptr<float>(h->lay.kv_scale) : nullptr;
   a.kv_seq = nullptr; a.row_base = nullptr;
@@ -374,8 +372,8 @@ pd_status enqueue_self_attention(pd_handle *h, int layer) {
 pd_status enqueue_cross_attention(pd_handle *h, int layer) {
   const int dt = h->cfg.dtype;
   AttnArgs a = attn_args(h, layer, false);
-  if (dt == PD_DTYPE_BF16 && h->have_tmap && cross_attn_tma_supported(h->dm, h->batch)) {
-    CU_TRY(h, launch_cross_attn_tma(a, h->tmap_kvc, h->kv8 ? h->tmap_kvc_v : h->tmap_kvc, h->cross_ctas, h->stream));   // merges its own partials
+  if (dt == PD_DTYPE_BF16 && h->have_tmap && cross_attn_tma_supported(h->dm)) {
+    CU_TRY(h, launch_cross_attn_tma(a, h->tmap_kvc, h->kv8 ? h->tmap_kvc_v : h->tmap_kvc, h->stream));   // merges its own partials
     h->own_launches++;
     return PD_OK;
   }
@@ -708,7 +706,8 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
     pd_status s = make_tensor_map(h);
     if (s != PD_OK) return bail(s);
     if (cross_attn_tma_prepare(dm.C, h->kv8) != cudaSuccess || cross_attn_tma_prepare(kTfGroup, h->kv8) != cudaSuccess) return bail(PD_ERR_CUDA);   // decode, teacher-forced groups
-    h->cross_ctas = cross_attn_ctas();
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0) h->sms = sms;
   }
   if (cfg->dtype == PD_DTYPE_BF16 && self_attn_tc_supported(dm) && self_attn_tc_prepare() != cudaSuccess) return bail(PD_ERR_CUDA);
   if (cfg->dtype == PD_DTYPE_BF16 && vocab_tc_supported(dm.d, dm.V) && reinterpret_cast<uintptr_t>(weights->lm_head) % 16 == 0) {
@@ -794,7 +793,7 @@ pd_status encode_prepare(pd_handle *h, const int32_t *ctx_len, int32_t batch, co
     return std::max(1, std::min(std::min(by_gpu, by_work), 8));
   };
   int ss = h->cfg.self_splits > 0 ? h->cfg.self_splits : core_splits(dm.SM * dm.PPS);
-  if (h->cfg.self_splits == 0 && self_tc(h)) ss = self_attn_tc_splits(dm, bh, h->cross_ctas / 2);   // the kernel uses as many of them as the lists need
+  if (h->cfg.self_splits == 0 && self_tc(h)) ss = self_attn_tc_splits(dm, bh, h->sms);   // the kernel uses as many of them as the lists need
   int cs = h->cfg.cross_splits > 0 ? h->cfg.cross_splits : core_splits(cdiv(dm.ctx, 32));
   if (ss > h->max_splits) ss = h->max_splits;
   if (cs > h->max_splits) cs = h->max_splits;
@@ -987,8 +986,8 @@ pd_status pd_collect_row(pd_handle *h, int32_t row, int32_t *tokens, int32_t *le
 
 // ---- the teacher-forced forward of Eq. 6 -----------------------------------------------------------------
 namespace {
-constexpr int kTfCrossBatch = 256;    // groups per cross-attention launch
-struct TfLayout { size_t tables, x, hb, qkv, rot, att, cq, co, ffn, logprob, part, tickets, logits, total; int logit_rows; };
+constexpr int kTfCrossBatch = 32768;    // groups per cross-attention launch (a grid dimension)
+struct TfLayout { size_t tables, x, hb, qkv, rot, att, cq, co, ffn, logprob, logits, total; int logit_rows; };
 
 TfLayout tf_layout(const Dims &dm, size_t rows, bool own_logits) {
   TfLayout L;
@@ -1005,8 +1004,6 @@ TfLayout tf_layout(const Dims &dm, size_t rows, bool own_logits) {
   L.co = reg(rows * dm.d * 2);
   L.ffn = reg(rows * dm.ff * 2);
   L.logprob = reg(rows * 4);
-  L.part = reg(cross_attn_tma_partial_bytes(kMaxCrossCtas, kTfGroup));
-  L.tickets = reg((size_t)kTfCrossBatch * dm.H * 4);
   L.logit_rows = 0;
   L.logits = off;
   if (own_logits) {
@@ -1094,7 +1091,6 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
   int32_t *d_grow0 = put(g_row0), *d_gn = put(g_n), *d_gseq = put(g_seq), *d_gctx = put(g_ctx);
   int32_t *d_brow0 = put(b_row0), *d_bn = put(b_n), *d_bsrow0 = put(b_srow0), *d_bsrows = put(b_srows), *d_bseq = put(b_seq), *d_bctx = put(b_ctx);
   CU_TRY(h, cudaMemcpyAsync(tab, tables.data(), tables.size() * 4, cudaMemcpyHostToDevice, s));
-  if (h->kv8) CU_TRY(h, cudaMemsetAsync(base + L.tickets, 0, (size_t)kTfCrossBatch * dm.H * 4, s));
 
   float *x = reinterpret_cast<float *>(base + L.x);
   void *hb = base + L.hb, *qkv = base + L.qkv, *att = base + L.att, *cq = base + L.cq, *co = base + L.co, *ffn = base + L.ffn;
@@ -1126,7 +1122,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
       da.kv_c = h->ptr<__nv_bfloat16>(h->lay.kv_c); da.layer = l; da.B = dm.B; da.ctx = dm.ctx;
       OWN(h, PD_PROF_CROSS_ATTN, launch_teacher_attn(da, false, s));
     }
-    for (size_t g0 = 0; g0 < G; g0 += kTfCrossBatch) {              // 8-bit context: groups as "sequences" of the batched kernel, 256 at a time
+    for (size_t g0 = 0; g0 < G; g0 += kTfCrossBatch) {              // 8-bit context: groups as "sequences" of the batched kernel
       AttnArgs a = attn_args(h, l, false);
       a.dm.C = kTfGroup;
       a.batch = (int)std::min<size_t>(kTfCrossBatch, G - g0);
@@ -1134,9 +1130,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
       a.st.n_active = d_gn + g0; a.st.ctx_len = d_gctx + g0;
       a.packed = 0;
       a.kv_seq = d_gseq + g0; a.row_base = d_grow0 + g0;
-      a.part_o = reinterpret_cast<float *>(base + L.part);
-      a.tickets = reinterpret_cast<int32_t *>(base + L.tickets);
-      OWN(h, PD_PROF_CROSS_ATTN, launch_cross_attn_tma(a, h->tmap_kvc, h->kv8 ? h->tmap_kvc_v : h->tmap_kvc, h->cross_ctas, s));
+      OWN(h, PD_PROF_CROSS_ATTN, launch_cross_attn_tma(a, h->tmap_kvc, h->kv8 ? h->tmap_kvc_v : h->tmap_kvc, s));
     }
     PD_TRY(gemm(h, false, M, dm.d, dm.d, co, lw[6], x, true, 1.f));
     OWN(h, PD_PROF_OTHER, launch_rmsnorm(dm, M, PD_DTYPE_BF16, x, lw[7], hb, s));

@@ -98,7 +98,7 @@ struct AttnArgs {
   const float *rel_bias;       // [H, rel_buckets]
   int rel_buckets;
   const float *bias_tab;       // [H, n_dist]: rel_bias[h][bucket(dist)] * log2(e), or null
-  int32_t *tickets;            // one arrival counter per (sequence, head), zero between launches
+  int32_t *tickets;            // self-attention: one arrival counter per (sequence, head), zero between launches
   // tensor-core self-attention with the step's KV-append inside it: the projection's output [rows][3 d] in
   // bf16 (fused_append = 1) or in fp32, to be rotated with rope_tab (fused_append = 2); 0 = the append kernel ran
   const void *qkv;
@@ -107,6 +107,7 @@ struct AttnArgs {
   // rows of q and out: 1 = the step's active rows packed back to back in (sequence, row) order, the step's keys/values are in the
   // cache, and the launch is a programmatic dependent of the one before it; 0 = row c of sequence b at b * C + c
   int packed;
+  int clear_status;            // stand-alone op: the kernel clears the status word itself
   // cross-attention over 8-bit keys/values: [layer][sequence][head][keys | values] fp32 scales (else null)
   const float *kv_scale;
   // cross-attention over row groups that are not one per sequence (the teacher-forced forward: many rows per
@@ -165,15 +166,12 @@ constexpr int kCoreRows = 16;            // rows per CTA of the plain-ALU attent
 cudaError_t attn_core_prepare(int dtype, bool self);      // once per device, outside any stream capture
 cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, bool pdl, cudaStream_t s);
 cudaError_t launch_attn_merge(const AttnArgs &a, int dtype, cudaStream_t s);
-constexpr int kMaxCrossCtas = 320;      // persistent cross-attention CTAs (two per SM) the scratch is sized for
-cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, int n_ctas, cudaStream_t s);
+cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, cudaStream_t s);
 cudaError_t encode_ctx_kv8_tensor_maps(CUtensorMap *map_k, CUtensorMap *map_v, const void *base, uint64_t n_blocks, uint64_t ctx,
                                        int *driver_code);
 cudaError_t launch_ctx_kv_quantize(const Dims &dm, int b0, int batch, int layer, const void *proj, const int32_t *ctx_len_dev,
                                    float *scale, float *amax, void *kv8, cudaStream_t s);
-size_t cross_attn_tma_partial_bytes(int n_ctas, int rows_per_seq);
-bool cross_attn_tma_supported(const Dims &dm, int batch);
-int cross_attn_ctas();                  // 2 x SM count of the current device, capped at kMaxCrossCtas
+bool cross_attn_tma_supported(const Dims &dm);
 cudaError_t launch_build_bias_table(const Dims &dm, const float *rel_bias, int rel_buckets, const int32_t *dist_bucket,
                                     float *bias_tab, cudaStream_t s);
 bool self_attn_tc_supported(const Dims &dm);
@@ -185,7 +183,6 @@ cudaError_t launch_argmax_sched(const Dims &dm, const DecState &st, int batch, c
 cudaError_t launch_pick_sched(const Dims &dm, const DecState &st, int batch, int tiles, const float *part_val,
                               const int32_t *part_idx, const float *term_val, const int32_t *teacher, cudaStream_t s);
 cudaError_t encode_ctx_kv_tensor_map(CUtensorMap *out, const void *base, uint64_t rows, int *driver_code);
-int cross_attn_tma_smem_bytes();
 cudaError_t cross_attn_tma_prepare(int rows_per_seq, bool fp8);   // once per device, outside any stream capture
 
 
@@ -291,8 +288,7 @@ cudaError_t launch_linear_tc(const LinearActMaps &map_a, const CUtensorMap &map_
 cudaError_t launch_transpose_bf16(int K, int N, const void *w, void *wt, cudaStream_t s);
 
 // ---- stand-alone cross-attention (attn_ops.cu) ---------------------------------------------
-size_t cross_attention_scratch_layout(int dtype, int batch, int rows_per_seq, int n_heads, int splits, size_t *off_tickets,
-                                      size_t *off_part_o, size_t *off_part_ml);
+size_t cross_attention_scratch_layout(int batch, int rows_per_seq, int n_heads, int splits, size_t *off_part_o, size_t *off_part_ml);
 bool cross_attention_args_ok(int dtype, int batch, int rows_per_seq, int n_heads, int max_ctx, float attn_scale, int splits);
 pd_status cross_attention_enqueue(int dtype, int batch, int rows_per_seq, int n_heads, int max_ctx, float attn_scale,
                                   int splits, const void *q, const void *kv, const int32_t *n_rows, const int32_t *ctx_len,
