@@ -1,0 +1,115 @@
+"""Small decodes, forwards and operator calls at the edges of the kernels' tiles and of the rules that choose between
+kernels, against the CPU oracle on the same seeded inputs.  Tolerances: the decode and forward bars of the other GPU tests
+(1e-4 fp32, 2e-2 bf16 on logits of this scale); the operator's follow from its roundings, stated beside them."""
+import numpy as np
+import pytest
+
+from paper_2506_23431_b200 import workload as W
+from tests import parity
+from tests.test_gpu_kernels import cross_case, oracle_cross
+from tests.test_gpu_parity import check
+from tests.test_gpu_teacher_forward import run_case
+
+pytestmark = pytest.mark.gpu
+
+BASE = dict(d_model=192, n_heads=3, n_layers=2, vocab=515, norm_gain_std=0.1, ctx=150, delta_t=1)
+T5, ROPE = W.POS_T5_BIAS, W.POS_ROPE
+
+DECODES = [
+    # storage, sequences, open rows per sequence, inner width, positions, longest subsequence, 8-bit context
+    ("bf16", 1, 1, 264, ROPE, 30, False),      # one row; an inner width that ends inside a 32-wide K unit
+    ("bf16", 1, 16, 1024, T5, 20, False),      # one full 16-row tile; the longest reduction that one CTA takes
+    ("bf16", 1, 17, 1048, ROPE, 20, False),    # one row in the second tile; a reduction over two CTAs, the second nearly empty
+    ("bf16", 3, 11, 520, T5, 14, True),        # sequences that share a row tile; 8-bit context
+    ("bf16", 4, 32, 2056, ROPE, 34, False),    # 128 rows: the most that run packed; three CTAs per reduction
+    ("bf16", 4, 32, 264, T5, 34, True),        # the same with two query tiles per sequence over 8-bit context
+    ("bf16", 3, 43, 264, T5, 45, False),       # 129 rows and more than 32 in a sequence: the kernels beyond
+    ("bf16", 5, 26, 264, ROPE, 28, False),     # 130 rows, unpacked, two query tiles
+    ("fp32", 1, 1, 264, ROPE, 30, False),
+    ("fp32", 1, 16, 1024, T5, 20, False),
+    ("fp32", 1, 17, 1032, ROPE, 20, False),    # second row tile, second chunk of attention rows, reduction over two CTAs
+    ("fp32", 2, 16, 520, T5, 18, False),       # 32 rows: the most that the fp32 products take
+    ("fp32", 3, 11, 264, ROPE, 14, False),     # 33 rows: library products
+    ("fp32", 1, 64, 264, T5, 66, False),       # four chunks of attention rows
+]
+
+
+@pytest.mark.parametrize("dtype,batch,rows,d_ff,pos,length,kv8", DECODES)
+def test_decode_at_row_and_reduction_edges(dtype, batch, rows, d_ff, pos, length, kv8):
+    base = W.CONFIGS["tiny" if dtype == "fp32" else "bart_base"]
+    # subsequences long enough for `rows` of them to be open at once; a few steps beyond that are compared
+    wl = base.scaled(name="edges", batch=batch, sub_max=rows, d_ff=d_ff, pos_mode=pos, max_sub_len=length, time_max=min(rows + 6, 96),
+                     length_dist=("uniform", max(1, length - 4), length), kv_c_dtype="e4m3" if kv8 else "same",
+                     **dict(BASE, ctx=144 if kv8 else 150))
+    s = check(wl, rows=[0, batch - 1] if batch > 1 else None, ragged=True, free_run=False)
+    assert s["max_err"] < parity.TOL[dtype]
+
+
+CROSS = [
+    # sequences, rows, heads, ctx -> CTAs per (sequence, head)
+    (1, 16, 18, 1300),     # 8, eleven tiles over eight CTAs
+    (1, 17, 18, 900),      # 8, two query tiles: fifteen records in the first CTA's ring
+    (1, 3, 19, 1300),      # 4
+    (37, 5, 1, 300),       # 4 by the segments, 2 by the three tiles
+    (38, 32, 1, 700),      # 2, two query tiles
+    (75, 1, 1, 520),       # 1, one tile beyond a multiple of the ring
+    (300, 2, 2, 40),       # more sequences than a launch once took
+    (2, 9, 2, 128),        # one tile exactly
+    (2, 9, 2, 129),        # and one key more
+]
+
+
+@pytest.mark.parametrize("batch,rows,heads,ctx", CROSS)
+def test_cross_attention_at_cluster_edges(batch, rows, heads, ctx):
+    """Unused rows come back as zeros and the status word clear, whatever the scratch held; two launches agree bit for bit."""
+    import torch
+    from paper_2506_23431_b200 import binding as B
+    q, kv, n_rows, ctx_len = cross_case(31, batch, rows, heads, ctx, "bf16")
+    ref = oracle_cross(q, kv, n_rows, ctx_len, heads, 0.125)
+    dev = torch.device("cuda", 0)
+    args = (torch.from_numpy(q).to(dev, torch.bfloat16), torch.from_numpy(kv).to(dev, torch.bfloat16),
+            torch.from_numpy(n_rows).to(dev), torch.from_numpy(ctx_len).to(dev), 0.125, 1)
+    scratch = torch.full((B.cross_attention_scratch_bytes(batch, rows, heads, 1),), 0x5a, dtype=torch.uint8, device=dev)
+    out = B.cross_attention(*args, scratch)
+    again = B.cross_attention(*args, scratch)
+    torch.cuda.synchronize()
+    assert int(scratch[:16].view(torch.int32)[2]) == 0
+    assert torch.equal(out.view(torch.int16), again.view(torch.int16))
+    got = out.float().cpu().numpy().astype(np.float64)
+    # weights and result are rounded to bf16 (2^-9 each, relative) and a row of weights sums to 1: twice 2^-9 of the largest value
+    assert np.abs(got - ref).max() <= 2 * 2.0 ** -9 * max(1.0, np.abs(kv[np.isfinite(kv)]).max())
+
+
+@pytest.mark.parametrize("rows,d_model,vocab", [(128, 64, 227), (129, 128, 451), (256, 64, 230)])
+def test_vocab_logits_at_row_tile_edges(rows, d_model, vocab):
+    """Both row-tile variants of the kernel, vocabularies whose logit rows start off every 16-byte boundary."""
+    import torch
+    from paper_2506_23431_b200 import binding as B
+    g = np.random.Generator(np.random.Philox(key=np.array([rows, vocab], dtype=np.uint64)))
+    hidden = W.bf16_round(g.standard_normal((rows, d_model), dtype=np.float32))
+    lm_head = W.bf16_round(0.05 * g.standard_normal((vocab, d_model), dtype=np.float32))
+    ref = hidden.astype(np.float64) @ lm_head.astype(np.float64).T
+    dev = torch.device("cuda", 0)
+    ids, best, logits = B.vocab_argmax(torch.from_numpy(hidden).to(dev, torch.bfloat16), torch.from_numpy(lm_head).to(dev, torch.bfloat16), want_logits=True)
+    got = logits.cpu().numpy()
+    # fp32 accumulation of d_model exact products: d_model * 2^-23 of the sum of their magnitudes
+    tol = d_model * 2.0 ** -23 * (np.abs(hidden).astype(np.float64) @ np.abs(lm_head).astype(np.float64).T).max()
+    assert np.abs(got - ref).max() <= tol
+    assert (ids.cpu().numpy() == got.argmax(axis=1)).all() and (best.cpu().numpy() == got.max(axis=1)).all()
+
+
+FORWARDS = [
+    # sequences, subsequences, longest, heads, vocabulary, positions
+    (3, 4, 15, 2, 301, ROPE),      # up to 64 rows a sequence: one block of 64; logit rows off the 16-byte boundary
+    (2, 5, 25, 2, 302, T5),        # several blocks of 64, the last one partly filled
+    (12, 16, 40, 6, 303, T5),      # enough blocks of 128 rows to fill the GPU
+    (12, 16, 40, 6, 304, ROPE),
+]
+
+
+@pytest.mark.parametrize("batch,sub_max,length,heads,vocab,pos", FORWARDS)
+def test_teacher_forward_at_block_edges(batch, sub_max, length, heads, vocab, pos):
+    wl = W.CONFIGS["bart_base"].scaled(name="tf_edges", n_layers=1, d_model=64 * heads, n_heads=heads, d_ff=256, vocab=vocab, norm_gain_std=0.1,
+                                       batch=batch, ctx=131, sub_max=sub_max, delta_t=2, max_sub_len=length,
+                                       length_dist=("uniform", max(0, length - 6), length), time_max=sub_max * 2 + length, pos_mode=pos)
+    assert run_case(wl, 2e-2) < 2e-2
