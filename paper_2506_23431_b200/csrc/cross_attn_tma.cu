@@ -4,7 +4,7 @@
 // contraction, so it runs on tensor cores; it stays HBM-bound (about S flop per byte).
 //
 // A (sequence, head) pair - its queries against its context - is a segment; a cluster of 1, 2, 4 or 8 CTAs
-// takes one, every CTA an equal share of its 128-key tiles, two CTAs per SM.  In every CTA a producer warp
+// takes one, every CTA an equal share of its 128-key tiles, two CTAs per SM (8-bit: four).  In every CTA a producer warp
 // streams the K and V tiles of its share (16 KB each, contiguous) through a ring of shared-memory stages
 // with TMA (cp.async.bulk.tensor.2d, 128-byte swizzle, completion on an mbarrier); four consumer warps each
 // take 32 keys of every tile: S = Q K^T with mma.sync m16n8k16 (bf16 in, fp32 accumulate), online softmax in
@@ -27,8 +27,7 @@
 // therefore 4 tig + {0, 1} | 4 tig + {2, 3} instead of 2 tig + {0, 1} | 2 tig + 8 + {0, 1}; queries
 // (score columns) are loaded with the same permutation, which a contraction does not see.  Queries and
 // softmax weights go through f16 (exact for bf16 queries in f16's range; 11 bits for the weights), the
-// key scale is folded into the score scale and the value scale into the final 1 / l.  Stages are 16 KB,
-// the ring six deep.
+// key scale is folded into the score scale and the value scale into the final 1 / l.  Stages are 16 KB.
 #include <cuda_fp16.h>
 
 #include "pd_internal.h"
@@ -36,16 +35,20 @@
 namespace pd {
 
 constexpr int XK = 128;                   // keys per tile
-// ring: three 32 KB stages (bf16) or six 16 KB stages (8-bit); with the merge scratch two CTAs fit an SM
-__host__ __device__ constexpr int xring_bytes(bool fp8) { return fp8 ? 96 * 1024 : 96 * 1024; }
+// CTAs per SM and the ring: two with three 32 KB stages (bf16), four with three 16 KB stages (8-bit, up to 16 rows).  The 8-bit
+// kernel waits on its own arithmetic between tiles more than on memory, so it wants warps rather than depth: 32 sequences x 16 heads x 2048
+// keys 33.5 us with two CTAs (96 KB rings), 36.8 with three (512 segments leave a thin second wave), 29.2 with four, the same with
+// two stages; its loads alone take 25.7 us.  The bf16 kernel is within 2 us of its loads alone (44.6 us there).  Two row tiles need the
+// registers of two CTAs per SM.
+__host__ __device__ constexpr int xctas(int mt, bool fp8) { return fp8 && mt == 1 ? 4 : 2; }      // CTAs per SM
+__host__ __device__ constexpr int xring_bytes(int mt, bool fp8) { return fp8 && mt == 1 ? 48 * 1024 : 96 * 1024; }
 // consumer warps: four, each taking 32 keys of a tile.  (Eight warps of 16 keys each were measured in both
 // variants and lost: 50.3 against 49.2 us per full bf16 launch, 31.9 against 28.7 us per 8-bit launch.)
 __host__ __device__ constexpr int xcw(bool fp8) { return fp8 ? 4 : 4; }
 __host__ __device__ constexpr int xthreads(bool fp8) { return (xcw(fp8) + 1) * 32; }
 constexpr int XREC_WORDS = 36;            // per lane and 16-row tile: 32 output values, 2 maxima, 2 sums
 constexpr int XREC_FLOATS = XREC_WORDS * 32;
-__host__ __device__ constexpr int xscratch_bytes(bool fp8) { return (xcw(fp8) / 2) * XREC_FLOATS * 4; }   // half the consumer warps' records for the tree merge
-__host__ __device__ constexpr int xsmem(bool fp8) { return xring_bytes(fp8) + xscratch_bytes(fp8) + 128 /*barriers*/ + 1024 /*alignment slack*/; }
+__host__ __device__ constexpr int xsmem(int mt, bool fp8) { return xring_bytes(mt, fp8) + 128 /*barriers*/ + 1024 /*alignment slack*/; }
 constexpr uint32_t XSPIN_LIMIT = 1u << 24;
 
 bool cross_attn_tma_supported(const Dims &dm) { return dm.C <= 32; }
@@ -376,12 +379,11 @@ __device__ __forceinline__ void store_rows(const TileAcc (&acc)[MT], __nv_bfloat
 // MT = 16-row query tiles (rows per sequence <= 16 * MT); FP8 = keys/values are E4M3 codes (tmap: the keys'
 // 128-byte lines, tmap_v: the transposed values), else bf16 (tmap alone: rows of 64 values)
 template <int MT, bool FP8>
-__global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const __grid_constant__ CUtensorMap tmap,
-                                                                          const __grid_constant__ CUtensorMap tmap_v, AttnArgs a) {
+__global__ void __launch_bounds__(xthreads(FP8), xctas(MT, FP8)) cross_attn_tma_kernel(const __grid_constant__ CUtensorMap tmap,
+                                                                                       const __grid_constant__ CUtensorMap tmap_v, AttnArgs a) {
   constexpr int XCW = xcw(FP8);
   constexpr int KPW = XK / XCW;
-  constexpr int XTILE_BYTES = XK * kDh * (FP8 ? 1 : 2), XSTAGE_BYTES = 2 * XTILE_BYTES, XSTAGES = xring_bytes(FP8) / XSTAGE_BYTES;
-  constexpr int XSCRATCH_BYTES = xscratch_bytes(FP8);
+  constexpr int XTILE_BYTES = XK * kDh * (FP8 ? 1 : 2), XSTAGE_BYTES = 2 * XTILE_BYTES, XSTAGES = xring_bytes(MT, FP8) / XSTAGE_BYTES;
   extern __shared__ uint8_t smem_raw[];
   __shared__ int before_s[XCW];
   const Dims &dm = a.dm;
@@ -389,8 +391,8 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
   const int ns = gridDim.x, rank = blockIdx.x, h = blockIdx.y, b = blockIdx.z, H = dm.H;
   const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
   uint8_t *smem_al = smem_raw + (base - smem_u32(smem_raw));
-  float *scratch = reinterpret_cast<float *>(smem_al + XSTAGES * XSTAGE_BYTES);
-  const uint32_t bar_full = base + XSTAGES * XSTAGE_BYTES + XSCRATCH_BYTES, bar_empty = bar_full + 8 * XSTAGES, bar_part = bar_empty + 8 * XSTAGES;
+  float *scratch = reinterpret_cast<float *>(smem_al);        // half the consumer warps' records for the tree merge, over the ring
+  const uint32_t bar_full = base + XSTAGES * XSTAGE_BYTES, bar_empty = bar_full + 8 * XSTAGES, bar_part = bar_empty + 8 * XSTAGES;
   const float *recv = reinterpret_cast<const float *>(smem_al);      // states of ranks 1 .. ns - 1, over the ring: [rank - 1][row tile][XREC_FLOATS]
 
   if (tid == 0) {
@@ -469,6 +471,7 @@ __global__ void __launch_bounds__(xthreads(FP8), 2) cross_attn_tma_kernel(const 
         if (lane == 0) mbar_arrive(bar_empty + 8 * s);
       }
     }
+    consumer_bar_sync<XCW * 32>();                      // the last tile is consumed: the ring is free
     // row sums across the quad, the warps' states into warp 0's
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
@@ -569,14 +572,14 @@ static int cross_cluster_size(const AttnArgs &a) {
   while (ns < 8 && 2 * ns <= tiles && 2 * ns * segs <= 148) ns *= 2;
   return ns;
 }
-static_assert(7 * 2 * XREC_FLOATS * 4 <= xring_bytes(false) && xring_bytes(true) == xring_bytes(false), "the states of a cluster fit over the ring");
+static_assert(7 * XREC_FLOATS * 4 <= xring_bytes(1, true) && 7 * 2 * XREC_FLOATS * 4 <= xring_bytes(2, true), "the states of a cluster fit over the ring");
 
 // rows_per_seq, fp8: the variant to prepare
 cudaError_t cross_attn_tma_prepare(int rows_per_seq, bool fp8) {
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if (rows_per_seq <= 16)
-    return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<1, true>, attr, xsmem(true)) : cudaFuncSetAttribute(cross_attn_tma_kernel<1, false>, attr, xsmem(false));
-  return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<2, true>, attr, xsmem(true)) : cudaFuncSetAttribute(cross_attn_tma_kernel<2, false>, attr, xsmem(false));
+    return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<1, true>, attr, xsmem(1, true)) : cudaFuncSetAttribute(cross_attn_tma_kernel<1, false>, attr, xsmem(1, false));
+  return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<2, true>, attr, xsmem(2, true)) : cudaFuncSetAttribute(cross_attn_tma_kernel<2, false>, attr, xsmem(2, false));
 }
 
 // 8-bit keys/values (a.kv_scale set): tmap = the keys' lines, tmap_v = the transposed values; else tmap alone.
@@ -590,7 +593,7 @@ cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, co
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ns, a.dm.H, a.batch);
   cfg.blockDim = dim3(xthreads(fp8), 1, 1);
-  cfg.dynamicSmemBytes = xsmem(fp8);
+  cfg.dynamicSmemBytes = xsmem(mt, fp8);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
