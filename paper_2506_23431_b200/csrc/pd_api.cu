@@ -1080,6 +1080,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
   if (scratch_bytes < L.total) return fail(h, PD_ERR_WORKSPACE, "pd_teacher_forward: scratch too small (pd_teacher_forward_scratch_bytes)");
   CU_TRY(h, cudaSetDevice(h->cfg.device));
   CU_TRY(h, teacher_attn_prepare());
+  CU_TRY(h, teacher_cross_tc_prepare());
   cudaStream_t s = h->stream;
   uint8_t *base = reinterpret_cast<uint8_t *>(scratch);
   int32_t *tab = reinterpret_cast<int32_t *>(base + L.tables);
@@ -1097,6 +1098,10 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
   const int M = (int)R;
   const bool rope = dm.pos_mode == PD_POS_ROPE;
   OWN(h, PD_PROF_OTHER, launch_gather_rows(M, dm.d, d_tok, h->w.embed, x, s));
+  CUtensorMap map_cq, map_ctx;
+  if (!h->kv8)
+    CU_TRY(h, encode_teacher_cross_maps(&map_cq, &map_ctx, cq, (uint64_t)M, (uint64_t)dm.d, h->ptr<void>(h->lay.kv_c),
+                                        (uint64_t)dm.L * dm.B * dm.H * 2 * dm.ctx));
   for (int l = 0; l < dm.L; ++l) {
     const void *const *lw = &h->layer_w[(size_t)l * kLayerTensors];
     OWN(h, PD_PROF_OTHER, launch_rmsnorm(dm, M, PD_DTYPE_BF16, x, lw[0], hb, s));
@@ -1112,7 +1117,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
     da.q = reinterpret_cast<const __nv_bfloat16 *>(qkv_b); da.out = reinterpret_cast<__nv_bfloat16 *>(att);
     da.row_sub = d_sub; da.row_tau = d_tau; da.grp_row0 = d_brow0; da.grp_n = d_bn; da.grp_key_row0 = d_bsrow0; da.grp_keys = d_bsrows;
     da.bias_tab = rope ? nullptr : h->ptr<float>(h->lay.bias_tab); da.n_dist = dm.n_dist;
-    OWN(h, PD_PROF_SELF_ATTN, launch_teacher_attn(da, true, s));
+    OWN(h, PD_PROF_SELF_ATTN, launch_teacher_self(da, s));
     PD_TRY(gemm(h, false, M, dm.d, dm.d, att, lw[2], x, true, 1.f));
     OWN(h, PD_PROF_OTHER, launch_rmsnorm(dm, M, PD_DTYPE_BF16, x, lw[3], hb, s));
     PD_TRY(gemm(h, false, M, dm.d, dm.d, hb, lw[4], cq, false, 0.f));
@@ -1120,7 +1125,8 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
       da.q = reinterpret_cast<const __nv_bfloat16 *>(cq); da.out = reinterpret_cast<__nv_bfloat16 *>(co);
       da.grp_keys = d_bctx; da.grp_seq = d_bseq;
       da.kv_c = h->ptr<__nv_bfloat16>(h->lay.kv_c); da.layer = l; da.B = dm.B; da.ctx = dm.ctx;
-      OWN(h, PD_PROF_CROSS_ATTN, launch_teacher_attn(da, false, s));
+      da.status = h->st.hdr + HDR_STATUS;
+      OWN(h, PD_PROF_CROSS_ATTN, launch_teacher_cross_tc(map_cq, map_ctx, da, s));
     }
     for (size_t g0 = 0; g0 < G; g0 += kTfCrossBatch) {              // 8-bit context: groups as "sequences" of the batched kernel
       AttnArgs a = attn_args(h, l, false);

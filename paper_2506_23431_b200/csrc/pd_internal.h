@@ -117,7 +117,7 @@ struct AttnArgs {
   const int32_t *row_base;
 };
 
-// ---- teacher-forced dense forward (teacher_kernels.cu) ------------------------------------------------
+// ---- teacher-forced dense forward (teacher_kernels.cu, teacher_cross_tc.cu) ------------------------------------------------
 struct DenseAttnArgs {
   int H, d, n_groups, block_rows;        // query rows per attention block: 128 or 64
   float scale_log2e;
@@ -132,9 +132,14 @@ struct DenseAttnArgs {
   // cross
   const __nv_bfloat16 *kv_c; int layer, B, ctx;
   const int32_t *grp_seq;                // [groups] the sequence whose context the block reads
+  int32_t *status;                       // error word (PD_ERR_TIMEOUT on an expired wait)
 };
 cudaError_t teacher_attn_prepare();      // once per device
-cudaError_t launch_teacher_attn(const DenseAttnArgs &a, bool self, cudaStream_t s);
+cudaError_t launch_teacher_self(const DenseAttnArgs &a, cudaStream_t s);
+cudaError_t teacher_cross_tc_prepare();  // once per device
+cudaError_t encode_teacher_cross_maps(CUtensorMap *map_q, CUtensorMap *map_kv, const void *q, uint64_t rows, uint64_t d, const void *kv_c,
+                                      uint64_t kv_rows);
+cudaError_t launch_teacher_cross_tc(const CUtensorMap &map_q, const CUtensorMap &map_kv, const DenseAttnArgs &a, cudaStream_t s);
 cudaError_t launch_rotate_rows(int rows, int d, const float *qkv, const int32_t *row_sub, const int32_t *row_tau, const float2 *rope_tab,
                                void *out, cudaStream_t s);
 cudaError_t launch_gather_rows(int rows, int d, const int32_t *row_tok, const void *embed, float *x, cudaStream_t s);

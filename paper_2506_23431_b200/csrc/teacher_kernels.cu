@@ -9,18 +9,14 @@ namespace pd {
 
 namespace {
 
-// Attention of up to 128 query rows of one sequence and head (one CTA; W warps of 16 MT rows each) over 64-key tiles that all
+// Self-attention of up to 128 query rows of one sequence and head (one CTA; W warps of 16 rows each) over 64-key tiles that all
 // warps share: a three-slot ring filled with 16-byte asynchronous copies (rows of 128 bytes, chunks swizzled), scores and
-// P.V on mma.sync, online softmax in the log2 domain; a warp owns its rows, so nothing is merged.
-// SELF = false: the keys are the sequence's context positions below ctx_len.  SELF = true: the keys are the sequence's own target
-// rows, with the dependency rule and the T5 bias applied to the accumulator fragment; the key walk ends at the first tile of a
+// P.V on mma.sync, online softmax in the log2 domain; a warp owns its rows, so nothing is merged.  The keys are the sequence's own
+// target rows, with the dependency rule and the T5 bias applied to the accumulator fragment; the key walk ends at the first tile of a
 // later subsequence.
-// What bounds it: with 128 rows per pass over the keys the tensor pipe (1075 cycles per tile) and the ldmatrix traffic that feeds
-// it (1024 cycles with 16 rows per warp, half of that with 32), not HBM.  11.5 k rows, 32 contexts of 2048, 16 heads, per layer:
-// cross-attention 640 us in groups of 32 rows on the decode kernel (every group reads its context again), 452 us here with 16 rows
-// per warp, 392 us with 32; self-attention 203 us in groups of 32 rows, 157 us with 16 rows per warp, 234 us with 32 (the mask needs
-// the registers).  So the context pass takes MT = 2 and the self pass MT = 1; where 128-row blocks would leave SMs without one,
-// both take 64-row blocks of MT = 1.
+// What bounds it: the mask and the bias, evaluated per pair.  11.5 k rows of 32 sequences, 16 heads, per layer: 203 us in groups of 32 rows
+// (every group reads its keys again), 157 us here with 16 rows per warp, 234 us with 32 (the mask needs the registers).  Where
+// 128-row blocks would leave SMs without one, 64-row blocks.
 constexpr int TK = 64, TSLOTS = 3, TMAXD = 640;
 constexpr int TSLOT_BYTES = TK * 256;            // 64 key rows, then 64 value rows
 constexpr int TATTN_SMEM = TSLOTS * TSLOT_BYTES + 128;
@@ -33,28 +29,21 @@ __device__ __forceinline__ void t_cp_async4(uint32_t dst, const void *src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
 }
 
-template <bool SELF, int W, int MT>
-__global__ void __launch_bounds__(W * 32, 16 / (W * MT)) teacher_attn_kernel(DenseAttnArgs a) {
+template <int W>
+__global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnArgs a) {
   using namespace mt;
   constexpr int TT = W * 32;
   extern __shared__ uint8_t t_raw[];
   __shared__ int ki_s[TSLOTS][TK], kt_s[TSLOTS][TK];
-  __shared__ float bias_s[SELF ? TMAXD : 1];
+  __shared__ float bias_s[TMAXD];
   const int grp = blockIdx.x, h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, tig = lane & 3;
   const int q0 = a.grp_row0[grp], nq = a.grp_n[grp];
   const uint32_t base = (smem_u32(t_raw) + 127u) & ~127u;
-  const size_t qld = SELF ? 3 * (size_t)a.d : (size_t)a.d, kld = SELF ? 3 * (size_t)a.d : (size_t)kDh;
-  const __nv_bfloat16 *kp, *vp;                  // row 0 of this head's keys and values
-  int nk, k0 = 0;
-  if (SELF) {
-    k0 = a.grp_key_row0[grp]; nk = a.grp_keys[grp];
-    kp = a.q + (size_t)k0 * kld + a.d + (size_t)h * kDh; vp = kp + a.d;
-  } else {
-    nk = a.grp_keys[grp];
-    kp = a.kv_c + ctx_kv_offset(a.layer, a.B, a.grp_seq[grp], a.H, h, 0, a.ctx); vp = kp + (size_t)a.ctx * kDh;
-  }
-  const bool use_bias = SELF && a.bias_tab != nullptr;
+  const size_t ld = 3 * (size_t)a.d;
+  const int k0 = a.grp_key_row0[grp], nk = a.grp_keys[grp];
+  const __nv_bfloat16 *kp = a.q + (size_t)k0 * ld + a.d + (size_t)h * kDh, *vp = kp + a.d;      // row 0 of this head's keys and values
+  const bool use_bias = a.bias_tab != nullptr;
   if (use_bias)
     for (int dd = tid; dd < a.n_dist; dd += TT) bias_s[dd] = a.bias_tab[(size_t)h * a.n_dist + dd];
 
@@ -65,18 +54,17 @@ __global__ void __launch_bounds__(W * 32, 16 / (W * MT)) teacher_attn_kernel(Den
     for (int i = 0; i < TK * 16 / TT; ++i) {     // chunks 0-7 of a row: keys, 8-15: values
       const int c = tid + i * TT, r = c >> 4, p = c & 15;
       const bool on = first + r < nk;            // absent keys: zero rows
-      const __nv_bfloat16 *src = (p < 8 ? kp : vp) + (on ? (size_t)(first + r) * kld : 0) + (p & 7) * 8;
+      const __nv_bfloat16 *src = (p < 8 ? kp : vp) + (on ? (size_t)(first + r) * ld : 0) + (p & 7) * 8;
       t_cp_async16(dst + (p >> 3) * (TK * 128) + swz(r, p & 7), src, on);
     }
-    if (SELF)
-      for (int i = tid; i < TK && first + i < nk; i += TT) {
-        t_cp_async4(smem_u32(&ki_s[slot][i]), a.row_sub + k0 + first + i);
-        t_cp_async4(smem_u32(&kt_s[slot][i]), a.row_tau + k0 + first + i);
-      }
+    for (int i = tid; i < TK && first + i < nk; i += TT) {
+      t_cp_async4(smem_u32(&ki_s[slot][i]), a.row_sub + k0 + first + i);
+      t_cp_async4(smem_u32(&kt_s[slot][i]), a.row_tau + k0 + first + i);
+    }
   };
   // tiles to walk: keys are sorted by subsequence, and nothing of a later one than the block's last row's is visible
   int n_tiles = (nk + TK - 1) / TK;
-  if (SELF) {
+  {
     const int q_i_max = a.row_sub[q0 + nq - 1];
     int lo = 0, hi = n_tiles;                    // first tile whose first key lies beyond
     while (lo < hi) {
@@ -90,30 +78,24 @@ __global__ void __launch_bounds__(W * 32, 16 / (W * MT)) teacher_attn_kernel(Den
     if (t < n_tiles) fetch(t);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  // this warp's query rows: 16 (MT warp + mt) + g, + 8
-  const int w0 = warp * 16 * MT;
-  uint32_t qf[MT][4][4];
-  int qi[MT][2], qt[MT][2], warp_i_max = 0x7fffffff;       // subsequence (-1: sees nothing) and timestamp of the rows
+  // this warp's query rows: 16 warp + g, + 8
+  const int w0 = warp * 16;
+  const int r_lo = w0 + g, r_hi = r_lo + 8;
+  const __nv_bfloat16 *q_lo = a.q + (size_t)(q0 + r_lo) * ld + (size_t)h * kDh + 2 * tig, *q_hi = q_lo + 8 * ld;
+  uint32_t qf[4][4];
 #pragma unroll
-  for (int mt_ = 0; mt_ < MT; ++mt_) {
-    const int r_lo = w0 + mt_ * 16 + g, r_hi = r_lo + 8;
-    const __nv_bfloat16 *q_lo = a.q + (size_t)(q0 + r_lo) * qld + (size_t)h * kDh + 2 * tig, *q_hi = q_lo + 8 * qld;
-#pragma unroll
-    for (int kk = 0; kk < 4; ++kk) {
-      qf[mt_][kk][0] = r_lo < nq ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16) : 0u;
-      qf[mt_][kk][1] = r_hi < nq ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16) : 0u;
-      qf[mt_][kk][2] = r_lo < nq ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8) : 0u;
-      qf[mt_][kk][3] = r_hi < nq ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8) : 0u;
-    }
-    if (SELF) {
-      qi[mt_][0] = r_lo < nq ? a.row_sub[q0 + r_lo] : -1; qt[mt_][0] = r_lo < nq ? a.row_tau[q0 + r_lo] : 0;
-      qi[mt_][1] = r_hi < nq ? a.row_sub[q0 + r_hi] : -1; qt[mt_][1] = r_hi < nq ? a.row_tau[q0 + r_hi] : 0;
-    }
+  for (int kk = 0; kk < 4; ++kk) {
+    qf[kk][0] = r_lo < nq ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16) : 0u;
+    qf[kk][1] = r_hi < nq ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16) : 0u;
+    qf[kk][2] = r_lo < nq ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8) : 0u;
+    qf[kk][3] = r_hi < nq ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8) : 0u;
   }
-  if (SELF) warp_i_max = w0 < nq ? a.row_sub[q0 + min(w0 + 16 * MT - 1, nq - 1)] : -1;
-  TileAcc acc[MT];
-#pragma unroll
-  for (int mt_ = 0; mt_ < MT; ++mt_) acc[mt_].clear();
+  // subsequence (-1: sees nothing) and timestamp of the rows
+  const int qi[2] = {r_lo < nq ? a.row_sub[q0 + r_lo] : -1, r_hi < nq ? a.row_sub[q0 + r_hi] : -1};
+  const int qt[2] = {r_lo < nq ? a.row_tau[q0 + r_lo] : 0, r_hi < nq ? a.row_tau[q0 + r_hi] : 0};
+  const int warp_i_max = w0 < nq ? a.row_sub[q0 + min(w0 + 15, nq - 1)] : -1;
+  TileAcc A;
+  A.clear();
   const float sl2 = a.scale_log2e;
 
   for (int tile = 0; tile < n_tiles; ++tile) {
@@ -122,85 +104,63 @@ __global__ void __launch_bounds__(W * 32, 16 / (W * MT)) teacher_attn_kernel(Den
     if (tile + TSLOTS - 1 < n_tiles) fetch(tile + TSLOTS - 1);
     asm volatile("cp.async.commit_group;" ::: "memory");
     const int slot = tile % TSLOTS, nv = min(TK, nk - tile * TK);
-    if (w0 >= nq || (SELF && ki_s[slot][0] > warp_i_max)) continue;      // no row of this warp sees the tile
+    if (w0 >= nq || ki_s[slot][0] > warp_i_max) continue;      // no row of this warp sees the tile
     const uint32_t kbase = base + slot * TSLOT_BYTES, vbase = kbase + TK * 128;
-    float sc[MT][8][4];
+    float sc[8][4];
 #pragma unroll
     for (int nt = 0; nt < 8; ++nt) {
-#pragma unroll
-      for (int mt_ = 0; mt_ < MT; ++mt_) sc[mt_][nt][0] = sc[mt_][nt][1] = sc[mt_][nt][2] = sc[mt_][nt][3] = 0.f;
+      sc[nt][0] = sc[nt][1] = sc[nt][2] = sc[nt][3] = 0.f;
 #pragma unroll
       for (int kq = 0; kq < 2; ++kq) {
         uint32_t b0, b1, b2, b3;
         ldsm_x4(kbase + swz(nt * 8 + (lane & 7), kq * 4 + (lane >> 3)), b0, b1, b2, b3);
+        mma_bf16(sc[nt], qf[2 * kq][0], qf[2 * kq][1], qf[2 * kq][2], qf[2 * kq][3], b0, b1);
+        mma_bf16(sc[nt], qf[2 * kq + 1][0], qf[2 * kq + 1][1], qf[2 * kq + 1][2], qf[2 * kq + 1][3], b2, b3);
+      }
+    }
+    // ---- scale, the dependency rule per pair (i' <= i and tau' <= tau), bias on the Manhattan distance (log2 domain)
 #pragma unroll
-        for (int mt_ = 0; mt_ < MT; ++mt_) {
-          mma_bf16(sc[mt_][nt], qf[mt_][2 * kq][0], qf[mt_][2 * kq][1], qf[mt_][2 * kq][2], qf[mt_][2 * kq][3], b0, b1);
-          mma_bf16(sc[mt_][nt], qf[mt_][2 * kq + 1][0], qf[mt_][2 * kq + 1][1], qf[mt_][2 * kq + 1][2], qf[mt_][2 * kq + 1][3], b2, b3);
+    for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+      for (int kx = 0; kx < 2; ++kx) {
+        const int e = nt * 8 + 2 * tig + kx;
+        const int ki = ki_s[slot][e], ktau = kt_s[slot][e];
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          float v = sc[nt][2 * hh + kx] * sl2;
+          const bool vis = e < nv && ki <= qi[hh] && ktau <= qt[hh];
+          if (use_bias && vis) v += bias_s[qt[hh] + qi[hh] - (ktau + ki)];
+          sc[nt][2 * hh + kx] = vis ? v : -INFINITY;
         }
       }
+    uint32_t pf[4][4];
+    float mx0 = -INFINITY, mx1 = -INFINITY;
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+      mx0 = fmaxf(mx0, fmaxf(sc[nt][0], sc[nt][1]));
+      mx1 = fmaxf(mx1, fmaxf(sc[nt][2], sc[nt][3]));
     }
-    // ---- SELF: scale, the dependency rule per pair (i' <= i and tau' <= tau), bias on the Manhattan distance (log2 domain);
-    // context: absent keys of the last tile; the scale joins the exponent below
-    if (SELF) {
+    mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1)); mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
+    mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1)); mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
+    const float mn0 = fmaxf(A.m0, mx0), mn1 = fmaxf(A.m1, mx1);
+    const float ref0 = mn0 == -INFINITY ? 0.f : mn0, ref1 = mn1 == -INFINITY ? 0.f : mn1;
+    const float c0 = ex2f(A.m0 - ref0), c1 = ex2f(A.m1 - ref1);
+    A.m0 = mn0; A.m1 = mn1;
+    float s0 = 0.f, s1 = 0.f;
 #pragma unroll
-      for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int kx = 0; kx < 2; ++kx) {
-          const int e = nt * 8 + 2 * tig + kx;
-          const int ki = ki_s[slot][e], ktau = kt_s[slot][e];
-#pragma unroll
-          for (int mt_ = 0; mt_ < MT; ++mt_)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-              float v = sc[mt_][nt][2 * hh + kx] * sl2;
-              const bool vis = e < nv && ki <= qi[mt_][hh] && ktau <= qt[mt_][hh];
-              if (use_bias && vis) v += bias_s[qt[mt_][hh] + qi[mt_][hh] - (ktau + ki)];
-              sc[mt_][nt][2 * hh + kx] = vis ? v : -INFINITY;
-            }
-        }
-    } else if (nv < TK) {
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-#pragma unroll
-          for (int mt_ = 0; mt_ < MT; ++mt_)
-            if (nt * 8 + 2 * tig + (x & 1) >= nv) sc[mt_][nt][x] = -INFINITY;
+    for (int nt = 0; nt < 8; ++nt) {
+      const float p0 = ex2f(sc[nt][0] - ref0), p1 = ex2f(sc[nt][1] - ref0);
+      const float p2 = ex2f(sc[nt][2] - ref1), p3 = ex2f(sc[nt][3] - ref1);
+      s0 += p0 + p1; s1 += p2 + p3;
+      pf[nt >> 1][(nt & 1) * 2] = pack_bf16(p0, p1);
+      pf[nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
     }
-    const float es = SELF ? 1.f : sl2;
-    uint32_t pf[MT][4][4];
+    A.l0 = A.l0 * c0 + s0; A.l1 = A.l1 * c1 + s1;
+    if (__any_sync(0xffffffffu, c0 != 1.f || c1 != 1.f)) {   // some row's running maximum moved
 #pragma unroll
-    for (int mt_ = 0; mt_ < MT; ++mt_) {
-      float mx0 = -INFINITY, mx1 = -INFINITY;
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt) {
-        mx0 = fmaxf(mx0, fmaxf(sc[mt_][nt][0], sc[mt_][nt][1]));
-        mx1 = fmaxf(mx1, fmaxf(sc[mt_][nt][2], sc[mt_][nt][3]));
-      }
-      mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1)); mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
-      mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1)); mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 2));
-      TileAcc &A = acc[mt_];
-      const float mn0 = fmaxf(A.m0, mx0 * es), mn1 = fmaxf(A.m1, mx1 * es);
-      const float ref0 = mn0 == -INFINITY ? 0.f : mn0, ref1 = mn1 == -INFINITY ? 0.f : mn1;
-      const float c0 = ex2f(A.m0 - ref0), c1 = ex2f(A.m1 - ref1);
-      A.m0 = mn0; A.m1 = mn1;
-      float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt) {
-        const float p0 = ex2f(fmaf(sc[mt_][nt][0], es, -ref0)), p1 = ex2f(fmaf(sc[mt_][nt][1], es, -ref0));
-        const float p2 = ex2f(fmaf(sc[mt_][nt][2], es, -ref1)), p3 = ex2f(fmaf(sc[mt_][nt][3], es, -ref1));
-        s0 += p0 + p1; s1 += p2 + p3;
-        pf[mt_][nt >> 1][(nt & 1) * 2] = pack_bf16(p0, p1);
-        pf[mt_][nt >> 1][(nt & 1) * 2 + 1] = pack_bf16(p2, p3);
-      }
-      A.l0 = A.l0 * c0 + s0; A.l1 = A.l1 * c1 + s1;
-      if (__any_sync(0xffffffffu, c0 != 1.f || c1 != 1.f)) {   // some row's running maximum moved
-#pragma unroll
-        for (int dn = 0; dn < 8; ++dn) { A.o[dn][0] *= c0; A.o[dn][1] *= c0; A.o[dn][2] *= c1; A.o[dn][3] *= c1; }
-      }
+      for (int dn = 0; dn < 8; ++dn) { A.o[dn][0] *= c0; A.o[dn][1] *= c0; A.o[dn][2] *= c1; A.o[dn][3] *= c1; }
     }
-    // ---- O += P (16 MT x 64 keys) . V (64 keys x 64)
+    // ---- O += P (16 x 64 keys) . V (64 keys x 64)
 #pragma unroll
     for (int kq = 0; kq < 4; ++kq) {
       const int key = kq * 16 + ((lane >> 3) & 1) * 8 + (lane & 7);
@@ -208,27 +168,19 @@ __global__ void __launch_bounds__(W * 32, 16 / (W * MT)) teacher_attn_kernel(Den
       for (int dp = 0; dp < 4; ++dp) {
         uint32_t b0, b1, b2, b3;
         ldsm_x4_t(vbase + swz(key, dp * 2 + (lane >> 4)), b0, b1, b2, b3);
-#pragma unroll
-        for (int mt_ = 0; mt_ < MT; ++mt_) {
-          mma_bf16(acc[mt_].o[2 * dp], pf[mt_][kq][0], pf[mt_][kq][1], pf[mt_][kq][2], pf[mt_][kq][3], b0, b1);
-          mma_bf16(acc[mt_].o[2 * dp + 1], pf[mt_][kq][0], pf[mt_][kq][1], pf[mt_][kq][2], pf[mt_][kq][3], b2, b3);
-        }
+        mma_bf16(A.o[2 * dp], pf[kq][0], pf[kq][1], pf[kq][2], pf[kq][3], b0, b1);
+        mma_bf16(A.o[2 * dp + 1], pf[kq][0], pf[kq][1], pf[kq][2], pf[kq][3], b2, b3);
       }
     }
   }
+  A.l0 += __shfl_xor_sync(0xffffffffu, A.l0, 1); A.l0 += __shfl_xor_sync(0xffffffffu, A.l0, 2);
+  A.l1 += __shfl_xor_sync(0xffffffffu, A.l1, 1); A.l1 += __shfl_xor_sync(0xffffffffu, A.l1, 2);
+  const float i0 = 1.f / A.l0, i1 = 1.f / A.l1;
+  __nv_bfloat16 *o_lo = a.out + (size_t)(q0 + r_lo) * a.d + (size_t)h * kDh + 2 * tig, *o_hi = o_lo + 8 * (size_t)a.d;
 #pragma unroll
-  for (int mt_ = 0; mt_ < MT; ++mt_) {
-    TileAcc &A = acc[mt_];
-    A.l0 += __shfl_xor_sync(0xffffffffu, A.l0, 1); A.l0 += __shfl_xor_sync(0xffffffffu, A.l0, 2);
-    A.l1 += __shfl_xor_sync(0xffffffffu, A.l1, 1); A.l1 += __shfl_xor_sync(0xffffffffu, A.l1, 2);
-    const float i0 = 1.f / A.l0, i1 = 1.f / A.l1;
-    const int r_lo = w0 + mt_ * 16 + g, r_hi = r_lo + 8;
-    __nv_bfloat16 *o_lo = a.out + (size_t)(q0 + r_lo) * a.d + (size_t)h * kDh + 2 * tig, *o_hi = o_lo + 8 * (size_t)a.d;
-#pragma unroll
-    for (int dn = 0; dn < 8; ++dn) {
-      if (r_lo < nq) *reinterpret_cast<__nv_bfloat162 *>(o_lo + dn * 8) = __floats2bfloat162_rn(A.o[dn][0] * i0, A.o[dn][1] * i0);
-      if (r_hi < nq) *reinterpret_cast<__nv_bfloat162 *>(o_hi + dn * 8) = __floats2bfloat162_rn(A.o[dn][2] * i1, A.o[dn][3] * i1);
-    }
+  for (int dn = 0; dn < 8; ++dn) {
+    if (r_lo < nq) *reinterpret_cast<__nv_bfloat162 *>(o_lo + dn * 8) = __floats2bfloat162_rn(A.o[dn][0] * i0, A.o[dn][1] * i0);
+    if (r_hi < nq) *reinterpret_cast<__nv_bfloat162 *>(o_hi + dn * 8) = __floats2bfloat162_rn(A.o[dn][2] * i1, A.o[dn][3] * i1);
   }
 }
 
@@ -312,21 +264,17 @@ __global__ void __launch_bounds__(256) target_logprob_kernel(int V, const float 
 
 cudaError_t teacher_attn_prepare() {
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(teacher_attn_kernel<false, 4, 2>, attr, TATTN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_attn_kernel<true, 8, 1>, attr, TATTN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_attn_kernel<false, 4, 1>, attr, TATTN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_attn_kernel<true, 4, 1>, attr, TATTN_SMEM);
+  cudaError_t e = cudaFuncSetAttribute(teacher_self_kernel<8>, attr, TATTN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_self_kernel<4>, attr, TATTN_SMEM);
   return e;
 }
 
-cudaError_t launch_teacher_attn(const DenseAttnArgs &a, bool self, cudaStream_t s) {
+cudaError_t launch_teacher_self(const DenseAttnArgs &a, cudaStream_t s) {
   if (a.n_groups < 1) return cudaSuccess;
-  if (self && a.bias_tab != nullptr && a.n_dist > TMAXD) return cudaErrorInvalidValue;      // the head's bias row is held in shared memory
+  if (a.bias_tab != nullptr && a.n_dist > TMAXD) return cudaErrorInvalidValue;      // the head's bias row is held in shared memory
   const dim3 grid(a.n_groups, a.H);
-  if (self && a.block_rows == 128) teacher_attn_kernel<true, 8, 1><<<grid, 256, TATTN_SMEM, s>>>(a);
-  else if (self) teacher_attn_kernel<true, 4, 1><<<grid, 128, TATTN_SMEM, s>>>(a);
-  else if (a.block_rows == 128) teacher_attn_kernel<false, 4, 2><<<grid, 128, TATTN_SMEM, s>>>(a);
-  else teacher_attn_kernel<false, 4, 1><<<grid, 128, TATTN_SMEM, s>>>(a);
+  if (a.block_rows == 128) teacher_self_kernel<8><<<grid, 256, TATTN_SMEM, s>>>(a);
+  else teacher_self_kernel<4><<<grid, 128, TATTN_SMEM, s>>>(a);
   return cudaGetLastError();
 }
 
