@@ -99,17 +99,41 @@ def test_vocab_logits_at_row_tile_edges(rows, d_model, vocab):
 
 
 FORWARDS = [
-    # sequences, subsequences, longest, heads, vocabulary, positions
-    (3, 4, 15, 2, 301, ROPE),      # up to 64 rows a sequence: one block of 64; logit rows off the 16-byte boundary
-    (2, 5, 25, 2, 302, T5),        # several blocks of 64, the last one partly filled
-    (12, 16, 40, 6, 303, T5),      # enough blocks of 128 rows to fill the GPU
-    (12, 16, 40, 6, 304, ROPE),
+    # sequences, subsequences, longest, heads, vocabulary, positions, context
+    (3, 4, 15, 2, 301, ROPE, 131),     # up to 64 rows a sequence: one block of 64; logit rows off the 16-byte boundary; three keys in a second tile
+    (2, 5, 25, 2, 302, T5, 128),       # several blocks of 64, the last one partly filled; one context tile exactly
+    (2, 5, 25, 2, 302, T5, 65),        # one key in the second half of a tile
+    (2, 2, 25, 2, 302, ROPE, 1),       # a context of one key
+    (12, 16, 40, 6, 303, T5, 131),     # enough blocks of 128 rows to fill the GPU
+    (12, 16, 40, 6, 304, ROPE, 400),   # more tiles than the ring holds
 ]
 
 
-@pytest.mark.parametrize("batch,sub_max,length,heads,vocab,pos", FORWARDS)
-def test_teacher_forward_at_block_edges(batch, sub_max, length, heads, vocab, pos):
+@pytest.mark.parametrize("batch,sub_max,length,heads,vocab,pos,ctx", FORWARDS)
+def test_teacher_forward_at_block_edges(batch, sub_max, length, heads, vocab, pos, ctx):
     wl = W.CONFIGS["bart_base"].scaled(name="tf_edges", n_layers=1, d_model=64 * heads, n_heads=heads, d_ff=256, vocab=vocab, norm_gain_std=0.1,
-                                       batch=batch, ctx=131, sub_max=sub_max, delta_t=2, max_sub_len=length,
+                                       batch=batch, ctx=ctx, sub_max=sub_max, delta_t=2, max_sub_len=length,
                                        length_dist=("uniform", max(0, length - 6), length), time_max=sub_max * 2 + length, pos_mode=pos)
     assert run_case(wl, 2e-2) < 2e-2
+
+
+def test_teacher_forward_when_the_running_maximum_moves():
+    """Sharp cross-attention: scores with a spread of several powers of two, so that rows meet larger ones tile after tile and what they
+    have summed is rescaled.  Queries and keys rounded to bf16 (2^-9 each) leave scores of up to 15 off by 0.06 at most, weights and
+    the layer's output off by as much relatively; the output projection takes that below the usual bar."""
+    from oracle import pipelined_decoder as O
+    from paper_2506_23431_b200.binding import PipelinedDecoder
+    from tests.test_gpu_teacher_forward import targets_of
+    wl = W.CONFIGS["bart_base"].scaled(name="tf_sharp", n_layers=1, d_model=128, n_heads=2, d_ff=256, vocab=300, norm_gain_std=0.1, batch=2, ctx=700,
+                                       sub_max=5, delta_t=2, max_sub_len=25, length_dist=("uniform", 15, 25), time_max=35, pos_mode=ROPE)
+    weights, mem, ctx_len = W.make_weights(wl), W.make_encoder_memory(wl), W.make_ctx_len(wl, ragged=True)
+    for name in ("l0.wq_c", "l0.wkv_c"):
+        weights[name] = W.bf16_round(7 * weights[name])
+    subs = targets_of(wl)
+    dec = PipelinedDecoder(wl.hyper(), weights, wl.batch)
+    dec.encode_context(dec.device_memory(mem), ctx_len, None)
+    logits = dec.teacher_forward(subs, want_logits=True)[2].cpu().numpy().astype(np.float64)
+    orc = O.PipelinedDecoderOracle(weights, wl.hyper())
+    ref = np.concatenate([orc.teacher_forward(mem[b], int(ctx_len[b]), subs[b])["logits"] for b in range(wl.batch)])
+    assert np.abs(logits - ref).max() <= 2e-2
+    dec.close()
