@@ -167,13 +167,14 @@ __global__ void __launch_bounds__(XC_THREADS, 2) teacher_cross_kernel(const __gr
   const uint32_t base = (c_smem_u32(c_raw) + 1023u) & ~1023u;
   const uint32_t q_s = base, ring = q_s + XC_Q;
   const uint32_t bar_q = ring + XC_STAGES * XC_STAGE, bar_full = bar_q + 8, bar_empty = bar_full + 8 * XC_STAGES, bar_s = bar_empty + 8 * XC_STAGES,
-                 bar_read = bar_s + 8, bar_p = bar_read + 8, bar_pv = bar_p + 8;
+                 bar_read = bar_s + 8, bar_p = bar_read + 8, bar_pv = bar_p + 16;
   if (tid == 0) {
     const uint32_t warps = (uint32_t)(nq + 31) / 32;       // softmax warps that have rows
     c_mbar_init(bar_q, 1);
     for (int s = 0; s < XC_STAGES; ++s) { c_mbar_init(bar_full + 8 * s, 1); c_mbar_init(bar_empty + 8 * s, 1); }
     c_mbar_init(bar_s, 1);
-    c_mbar_init(bar_read, warps); c_mbar_init(bar_p, warps);
+    c_mbar_init(bar_read, warps);
+    c_mbar_init(bar_p, warps); c_mbar_init(bar_p + 8, warps);
     c_mbar_init(bar_pv, 1); c_mbar_init(bar_pv + 8, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(XC_THREADS, 2) teacher_cross_kernel(const __gr
           c_fence_after();
           scores(tile + 1);
         }
-        if (!ok || !c_mbar_wait(bar_p, (uint32_t)j & 1u)) { ok = false; break; }
+        if (!ok || !c_mbar_wait(bar_p + 8 * (j & 1), (uint32_t)(j >> 1) & 1u)) { ok = false; break; }
         c_fence_after();
 #pragma unroll
         for (int k = 0; k < XC_H / 16; ++k)                 // 16 keys = 8 columns of weights, 16 rows of values
@@ -312,7 +313,10 @@ __global__ void __launch_bounds__(XC_THREADS, 2) teacher_cross_kernel(const __gr
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       c_fence_before();
       __syncwarp();
-      if (lane == 0) c_mbar_arrive(bar_p);
+      // A barrier each for even and odd halves: a warp arrives for half j behind its wait for the products of half j - 2, which start when
+      // every warp has arrived for that one, so no arrival is ever counted into the half before.  (With one barrier for all halves a
+      // warp could arrive for j while another still rescales O for j - 1, whose products then started on unfinished weights.)
+      if (lane == 0) c_mbar_arrive(bar_p + 8 * (j & 1));
     }
     if (ok && !c_mbar_wait(bar_pv + 8 * ((n_halves - 1) & 1), (uint32_t)((n_halves - 1) >> 1) & 1u)) ok = false;
     if (__all_sync(0xffffffffu, ok)) {

@@ -137,3 +137,41 @@ def test_teacher_forward_when_the_running_maximum_moves():
     ref = np.concatenate([orc.teacher_forward(mem[b], int(ctx_len[b]), subs[b])["logits"] for b in range(wl.batch)])
     assert np.abs(logits - ref).max() <= 2e-2
     dec.close()
+
+
+@pytest.mark.parametrize("ctx", [65, 700])
+def test_teacher_forward_when_one_warp_of_a_block_lags(ctx):
+    """Rows of one 32-row group meet a larger score half after half (their keys grow along the context) and rescale what they have summed;
+    the other groups' queries are near zero and never do: the groups of a block drift apart.  Repeats agree bit for bit, and the oracle's
+    forward within the bar of the test above (two halves: the shortest context with a hand-over)."""
+    from oracle import pipelined_decoder as O
+    from paper_2506_23431_b200.binding import PipelinedDecoder
+    wl = W.CONFIGS["bart_base"].scaled(name="tf_lag", n_layers=1, d_model=128, n_heads=2, d_ff=256, vocab=300, norm_gain_std=0.0, batch=8, ctx=ctx,
+                                       sub_max=5, delta_t=2, max_sub_len=31, length_dist=("uniform", 31, 31), time_max=42, pos_mode=ROPE)
+    weights, mem, ctx_len = W.make_weights(wl), W.make_encoder_memory(wl), np.full(wl.batch, ctx, np.int32)
+    # words 3 .. 149 live in the first half of the columns, the others and <bos> in the second; only the first half makes queries
+    g = np.random.Generator(np.random.Philox(key=np.array([ctx, 77], dtype=np.uint64)))
+    embed = g.standard_normal((300, 128), dtype=np.float32)
+    embed[3:150, 64:] = 0
+    embed[:3, :64] = 0
+    embed[150:, :64] = 0
+    weights["embed"] = W.bf16_round(embed)
+    weights["l0.wq_c"][64:] = 0
+    for name in ("l0.wq_c", "l0.wkv_c"):
+        weights[name] = W.bf16_round(8 * weights[name])
+    mem = W.bf16_round(mem * np.linspace(0.1, 1.3, ctx, dtype=np.float32)[None, :, None])
+    words = g.integers(150, 300, size=(wl.batch, 5, 31))
+    for b in range(wl.batch):
+        words[b, b % 4] = g.integers(3, 150, size=31)          # rows 32 i .. 32 i + 31 are subsequence i + 1's (31 words and <bos>)
+    subs = words.tolist()
+    dec = PipelinedDecoder(wl.hyper(), weights, wl.batch)
+    dec.encode_context(dec.device_memory(mem), ctx_len, None)
+    runs = [dec.teacher_forward(subs, want_logits=True)[2].cpu().numpy() for _ in range(12)]
+    orc = O.PipelinedDecoderOracle(weights, wl.hyper())
+    for r in runs[1:]:
+        assert np.array_equal(r, runs[0])
+    rows = 5 * 32
+    for b in (0, 1, 2, 3):
+        ref = orc.teacher_forward(mem[b], ctx, subs[b])["logits"]
+        assert np.abs(runs[0][b * rows:(b + 1) * rows] - ref).max() <= 2e-2
+    dec.close()
