@@ -216,7 +216,7 @@ PD_API pd_status pd_collect_row(pd_handle *h, int32_t row, int32_t *tokens, int3
  *                sum over all subsequences of lens + 1 rows (own_logits = 1 when `logits` is NULL: the library then
  *                works through the vocabulary projection in chunks of rows inside the scratch)
  *   logprob      host [rows] or NULL: log P(target) per row, rows in (sequence, subsequence, position) order
- *   logits       device fp32 [rows, vocab] or NULL: every row's logits (tests)
+ *   logits       device fp32 [rows, vocab] or NULL: every row's logits (any float's alignment: a slice of a larger buffer will do)
  *   rows_out, loss_out  host or NULL: the row count, and Eq. 6's L = - sum of logprob
  * bf16 path with at most 32 rows per sequence in pd_step (the tensor-core cross-attention kernel) only, else
  * PD_ERR_UNSUPPORTED.  Synchronises. */

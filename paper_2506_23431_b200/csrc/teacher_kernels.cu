@@ -232,7 +232,8 @@ __global__ void __launch_bounds__(256) target_logprob_kernel(int V, const float 
     if (x > m) { s *= expf(m - x); m = x; }
     if (m > -INFINITY) s += expf(x - m);
   };
-  const int head = min(V, (int)((4u - (unsigned)(((size_t)blockIdx.x * V) & 3u)) & 3u));
+  // scalar up to the row's first 16-byte boundary: the caller's buffer may itself start between two
+  const int head = min(V, (int)((16u - (unsigned)(reinterpret_cast<uintptr_t>(row) & 15u)) & 15u) / 4);
   const int nvec = (V - head) / 4;
   if (tid < head) take(row[tid]);
   const float4 *body = reinterpret_cast<const float4 *>(row + head);

@@ -175,3 +175,40 @@ def test_teacher_forward_when_one_warp_of_a_block_lags(ctx):
         ref = orc.teacher_forward(mem[b], ctx, subs[b])["logits"]
         assert np.abs(runs[0][b * rows:(b + 1) * rows] - ref).max() <= 2e-2
     dec.close()
+
+
+@pytest.mark.parametrize("vocab", [301, 304])
+def test_teacher_forward_into_a_slice_of_a_larger_buffer(vocab):
+    """The caller's logits start at any float: rows of a larger buffer, one to three floats off a 16-byte boundary.  The same rows through
+    another order of fp32 sums: 300 terms, 300 x 2^-24 relative of a log-probability of a few units; the logits 128 terms of products."""
+    import ctypes as C
+
+    import torch
+    from paper_2506_23431_b200 import binding as B
+    from tests.test_gpu_teacher_forward import targets_of
+    wl = W.CONFIGS["bart_base"].scaled(name="tf_slice", n_layers=1, d_model=128, n_heads=2, d_ff=256, vocab=vocab, norm_gain_std=0.1, batch=2, ctx=96,
+                                       sub_max=4, delta_t=2, max_sub_len=15, length_dist=("uniform", 5, 15), time_max=25, pos_mode=ROPE)
+    subs = targets_of(wl)
+    dec = B.PipelinedDecoder(wl.hyper(), W.make_weights(wl), wl.batch)
+    dec.encode_context(dec.device_memory(W.make_encoder_memory(wl)), W.make_ctx_len(wl), None)
+    lp, loss, want = dec.teacher_forward(subs, want_logits=True)
+    rows = len(lp)
+    n_sub = np.array([len(s) for s in subs], np.int32)
+    lens, toks = np.zeros((wl.batch, wl.sub_max), np.int32), np.zeros((wl.batch, wl.sub_max, wl.max_sub_len), np.int32)
+    for b, seq in enumerate(subs):
+        for i, sub in enumerate(seq):
+            lens[b, i], toks[b, i, :len(sub)] = len(sub), sub
+    nbytes = int(B._lib.pd_teacher_forward_scratch_bytes(dec._h, rows, 0))
+    scratch = torch.empty(nbytes, dtype=torch.uint8, device=dec.device)
+    for off in (1, 2, 3):
+        buf = torch.full((off + (rows + 1) * vocab,), 7.0, device=dec.device)
+        torch.cuda.synchronize()
+        got_lp, n, got_loss = np.empty(rows, np.float32), C.c_int32(0), C.c_double(0.0)
+        st = B._lib.pd_teacher_forward(dec._h, B._p(n_sub), B._p(lens), B._p(toks), None, C.c_void_p(scratch.data_ptr()), C.c_size_t(nbytes),
+                                       got_lp.ctypes.data_as(C.POINTER(C.c_float)), C.c_void_p(buf.data_ptr() + 4 * off), C.byref(n), C.byref(got_loss))
+        assert st == 0 and n.value == rows
+        got = buf[off:off + rows * vocab].reshape(rows, vocab)
+        assert (got - want).abs().max().item() <= 1e-4
+        assert (buf[:off] == 7).all() and (buf[off + rows * vocab:] == 7).all()          # nothing beside the slice
+        assert np.abs(got_lp - lp).max() <= 1e-4 and abs(got_loss.value - loss) <= 1e-4 * rows
+    dec.close()
