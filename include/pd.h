@@ -105,7 +105,8 @@ typedef struct {
  * are row-major [in, out] (y = x W).  Per layer, in this order: norm1 [d], wqkv [d, 3d]
  * (columns q | k | v, head-major), wo [d, d], norm2 [d], wq_c [d, d], wkv_c [d, 2d] (columns
  * k | v), wo_c [d, d], norm3 [d], w1 [d, d_ff], w2 [d_ff, d].  The decoder layer is pre-RMSNorm,
- * bias-free, ReLU feed-forward, untied output head. */
+ * bias-free, ReLU feed-forward, untied output head.  embed and the norm gains may start at any
+ * value (slices of larger buffers). */
 typedef struct {
   const void *embed;        /* [vocab, d]                                   */
   const void *const *layer; /* host array of n_layers*10 device pointers    */

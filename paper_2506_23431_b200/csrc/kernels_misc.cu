@@ -190,17 +190,14 @@ __global__ void __launch_bounds__(128) embed_packed_kernel(Dims dm, DecState st,
   if (c >= S) return;
   const size_t m = (size_t)(before + c);
   if (tid == 0) row_meta_packed[m] = st.row_meta[r];
-  const uint2 *e = reinterpret_cast<const uint2 *>(embed + (size_t)tok * dm.d);       // four columns per thread; d is a multiple of 64
-  const uint2 *g = reinterpret_cast<const uint2 *>(gain);
+  const __nv_bfloat16 *e = embed + (size_t)tok * dm.d;       // four columns per thread; d is a multiple of 64
   float ss = 0.f;
   for (int q = tid; q < dm.d / 4; q += 128) {
-    const uint2 ev = e[q], gv = g[q];
-    const __nv_bfloat162 *e2 = reinterpret_cast<const __nv_bfloat162 *>(&ev), *g2 = reinterpret_cast<const __nv_bfloat162 *>(&gv);
-    const float2 a = __bfloat1622float2(e2[0]), bb = __bfloat1622float2(e2[1]), ga = __bfloat1622float2(g2[0]), gb = __bfloat1622float2(g2[1]);
-    *reinterpret_cast<float4 *>(x + m * dm.d + 4 * q) = make_float4(a.x, a.y, bb.x, bb.y);
-    const __nv_bfloat162 o0 = __floats2bfloat162_rn(a.x * ga.x, a.y * ga.y), o1 = __floats2bfloat162_rn(bb.x * gb.x, bb.y * gb.y);
+    const float4 v = load4_table(e + 4 * q), g = load4_table(gain + 4 * q);
+    *reinterpret_cast<float4 *>(x + m * dm.d + 4 * q) = v;
+    const __nv_bfloat162 o0 = __floats2bfloat162_rn(v.x * g.x, v.y * g.y), o1 = __floats2bfloat162_rn(v.z * g.z, v.w * g.w);
     *reinterpret_cast<uint2 *>(xg + m * dm.d + 4 * q) = make_uint2(*reinterpret_cast<const uint32_t *>(&o0), *reinterpret_cast<const uint32_t *>(&o1));
-    ss += a.x * a.x + a.y * a.y + bb.x * bb.x + bb.y * bb.y;
+    ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
   }
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   if ((tid & 31) == 0) red[tid >> 5] = ss;
@@ -220,13 +217,6 @@ cudaError_t launch_embed_packed(const Dims &dm, const DecState &st, int batch, c
 // (rows are multiples of 64 columns, at most 4096): one 16-byte load each, kept in registers over the sum.
 constexpr int RN_THREADS = 256;
 
-template <typename T> __device__ __forceinline__ float4 load4(const T *p);
-template <> __device__ __forceinline__ float4 load4<float>(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-template <> __device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16 *p) {
-  const uint2 w = *reinterpret_cast<const uint2 *>(p);
-  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.y));
-  return make_float4(a.x, a.y, b.x, b.y);
-}
 __device__ __forceinline__ void store4(float *p, const float4 &v) { *reinterpret_cast<float4 *>(p) = v; }
 __device__ __forceinline__ void store4(__nv_bfloat16 *p, const float4 &v) {
   const __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
@@ -242,7 +232,7 @@ __global__ void __launch_bounds__(1024) rmsnorm_kernel(int d, float eps, const f
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f), gn = v;
   if (on) {
     v = *reinterpret_cast<const float4 *>(x + (size_t)blockIdx.x * d + c);
-    gn = load4<T>(gain + c);
+    gn = load4_table(gain + c);
   }
   float ss = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);

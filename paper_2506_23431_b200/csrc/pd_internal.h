@@ -39,6 +39,21 @@ __host__ __device__ __forceinline__ size_t ctx_kv_offset(int layer, int B, int b
   return (((((size_t)layer * B + b) * H + h) * 2 + is_v) * ctx) * kDh;
 }
 
+// Four neighbouring values of a table the caller laid out (embedding, norm gains), whose base is only known to be aligned to one value.
+// One test per thread, the same in all of them; a table off the boundary costs four loads instead of one.
+__device__ __forceinline__ float4 load4_table(const float *p) {
+  if ((reinterpret_cast<uintptr_t>(p) & 15) == 0) return *reinterpret_cast<const float4 *>(p);
+  return make_float4(p[0], p[1], p[2], p[3]);
+}
+__device__ __forceinline__ float4 load4_table(const __nv_bfloat16 *p) {
+  if ((reinterpret_cast<uintptr_t>(p) & 7) == 0) {
+    const uint2 w = *reinterpret_cast<const uint2 *>(p);
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+  }
+  return make_float4(__bfloat162float(p[0]), __bfloat162float(p[1]), __bfloat162float(p[2]), __bfloat162float(p[3]));
+}
+
 // header words of the state block
 enum { HDR_STEP_T = 0, HDR_ALL_DONE = 1, HDR_STATUS = 2, HDR_PAGE_BUMP = 3, HDR_BATCH = 4, HDR_N_DONE = 5,
        HDR_TICKET = 6, HDR_WORDS = 16 };

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(PF_T, 1) proj_f32_kernel(ProjF32Args a) {
   const int ce = 2 * (tid & 15), rl = tid >> 4;       // this thread's pair of columns and row of a tile in the epilogue
   const int col = n0 + ce;
   float2 gn = make_float2(0.f, 0.f);
-  if (EPI == PROJ_RESID) gn = *reinterpret_cast<const float2 *>(a.gain_next + col);
+  if (EPI == PROJ_RESID) gn = make_float2(a.gain_next[col], a.gain_next[col + 1]);      // (the caller's, aligned to one value)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (CLUSTER) f_cluster_wait();
 

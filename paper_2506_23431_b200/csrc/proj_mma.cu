@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(PJ_T, 2) proj_mma_kernel(ProjArgs a) {
   if (blockIdx.y == 0) count();
   const int ce = 2 * (tid & 15);                      // this thread's pair of columns in the epilogue (sixteen threads per row)
   float2 gn = make_float2(0.f, 0.f);
-  if (EPI == PROJ_RESID) gn = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(a.gain_next + n0 + ce));
+  if (EPI == PROJ_RESID) gn = make_float2(__bfloat162float(a.gain_next[n0 + ce]), __bfloat162float(a.gain_next[n0 + ce + 1]));      // (the caller's, aligned to one value)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (CLUSTER) j_cluster_wait();
 

@@ -206,12 +206,8 @@ __global__ void __launch_bounds__(256) rotate_rows_kernel(int d, const float *__
 __global__ void gather_rows_kernel(int d, const int32_t *__restrict__ row_tok, const __nv_bfloat16 *__restrict__ embed,
                                    float *__restrict__ x) {
   const int r = blockIdx.x;
-  const uint2 *e = reinterpret_cast<const uint2 *>(embed + (size_t)row_tok[r] * d);      // four columns per thread; d is a multiple of 64
-  for (int c = threadIdx.x; c < d / 4; c += blockDim.x) {
-    const uint2 w = e[c];
-    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w.y));
-    *reinterpret_cast<float4 *>(x + (size_t)r * d + 4 * c) = make_float4(a.x, a.y, b.x, b.y);
-  }
+  const __nv_bfloat16 *e = embed + (size_t)row_tok[r] * d;      // four columns per thread; d is a multiple of 64
+  for (int c = threadIdx.x; c < d / 4; c += blockDim.x) *reinterpret_cast<float4 *>(x + (size_t)r * d + 4 * c) = load4_table(e + 4 * c);
 }
 
 // logprob[r] = logits[r][target] - log sum_v exp(logits[r][v])   (the row's term of Eq. 6).  One pass over the row (every thread

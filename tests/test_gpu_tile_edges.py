@@ -212,3 +212,49 @@ def test_teacher_forward_into_a_slice_of_a_larger_buffer(vocab):
         assert (buf[:off] == 7).all() and (buf[off + rows * vocab:] == 7).all()          # nothing beside the slice
         assert np.abs(got_lp - lp).max() <= 1e-4 and abs(got_loss.value - loss) <= 1e-4 * rows
     dec.close()
+
+
+@pytest.mark.parametrize("dtype,batch", [("bf16", 2), ("bf16", 20), ("fp32", 2), ("fp32", 5)])
+def test_embedding_and_gains_that_start_at_any_value(dtype, batch):
+    """embed and every norm gain one value into larger buffers, on the packed, the library and both fp32 paths of a step and in the one-pass
+    forward: the same bits as from tables of their own."""
+    import ctypes as C
+
+    import torch
+    from paper_2506_23431_b200 import binding as B
+    wl = W.CONFIGS["tiny" if dtype == "fp32" else "bart_base"].scaled(
+        name="tables", batch=batch, n_layers=2, d_model=128, n_heads=2, d_ff=256, vocab=301, norm_gain_std=0.1, ctx=96, sub_max=7, delta_t=2,
+        max_sub_len=15, length_dist=("uniform", 5, 15), time_max=26, pos_mode=ROPE)
+    mem, ctx_len, forced = W.make_encoder_memory(wl), W.make_ctx_len(wl), W.make_forced_len(wl)
+    subs = [[[5, 6, 7 + b], [8, 9]] for b in range(batch)]
+    dec = B.PipelinedDecoder(wl.hyper(), W.make_weights(wl), wl.batch, store_logits=True)
+
+    def results():
+        dec.encode_context(dec.device_memory(mem), ctx_len, forced)
+        lp = dec.teacher_forward(subs)[0] if dtype == "bf16" else np.zeros(1)
+        dec.run()
+        return [lp, dec.get_logits()[0], dec.collect()["tokens"]]
+    want = results()
+
+    def shifted(t):
+        buf = torch.empty(t.numel() + 1, dtype=t.dtype, device=t.device)
+        buf[1:] = t.reshape(-1)
+        return buf
+    tables = ["embed", "final_norm"] + [f"l{l}.norm{k}" for l in range(wl.n_layers) for k in (1, 2, 3)]
+    keep = {k: shifted(dec._w[k]) for k in tables}
+    at = {k: t.data_ptr() + t.element_size() for k, t in keep.items()}
+    for l in range(wl.n_layers):
+        for j, name in enumerate(B.LAYER_TENSORS):
+            dec._layer_ptrs[l * len(B.LAYER_TENSORS) + j] = at.get(f"l{l}.{name}", dec._w[f"l{l}.{name}"].data_ptr())
+    w = B.PdWeights()
+    w.embed, w.final_norm, w.lm_head, w.rel_bias = at["embed"], at["final_norm"], dec._w["lm_head"].data_ptr(), None
+    w.layer = C.cast(dec._layer_ptrs, C.POINTER(C.c_void_p))
+    torch.cuda.synchronize()
+    B._lib.pd_destroy(dec._h)
+    dec._h = B._H()
+    st = B._lib.pd_init(C.byref(dec.cfg), C.byref(w), C.c_void_p((dec._ws.data_ptr() + 255) // 256 * 256), C.c_size_t(dec.workspace_bytes),
+                        C.c_void_p(dec.stream.cuda_stream), C.byref(dec._h))
+    assert st == 0
+    for a, b in zip(want, results()):
+        assert np.array_equal(a, b)
+    dec.close()
