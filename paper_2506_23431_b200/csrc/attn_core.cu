@@ -57,7 +57,7 @@ template <typename T, bool SELF>
 __global__ void __launch_bounds__(NT) attn_core_kernel(AttnArgs a) {
   const Dims &dm = a.dm;
   const int n_chunk = (dm.C + kCoreRows - 1) / kCoreRows;
-  const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z / n_chunk, c0 = (blockIdx.z % n_chunk) * kCoreRows;
+  const int split = blockIdx.x / n_chunk, h = blockIdx.y, b = blockIdx.z, c0 = (blockIdx.x % n_chunk) * kCoreRows;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   __shared__ __align__(16) float Qs[kCoreRows][kDh];
   extern __shared__ __align__(16) uint8_t core_raw[];   // the warps' tiles (then their (O, m, l)), the warps' weights
@@ -277,7 +277,8 @@ cudaError_t attn_core_prepare(int dtype, bool self) {
 // what it writes is read behind the wait (queries, the step's keys/values).
 cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, bool pdl, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.splits, a.dm.H, a.batch * ((a.dm.C + kCoreRows - 1) / kCoreRows));
+  // chunks share a dimension with the splits: the sequences alone may fill theirs (the entry points take 65535)
+  cfg.gridDim = dim3(a.splits * ((a.dm.C + kCoreRows - 1) / kCoreRows), a.dm.H, a.batch);
   cfg.blockDim = dim3(NT, 1, 1);
   cfg.dynamicSmemBytes = dtype == PD_DTYPE_BF16 ? core_smem<__nv_bfloat16>() : core_smem<float>();
   cfg.stream = s;

@@ -258,3 +258,23 @@ def test_embedding_and_gains_that_start_at_any_value(dtype, batch):
     for a, b in zip(want, results()):
         assert np.array_equal(a, b)
     dec.close()
+
+
+@pytest.mark.parametrize("dtype,batch,rows", [("fp32", 16384, 49), ("fp32", 40000, 17), ("bf16", 22000, 33), ("bf16", 65535, 2)])
+def test_cross_attention_of_many_sequences(dtype, batch, rows):
+    """More sequences than a grid dimension holds chunks of rows.  The first, a middle and the last sequence against fp64; tolerances as
+    for the operator's other tests (fp32 sums of 8 keys; bf16: weights and result rounded, 2^-9 each)."""
+    import torch
+    from paper_2506_23431_b200 import binding as B
+    dev, td = torch.device("cuda", 0), torch.float32 if dtype == "fp32" else torch.bfloat16
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(batch)
+    q = torch.randn(batch, rows, 64, generator=gen, device=dev).to(td)
+    kv = torch.randn(batch, 1, 2, 8, 64, generator=gen, device=dev).to(td)
+    n_rows = torch.full((batch,), rows, dtype=torch.int32, device=dev)
+    ctx_len = torch.full((batch,), 7, dtype=torch.int32, device=dev)
+    out = B.cross_attention(q, kv, n_rows, ctx_len, 0.125, 1)
+    for b in (0, batch // 2, batch - 1):
+        w = torch.softmax(0.125 * q[b].double() @ kv[b, 0, 0, :7].double().T, -1)
+        ref = w @ kv[b, 0, 1, :7].double()
+        assert (out[b].double() - ref).abs().max().item() <= (2e-5 if dtype == "fp32" else 2 * 2.0 ** -9 * kv[b].abs().max().item())
