@@ -46,6 +46,10 @@ template <bool SWZ> __device__ __forceinline__ float4 key4(const __nv_bfloat16 *
   return make_float4(a.x, a.y, b.x, b.y);
 }
 
+// A maximum as the point of reference of exponentials: with nothing visible yet (-inf) any finite one gives them weight 0, and a score that is
+// no number keeps a weight that is none, whichever warp or split meets it.
+__device__ __forceinline__ float finite(float m) { return m == -INFINITY ? 0.f : m; }
+
 // One CTA = one (split, head, sequence, chunk of up to 16 rows).  Its eight warps work alone on every eighth 32-key tile: a lane
 // holds one key for the scores (queries come as broadcasts from shared memory) and two columns of the output for
 // P.V; online softmax per warp, one merge at the end.  Each warp has room for one tile of keys and one of values: the
@@ -187,7 +191,7 @@ __global__ void __launch_bounds__(NT) attn_core_kernel(AttnArgs a) {
       for (int u = 0; u < 4; ++u) {
         m_old[u] = __shfl_sync(0xffffffffu, m_run, s0 + u);
         mx[u] = fmaxf(m_old[u], mx[u]);
-        p[u] = mx[u] == -INFINITY ? 0.f : exp2f(sc[u] - mx[u]);
+        p[u] = exp2f(sc[u] - finite(mx[u]));
         sum[u] = p[u];
         ps[(s0 + u) * PP + lane] = p[u];
       }
@@ -198,7 +202,7 @@ __global__ void __launch_bounds__(NT) attn_core_kernel(AttnArgs a) {
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (lane == s0 + u) {
-          corr = m_old[u] == -INFINITY ? 0.f : exp2f(m_old[u] - mx[u]);
+          corr = exp2f(m_old[u] - finite(mx[u]));
           m_run = mx[u]; l_run = l_run * corr + sum[u];
         }
     }
@@ -248,9 +252,7 @@ __global__ void __launch_bounds__(NT) attn_core_kernel(AttnArgs a) {
     float L = 0.f, O = 0.f;
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
-      const float m = mm[w * kCoreRows + s];
-      if (m == -INFINITY) continue;
-      const float f = exp2f(m - M);
+      const float f = exp2f(mm[w * kCoreRows + s] - finite(M));
       L += ml[w * kCoreRows + s] * f;
       O += mo[(w * kCoreRows + s) * kDh + dim] * f;
     }
@@ -306,9 +308,7 @@ __global__ void attn_merge_kernel(AttnArgs a) {
     for (int s = 0; s < a.splits; ++s) M = fmaxf(M, a.part_ml[(p0 + s) * 2]);
     float L = 0.f, O = 0.f;
     for (int s = 0; s < a.splits; ++s) {
-      float m = a.part_ml[(p0 + s) * 2];
-      if (m == -INFINITY) continue;
-      float w = exp2f(m - M);
+      float w = exp2f(a.part_ml[(p0 + s) * 2] - finite(M));
       L += a.part_ml[(p0 + s) * 2 + 1] * w;
       O += a.part_o[(p0 + s) * kDh + dim] * w;
     }

@@ -278,3 +278,34 @@ def test_cross_attention_of_many_sequences(dtype, batch, rows):
         w = torch.softmax(0.125 * q[b].double() @ kv[b, 0, 0, :7].double().T, -1)
         ref = w @ kv[b, 0, 1, :7].double()
         assert (out[b].double() - ref).abs().max().item() <= (2e-5 if dtype == "fp32" else 2 * 2.0 ** -9 * kv[b].abs().max().item())
+
+
+@pytest.mark.parametrize("dtype,rows", [("fp32", 4), ("bf16", 4), ("bf16", 40)])
+@pytest.mark.parametrize("first,last", [(0, 32), (32, 64), (96, 97), (256, 300)])
+def test_cross_attention_with_keys_out_of_range(dtype, rows, first, last):
+    """Keys that are no numbers make the head's rows none, wherever their tile falls; keys whose scores overflow to -inf weigh nothing.  The
+    other head is not touched.  Both attention kernels, one split and three; tolerance as for the operator's other tests."""
+    import torch
+    from paper_2506_23431_b200 import binding as B
+    dev, td = torch.device("cuda", 0), torch.float32 if dtype == "fp32" else torch.bfloat16
+    gen = torch.Generator(device=dev)
+    gen.manual_seed(first)
+    q = (0.5 + torch.rand(1, rows, 128, generator=gen, device=dev)).to(td)
+    kv = torch.randn(1, 2, 2, 300, 64, generator=gen, device=dev).to(td)
+    n_rows = torch.full((1,), rows, dtype=torch.int32, device=dev)
+    ctx_len = torch.full((1,), 300, dtype=torch.int32, device=dev)
+    for splits in (1, 3):
+        for bad in (float("nan"), -3e38):
+            keys = kv.clone()
+            keys[0, 1, 0, first:last] = bad
+            out = B.cross_attention(q, keys, n_rows, ctx_len, 0.125, splits)[0].double()
+            for h in (0, 1):
+                got = out[:, 64 * h:64 * h + 64]
+                if h == 1 and bad != bad:
+                    assert torch.isnan(got).all()
+                    continue
+                s = 0.125 * q[0, :, 64 * h:64 * h + 64].double() @ kv[0, h, 0].double().T
+                if h == 1:
+                    s[:, first:last] = -float("inf")
+                ref = torch.softmax(s, -1) @ kv[0, h, 1].double()
+                assert (got - ref).abs().max().item() <= (2e-5 if dtype == "fp32" else 2 * 2.0 ** -9 * kv.abs().max().item())
