@@ -219,14 +219,16 @@ __global__ void __launch_bounds__(256) target_logprob_kernel(int V, const float 
   const int tid = threadIdx.x;
   const float *row = logits + (size_t)blockIdx.x * V;
   float m = -INFINITY, s = 0.f;
+  auto finite = [](float mx) { return mx > -INFINITY ? mx : 0.f; };      // so that a NaN among logits of -inf stays one in the sum
   auto take4 = [&](const float4 &x) {
     const float mx = fmaxf(fmaxf(x.x, x.y), fmaxf(x.z, x.w));
     if (mx > m) { s *= expf(m - mx); m = mx; }
-    if (m > -INFINITY) s += (expf(x.x - m) + expf(x.y - m)) + (expf(x.z - m) + expf(x.w - m));
+    const float r = finite(m);
+    s += (expf(x.x - r) + expf(x.y - r)) + (expf(x.z - r) + expf(x.w - r));
   };
   auto take = [&](float x) {
     if (x > m) { s *= expf(m - x); m = x; }
-    if (m > -INFINITY) s += expf(x - m);
+    s += expf(x - finite(m));
   };
   // scalar up to the row's first 16-byte boundary: the caller's buffer may itself start between two
   const int head = min(V, (int)((16u - (unsigned)(reinterpret_cast<uintptr_t>(row) & 15u)) & 15u) / 4);
@@ -243,9 +245,9 @@ __global__ void __launch_bounds__(256) target_logprob_kernel(int V, const float 
   }
   for (; q < nvec; q += 256) take4(__ldcs(body + q));
   for (int v = head + 4 * nvec + tid; v < V; v += 256) take(row[v]);
-  auto join = [](float &ma, float &sa, float mb, float sb) {
-    const float mx = fmaxf(ma, mb);
-    if (mx > -INFINITY) sa = sa * expf(ma - mx) + sb * expf(mb - mx);
+  auto join = [&](float &ma, float &sa, float mb, float sb) {
+    const float mx = fmaxf(ma, mb), r = finite(mx);
+    sa = sa * expf(ma - r) + sb * expf(mb - r);
     ma = mx;
   };
   for (int o = 16; o > 0; o >>= 1) join(m, s, __shfl_xor_sync(0xffffffffu, m, o), __shfl_xor_sync(0xffffffffu, s, o));

@@ -309,3 +309,37 @@ def test_cross_attention_with_keys_out_of_range(dtype, rows, first, last):
                     s[:, first:last] = -float("inf")
                 ref = torch.softmax(s, -1) @ kv[0, h, 1].double()
                 assert (got - ref).abs().max().item() <= (2e-5 if dtype == "fp32" else 2 * 2.0 ** -9 * kv.abs().max().item())
+
+
+@pytest.mark.parametrize("vocab", [301, 2304])
+@pytest.mark.parametrize("first", [0, 4, 297])
+def test_log_probabilities_of_logits_out_of_range(vocab, first):
+    """Four output vectors that are no numbers (a thread's first load of a row among them) leave no row a log-probability; four whose logits
+    overflow to -inf take no part in the sums: the row's log-probability is that of the other words."""
+    from paper_2506_23431_b200.binding import PipelinedDecoder
+    wl = W.CONFIGS["bart_base"].scaled(name="tf_nan", n_layers=1, d_model=128, n_heads=2, d_ff=256, vocab=vocab, norm_gain_std=0.1, batch=1, ctx=40,
+                                       sub_max=2, delta_t=2, max_sub_len=15, length_dist=("uniform", 5, 15), time_max=25, pos_mode=ROPE)
+    weights = W.make_weights(wl)
+    # the embedding's first column dominates and the final norm keeps nothing else: every hidden state is +c, 0, 0, ...
+    weights["embed"][:, 0] = 64.0
+    weights["final_norm"][:] = 0
+    weights["final_norm"][0] = 1
+    subs = [[[20, 21, 22], [23]]]
+    lp = {}
+    for bad in (0.0, np.nan, -3e38):
+        w = dict(weights, lm_head=weights["lm_head"].copy())
+        w["lm_head"][first:first + 4, 0] = bad
+        w["lm_head"][wl.sep_id, 0] = weights["lm_head"][wl.sep_id, 0]
+        dec = PipelinedDecoder(wl.hyper(), w, wl.batch)
+        dec.encode_context(dec.device_memory(W.make_encoder_memory(wl)), [wl.ctx], None)
+        lp[str(bad)], _, logits = dec.teacher_forward(subs, want_logits=True)
+        z = logits.cpu().numpy().astype(np.float64)
+        tgt = [20, 21, 22, wl.sep_id, 23, wl.sep_id]
+        if bad == bad:
+            keep = np.isfinite(z)
+            assert (~keep).sum() == (0 if bad == 0 else 6 * (4 - (first <= wl.sep_id < first + 4)))
+            want = [z[r, t] - np.log(np.exp(z[r][keep[r]] - z[r][keep[r]].max()).sum()) - z[r][keep[r]].max() for r, t in enumerate(tgt)]
+            assert np.abs(lp[str(bad)] - want).max() <= 1e-4
+        else:
+            assert np.isnan(lp[str(bad)]).all()
+        dec.close()
