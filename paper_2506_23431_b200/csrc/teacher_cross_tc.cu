@@ -13,6 +13,8 @@
 // documents of 1000 in 64-row blocks, 12 heads: 13.9 us against 17.5 us.  The loads and products alone, without the exponentials, take 176 us.
 // Every mbarrier wait is bounded: on expiry the kernel records PD_ERR_TIMEOUT, stops waiting, falls through to the
 // common exit and frees its tensor memory.
+#include <float.h>
+
 #include "pd_internal.h"
 
 namespace pd {
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(XC_THREADS, 2) teacher_cross_kernel(const __gr
       for (int i = 0; i < 64; ++i) mx[i & 3] = fmaxf(mx[i & 3], __uint_as_float(r[i]));
       const float m = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sl2;
       if (j == 0) {
-        m_used = m;
+        m_used = fmaxf(m, -FLT_MAX);                        // (finite also where all 64 scores have overflowed to -inf: they weigh 0)
       } else if (__any_sync(0xffffffffu, m > m_used + XC_LAG)) {      // some row's maximum has moved too far: rescale this warp's rows of O
         if (!c_mbar_wait(bar_pv + 8 * ((j - 1) & 1), (uint32_t)((j - 1) >> 1) & 1u)) { ok = false; break; }
         __syncwarp();

@@ -343,3 +343,31 @@ def test_log_probabilities_of_logits_out_of_range(vocab, first):
         else:
             assert np.isnan(lp[str(bad)]).all()
         dec.close()
+
+
+@pytest.mark.parametrize("ctx,bad", [(130, (0, 64)), (130, (0, 128)), (300, (64, 200)), (64, (0, 63))])
+def test_teacher_forward_with_keys_whose_scores_overflow(ctx, bad):
+    """Keys that score -inf with every query - a row's whole first half tile among them - weigh nothing: the forward over a context that
+    holds them equals the oracle's over the rest (cross-attention has no positions)."""
+    from oracle import pipelined_decoder as O
+    from paper_2506_23431_b200.binding import PipelinedDecoder
+    wl = W.CONFIGS["bart_base"].scaled(name="tf_over", n_layers=1, d_model=128, n_heads=2, d_ff=256, vocab=301, norm_gain_std=0.1, batch=1, ctx=ctx,
+                                       sub_max=5, delta_t=2, max_sub_len=15, length_dist=("uniform", 10, 15), time_max=25, pos_mode=ROPE)
+    weights, mem, subs = W.make_weights(wl), W.make_encoder_memory(wl), [[[5, 6, 7, 8], [9, 10], [11] * 15, [12] * 15, [13] * 15]]
+    # every query is positive (the first column of every state dominates and feeds all of wq_c's columns), the bad positions' keys
+    # are -2e38 in every column; values take nothing from the column that makes them so
+    weights["embed"][:, 0] = 8.0
+    weights["l0.wq_c"][0] = 0.5
+    weights["l0.wkv_c"][0, :128], weights["l0.wkv_c"][0, 128:] = 1.0, 0.0
+    mem[0, :, 0] = 0
+    weights = {k: W.bf16_round(v) if k != "rel_bias" else v for k, v in weights.items()}
+    worse = mem.copy()
+    worse[0, bad[0]:bad[1], 0] = -2e38
+    keep = np.ones(ctx, bool)
+    keep[bad[0]:bad[1]] = False
+    dec = PipelinedDecoder(wl.hyper(), weights, wl.batch)
+    dec.encode_context(dec.device_memory(W.bf16_round(worse)), [ctx], None)
+    got = dec.teacher_forward(subs, want_logits=True)[2].cpu().numpy()
+    ref = O.PipelinedDecoderOracle(weights, wl.hyper()).teacher_forward(mem[0][keep], int(keep.sum()), subs[0])["logits"]
+    assert np.abs(got - ref).max() <= 2e-2
+    dec.close()
