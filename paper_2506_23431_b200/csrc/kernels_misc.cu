@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(1024) rmsnorm_kernel(int d, float eps, const f
     v = *reinterpret_cast<const float4 *>(x + (size_t)blockIdx.x * d + c);
     gn = load4_table(gain + c);
   }
-  float ss = v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
+  float ss = fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.x, v.x, v.y * v.y)));      // (written out: the same bits however the code around it is compiled)
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ss;
   __syncthreads();
