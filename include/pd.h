@@ -308,7 +308,8 @@ PD_API pd_status pd_get_stats(pd_handle *h, int64_t *stats);
  *                (the kernels clamp what they read to these ranges, so a bad value gives a wrong
  *                result for that sequence, never an access outside the tensors)
  *   splits       1..32: split-K factor over the context of the plain-ALU kernel (fp32, or more
- *                than 32 rows per sequence; partials are merged by a second kernel).  The bf16
+ *                than 32 rows per sequence; partials are merged by a second kernel), at most one
+ *                per 256 positions of max_ctx in use.  The bf16
  *                tensor-core kernel spreads the context tiles over the GPU by itself.
  *   scratch      device, 256-byte aligned, at least pd_cross_attention_scratch_bytes(...): a
  *                256-byte header (int32 word 2 receives PD_ERR_TIMEOUT if a bounded wait inside

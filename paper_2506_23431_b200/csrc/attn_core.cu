@@ -6,30 +6,31 @@
 // These are the fp32 path of every configuration and the bf16 path when a sequence has more
 // than 32 rows; otherwise bf16 runs the tensor-core kernels in self_attn_tc.cu and
 // cross_attn_tma.cu.
+#include <type_traits>
+
 #include "pd_internal.h"
 
 namespace pd {
 
-template <typename T> __device__ __forceinline__ float ld_f(const T *p);
-template <> __device__ __forceinline__ float ld_f<float>(const float *p) { return *p; }
-template <> __device__ __forceinline__ float ld_f<__nv_bfloat16>(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
 template <typename T> __device__ __forceinline__ void st_f(T *p, float v);
 template <> __device__ __forceinline__ void st_f<float>(float *p, float v) { *p = v; }
 template <> __device__ __forceinline__ void st_f<__nv_bfloat16>(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void st_f2(float *p, float x, float y) { *reinterpret_cast<float2 *>(p) = make_float2(x, y); }
+__device__ __forceinline__ void st_f2(__nv_bfloat16 *p, float x, float y) { *reinterpret_cast<__nv_bfloat162 *>(p) = __floats2bfloat162_rn(x, y); }
 template <typename T> __device__ __forceinline__ float2 ld_f2(const T *p);
 template <> __device__ __forceinline__ float2 ld_f2<float>(const float *p) { return *reinterpret_cast<const float2 *>(p); }
 template <> __device__ __forceinline__ float2 ld_f2<__nv_bfloat16>(const __nv_bfloat16 *p) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p)); }
 
 constexpr int TK = 32;            // keys per tile: one per lane
-constexpr int NT = 256;           // threads per CTA
-constexpr int NW = NT / 32;
+constexpr int NW = 8;             // warps per CTA at most
+constexpr int REG_WARPS = 12;     // warps the registers are shared out for: 168 each, three warps per quarter of an SM (two with any more)
 constexpr int MAXD = 512;         // longest distance table held in shared memory
 constexpr int PP = TK + 4;        // floats per row of a warp's weights
 
 template <typename T> __host__ __device__ constexpr int row_bytes() { return kDh * (int)sizeof(T) + 16; }      // padded: lanes read rows of their own without conflicts
-template <typename T> constexpr int ring_bytes() { return NW * 2 * TK * row_bytes<T>(); }                      // per warp one tile of keys and one of values
-constexpr int MERGE_BYTES = NW * kCoreRows * (kDh + 2) * 4;
-template <typename T> constexpr int core_smem() { return (ring_bytes<T>() > MERGE_BYTES ? ring_bytes<T>() : MERGE_BYTES) + NW * kCoreRows * PP * 4; }
+template <typename T> __host__ __device__ constexpr int ring_bytes() { return 2 * TK * row_bytes<T>(); }      // per warp: one tile of keys and one of values
+template <typename T> constexpr int core_smem(int warps) { return warps * (ring_bytes<T>() + kCoreRows * PP * 4); }
+static_assert(ring_bytes<__nv_bfloat16>() >= kCoreRows * (kDh + 2) * 4, "a warp's (O, m, l) fits over its ring");
 
 __device__ __forceinline__ void c_cp_async16(uint32_t dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -50,19 +51,20 @@ template <bool SWZ> __device__ __forceinline__ float4 key4(const __nv_bfloat16 *
 // no number keeps a weight that is none, whichever warp or split meets it.
 __device__ __forceinline__ float finite(float m) { return m == -INFINITY ? 0.f : m; }
 
-// One CTA = one (split, head, sequence, chunk of up to 16 rows).  Its eight warps work alone on every eighth 32-key tile: a lane
+// One CTA = one (split, head, sequence, chunk of up to 16 rows).  Its warps, eight at most, work alone on every eighth 32-key tile: a lane
 // holds one key for the scores (queries come as broadcasts from shared memory) and two columns of the output for
 // P.V; online softmax per warp, one merge at the end.  Each warp has room for one tile of keys and one of values: the
 // next keys travel while the weights meet the values, the next values while the next scores are taken.
 // What bounds it at decode sizes is the chain of latencies of a tile, so nothing in the walk waits for another warp.  (Tiles
 // staged for the whole CTA with five barriers each: 19.3 us for 4 rows over 256 fp32 keys, against 7.9 us;
 // 16 x 12 heads x 1000 keys, 9 rows: 87 us against 62-65 us.)
-template <typename T, bool SELF>
-__global__ void __launch_bounds__(NT) attn_core_kernel(AttnArgs a) {
+// FULL = all NW warps (the count then folds into every address and loop), else as many as the launch has.
+template <typename T, bool SELF, bool FULL>
+__global__ void __launch_bounds__(REG_WARPS * 32) attn_core_kernel(AttnArgs a) {
   const Dims &dm = a.dm;
   const int n_chunk = (dm.C + kCoreRows - 1) / kCoreRows;
   const int split = blockIdx.x / n_chunk, h = blockIdx.y, b = blockIdx.z, c0 = (blockIdx.x % n_chunk) * kCoreRows;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = FULL ? NW : (int)blockDim.x >> 5, nt = nw * 32;
   __shared__ __align__(16) float Qs[kCoreRows][kDh];
   extern __shared__ __align__(16) uint8_t core_raw[];   // the warps' tiles (then their (O, m, l)), the warps' weights
   __shared__ float bias_d[SELF ? MAXD : 1];
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(NT) attn_core_kernel(AttnArgs a) {
   const int t = SELF ? a.st.hdr[HDR_STEP_T] - a.st.t0[b] : 0;        // the sequence's own step
   const bool use_bias = SELF && dm.pos_mode == PD_POS_T5_BIAS;
   if (use_bias)
-    for (int dd = tid; dd < dm.n_dist && dd < MAXD; dd += NT)
+    for (int dd = tid; dd < dm.n_dist && dd < MAXD; dd += nt)
       bias_d[dd] = a.rel_bias[h * a.rel_buckets + a.dist_bucket[dd]] * 1.4426950408889634f;  // log2 domain
   if (tid < kCoreRows) sub_s[tid] = (SELF && tid < S) ? a.st.row_sub[row0 + tid] : 0;
   int n_tiles, ctx_len = 0;
@@ -88,17 +90,17 @@ __global__ void __launch_bounds__(NT) attn_core_kernel(AttnArgs a) {
   }
   constexpr int RB = row_bytes<T>();
   constexpr bool SWZ = SELF && sizeof(T) == 2;
-  uint8_t *ring = core_raw + warp * 2 * TK * RB;
+  uint8_t *ring = core_raw + warp * ring_bytes<T>();
   const uint32_t ring_k = (uint32_t)__cvta_generic_to_shared(ring), ring_v = ring_k + TK * RB;
-  float *ps = reinterpret_cast<float *>(core_raw + (ring_bytes<T>() > MERGE_BYTES ? ring_bytes<T>() : MERGE_BYTES)) + warp * kCoreRows * PP;
+  float *ps = reinterpret_cast<float *>(core_raw + nw * ring_bytes<T>()) + warp * kCoreRows * PP;
 
   struct Tile { int n_valid, k_sub, k_tau0; const T *kp; };      // keys that exist (0: the walk is over), subsequence, first timestamp
-  int at = split * NW + warp;
+  int at = split * nw + warp;
   const size_t v_off = SELF ? kDh : (size_t)dm.ctx * kDh, kstride = SELF ? 2 * kDh : kDh;
   auto next_tile = [&]() {
     Tile x;
     x.n_valid = 0; x.k_sub = 0; x.k_tau0 = 0; x.kp = nullptr;
-    for (; at < n_tiles && x.n_valid <= 0; at += a.splits * NW) {
+    for (; at < n_tiles && x.n_valid <= 0; at += a.splits * nw) {
       if (SELF) {
         const int ksub = at / dm.PPS + 1, j = at % dm.PPS;
         const int sidx = b * dm.SM + ksub - 1, e0 = j * dm.P;
@@ -132,11 +134,13 @@ __global__ void __launch_bounds__(NT) attn_core_kernel(AttnArgs a) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   T *out = (T *)a.out;
   if (split == 0)                                       // rows beyond the active ones stay zero
-    for (int idx = tid; idx < (min(kCoreRows, dm.C - c0) - max(S, 0)) * kDh; idx += NT)
+    for (int idx = tid; idx < (min(kCoreRows, dm.C - c0) - max(S, 0)) * kDh; idx += nt)
       st_f<T>(out + (size_t)(row0 + max(S, 0) + idx / kDh) * dm.d + h * kDh + idx % kDh, 0.f);
   if (S <= 0) return;
-  for (int idx = tid; idx < kCoreRows * kDh; idx += NT)
-    Qs[idx / kDh][idx % kDh] = idx < S * kDh ? ld_f<T>((const T *)a.q + (size_t)(row0 + idx / kDh) * dm.d + h * kDh + idx % kDh) : 0.f;
+  for (int idx = tid; idx < kCoreRows * kDh / 4; idx += nt) {        // four columns at a time: a CTA may have only one warp
+    const int r = idx / (kDh / 4), c = 4 * (idx % (kDh / 4));
+    *reinterpret_cast<float4 *>(&Qs[r][c]) = r < S ? key4<false>((const T *)a.q + (size_t)(row0 + r) * dm.d + h * kDh, 0, c / 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
   __syncthreads();
 
   float o[kCoreRows][2];
@@ -238,59 +242,76 @@ __global__ void __launch_bounds__(NT) attn_core_kernel(AttnArgs a) {
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   // ---- merge of the warps
   __syncthreads();
-  float *mo = reinterpret_cast<float *>(core_raw), *mm = mo + NW * kCoreRows * kDh, *ml = mm + NW * kCoreRows;
+  float *mo = reinterpret_cast<float *>(core_raw), *mm = mo + nw * kCoreRows * kDh, *ml = mm + nw * kCoreRows;
 #pragma unroll
   for (int s = 0; s < kCoreRows; ++s)
     if (s < S) *reinterpret_cast<float2 *>(&mo[(warp * kCoreRows + s) * kDh + 2 * lane]) = make_float2(o[s][0], o[s][1]);
   if (lane < S) { mm[warp * kCoreRows + lane] = m_run; ml[warp * kCoreRows + lane] = l_run; }
   __syncthreads();
-  for (int idx = tid; idx < S * kDh; idx += NT) {
-    const int s = idx / kDh, dim = idx % kDh, r = row0 + s;
-    float M = -INFINITY;
+  for (int s = warp; s < S; s += nw) {                  // a row per warp, two columns per lane
+    const int r = row0 + s;
+    float m[NW], M = -INFINITY, L = 0.f;               // (absent warps: -inf, weight 0; their loads do not wait for one another's test)
 #pragma unroll
-    for (int w = 0; w < NW; ++w) M = fmaxf(M, mm[w * kCoreRows + s]);
-    float L = 0.f, O = 0.f;
+    for (int w = 0; w < NW; ++w) { m[w] = w < nw ? mm[w * kCoreRows + s] : -INFINITY; M = fmaxf(M, m[w]); }
+    float2 O = make_float2(0.f, 0.f);
 #pragma unroll
     for (int w = 0; w < NW; ++w) {
-      const float f = exp2f(mm[w * kCoreRows + s] - finite(M));
-      L += ml[w * kCoreRows + s] * f;
-      O += mo[(w * kCoreRows + s) * kDh + dim] * f;
+      const float f = exp2f(m[w] - finite(M)), l = w < nw ? ml[w * kCoreRows + s] : 0.f;
+      const float2 u = w < nw ? *reinterpret_cast<const float2 *>(&mo[(w * kCoreRows + s) * kDh + 2 * lane]) : make_float2(0.f, 0.f);
+      L += l * f;
+      O.x += u.x * f; O.y += u.y * f;
     }
     if (a.splits == 1) {
-      st_f<T>(out + (size_t)r * dm.d + h * kDh + dim, O / L);
+      st_f2(out + (size_t)r * dm.d + h * kDh + 2 * lane, O.x / L, O.y / L);
     } else {
       const size_t pi = ((size_t)r * dm.H + h) * a.splits + split;
-      a.part_o[pi * kDh + dim] = O;
-      if (dim == 0) { a.part_ml[pi * 2] = M; a.part_ml[pi * 2 + 1] = L; }
+      *reinterpret_cast<float2 *>(a.part_o + pi * kDh + 2 * lane) = O;
+      if (lane == 0) { a.part_ml[pi * 2] = M; a.part_ml[pi * 2 + 1] = L; }
     }
   }
 }
 
-cudaError_t attn_core_prepare(int dtype, bool self) {
+template <typename T, bool SELF>
+static cudaError_t prepare_core() {
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  if (dtype == PD_DTYPE_BF16)
-    return self ? cudaFuncSetAttribute(attn_core_kernel<__nv_bfloat16, true>, attr, core_smem<__nv_bfloat16>())
-                : cudaFuncSetAttribute(attn_core_kernel<__nv_bfloat16, false>, attr, core_smem<__nv_bfloat16>());
-  return self ? cudaFuncSetAttribute(attn_core_kernel<float, true>, attr, core_smem<float>())
-              : cudaFuncSetAttribute(attn_core_kernel<float, false>, attr, core_smem<float>());
+  const cudaError_t e = cudaFuncSetAttribute(attn_core_kernel<T, SELF, true>, attr, core_smem<T>(NW));
+  return e != cudaSuccess ? e : cudaFuncSetAttribute(attn_core_kernel<T, SELF, false>, attr, core_smem<T>(NW));
 }
+cudaError_t attn_core_prepare(int dtype, bool self) {
+  if (dtype == PD_DTYPE_BF16) return self ? prepare_core<__nv_bfloat16, true>() : prepare_core<__nv_bfloat16, false>();
+  return self ? prepare_core<float, true>() : prepare_core<float, false>();
+}
+
+// The tiles of a round of eight warps per split: with fewer, a split adds a launch and takes no tile off any warp's walk.
+int attn_core_splits_useful(int ctx) { return (ctx + NW * TK - 1) / (NW * TK); }
 
 // pdl: launched as a programmatic dependent of the kernel before it - only where that kernel writes none of the state, and
 // what it writes is read behind the wait (queries, the step's keys/values).
 cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, bool pdl, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
-  // chunks share a dimension with the splits: the sequences alone may fill theirs (the entry points take 65535)
-  cfg.gridDim = dim3(a.splits * ((a.dm.C + kCoreRows - 1) / kCoreRows), a.dm.H, a.batch);
-  cfg.blockDim = dim3(NT, 1, 1);
-  cfg.dynamicSmemBytes = dtype == PD_DTYPE_BF16 ? core_smem<__nv_bfloat16>() : core_smem<float>();
+  // Chunks share a dimension with the splits: the sequences alone may fill theirs (the entry points take 65535).
+  const int chunks = (a.dm.C + kCoreRows - 1) / kCoreRows;
+  cfg.gridDim = dim3(a.splits * chunks, a.dm.H, a.batch);
+  // Warps: with a CTA per SM at most, all eight (they share the loads ahead of the walk).  Beyond that no more than there are tiles for, and as
+  // few as keep the number of rounds: a warp without a tile holds 12 - 20 KB of shared memory that another CTA could use.  64 sequences x
+  // 12 heads, fp32: 20 rows over 64 keys 92 us with eight warps each, 33 with two; 33 rows over 300 keys 269 us, 162 with five.
+  const int tiles = self ? a.dm.SM * a.dm.PPS : (a.dm.ctx + TK - 1) / TK, each = (tiles + a.splits - 1) / a.splits;
+  const int rounds = (each + NW - 1) / NW;
+  const int warps = (long long)a.splits * chunks * a.dm.H * a.batch <= 148 ? NW : (each + rounds - 1) / rounds;
+  cfg.blockDim = dim3(32 * warps, 1, 1);
+  cfg.dynamicSmemBytes = dtype == PD_DTYPE_BF16 ? core_smem<__nv_bfloat16>(warps) : core_smem<float>(warps);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = pdl ? 1 : 0;
-  if (dtype == PD_DTYPE_BF16)
-    return self ? cudaLaunchKernelEx(&cfg, attn_core_kernel<__nv_bfloat16, true>, a) : cudaLaunchKernelEx(&cfg, attn_core_kernel<__nv_bfloat16, false>, a);
-  return self ? cudaLaunchKernelEx(&cfg, attn_core_kernel<float, true>, a) : cudaLaunchKernelEx(&cfg, attn_core_kernel<float, false>, a);
+  auto launch = [&](auto full) {
+    constexpr bool F = decltype(full)::value;
+    if (dtype == PD_DTYPE_BF16)
+      return self ? cudaLaunchKernelEx(&cfg, attn_core_kernel<__nv_bfloat16, true, F>, a) : cudaLaunchKernelEx(&cfg, attn_core_kernel<__nv_bfloat16, false, F>, a);
+    return self ? cudaLaunchKernelEx(&cfg, attn_core_kernel<float, true, F>, a) : cudaLaunchKernelEx(&cfg, attn_core_kernel<float, false, F>, a);
+  };
+  return warps == NW ? launch(std::true_type()) : launch(std::false_type());
 }
 
 // Merge of the split-K partials (m, l, o) of one row and head: the usual log-sum-exp rescale.

@@ -2,6 +2,8 @@
 // launches, on caller-supplied queries and context keys/values, without a decoder handle.
 #include <string.h>
 
+#include <algorithm>
+
 #include "pd_internal.h"
 
 using namespace pd;
@@ -59,10 +61,11 @@ pd_status cross_attention_enqueue(int dtype, int batch, int rows_per_seq, int n_
     a.clear_status = 1;      // one launch is the whole call: a separate clear of the header cost 2 us
     return launch_cross_attn_tma(a, tmap, tmap, s) == cudaSuccess ? PD_OK : PD_ERR_CUDA;
   }
+  a.splits = std::min(splits, attn_core_splits_useful(max_ctx));
   if (cudaMemsetAsync(base, 0, kOpHeaderBytes, s) != cudaSuccess) return PD_ERR_CUDA;
   if (attn_core_prepare(dtype, false) != cudaSuccess) return PD_ERR_CUDA;
   if (launch_attn_core(a, dtype, false, false, s) != cudaSuccess) return PD_ERR_CUDA;
-  if (splits > 1 && launch_attn_merge(a, dtype, s) != cudaSuccess) return PD_ERR_CUDA;
+  if (a.splits > 1 && launch_attn_merge(a, dtype, s) != cudaSuccess) return PD_ERR_CUDA;
   return PD_OK;
 }
 

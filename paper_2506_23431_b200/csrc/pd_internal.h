@@ -184,6 +184,7 @@ cudaError_t launch_ctx_kv_relayout(const Dims &dm, int b0, int batch, int layer,
                                    cudaStream_t s);
 constexpr int kCoreRows = 16;            // rows per CTA of the plain-ALU attention kernel
 cudaError_t attn_core_prepare(int dtype, bool self);      // once per device, outside any stream capture
+int attn_core_splits_useful(int ctx);    // more splits than this over a context of ctx positions would not shorten any warp's walk
 cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, bool pdl, cudaStream_t s);
 cudaError_t launch_attn_merge(const AttnArgs &a, int dtype, cudaStream_t s);
 cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, cudaStream_t s);

@@ -371,3 +371,19 @@ def test_teacher_forward_with_keys_whose_scores_overflow(ctx, bad):
     ref = O.PipelinedDecoderOracle(weights, wl.hyper()).teacher_forward(mem[0][keep], int(keep.sum()), subs[0])["logits"]
     assert np.abs(got - ref).max() <= 2e-2
     dec.close()
+
+
+@pytest.mark.parametrize("dtype,rows", [("fp32", 1), ("fp32", 17), ("bf16", 33)])
+@pytest.mark.parametrize("ctx,splits", [(1, 1), (32, 4), (33, 1), (257, 2), (300, 4), (515, 3)])
+def test_plain_alu_attention_with_few_tiles_per_cta(dtype, rows, ctx, splits):
+    """More (sequence, head, chunk) triples than SMs, so that a CTA has as many warps as it has tiles for: one to eight, with ragged contexts
+    and rows, one split and several; tolerances as for the operator's other tests."""
+    import torch
+    from paper_2506_23431_b200 import binding as B
+    q, kv, n_rows, ctx_len = cross_case(ctx, 40, rows, 4, ctx, dtype)
+    ref = oracle_cross(q, kv, n_rows, ctx_len, 4, 0.125)
+    dev, td = torch.device("cuda", 0), torch.float32 if dtype == "fp32" else torch.bfloat16
+    out = B.cross_attention(torch.from_numpy(q).to(dev, td), torch.from_numpy(kv).to(dev, td), torch.from_numpy(n_rows).to(dev),
+                            torch.from_numpy(ctx_len).to(dev), 0.125, splits)
+    tol = 2e-5 if dtype == "fp32" else 2 * 2.0 ** -9 * max(1.0, np.abs(kv[np.isfinite(kv)]).max())
+    assert np.abs(out.float().cpu().numpy().astype(np.float64) - ref).max() <= tol
