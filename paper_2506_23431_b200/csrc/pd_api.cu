@@ -715,7 +715,7 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
     if (encode_vocab_maps(&h->vmaps, h->ptr<void>(L.hbuf), (uint64_t)dm.B * dm.C, weights->lm_head, (uint64_t)dm.V,
                           (uint64_t)dm.d, &code) != cudaSuccess)
       return bail(PD_ERR_CUDA);
-    if (vocab_tc_prepare(1) != cudaSuccess || vocab_tc_prepare(dm.B * dm.C) != cudaSuccess) return bail(PD_ERR_CUDA);   // (a smaller batch may take the other variant)
+    if (vocab_tc_prepare(1, dm.V, cfg->store_logits != 0) != cudaSuccess || vocab_tc_prepare(dm.B * dm.C, dm.V, cfg->store_logits != 0) != cudaSuccess) return bail(PD_ERR_CUDA);   // (a smaller batch may take the other variant)
     h->vocab_tc = true;
   }
   if (h->vocab_tc && h->have_tmap && self_attn_tc_supported(dm)) {
@@ -1152,7 +1152,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
     if (dm.V % 4 == 0 || !h->vocab_tc) return gemm(h, true, n, dm.V, dm.d, rows_hb, h->w.lm_head, out, true, 0.f);
     VocabMaps maps;
     CU_TRY(h, encode_vocab_maps(&maps, rows_hb, (uint64_t)n, h->w.lm_head, (uint64_t)dm.V, (uint64_t)dm.d, nullptr));
-    CU_TRY(h, vocab_tc_prepare(n));
+    CU_TRY(h, vocab_tc_prepare(n, dm.V, true));
     VocabArgs va;
     memset(&va, 0, sizeof(va));
     va.m_fixed = n; va.V = dm.V; va.K = dm.d; va.rows_cap = n; va.eos = -1; va.sep = -1; va.logits = out; va.status = h->st.hdr + HDR_STATUS;

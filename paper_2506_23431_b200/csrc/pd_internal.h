@@ -228,7 +228,7 @@ struct VocabMaps { CUtensorMap a, a32, b; };   // hidden rows (128-row and 32-ro
 int vocab_tc_slice(int V);
 int vocab_tc_tiles(int V);
 bool vocab_tc_supported(int K, int V);
-cudaError_t vocab_tc_prepare(int rows_cap);   // the variant for this many rows: once per device, outside any stream capture
+cudaError_t vocab_tc_prepare(int rows_cap, int V, bool logits);   // the variant for this many rows and ids, logits stored or not: once per device, outside any stream capture
 cudaError_t encode_vocab_maps(VocabMaps *m, const void *hidden, uint64_t rows, const void *lm_head, uint64_t vocab, uint64_t K,
                               int *driver_code);
 cudaError_t launch_vocab_tc(const VocabMaps &m, const VocabArgs &a, cudaStream_t s);

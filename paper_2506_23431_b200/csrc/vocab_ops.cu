@@ -74,7 +74,7 @@ pd_status pd_vocab_argmax(int32_t rows, int32_t d_model, int32_t vocab, const vo
   VocabMaps maps;
   if (encode_vocab_maps(&maps, hidden, (uint64_t)rows, lm_head, (uint64_t)vocab, (uint64_t)d_model, nullptr) != cudaSuccess)
     return PD_ERR_CUDA;
-  if (vocab_tc_prepare(rows) != cudaSuccess) return PD_ERR_CUDA;
+  if (vocab_tc_prepare(rows, vocab, logits != nullptr) != cudaSuccess) return PD_ERR_CUDA;
   VocabArgs a;
   a.n_active = nullptr; a.batch = 0; a.m_fixed = rows; a.V = vocab; a.K = d_model; a.rows_cap = rows;
   a.eos = -1; a.sep = -1;

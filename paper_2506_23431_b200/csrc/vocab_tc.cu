@@ -10,7 +10,7 @@
 // of lm_head; more rows take more passes, which re-read the slice from L2).  The number of rows is
 // read on the device (the sum of the sequences' active rows), so work follows the rows that exist,
 // not the allocated maximum.  Warp 0 streams 64-column blocks of hidden and lm_head into a
-// shared-memory ring of two or three stages with TMA (128-byte swizzle, mbarrier completion; of a ragged last row
+// shared-memory ring of two to four stages with TMA (128-byte swizzle, mbarrier completion; of a ragged last row
 // tile only the 32-row boxes that hold rows travel; the first lm_head blocks, which do not depend on the
 // kernel before, are requested ahead of the programmatic-dependency wait); one lane of
 // warp 1 issues tcgen05.mma (M 128, N 224, K 16, bf16 in, fp32 accumulators in tensor memory) and
@@ -38,11 +38,11 @@ constexpr int VT_LOGIT_BYTES = 4 * 32 * VT_LPITCH * 4;
 // TILES = row tiles (accumulators) per pass.  Up to 128 rows one is enough, and half the stage and half of tensor memory let two
 // CTAs share an SM: all slices of a vocabulary of 50265 are then resident at once, and one CTA's epilogue runs under the
 // other's copies.  100 rows x 50265 ids of width 768, logits stored, per launch: 23.6 us, against 34.4 us with the two-tile form
-// (one CTA per SM, two rounds).
-__host__ __device__ constexpr int vt_stages(int tiles) { return tiles == 1 ? 2 : 3; }
+// (one CTA per SM, two rounds).  STAGES of the ring: what the shared memory of an SM holds - two for each of two CTAs; where there are
+// no more slices than SMs a CTA has one to itself, and takes four (17 rows x 20081 ids of width 768: logits stored: 22.5 us with two, 20.6 us with four).
 __host__ __device__ constexpr int vt_stage_bytes(int tiles) { return tiles * VT_A_BYTES + VT_B_BYTES; }
 __host__ __device__ constexpr int vt_tmem_cols(int tiles) { return 256 * tiles; }      // accumulator j at column 256 j
-constexpr int vt_smem(int tiles) { return vt_stages(tiles) * vt_stage_bytes(tiles) + 128 /*barriers*/ + VT_LOGIT_BYTES + 1024 /*alignment slack*/; }
+constexpr int vt_smem(int tiles, int stages) { return stages * vt_stage_bytes(tiles) + 128 /*barriers*/ + VT_LOGIT_BYTES + 1024 /*alignment slack*/; }
 constexpr uint32_t VT_SPIN_LIMIT = 1u << 24;
 // instruction descriptor of kind::f16: D fp32, A and B bf16, both K-major, N >> 3 at bit 17, M >> 4 at bit 24
 __device__ __forceinline__ uint32_t v_idesc(int n) {
@@ -136,11 +136,12 @@ __device__ __forceinline__ void v_tmem_ld16(uint32_t taddr, uint32_t (&r)[32]) {
 __device__ __forceinline__ void v_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void v_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-template <int TILES>
-__global__ void __launch_bounds__(VT_THREADS, TILES == 1 ? 2 : 1)
+// LOGITS: they are stored (without that code the compiler keeps the walk over a row's columns tighter).
+template <int TILES, int STAGES, bool LOGITS>
+__global__ void __launch_bounds__(VT_THREADS, TILES == 1 && STAGES == 2 ? 2 : 1)
 vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_a32,
                 const __grid_constant__ CUtensorMap map_b, VocabArgs a) {
-  constexpr int VT_STAGES = vt_stages(TILES), VT_STAGE_BYTES = vt_stage_bytes(TILES), VT_TMEM_COLS = vt_tmem_cols(TILES);
+  constexpr int VT_STAGES = STAGES, VT_STAGE_BYTES = vt_stage_bytes(TILES), VT_TMEM_COLS = vt_tmem_cols(TILES);
   extern __shared__ uint8_t v_smem_raw[];
   __shared__ uint32_t tmem_base_s;
   __shared__ int red_s[VT_THREADS / 32];
@@ -272,16 +273,16 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     float *lblk = reinterpret_cast<float *>(v_smem_raw + (base - v_smem_u32(v_smem_raw)) + VT_STAGES * VT_STAGE_BYTES + 128) + quarter * 32 * VT_LPITCH;
     for (int p = 0; p < n_pass; ++p) {
       const int tiles = min(TILES, n_tt - TILES * p);
-      for (int j = 0; j < tiles; ++j) {                  // the rows' norm scales, while the product runs (each lane reads back its own)
+      for (int j = 0; j < tiles && a.ssq != nullptr; ++j) {      // the rows' norm scales, while the product runs (each lane reads back its own)
         const int m = (TILES * p + j) * VT_M + quarter * 32 + lane;
         float s0 = 0.f, s1 = 0.f;
-        if (a.ssq != nullptr && m < Mc) {
+        if (m < Mc) {
           const float *q = a.ssq + (size_t)m * a.ssq_stride;
           int pp = 0;
           for (; pp + 1 < a.parts; pp += 2) { s0 += __ldcg(q + pp); s1 += __ldcg(q + pp + 1); }
           if (pp < a.parts) s0 += __ldcg(q + pp);
         }
-        inv_s[j * VT_M + quarter * 32 + lane] = a.ssq != nullptr ? rsqrtf((s0 + s1) * a.inv_width + a.eps) : 1.f;
+        inv_s[j * VT_M + quarter * 32 + lane] = rsqrtf((s0 + s1) * a.inv_width + a.eps);
       }
       if (ok && !v_mbar_wait(bar_acc_full, (uint32_t)p & 1u)) ok = false;
       if (!ok) break;
@@ -290,7 +291,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         const int m = (TILES * p + j) * VT_M + quarter * 32 + lane;
         float bv = -INFINITY, te = -INFINITY, ts = -INFINITY;
         int bi = INT_MAX;
-        const float inv = inv_s[j * VT_M + quarter * 32 + lane];
+        const float inv = a.ssq != nullptr ? inv_s[j * VT_M + quarter * 32 + lane] : 1.f;
 #pragma unroll 1
         for (int c = 0; c * 32 < wn; ++c) {              // 32 columns at a time; a slice of an odd number of 16s ends with 16
           uint32_t r[32];
@@ -303,17 +304,21 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
             for (int i = 16; i < 32; ++i) r[i] = 0xff800000u;    // -inf: never a maximum, never stored (beyond the slice)
           }
           const int v0 = v_tile0 + c * 32;
+          if (a.ssq != nullptr) {                        // (a pass over the registers of its own: without a norm in front it is skipped)
+#pragma unroll
+            for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * inv);
+          }
           const bool special = ncol < 32 || v0 + 32 > a.V || (a.eos >= v0 && a.eos < v0 + 32) || (a.sep >= v0 && a.sep < v0 + 32);
           if (!special) {
 #pragma unroll
             for (int i = 0; i < 32; ++i) {               // ascending ids and a strict compare: ties keep the lowest id
-              const float x = __uint_as_float(r[i]) * inv;
+              const float x = __uint_as_float(r[i]);
               if (x > bv) { bv = x; bi = v0 + i; }
             }
           } else {
 #pragma unroll
             for (int i = 0; i < 32; ++i) {
-              const float x = __uint_as_float(r[i]) * inv;
+              const float x = __uint_as_float(r[i]);
               const int v = v0 + i;
               if (v >= a.V || i >= ncol) continue;
               if (v == a.eos) te = x;
@@ -321,13 +326,13 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
               else if (x > bv) { bv = x; bi = v; }
             }
           }
-          if (a.logits != nullptr) {
+          if (LOGITS) {
             // a thread holds 32 columns of its row: turned in shared memory, so that a warp stores 32 columns of one row at a
             // time (stored from the registers, every lane of a store touched another line: 48.8 us per launch at 100 rows
             // x 50265 ids of width 768, against 34.4 us)
             float *blk = lblk + lane * VT_LPITCH;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) blk[i] = __uint_as_float(r[i]) * inv;
+            for (int i = 0; i < 32; ++i) blk[i] = __uint_as_float(r[i]);
             __syncwarp();
             const int m0 = (TILES * p + j) * VT_M + quarter * 32, mr = min(32, Mc - m0);
             if (lane < ncol && v0 + lane < a.V) {
@@ -378,9 +383,17 @@ cudaError_t encode_vocab_maps(VocabMaps *m, const void *hidden, uint64_t rows, c
 
 bool vocab_tc_supported(int K, int V) { return K >= VT_BK && K % VT_BK == 0 && V >= 1; }
 
-cudaError_t vocab_tc_prepare(int rows_cap) {
-  return rows_cap <= VT_M ? cudaFuncSetAttribute(vocab_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, vt_smem(1))
-                          : cudaFuncSetAttribute(vocab_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, vt_smem(2));
+// The variant for this many rows and ids: f(kernel, its dynamic shared memory).
+template <bool LOGITS, typename F>
+static cudaError_t with_variant(int rows_cap, int V, F f) {
+  if (rows_cap > VT_M) return f(vocab_tc_kernel<2, 3, LOGITS>, vt_smem(2, 3));
+  if (vocab_tc_tiles(V) <= VT_SMS) return f(vocab_tc_kernel<1, 4, LOGITS>, vt_smem(1, 4));
+  return f(vocab_tc_kernel<1, 2, LOGITS>, vt_smem(1, 2));
+}
+
+cudaError_t vocab_tc_prepare(int rows_cap, int V, bool logits) {
+  auto set = [](auto kernel, int smem) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
+  return logits ? with_variant<true>(rows_cap, V, set) : with_variant<false>(rows_cap, V, set);
 }
 
 // Launched as a programmatic dependent of the kernel before it in the stream (the packed final norm or the last
@@ -391,14 +404,16 @@ cudaError_t launch_vocab_tc(const VocabMaps &m, const VocabArgs &a_in, cudaStrea
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(vocab_tc_tiles(a.V), 1, 1);
   cfg.blockDim = dim3(VT_THREADS, 1, 1);
-  cfg.dynamicSmemBytes = a.rows_cap <= VT_M ? vt_smem(1) : vt_smem(2);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr; cfg.numAttrs = 1;
-  return a.rows_cap <= VT_M ? cudaLaunchKernelEx(&cfg, vocab_tc_kernel<1>, m.a, m.a32, m.b, a)
-                            : cudaLaunchKernelEx(&cfg, vocab_tc_kernel<2>, m.a, m.a32, m.b, a);
+  auto launch = [&](auto kernel, int smem) {
+    cfg.dynamicSmemBytes = smem;
+    return cudaLaunchKernelEx(&cfg, kernel, m.a, m.a32, m.b, a);
+  };
+  return a.logits != nullptr ? with_variant<true>(a.rows_cap, a.V, launch) : with_variant<false>(a.rows_cap, a.V, launch);
 }
 
 }  // namespace pd
