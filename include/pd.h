@@ -275,7 +275,8 @@ PD_API pd_status pd_profile_read(pd_handle *h, double *ms, int64_t *launches);
  * self-attention (which = PD_PROF_SELF_ATTN) or cross-attention (PD_PROF_CROSS_ATTN) launches of
  * all layers, one layer after the other, `reps` times back to back after one warm-up pass,
  * between two CUDA events, and returns the average device time per layer launch (merge kernel
- * included when the step is split) in microseconds.  Successive layers read different memory, so
+ * included when the step is split) in microseconds.  No launch overlaps with another (in a decode step
+ * they may be programmatic dependents of the kernel before).  Successive layers read different memory, so
  * with per-layer keys/values beyond the L2 size the launches stay HBM-bound.  The decode state is
  * not changed (the attention outputs of the last layer are rewritten with the same values).
  * Synchronises. */

@@ -285,9 +285,9 @@ cudaError_t attn_core_prepare(int dtype, bool self) {
 // The tiles of a round of eight warps per split: with fewer, a split adds a launch and takes no tile off any warp's walk.
 int attn_core_splits_useful(int ctx) { return (ctx + NW * TK - 1) / (NW * TK); }
 
-// pdl: launched as a programmatic dependent of the kernel before it - only where that kernel writes none of the state, and
+// a.pdl: launched as a programmatic dependent of the kernel before it - only where that kernel writes none of the state, and
 // what it writes is read behind the wait (queries, the step's keys/values).
-cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, bool pdl, cudaStream_t s) {
+cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   // Chunks share a dimension with the splits: the sequences alone may fill theirs (the entry points take 65535).
   const int chunks = (a.dm.C + kCoreRows - 1) / kCoreRows;
@@ -304,7 +304,7 @@ cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, bool pdl, 
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = pdl ? 1 : 0;
+  cfg.attrs = attr; cfg.numAttrs = a.pdl ? 1 : 0;
   auto launch = [&](auto full) {
     constexpr bool F = decltype(full)::value;
     if (dtype == PD_DTYPE_BF16)

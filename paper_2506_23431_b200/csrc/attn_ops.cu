@@ -64,7 +64,7 @@ pd_status cross_attention_enqueue(int dtype, int batch, int rows_per_seq, int n_
   a.splits = std::min(splits, attn_core_splits_useful(max_ctx));
   if (cudaMemsetAsync(base, 0, kOpHeaderBytes, s) != cudaSuccess) return PD_ERR_CUDA;
   if (attn_core_prepare(dtype, false) != cudaSuccess) return PD_ERR_CUDA;
-  if (launch_attn_core(a, dtype, false, false, s) != cudaSuccess) return PD_ERR_CUDA;
+  if (launch_attn_core(a, dtype, false, s) != cudaSuccess) return PD_ERR_CUDA;
   if (a.splits > 1 && launch_attn_merge(a, dtype, s) != cudaSuccess) return PD_ERR_CUDA;
   return PD_OK;
 }

@@ -583,7 +583,7 @@ cudaError_t cross_attn_tma_prepare(int rows_per_seq, bool fp8) {
 }
 
 // 8-bit keys/values (a.kv_scale set): tmap = the keys' lines, tmap_v = the transposed values; else tmap alone.
-// Packed rows (a.packed): launched as a programmatic dependent of the query projection before it, which writes none of the keys,
+// a.pdl: launched as a programmatic dependent of the query projection before it, which writes none of the keys,
 // values, row counts and context lengths, so the first tiles travel while that kernel runs.
 cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, cudaStream_t s) {
   const int mt = (a.dm.C + 15) / 16;
@@ -600,7 +600,7 @@ cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, co
   attr[0].val.clusterDim.x = ns; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = a.packed ? 2 : 1;
+  cfg.attrs = attr; cfg.numAttrs = a.pdl ? 2 : 1;
   if (mt == 1) return fp8 ? cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, true>, tmap, tmap_v, a) : cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, false>, tmap, tmap_v, a);
   return fp8 ? cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, true>, tmap, tmap_v, a) : cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, false>, tmap, tmap_v, a);
 }

@@ -327,7 +327,8 @@ bool packed_path(const pd_handle *h) {
   return h->packed_ok && h->batch * h->dm.C <= kPackedMaxRows && cross_attn_tma_supported(h->dm);
 }
 
-AttnArgs attn_args(pd_handle *h, int layer, bool self) {
+// alone: not to overlap with the launch before (timing)
+AttnArgs attn_args(pd_handle *h, int layer, bool self, bool alone) {
   AttnArgs a;
   a.dm = h->dm; a.st = h->st; a.layer = layer; a.batch = h->batch;
   a.splits = self ? h->self_splits : h->cross_splits;
@@ -344,6 +345,7 @@ AttnArgs attn_args(pd_handle *h, int layer, bool self) {
   a.qkv = h->ptr<void>(h->lay.qkv);
   a.fused_append = self ? fused_append(h) : 0;
   a.packed = packed_path(h) ? 1 : 0;
+  a.pdl = (a.packed || h->f32_own) && !alone ? 1 : 0;
   a.clear_status = 0;
   a.rope_tab = h->ptr<float2>(h->lay.rope_tab);
   a.kv_scale = (!self && h->kv8) ? h->ptr<float>(h->lay.kv_scale) : nullptr;
@@ -354,30 +356,30 @@ AttnArgs attn_args(pd_handle *h, int layer, bool self) {
 // Pipelined self-attention of one layer.  The tensor-core kernel appends the step's keys/values itself and
 // merges its splits in the same launch; the plain-ALU kernel follows the append kernel and, when split,
 // is followed by the merge kernel.
-pd_status enqueue_self_attention(pd_handle *h, int layer) {
+pd_status enqueue_self_attention(pd_handle *h, int layer, bool alone = false) {
   const int dt = h->cfg.dtype;
-  AttnArgs a = attn_args(h, layer, true);
+  AttnArgs a = attn_args(h, layer, true, alone);
   if (self_tc(h)) {
     CU_TRY(h, launch_self_attn_tc(a, h->stream));
     h->own_launches++;
     return PD_OK;
   }
-  CU_TRY(h, launch_attn_core(a, dt, true, h->f32_own, h->stream));
+  CU_TRY(h, launch_attn_core(a, dt, true, h->stream));
   h->own_launches++;
   if (a.splits > 1) { CU_TRY(h, launch_attn_merge(a, dt, h->stream)); h->own_launches++; }
   return PD_OK;
 }
 
 // Batched cross-attention of one layer.
-pd_status enqueue_cross_attention(pd_handle *h, int layer) {
+pd_status enqueue_cross_attention(pd_handle *h, int layer, bool alone = false) {
   const int dt = h->cfg.dtype;
-  AttnArgs a = attn_args(h, layer, false);
+  AttnArgs a = attn_args(h, layer, false, alone);
   if (dt == PD_DTYPE_BF16 && h->have_tmap && cross_attn_tma_supported(h->dm)) {
     CU_TRY(h, launch_cross_attn_tma(a, h->tmap_kvc, h->kv8 ? h->tmap_kvc_v : h->tmap_kvc, h->stream));   // merges its own partials
     h->own_launches++;
     return PD_OK;
   }
-  CU_TRY(h, launch_attn_core(a, dt, false, h->f32_own, h->stream));
+  CU_TRY(h, launch_attn_core(a, dt, false, h->stream));
   h->own_launches++;
   if (a.splits > 1) { CU_TRY(h, launch_attn_merge(a, dt, h->stream)); h->own_launches++; }
   return PD_OK;
@@ -1129,7 +1131,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
       OWN(h, PD_PROF_CROSS_ATTN, launch_teacher_cross_tc(map_cq, map_ctx, da, s));
     }
     for (size_t g0 = 0; g0 < G; g0 += kTfCrossBatch) {              // 8-bit context: groups as "sequences" of the batched kernel
-      AttnArgs a = attn_args(h, l, false);
+      AttnArgs a = attn_args(h, l, false, true);
       a.dm.C = kTfGroup;
       a.batch = (int)std::min<size_t>(kTfCrossBatch, G - g0);
       a.q = cq; a.out = co;
@@ -1350,7 +1352,7 @@ pd_status pd_time_attention(pd_handle *h, int32_t which, int32_t reps, float *av
   for (int rep = -1; rep < reps && st == PD_OK; ++rep) {       // rep -1 is a warm-up pass
     if (rep == 0) cudaEventRecord(a, h->stream);
     for (int l = 0; l < h->dm.L && st == PD_OK; ++l)
-      st = which == PD_PROF_SELF_ATTN ? enqueue_self_attention(h, l) : enqueue_cross_attention(h, l);
+      st = which == PD_PROF_SELF_ATTN ? enqueue_self_attention(h, l, true) : enqueue_cross_attention(h, l, true);
   }
   cudaEventRecord(b, h->stream);
   cudaError_t e = cudaStreamSynchronize(h->stream);

@@ -119,9 +119,10 @@ struct AttnArgs {
   const void *qkv;
   int fused_append;
   const float2 *rope_tab;
-  // rows of q and out: 1 = the step's active rows packed back to back in (sequence, row) order, the step's keys/values are in the
-  // cache, and the launch is a programmatic dependent of the one before it; 0 = row c of sequence b at b * C + c
+  // rows of q and out: 1 = the step's active rows packed back to back in (sequence, row) order, and the step's keys/values are in the
+  // cache; 0 = row c of sequence b at b * C + c
   int packed;
+  int pdl;                     // launch as a programmatic dependent of the kernel before, which writes none of the state
   int clear_status;            // stand-alone op: the kernel clears the status word itself
   // cross-attention over 8-bit keys/values: [layer][sequence][head][keys | values] fp32 scales (else null)
   const float *kv_scale;
@@ -185,7 +186,7 @@ cudaError_t launch_ctx_kv_relayout(const Dims &dm, int b0, int batch, int layer,
 constexpr int kCoreRows = 16;            // rows per CTA of the plain-ALU attention kernel
 cudaError_t attn_core_prepare(int dtype, bool self);      // once per device, outside any stream capture
 int attn_core_splits_useful(int ctx);    // more splits than this over a context of ctx positions would not shorten any warp's walk
-cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, bool pdl, cudaStream_t s);
+cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, cudaStream_t s);
 cudaError_t launch_attn_merge(const AttnArgs &a, int dtype, cudaStream_t s);
 cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, cudaStream_t s);
 cudaError_t encode_ctx_kv8_tensor_maps(CUtensorMap *map_k, CUtensorMap *map_v, const void *base, uint64_t n_blocks, uint64_t ctx,

@@ -711,7 +711,7 @@ cudaError_t launch_self_attn_tc(const AttnArgs &a, cudaStream_t s) {
   int dev = 0, sms = 148;
   if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const bool roomy = (long long)a.splits * a.dm.H * a.batch <= 4LL * sms;      // all CTAs resident at four per SM
-  cudaLaunchConfig_t cfg = {};             // packed form: a programmatic dependent of the projection
+  cudaLaunchConfig_t cfg = {};             // packed form (a.pdl: a programmatic dependent of the projection)
   cfg.gridDim = grid;
   cfg.blockDim = dim3(STHREADS, 1, 1);
   cfg.dynamicSmemBytes = smem;
@@ -719,7 +719,7 @@ cudaError_t launch_self_attn_tc(const AttnArgs &a, cudaStream_t s) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
+  cfg.attrs = attr; cfg.numAttrs = a.pdl ? 1 : 0;
 #define PD_SELF_LAUNCH(MT_, P_)                                                                            \
   do {                                                                                                   \
     if (a.packed && roomy) return cudaLaunchKernelEx(&cfg, self_attn_tc_kernel<MT_, P_, 3, 4>, a);             \

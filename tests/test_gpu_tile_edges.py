@@ -387,3 +387,27 @@ def test_plain_alu_attention_with_few_tiles_per_cta(dtype, rows, ctx, splits):
                             torch.from_numpy(ctx_len).to(dev), 0.125, splits)
     tol = 2e-5 if dtype == "fp32" else 2 * 2.0 ** -9 * max(1.0, np.abs(kv[np.isfinite(kv)]).max())
     assert np.abs(out.float().cpu().numpy().astype(np.float64) - ref).max() <= tol
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("which", ["self_attn", "cross_attn"])
+def test_timed_attention_launches_do_not_overlap(dtype, which):
+    """pd_time_attention reports the duration of a launch, so none may begin under the one before (as they do inside a step)."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+    from paper_2506_23431_b200.binding import PipelinedDecoder
+    wl = W.CONFIGS["bart_base" if dtype == "bf16" else "tiny"].scaled(name="timed", batch=2, ctx=700, n_layers=4, sub_max=6, vocab=500)
+    dec = PipelinedDecoder(wl.hyper(), W.make_weights(wl), wl.batch)
+    dec.encode_context(dec.device_memory(W.make_encoder_memory(wl)), W.make_ctx_len(wl), W.make_forced_len(wl))
+    for _ in range(4):
+        dec.step()
+    dec.time_attention(which, 1)
+    torch.cuda.synchronize()
+    with profile(activities=[ProfilerActivity.CUDA]) as prof:
+        assert dec.time_attention(which, 5) > 0
+    spans = sorted((e.time_range.start, e.time_range.end) for e in prof.events() if "attn" in e.name)
+    dec.close()
+    if not spans:
+        pytest.skip("the profiler records no kernels here")
+    assert len(spans) >= 6 * wl.n_layers
+    assert all(b[0] >= a[1] for a, b in zip(spans, spans[1:]))
