@@ -297,7 +297,7 @@ cudaError_t launch_attn_core(const AttnArgs &a, int dtype, bool self, cudaStream
   // 12 heads, fp32: 20 rows over 64 keys 92 us with eight warps each, 33 with two; 33 rows over 300 keys 269 us, 162 with five.
   const int tiles = self ? a.dm.SM * a.dm.PPS : (a.dm.ctx + TK - 1) / TK, each = (tiles + a.splits - 1) / a.splits;
   const int rounds = (each + NW - 1) / NW;
-  const int warps = (long long)a.splits * chunks * a.dm.H * a.batch <= 148 ? NW : (each + rounds - 1) / rounds;
+  const int warps = (long long)a.splits * chunks * a.dm.H * a.batch <= kSms ? NW : (each + rounds - 1) / rounds;
   cfg.blockDim = dim3(32 * warps, 1, 1);
   cfg.dynamicSmemBytes = dtype == PD_DTYPE_BF16 ? core_smem<__nv_bfloat16>(warps) : core_smem<float>(warps);
   cfg.stream = s;

@@ -12,10 +12,8 @@
 // shared memory into warp 0; in a cluster the other CTAs push that state into the first one's shared memory,
 // which merges them in rank order (deterministic) and writes the output.  A segment without an active
 // row ends at once, and the hardware's block scheduler fills its place.
-// (Before, a persistent grid walked one list of all tiles, cut where segments were few, with partial
-// records merged through global memory; a prefix over the sequences preceded the first load.  Per launch, then -> now, us, bf16,
-// sequences x heads x context x rows: 1 x 12 x 777 x 8 12.4 -> 6.2, 4 x 12 x 777 x 8 14.5 -> 8.3, 8 x 16 x 4096 x 10 30.9 -> 26.7,
-// 16 x 12 x 1000 x 9 15.8 -> 13.9, 32 x 16 x 2048 x 12 48.4 -> 45.4, 64 x 12 x 1024 x 7 39.3 -> 37.9.)
+// Per launch, us, bf16, sequences x heads x context x rows: 1 x 12 x 777 x 8 6.2, 4 x 12 x 777 x 8 8.3, 8 x 16 x 4096 x 10 26.7,
+// 16 x 12 x 1000 x 9 13.9, 32 x 16 x 2048 x 12 45.4, 64 x 12 x 1024 x 7 37.9.
 // Every mbarrier wait is bounded: on expiry the kernel records PD_ERR_TIMEOUT and drains.
 //
 // 8-bit variant (FP8 = true): the context keys/values are E4M3 codes with one scale per (layer,
@@ -42,10 +40,9 @@ constexpr int XK = 128;                   // keys per tile
 // registers of two CTAs per SM.
 __host__ __device__ constexpr int xctas(int mt, bool fp8) { return fp8 && mt == 1 ? 4 : 2; }      // CTAs per SM
 __host__ __device__ constexpr int xring_bytes(int mt, bool fp8) { return fp8 && mt == 1 ? 48 * 1024 : 96 * 1024; }
-// consumer warps: four, each taking 32 keys of a tile.  (Eight warps of 16 keys each were measured in both
+// consumer warps, each taking 32 keys of a tile.  (Eight warps of 16 keys each were measured in both
 // variants and lost: 50.3 against 49.2 us per full bf16 launch, 31.9 against 28.7 us per 8-bit launch.)
-__host__ __device__ constexpr int xcw(bool fp8) { return fp8 ? 4 : 4; }
-__host__ __device__ constexpr int xthreads(bool fp8) { return (xcw(fp8) + 1) * 32; }
+constexpr int XCW = 4, XTHREADS = (XCW + 1) * 32;
 constexpr int XREC_WORDS = 36;            // per lane and 16-row tile: 32 output values, 2 maxima, 2 sums
 constexpr int XREC_FLOATS = XREC_WORDS * 32;
 __host__ __device__ constexpr int xsmem(int mt, bool fp8) { return xring_bytes(mt, fp8) + 128 /*barriers*/ + 1024 /*alignment slack*/; }
@@ -225,7 +222,7 @@ __device__ __forceinline__ void load_queries(uint32_t (&qf)[MT][4][4], const __n
 template <int MT, bool FP8>
 __device__ __forceinline__ void tile_step(TileAcc (&acc)[MT], const uint32_t (&qf)[MT][4][4], uint32_t kbase, uint32_t vbase, int key0, int kb,
                                           int ctx_len, float seg_sl2, int lane) {
-  constexpr int KPW = XK / xcw(FP8), NTW = KPW / 8, KSW = KPW / 16;      // keys per warp and tile; 8-key score tiles, 16-key P.V steps
+  constexpr int KPW = XK / XCW, NTW = KPW / 8, KSW = KPW / 16;      // keys per warp and tile; 8-key score tiles, 16-key P.V steps
   const int tig = lane & 3;
   const bool ragged = key0 + KPW > ctx_len;
   // Rows at or beyond ctx_len hold whatever follows in memory.  Their weights are exactly 0 below;
@@ -379,9 +376,8 @@ __device__ __forceinline__ void store_rows(const TileAcc (&acc)[MT], __nv_bfloat
 // MT = 16-row query tiles (rows per sequence <= 16 * MT); FP8 = keys/values are E4M3 codes (tmap: the keys'
 // 128-byte lines, tmap_v: the transposed values), else bf16 (tmap alone: rows of 64 values)
 template <int MT, bool FP8>
-__global__ void __launch_bounds__(xthreads(FP8), xctas(MT, FP8)) cross_attn_tma_kernel(const __grid_constant__ CUtensorMap tmap,
+__global__ void __launch_bounds__(XTHREADS, xctas(MT, FP8)) cross_attn_tma_kernel(const __grid_constant__ CUtensorMap tmap,
                                                                                        const __grid_constant__ CUtensorMap tmap_v, AttnArgs a) {
-  constexpr int XCW = xcw(FP8);
   constexpr int KPW = XK / XCW;
   constexpr int XTILE_BYTES = XK * kDh * (FP8 ? 1 : 2), XSTAGE_BYTES = 2 * XTILE_BYTES, XSTAGES = xring_bytes(MT, FP8) / XSTAGE_BYTES;
   extern __shared__ uint8_t smem_raw[];
@@ -421,7 +417,7 @@ __global__ void __launch_bounds__(xthreads(FP8), xctas(MT, FP8)) cross_attn_tma_
   __nv_bfloat16 *out = (__nv_bfloat16 *)a.out;
   if (a.clear_status && rank == 0 && h == 0 && b == 0 && tid == 0) a.st.hdr[HDR_STATUS] = 0;      // stand-alone op: its scratch comes as it is; a wait can expire only long after this
   if (!a.packed && a.row_base == nullptr && rank == 0)  // rows of the sequence beyond its active ones come back as zeros
-    for (int idx = tid; idx < (dm.C - S) * (kDh / 8); idx += xthreads(FP8))
+    for (int idx = tid; idx < (dm.C - S) * (kDh / 8); idx += XTHREADS)
       *reinterpret_cast<uint4 *>(out + (size_t)(row0 + S + idx / (kDh / 8)) * dm.d + h * kDh + (idx % (kDh / 8)) * 8) = make_uint4(0u, 0u, 0u, 0u);
   const int nt = S > 0 ? (ctx_len + XK - 1) / XK : 0;
   const int lo = nt * rank / ns, hi = nt * (rank + 1) / ns;
@@ -569,7 +565,7 @@ static int cross_cluster_size(const AttnArgs &a) {
   const long long segs = (long long)a.batch * a.dm.H;
   const int tiles = (a.dm.ctx + XK - 1) / XK;
   int ns = 1;
-  while (ns < 8 && 2 * ns <= tiles && 2 * ns * segs <= 148) ns *= 2;
+  while (ns < 8 && 2 * ns <= tiles && 2 * ns * segs <= kSms) ns *= 2;
   return ns;
 }
 static_assert(7 * XREC_FLOATS * 4 <= xring_bytes(1, true) && 7 * 2 * XREC_FLOATS * 4 <= xring_bytes(2, true), "the states of a cluster fit over the ring");
@@ -592,7 +588,7 @@ cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, co
   const int ns = cross_cluster_size(a);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ns, a.dm.H, a.batch);
-  cfg.blockDim = dim3(xthreads(fp8), 1, 1);
+  cfg.blockDim = dim3(XTHREADS, 1, 1);
   cfg.dynamicSmemBytes = xsmem(mt, fp8);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];

@@ -327,7 +327,7 @@ __global__ void relu_kernel(uint4 *buf, size_t n16) {
 
 cudaError_t launch_relu(int dtype, void *buf, size_t n, cudaStream_t s) {
   const size_t n16 = n * (dtype == PD_DTYPE_BF16 ? 2 : 4) / 16;
-  int blocks = (int)std::min<size_t>((n16 + 255) / 256, 148 * 8);
+  int blocks = (int)std::min<size_t>((n16 + 255) / 256, kSms * 8);
   if (blocks < 1) blocks = 1;
   if (dtype == PD_DTYPE_BF16) relu_kernel<__nv_bfloat16><<<blocks, 256, 0, s>>>((uint4 *)buf, n16);
   else relu_kernel<float><<<blocks, 256, 0, s>>>((uint4 *)buf, n16);
@@ -442,7 +442,7 @@ cudaError_t launch_ctx_kv_relayout(const Dims &dm, int b0, int batch, int layer,
                                    cudaStream_t s) {
   const int esize = dtype == PD_DTYPE_BF16 ? 2 : 4, blocks = (dm.ctx + 63) / 64;
   // few positions: the heads are spread over more CTAs
-  int gz = 2 * 148 / (blocks * batch);
+  int gz = 2 * kSms / (blocks * batch);
   if (gz > (2 * dm.H + 7) / 8) gz = (2 * dm.H + 7) / 8;
   if (gz < 1) gz = 1;
   ctx_kv_relayout_kernel<<<dim3(blocks, batch, gz), 256, 0, s>>>(dm, b0, layer, esize, (const uint4 *)proj, (uint4 *)kv_c);

@@ -189,7 +189,7 @@ struct pd_handle {
   int batch = 0;
   bool encoded = false;
   int self_splits = 1, cross_splits = 1;
-  int sms = 148;
+  int sms = kSms;
   int steps_enqueued = 0;
   bool teacher_clear = false;
   // graph
@@ -318,10 +318,11 @@ int fused_append(const pd_handle *h) {
 
 // The packed decode path: every active row of a step in one packed row list, the layers' products on proj_mma.cu, every launch a
 // programmatic dependent of the one before it.  For few rows, where a step is a chain of launch and load latencies: the products
-// take less than cuBLAS with its norm kernels up to about 128 allocated rows (per layer, 90 active rows of 128 at width 768: 30 us
-// against 31 us, 6 of 8: 16 us against 31 us), and the dependent launches give the attentions a head start.  With more rows
-// the products are bound by the bytes their 32-column slices read again for every row group (190 of 512 at width 1024:
-// 58 us against 40 us): there the unpacked path below, with cuBLAS over the allocated rows, stays.
+// take less than cuBLAS with its norm kernels up to about 90 active rows (per layer, at width 768: 90 active of 128 allocated 30 us
+// against 31 us, 6 of 8 16 us against 31 us), and the dependent launches give the attentions a head start.  With more rows
+// the products are bound by the bytes their 32-column slices read again for every row group (190 active of 512 at width 1024:
+// 58 us against 40 us): there the unpacked path below, with cuBLAS over the allocated rows, stays.  The rule goes by allocated rows, which
+// the host knows when it captures a step; how many are active only the device knows, so a large handle's short start and tail stay unpacked.
 constexpr int kPackedMaxRows = 128;
 bool packed_path(const pd_handle *h) {
   return h->packed_ok && h->batch * h->dm.C <= kPackedMaxRows && cross_attn_tma_supported(h->dm);
@@ -791,7 +792,7 @@ pd_status encode_prepare(pd_handle *h, const int32_t *ctx_len, int32_t batch, co
   auto cdiv = [](int a, int b) { return (a + b - 1) / b; };
   const int bh = batch * dm.H, ctas = bh * cdiv(dm.C, kCoreRows);
   auto core_splits = [&](int tiles) {
-    const int by_gpu = cdiv(2 * 148, ctas), by_work = tiles / (4 * 8);
+    const int by_gpu = cdiv(2 * kSms, ctas), by_work = tiles / (4 * 8);
     return std::max(1, std::min(std::min(by_gpu, by_work), 8));
   };
   int ss = h->cfg.self_splits > 0 ? h->cfg.self_splits : core_splits(dm.SM * dm.PPS);
@@ -1068,7 +1069,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
     seq_row0.push_back(srow0); seq_rows.push_back(srows);
     blocks128 += (srows + 127) / 128;
   }
-  const int block_rows = blocks128 * dm.H >= 2 * 148 ? 128 : 64;
+  const int block_rows = blocks128 * dm.H >= 2 * kSms ? 128 : 64;
   for (int b = 0; b < h->batch; ++b)
     for (int r = 0; r < seq_rows[b]; r += block_rows) {
       b_row0.push_back(seq_row0[b] + r); b_n.push_back(std::min(block_rows, seq_rows[b] - r));

@@ -13,6 +13,7 @@ namespace pd {
 constexpr int kDh = 64;          // head width the kernels are written for
 constexpr int kMaxRows = 64;     // most subsequences active at once per sequence (sub_max <= 64)
 constexpr int kLayerTensors = 10;
+constexpr int kSms = 148;        // SMs of a B200: the rules that choose splits, clusters, slices and row groups are measured on that many
 constexpr size_t kOpHeaderBytes = 256;   // header (HDR_* words) at the start of a stand-alone op's scratch
 
 // KV pool layout: [layer][page][head][entry][K 64 | V 64].  One (page, head) block holds its

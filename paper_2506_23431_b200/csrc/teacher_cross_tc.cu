@@ -8,9 +8,10 @@
 // of P V (through shared memory instead, with 64-key products, both operands' reads and the fences cost 16 us of 205).
 // The running maximum lags: O is rescaled only when a row's maximum has grown by more than 2^8, so that the usual
 // half leaves O alone (weights up to 2^8 lose nothing in bf16, and the same stale maximum divides out).
-// What bounds it: 64 x 128 exponentials per half (512 cycles at 16 a cycle) - two CTAs keep that pipe busy while the other waits for its
-// products.  11.5 k rows, 32 contexts of 2048, 16 heads, per layer: 189 us, where mma.sync (32 rows per warp, 64-key tiles) took 389 us; 3
-// documents of 1000 in 64-row blocks, 12 heads: 13.9 us against 17.5 us.  The loads and products alone, without the exponentials, take 176 us.
+// What bounds it: the loads and products and their hand-overs between the warps - without the exponentials a launch takes 176 of its
+// 190 us.  Two CTAs per SM, so that one's exponentials (64 x 128 per half, 512 cycles at 16 a cycle) run under the other's products.  11.5 k rows, 32
+// contexts of 2048, 16 heads, per layer: 190 us, where mma.sync (32 rows per warp, 64-key tiles) took 389 us; 3 documents of 1000 in 64-row
+// blocks, 12 heads: 13.9 us against 17.5 us.
 // Every mbarrier wait is bounded: on expiry the kernel records PD_ERR_TIMEOUT, stops waiting, falls through to the
 // common exit and frees its tensor memory.
 #include <float.h>

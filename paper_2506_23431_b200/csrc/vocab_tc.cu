@@ -25,7 +25,6 @@
 namespace pd {
 
 constexpr int VT_N = 224;                       // most vocabulary ids per CTA (the N of one tcgen05.mma; the slice in use is a.wn)
-constexpr int VT_SMS = 148;                     // SMs the slice width is balanced for
 constexpr int VT_M = 128;                       // rows per accumulator
 constexpr int VT_BK = 64;                       // columns of K per stage (128 bytes: one swizzle span)
 constexpr int VT_THREADS = 192;                 // producer warp, MMA warp, four epilogue warps
@@ -53,8 +52,8 @@ __device__ __forceinline__ uint32_t v_idesc(int n) {
 // number of rounds the widest slice (224) would need; at least 64 (narrower slices only multiply the
 // re-reads of the hidden rows), and no wider than V needs.
 int vocab_tc_slice(int V) {
-  const int k = (V + VT_SMS * VT_N - 1) / (VT_SMS * VT_N);
-  int wn = ((V + VT_SMS * k - 1) / (VT_SMS * k) + 15) / 16 * 16;
+  const int k = (V + kSms * VT_N - 1) / (kSms * VT_N);
+  int wn = ((V + kSms * k - 1) / (kSms * k) + 15) / 16 * 16;
   if (wn < 64) wn = 64;
   if (wn > VT_N) wn = VT_N;
   const int need = (V + 15) / 16 * 16;
@@ -387,7 +386,7 @@ bool vocab_tc_supported(int K, int V) { return K >= VT_BK && K % VT_BK == 0 && V
 template <bool LOGITS, typename F>
 static cudaError_t with_variant(int rows_cap, int V, F f) {
   if (rows_cap > VT_M) return f(vocab_tc_kernel<2, 3, LOGITS>, vt_smem(2, 3));
-  if (vocab_tc_tiles(V) <= VT_SMS) return f(vocab_tc_kernel<1, 4, LOGITS>, vt_smem(1, 4));
+  if (vocab_tc_tiles(V) <= kSms) return f(vocab_tc_kernel<1, 4, LOGITS>, vt_smem(1, 4));
   return f(vocab_tc_kernel<1, 2, LOGITS>, vt_smem(1, 2));
 }
 
