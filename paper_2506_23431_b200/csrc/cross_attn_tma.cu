@@ -406,7 +406,8 @@ __global__ void __launch_bounds__(XTHREADS, xctas(MT, FP8)) cross_attn_tma_kerne
     if (lane == 0) before_s[warp] = before;
   }
   __syncthreads();
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // (8-bit: the kernel behind does not start early, see the launcher)
+  if (!FP8) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int kv_b = a.kv_seq != nullptr ? a.kv_seq[b] : b;      // the sequence whose context this group reads
   int row0 = a.row_base != nullptr ? a.row_base[b] : b * dm.C;
   if (a.packed) {
@@ -581,6 +582,9 @@ cudaError_t cross_attn_tma_prepare(int rows_per_seq, bool fp8) {
 // 8-bit keys/values (a.kv_scale set): tmap = the keys' lines, tmap_v = the transposed values; else tmap alone.
 // a.pdl: launched as a programmatic dependent of the query projection before it, which writes none of the keys,
 // values, row counts and context lengths, so the first tiles travel while that kernel runs.
+// The 8-bit launches neither begin early nor let the kernel behind begin early.  Their small CTAs piled up on the few SMs that the kernel before had
+// left (a step of six layers, 128 segments of 4096 keys: 0.46 ms; 0.41 ms with the kernel before the clusters), and with the next kernels
+// resident beside them decodes did not repeat bit for bit.
 cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, cudaStream_t s) {
   const int mt = (a.dm.C + 15) / 16;
   const bool fp8 = a.kv_scale != nullptr;
@@ -596,7 +600,7 @@ cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, co
   attr[0].val.clusterDim.x = ns; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = a.pdl ? 2 : 1;
+  cfg.attrs = attr; cfg.numAttrs = a.pdl && !fp8 ? 2 : 1;
   if (mt == 1) return fp8 ? cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, true>, tmap, tmap_v, a) : cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, false>, tmap, tmap_v, a);
   return fp8 ? cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, true>, tmap, tmap_v, a) : cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, false>, tmap, tmap_v, a);
 }

@@ -411,3 +411,25 @@ def test_timed_attention_launches_do_not_overlap(dtype, which):
         pytest.skip("the profiler records no kernels here")
     assert len(spans) >= 6 * wl.n_layers
     assert all(b[0] >= a[1] for a, b in zip(spans, spans[1:]))
+
+
+@pytest.mark.parametrize("kv8", [True, False])
+@pytest.mark.parametrize("batch,heads,ctx", [(16, 12, 1024), (16, 16, 512), (8, 12, 2048), (2, 4, 96)])
+def test_decodes_of_few_rows_repeat_bit_for_bit(batch, heads, ctx, kv8):
+    """The packed path, whose launches overlap: residual stream and tokens of a whole decode, again and again, on one handle."""
+    from paper_2506_23431_b200 import binding as B
+    wl = W.CONFIGS["bart_base"].scaled(name="repeat", batch=batch, n_layers=4, d_model=64 * heads, n_heads=heads, d_ff=256 * heads, vocab=2000, ctx=ctx,
+                                       sub_max=8, delta_t=4, max_sub_len=24, length_dist=("uniform", 10, 24), time_max=40, pos_mode=T5,
+                                       kv_c_dtype="e4m3" if kv8 else "same")
+    dec = B.PipelinedDecoder(wl.hyper(), W.make_weights(wl), wl.batch)
+    mem, ctx_len, forced = dec.device_memory(W.make_encoder_memory(wl)), W.make_ctx_len(wl), W.make_forced_len(wl)
+    first = None
+    for _ in range(12):
+        dec.encode_context(mem, ctx_len, forced)
+        for _ in range(36):
+            dec.step()
+        rows = dec.batch * dec.rows_per_seq
+        got = (dec.debug_read(B.PD_BUF_X, np.float32, rows * wl.d_model).copy(), dec.get_chosen().copy())
+        first = first or got
+        assert np.array_equal(got[0], first[0]) and np.array_equal(got[1], first[1])
+    dec.close()
