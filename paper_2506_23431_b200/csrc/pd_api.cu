@@ -176,6 +176,8 @@ struct pd_handle {
   bool vocab_tc = false;
   bool packed_ok = false;          // bf16, and every kernel of the packed path takes this configuration
   bool f32_own = false;            // fp32: the layers' products on proj_f32 (at most 32 allocated rows)
+  std::vector<ProjTcWeightMaps> tc_w;   // per layer and product: the weights of proj_tc; empty: not usable
+  ProjTcActMaps tc_act[4];         // its activations: normalised input, self-attention output, cross-attention output, feed-forward rows
   bool rows_packed = false;        // the last step left the activation buffers packed (pd_debug_read)
   // pd_generate_host: host-to-device copies of the encoder memory run on a stream of their own, in
   // chunks of sequences, so that the context projection of one chunk overlaps the copy of the next
@@ -316,6 +318,15 @@ int fused_append(const pd_handle *h) {
   return h->dm.PPS >= 2 ? 2 : 0;
 }
 
+// The products of a layer that the packed path runs on its own kernels: weight tensor, activations (index into tc_act), epilogue
+enum { P_QKV, P_SELF_O, P_CROSS_Q, P_CROSS_O, P_UP, P_DOWN, P_COUNT };
+struct Product { int weight, act, epi; };
+constexpr Product kProducts[P_COUNT] = {{1, 0, PROJ_QKV}, {2, 1, PROJ_RESID}, {4, 0, PROJ_STORE}, {6, 2, PROJ_RESID}, {8, 0, PROJ_RELU}, {9, 3, PROJ_RESID}};
+void product_shape(const Dims &dm, int p, int &K, int &N) {
+  K = p == P_DOWN ? dm.ff : dm.d;
+  N = p == P_QKV ? 3 * dm.d : p == P_UP ? dm.ff : dm.d;
+}
+
 // The packed decode path: every active row of a step in one packed row list, the layers' products on proj_mma.cu, every launch a
 // programmatic dependent of the one before it.  For few rows, where a step is a chain of launch and load latencies: the products
 // take less than cuBLAS with its norm kernels up to about 90 active rows (per layer, at width 768: 90 active of 128 allocated 30 us
@@ -323,9 +334,9 @@ int fused_append(const pd_handle *h) {
 // the products are bound by the bytes their 32-column slices read again for every row group (190 active of 512 at width 1024:
 // 58 us against 40 us): there the unpacked path below, with cuBLAS over the allocated rows, stays.  The rule goes by allocated rows, which
 // the host knows when it captures a step; how many are active only the device knows, so a large handle's short start and tail stay unpacked.
-constexpr int kPackedMaxRows = 128;
+constexpr int kPackedMaxRows = 128, kPackedMaxRowsTc = 1024;
 bool packed_path(const pd_handle *h) {
-  return h->packed_ok && h->batch * h->dm.C <= kPackedMaxRows && cross_attn_tma_supported(h->dm);
+  return h->packed_ok && h->batch * h->dm.C <= (h->tc_w.empty() ? kPackedMaxRows : kPackedMaxRowsTc) && cross_attn_tma_supported(h->dm);
 }
 
 // alone: not to overlap with the launch before (timing)
@@ -420,35 +431,46 @@ pd_status enqueue_step_packed(pd_handle *h) {
   p.x = h->ptr<float>(L.x); p.ssq_out = ssq;
   p.row_meta = h->ptr<int4>(L.row_meta_packed); p.rope_tab = rope ? h->ptr<float2>(L.rope_tab) : nullptr;
   p.kv_pool = h->ptr<__nv_bfloat16>(L.kv_pool); p.pool = dm.pool; p.P = dm.P; p.raw_f32 = rope ? 1 : 0;
+  p.status = h->st.hdr + HDR_STATUS;
   auto bf = [](const void *q) { return static_cast<const __nv_bfloat16 *>(q); };
+  auto product = [&](int l, int which, ProjArgs a) -> pd_status {
+    const Product &pr = kProducts[which];
+    product_shape(dm, which, a.K, a.N);
+    a.w = bf(h->layer_w[(size_t)l * kLayerTensors + pr.weight]);
+    if (!h->tc_w.empty() && proj_tc_better(a.K, a.N, p.rows_cap))
+      OWN(h, PD_PROF_GEMM, launch_proj_tc(pr.epi, h->tc_w[(size_t)l * P_COUNT + which], h->tc_act[pr.act], a, s));
+    else
+      OWN(h, PD_PROF_GEMM, launch_proj_mma(pr.epi, a, s));
+    return PD_OK;
+  };
   OWN(h, PD_PROF_OTHER, launch_embed_packed(dm, h->st, h->batch, h->w.embed, p.x, h->layer_w[0], hb, ssq, p.ssq_stride,
                                             h->ptr<int4>(L.row_meta_packed), h->ptr<int32_t>(L.row_at), s));
   for (int l = 0; l < dm.L; ++l) {
     const void *const *lw = &h->layer_w[(size_t)l * kLayerTensors];
     ProjArgs a = p;                                   // queries, keys, values; the cache append
-    a.act = hb; a.w = bf(lw[1]); a.K = dm.d; a.N = 3 * dm.d; a.layer = l;
+    a.act = hb; a.layer = l;
     if (l == 0) a.parts_in = 1;                       // the embedding kernel leaves whole sums
     a.out = h->ptr<__nv_bfloat16>(L.qbuf); a.raw = l == dm.L - 1 ? h->ptr<void>(L.qkv) : nullptr;
-    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_QKV, a, s));
+    PD_TRY(product(l, P_QKV, a));
     {
       ProfScope ps(h, PD_PROF_SELF_ATTN);
       PD_TRY(enqueue_self_attention(h, l));
     }
-    a = p; a.act = h->ptr<__nv_bfloat16>(L.self_out); a.w = bf(lw[2]); a.K = dm.d; a.N = dm.d; a.out = hb; a.gain_next = bf(lw[3]);
-    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_RESID, a, s));
-    a = p; a.act = hb; a.w = bf(lw[4]); a.K = dm.d; a.N = dm.d; a.out = h->ptr<__nv_bfloat16>(L.cq);
-    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_STORE, a, s));
+    a = p; a.act = h->ptr<__nv_bfloat16>(L.self_out); a.out = hb; a.gain_next = bf(lw[3]);
+    PD_TRY(product(l, P_SELF_O, a));
+    a = p; a.act = hb; a.out = h->ptr<__nv_bfloat16>(L.cq);
+    PD_TRY(product(l, P_CROSS_Q, a));
     {
       ProfScope ps(h, PD_PROF_CROSS_ATTN);
       PD_TRY(enqueue_cross_attention(h, l));
     }
-    a = p; a.act = h->ptr<__nv_bfloat16>(L.cross_out); a.w = bf(lw[6]); a.K = dm.d; a.N = dm.d; a.out = hb; a.gain_next = bf(lw[7]);
-    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_RESID, a, s));
-    a = p; a.act = hb; a.w = bf(lw[8]); a.K = dm.d; a.N = dm.ff; a.out = h->ptr<__nv_bfloat16>(L.ffn);
-    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_RELU, a, s));
-    a = p; a.act = h->ptr<__nv_bfloat16>(L.ffn); a.w = bf(lw[9]); a.K = dm.ff; a.N = dm.d; a.out = hb;
+    a = p; a.act = h->ptr<__nv_bfloat16>(L.cross_out); a.out = hb; a.gain_next = bf(lw[7]);
+    PD_TRY(product(l, P_CROSS_O, a));
+    a = p; a.act = hb; a.out = h->ptr<__nv_bfloat16>(L.ffn);
+    PD_TRY(product(l, P_UP, a));
+    a = p; a.act = h->ptr<__nv_bfloat16>(L.ffn); a.out = hb;
     a.gain_next = bf(l + 1 < dm.L ? h->layer_w[(size_t)(l + 1) * kLayerTensors] : h->w.final_norm);
-    OWN(h, PD_PROF_GEMM, launch_proj_mma(PROJ_RESID, a, s));
+    PD_TRY(product(l, P_DOWN, a));
   }
   return enqueue_vocab(h, ssq);
 }
@@ -723,10 +745,27 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
   }
   if (h->vocab_tc && h->have_tmap && self_attn_tc_supported(dm)) {
     h->packed_ok = true;
-    const int spec[6][3] = {{1, dm.d, 3 * dm.d}, {2, dm.d, dm.d}, {4, dm.d, dm.d}, {6, dm.d, dm.d}, {8, dm.d, dm.ff}, {9, dm.ff, dm.d}};
+    bool tc = true;
     for (int l = 0; l < dm.L; ++l)
-      for (const auto &sp : spec)
-        h->packed_ok = h->packed_ok && proj_mma_supported(sp[1], sp[2], h->layer_w[(size_t)l * kLayerTensors + sp[0]]);
+      for (int q = 0; q < P_COUNT; ++q) {
+        int K, N;
+        product_shape(dm, q, K, N);
+        h->packed_ok = h->packed_ok && proj_mma_supported(K, N, h->layer_w[(size_t)l * kLayerTensors + kProducts[q].weight]);
+        tc = tc && proj_tc_supported(K, N);
+      }
+    if (h->packed_ok && tc) {
+      const Region *act[4] = {&L.hbuf, &L.self_out, &L.cross_out, &L.ffn};
+      bool good = proj_tc_prepare() == cudaSuccess;
+      for (int i = 0; i < 4; ++i)
+        good = good && encode_proj_tc_act_maps(&h->tc_act[i], h->ptr<void>(*act[i]), (uint64_t)dm.B * dm.C, i == 3 ? dm.ff : dm.d) == cudaSuccess;
+      h->tc_w.resize((size_t)dm.L * P_COUNT);
+      for (size_t i = 0; i < h->tc_w.size(); ++i) {
+        int K, N;
+        product_shape(dm, (int)(i % P_COUNT), K, N);
+        good = good && encode_proj_tc_weight_maps(&h->tc_w[i], h->layer_w[i / P_COUNT * kLayerTensors + kProducts[i % P_COUNT].weight], K, N) == cudaSuccess;
+      }
+      if (!good) return bail(PD_ERR_CUDA);
+    }
     if (h->packed_ok && (proj_mma_prepare() != cudaSuccess ||
                          cudaMemsetAsync(h->ptr<void>(L.row_at), 0xFF, L.row_at.bytes, h->stream) != cudaSuccess ||
                          cudaStreamSynchronize(h->stream) != cudaSuccess))

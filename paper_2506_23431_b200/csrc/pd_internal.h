@@ -256,11 +256,23 @@ struct ProjArgs {
   const int4 *row_meta; const float2 *rope_tab;
   __nv_bfloat16 *kv_pool; int layer, pool, P;
   void *raw; int raw_f32;
+  int32_t *status;           // proj_tc: error word (PD_ERR_TIMEOUT on an expired wait)
+  int groups;                // proj_tc: row groups that give every SM one CTA (set by the launcher)
 };
 bool proj_mma_supported(int K, int N, const void *w);
 int proj_mma_parts(int N);               // column tiles = parts of ssq_out
 cudaError_t proj_mma_prepare();          // once per device, outside any stream capture
 cudaError_t launch_proj_mma(int epi, const ProjArgs &a, cudaStream_t s);
+
+// ---- the same layers over more rows, on tcgen05 (proj_tc.cu) -----------------------------------------------
+struct ProjTcWeightMaps { CUtensorMap k[2]; };     // weights [K][N]: boxes of 64 columns and 128 or 256 of K
+struct ProjTcActMaps { CUtensorMap box[4]; };      // activations [rows][K]: boxes of 16, 32, 48 or 64 rows, and 256 (48, 64 rows: 128) of K
+bool proj_tc_supported(int K, int N);
+bool proj_tc_better(int K, int N, int rows_cap);      // than proj_mma
+cudaError_t proj_tc_prepare();           // once per device, outside any stream capture
+cudaError_t encode_proj_tc_weight_maps(ProjTcWeightMaps *out, const void *w, uint64_t K, uint64_t N);
+cudaError_t encode_proj_tc_act_maps(ProjTcActMaps *out, const void *act, uint64_t rows, uint64_t K);
+cudaError_t launch_proj_tc(int epi, const ProjTcWeightMaps &map_w, const ProjTcActMaps &maps, const ProjArgs &a, cudaStream_t s);
 
 // ---- the same layers in fp32 over few unpacked rows (proj_f32.cu) ---------------------------------------
 struct ProjF32Args {

@@ -433,3 +433,29 @@ def test_decodes_of_few_rows_repeat_bit_for_bit(batch, heads, ctx, kv8):
         first = first or got
         assert np.array_equal(got[0], first[0]) and np.array_equal(got[1], first[1])
     dec.close()
+
+
+PACKED = [
+    # sequences, open rows per sequence, inner width, positions, longest subsequence, 8-bit context
+    (5, 26, 64, ROPE, 28, False),       # 130 rows allocated: the fewest that take the tensor-memory products; an inner width of one block
+    (9, 31, 1088, T5, 33, True),        # a reduction over two pairs of CTAs, the second one block shorter
+    (16, 32, 2112, ROPE, 34, False),    # 512 rows: three pairs; row groups grow past one per SM
+    (32, 32, 4160, T5, 36, False),      # 1024 rows, the most that run packed; four pairs, the last one block longer or shorter
+    (40, 7, 256, ROPE, 40, False),      # two pages per subsequence
+]
+
+
+@pytest.mark.parametrize("batch,rows,d_ff,pos,length,kv8", PACKED)
+def test_decode_on_tensor_memory_products(batch, rows, d_ff, pos, length, kv8):
+    """More rows than the register products take: rows of 1 to all of a group, widths that end inside a slice of columns (192, 576)."""
+    wl = W.CONFIGS["bart_base"].scaled(name="packed", batch=batch, sub_max=rows, d_ff=d_ff, pos_mode=pos, max_sub_len=length, time_max=min(rows + 6, 96),
+                                       length_dist=("uniform", max(1, length - 4), length), kv_c_dtype="e4m3" if kv8 else "same",
+                                       **dict(BASE, ctx=144 if kv8 else 150))
+    s = check(wl, rows=[0, batch - 1], ragged=True, free_run=False)
+    assert s["max_err"] < parity.TOL["bf16"]
+
+
+@pytest.mark.parametrize("kv8", [True, False])
+@pytest.mark.parametrize("batch,heads,ctx", [(24, 16, 512), (40, 12, 300)])
+def test_decodes_of_many_packed_rows_repeat_bit_for_bit(batch, heads, ctx, kv8):
+    test_decodes_of_few_rows_repeat_bit_for_bit(batch, heads, ctx // 16 * 16, kv8)
