@@ -431,14 +431,13 @@ pd_status enqueue_step_packed(pd_handle *h) {
   p.x = h->ptr<float>(L.x); p.ssq_out = ssq;
   p.row_meta = h->ptr<int4>(L.row_meta_packed); p.rope_tab = rope ? h->ptr<float2>(L.rope_tab) : nullptr;
   p.kv_pool = h->ptr<__nv_bfloat16>(L.kv_pool); p.pool = dm.pool; p.P = dm.P; p.raw_f32 = rope ? 1 : 0;
-  p.status = h->st.hdr + HDR_STATUS;
   auto bf = [](const void *q) { return static_cast<const __nv_bfloat16 *>(q); };
   auto product = [&](int l, int which, ProjArgs a) -> pd_status {
     const Product &pr = kProducts[which];
     product_shape(dm, which, a.K, a.N);
     a.w = bf(h->layer_w[(size_t)l * kLayerTensors + pr.weight]);
     if (!h->tc_w.empty() && proj_tc_better(a.K, a.N, p.rows_cap))
-      OWN(h, PD_PROF_GEMM, launch_proj_tc(pr.epi, h->tc_w[(size_t)l * P_COUNT + which], h->tc_act[pr.act], a, s));
+      OWN(h, PD_PROF_GEMM, launch_proj_tc(pr.epi, h->tc_w[(size_t)l * P_COUNT + which], h->tc_act[pr.act], a, h->st.hdr + HDR_STATUS, s));
     else
       OWN(h, PD_PROF_GEMM, launch_proj_mma(pr.epi, a, s));
     return PD_OK;

@@ -256,8 +256,6 @@ struct ProjArgs {
   const int4 *row_meta; const float2 *rope_tab;
   __nv_bfloat16 *kv_pool; int layer, pool, P;
   void *raw; int raw_f32;
-  int32_t *status;           // proj_tc: error word (PD_ERR_TIMEOUT on an expired wait)
-  int groups;                // proj_tc: row groups that give every SM one CTA (set by the launcher)
 };
 bool proj_mma_supported(int K, int N, const void *w);
 int proj_mma_parts(int N);               // column tiles = parts of ssq_out
@@ -272,7 +270,7 @@ bool proj_tc_better(int K, int N, int rows_cap);      // than proj_mma
 cudaError_t proj_tc_prepare();           // once per device, outside any stream capture
 cudaError_t encode_proj_tc_weight_maps(ProjTcWeightMaps *out, const void *w, uint64_t K, uint64_t N);
 cudaError_t encode_proj_tc_act_maps(ProjTcActMaps *out, const void *act, uint64_t rows, uint64_t K);
-cudaError_t launch_proj_tc(int epi, const ProjTcWeightMaps &map_w, const ProjTcActMaps &maps, const ProjArgs &a, cudaStream_t s);
+cudaError_t launch_proj_tc(int epi, const ProjTcWeightMaps &map_w, const ProjTcActMaps &maps, const ProjArgs &a, int32_t *status, cudaStream_t s);
 
 // ---- the same layers in fp32 over few unpacked rows (proj_f32.cu) ---------------------------------------
 struct ProjF32Args {

@@ -147,10 +147,15 @@ __device__ __forceinline__ uint32_t t_pack2(float lo, float hi) {
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
+struct ProjTcArgs : ProjArgs {
+  int groups;                // row groups that give every SM one CTA
+  int32_t *status;           // error word (PD_ERR_TIMEOUT on an expired wait)
+};
+
 // Grid (2 x column slices, row groups, K splits), cluster (2, 1, K splits).
 template <int EPI, bool SPLIT>
 __global__ void __launch_bounds__(PT_THREADS, 2)
-proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_constant__ ProjTcActMaps maps, ProjArgs a) {
+proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_constant__ ProjTcActMaps maps, ProjTcArgs a) {
   extern __shared__ uint8_t t_raw[];
   __shared__ uint32_t tmem_base_s;
   __shared__ int rows_s[PT_THREADS / 32];
@@ -528,10 +533,11 @@ cudaError_t encode_proj_tc_act_maps(ProjTcActMaps *out, const void *act, uint64_
   return cudaSuccess;
 }
 
-cudaError_t launch_proj_tc(int epi, const ProjTcWeightMaps &map_w, const ProjTcActMaps &maps, const ProjArgs &a_in, cudaStream_t s) {
-  ProjArgs a = a_in;
+cudaError_t launch_proj_tc(int epi, const ProjTcWeightMaps &map_w, const ProjTcActMaps &maps, const ProjArgs &a_in, int32_t *status, cudaStream_t s) {
+  ProjTcArgs a;
+  static_cast<ProjArgs &>(a) = a_in;
   const Plan p = plan(a.K, a.N, a.rows_cap);
-  a.groups = p.groups;
+  a.groups = p.groups; a.status = status;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * p.slices, p.gy, p.ks);
   cfg.blockDim = dim3(PT_THREADS, 1, 1);
