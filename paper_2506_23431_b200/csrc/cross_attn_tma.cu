@@ -227,8 +227,7 @@ __device__ __forceinline__ void tile_step(TileAcc (&acc)[MT], const uint32_t (&q
   const bool ragged = key0 + KPW > ctx_len;
   // Rows at or beyond ctx_len hold whatever follows in memory.  Their weights are exactly 0 below;
   // the value fragments of those keys are cleared in registers after ldmatrix, so that 0 never
-  // multiplies a non-finite.  (Nothing but TMA ever writes a stage: zeroing the rows in shared
-  // memory raced with the next bulk copy into the stage, proxy fence or not.)
+  // multiplies a non-finite.
   // ---- scores: S[mt][nt] = Q (16 x 64) . K^T (64 x 8 keys)
   float sc[MT][NTW][4];
 #pragma unroll
@@ -406,8 +405,7 @@ __global__ void __launch_bounds__(XTHREADS, xctas(MT, FP8)) cross_attn_tma_kerne
     if (lane == 0) before_s[warp] = before;
   }
   __syncthreads();
-  // (8-bit: the kernel behind does not start early, see the launcher)
-  if (!FP8) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int kv_b = a.kv_seq != nullptr ? a.kv_seq[b] : b;      // the sequence whose context this group reads
   int row0 = a.row_base != nullptr ? a.row_base[b] : b * dm.C;
   if (a.packed) {
@@ -437,6 +435,10 @@ __global__ void __launch_bounds__(XTHREADS, xctas(MT, FP8)) cross_attn_tma_kerne
       for (int it = 0; it < hi - lo; ++it) {
         const int s = it % XSTAGES;
         if (!mbar_wait(bar_empty + 8 * s, (((uint32_t)(it / XSTAGES)) & 1u) ^ 1u)) { ok = false; break; }
+        // The stage was read through the generic proxy and is filled through the async one.  Without this fence a copy overtook the last
+        // ldmatrix of the slowest warp: a 32-byte sector of the values, one decode in a few where the launches before and after overlap
+        // this one.  (In the consumer warps, ahead of their arrival, it holds as well, and costs them 36 cycles a tile.)
+        if (it >= XSTAGES) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_expect_tx(bar_full + 8 * s, XSTAGE_BYTES);
         const uint32_t dst = base + s * XSTAGE_BYTES;
         if (FP8) {
@@ -582,9 +584,6 @@ cudaError_t cross_attn_tma_prepare(int rows_per_seq, bool fp8) {
 // 8-bit keys/values (a.kv_scale set): tmap = the keys' lines, tmap_v = the transposed values; else tmap alone.
 // a.pdl: launched as a programmatic dependent of the query projection before it, which writes none of the keys,
 // values, row counts and context lengths, so the first tiles travel while that kernel runs.
-// The 8-bit launches neither begin early nor let the kernel behind begin early.  Their small CTAs piled up on the few SMs that the kernel before had
-// left (a step of six layers, 128 segments of 4096 keys: 0.46 ms; 0.41 ms with the kernel before the clusters), and with the next kernels
-// resident beside them decodes did not repeat bit for bit.
 cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, cudaStream_t s) {
   const int mt = (a.dm.C + 15) / 16;
   const bool fp8 = a.kv_scale != nullptr;
@@ -600,7 +599,7 @@ cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, co
   attr[0].val.clusterDim.x = ns; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = a.pdl && !fp8 ? 2 : 1;
+  cfg.attrs = attr; cfg.numAttrs = a.pdl ? 2 : 1;
   if (mt == 1) return fp8 ? cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, true>, tmap, tmap_v, a) : cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, false>, tmap, tmap_v, a);
   return fp8 ? cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, true>, tmap, tmap_v, a) : cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, false>, tmap, tmap_v, a);
 }
