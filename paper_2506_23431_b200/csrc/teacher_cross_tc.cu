@@ -65,27 +65,35 @@ __device__ __forceinline__ void c_tma_load_2d(uint32_t dst, const CUtensorMap *t
       : "memory");
 }
 // Shared-memory matrix descriptor of rows of 128 bytes, 128-byte swizzle, 1024 B between groups of eight rows.  The same words serve
-// a K-major operand (rows = M or N) and, with one 64-wide span of it, an MN-major one (rows = K).
-__device__ __forceinline__ uint64_t c_smem_desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (64ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
+// a K-major operand (rows = M or N) and, with one 64-wide span of it, an MN-major one (rows = K).  Low word: address >> 4; the high one is constant.
+constexpr uint32_t XC_DESC_HI = 64u | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t c_desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (64u << 16); }
+// One lane of a converged warp.
+__device__ __forceinline__ bool c_elect() {
+  uint32_t on;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(on));
+  return on != 0;
 }
 // instruction descriptor of kind::f16: D fp32, A and B bf16, N >> 3 at bit 17, M >> 4 at bit 24; bit 16: B is MN-major
 constexpr uint32_t xc_idesc(int n) { return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(XC_M >> 4) << 24); }
-__device__ __forceinline__ void c_mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void c_mma_bf16(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %5};\n\t"
+      "mov.b64 db, {%2, %5};\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}"
+      ::"r"(tmem_d), "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "n"(XC_DESC_HI)
       : "memory");
 }
 // A from tensor memory: two consecutive K values per 32-bit column, one row per lane
-__device__ __forceinline__ void c_mma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void c_mma_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint32_t blo, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+      "mov.b64 db, {%2, %5};\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n\t}"
+      ::"r"(tmem_d), "r"(tmem_a), "r"(blo), "r"(idesc), "r"(accumulate), "n"(XC_DESC_HI)
       : "memory");
 }
 __device__ __forceinline__ void c_mma_commit(uint32_t bar) {
@@ -209,32 +217,36 @@ __global__ void __launch_bounds__(XC_THREADS, 2) teacher_cross_kernel(const __gr
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ products (one lane)
-    if (lane == 0) {
-      auto scores = [&](int tile) {
-        const int s = tile % XC_STAGES;
-        if (!c_mbar_wait(bar_full + 8 * s, (uint32_t)(tile / XC_STAGES) & 1u)) { ok = false; return; }
-        c_fence_after();
+    // ------------------------------------------------------------------ products (one lane).  The whole warp walks: in a loop that a single lane
+    // walks the descriptors stay out of the uniform registers the products read, and a product costs 128 cycles to issue where it takes 52 to 68
+    const uint32_t q_lo = c_desc_lo(q_s), ring_lo = c_desc_lo(ring);
+    auto scores = [&](int tile) {
+      const int s = tile % XC_STAGES;
+      if (!c_mbar_wait(bar_full + 8 * s, (uint32_t)(tile / XC_STAGES) & 1u)) { ok = false; return; }
+      c_fence_after();
+      if (c_elect()) {
 #pragma unroll
         for (int k = 0; k < kDh / 16; ++k)
-          c_mma_bf16(tmem, c_smem_desc(q_s + k * 32), c_smem_desc(ring + s * XC_STAGE + k * 32), xc_idesc(XC_K), k > 0 ? 1u : 0u);
+          c_mma_bf16(tmem, q_lo + k * 2, ring_lo + s * (XC_STAGE >> 4) + k * 2, xc_idesc(XC_K), k > 0 ? 1u : 0u);
         c_mma_commit(bar_s);
-      };
-      ok = c_mbar_wait(bar_q, 0);
-      if (ok) scores(0);
-      for (int j = 0; j < n_halves && ok; ++j) {
-        const int tile = j >> 1, s = tile % XC_STAGES;
-        if ((j & 1) != 0 && tile + 1 < n_tiles) {           // the tile's scores are all read: the next one's
-          if (!c_mbar_wait(bar_read, (uint32_t)tile & 1u)) { ok = false; break; }
-          c_fence_after();
-          scores(tile + 1);
-        }
-        if (!ok || !c_mbar_wait(bar_p + 8 * (j & 1), (uint32_t)(j >> 1) & 1u)) { ok = false; break; }
+      }
+    };
+    ok = c_mbar_wait(bar_q, 0);
+    if (ok) scores(0);
+    for (int j = 0; j < n_halves && ok; ++j) {
+      const int tile = j >> 1, s = tile % XC_STAGES;
+      if ((j & 1) != 0 && tile + 1 < n_tiles) {             // the tile's scores are all read: the next one's
+        if (!c_mbar_wait(bar_read, (uint32_t)tile & 1u)) { ok = false; break; }
         c_fence_after();
+        scores(tile + 1);
+      }
+      if (!ok || !c_mbar_wait(bar_p + 8 * (j & 1), (uint32_t)(j >> 1) & 1u)) { ok = false; break; }
+      c_fence_after();
+      if (c_elect()) {
+        const uint32_t v_lo = ring_lo + s * (XC_STAGE >> 4) + (XC_TILE >> 4) + (j & 1) * (XC_TILE / 2 >> 4);
 #pragma unroll
         for (int k = 0; k < XC_H / 16; ++k)                 // 16 keys = 8 columns of weights, 16 rows of values
-          c_mma_bf16_ta(tmem + XC_O, tmem + XC_W + (uint32_t)((j & 1) * 32 + k * 8),
-                        c_smem_desc(ring + s * XC_STAGE + XC_TILE + (j & 1) * (XC_TILE / 2) + k * 2048), xc_idesc(kDh) | (1u << 16),
+          c_mma_bf16_ta(tmem + XC_O, tmem + XC_W + (uint32_t)((j & 1) * 32 + k * 8), v_lo + k * (2048 >> 4), xc_idesc(kDh) | (1u << 16),
                         (j > 0 || k > 0) ? 1u : 0u);
         if ((j & 1) != 0) c_mma_commit(bar_empty + 8 * s);
         c_mma_commit(bar_pv + 8 * (j & 1));

@@ -92,17 +92,24 @@ __device__ __forceinline__ void v_tma_load_2d(uint32_t dst, const CUtensorMap *t
       ::"r"(dst), "l"(tmap), "r"(bar), "r"(x), "r"(y)
       : "memory");
 }
-// Shared-memory matrix descriptor of a K-major tile whose rows are 128 bytes, 128-byte swizzle:
-// start address >> 4, leading offset 16 B (unused by swizzled K-major), 1024 B between 8-row groups.
-__device__ __forceinline__ uint64_t v_smem_desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | (64ull << 32) | (1ull << 46) | (2ull << 61);
+// Shared-memory matrix descriptor of a K-major tile whose rows are 128 bytes, 128-byte swizzle, 1024 B between 8-row groups.  Low word:
+// address >> 4 (and the leading offset, unused by swizzled K-major); the high one is constant.
+constexpr uint32_t VT_DESC_HI = 64u | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t v_desc_lo(uint32_t saddr) { return ((saddr & 0x3FFFFu) >> 4) | (1u << 16); }
+// One lane of a converged warp.
+__device__ __forceinline__ bool v_elect() {
+  uint32_t on;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(on));
+  return on != 0;
 }
-__device__ __forceinline__ void v_mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+__device__ __forceinline__ void v_mma_bf16(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "mov.b64 da, {%1, %5};\n\t"
+      "mov.b64 db, {%2, %5};\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}"
+      ::"r"(tmem_d), "r"(alo), "r"(blo), "r"(idesc), "r"(accumulate), "n"(VT_DESC_HI)
       : "memory");
 }
 // The barrier gets one arrival once every tcgen05.mma issued so far by this thread has finished.
@@ -239,30 +246,30 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issue (one lane)
-    if (lane == 0) {
-      int it = 0;
-      const uint32_t idesc = v_idesc(wn);
-      for (int p = 0; p < n_pass && ok; ++p) {
-        const int tiles = min(TILES, n_tt - TILES * p);
-        // the epilogue must be done with the previous pass's accumulators
-        if (!v_mbar_wait(bar_acc_empty, ((uint32_t)p & 1u) ^ 1u)) { ok = false; break; }
+    // ------------------------------------------------------------------ MMA issue (one lane).  The whole warp walks: in a loop that a single lane
+    // walks the descriptors stay out of the uniform registers the products read, and a product costs 128 cycles to issue where it takes 90
+    int s = 0;
+    uint32_t u = 0;
+    const uint32_t idesc = v_idesc(wn);
+    for (int p = 0; p < n_pass && ok; ++p) {
+      const int tiles = min(TILES, n_tt - TILES * p);
+      // the epilogue must be done with the previous pass's accumulators
+      if (!v_mbar_wait(bar_acc_empty, ((uint32_t)p & 1u) ^ 1u)) { ok = false; break; }
+      v_fence_after();
+      for (int kb = 0; kb < nkb; ++kb) {
+        if (!v_mbar_wait(bar_full + 8 * s, u & 1u)) { ok = false; break; }
         v_fence_after();
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = it % VT_STAGES;
-          const uint32_t u = (uint32_t)(it / VT_STAGES);
-          if (!v_mbar_wait(bar_full + 8 * s, u & 1u)) { ok = false; break; }
-          v_fence_after();
-          const uint32_t sa = base + s * VT_STAGE_BYTES, sb = sa + TILES * VT_A_BYTES;
+        if (v_elect()) {
+          const uint32_t sa = v_desc_lo(base + s * VT_STAGE_BYTES), sb = sa + (TILES * VT_A_BYTES >> 4);
           for (int j = 0; j < tiles; ++j)
 #pragma unroll
-            for (int k4 = 0; k4 < VT_BK / 16; ++k4)      // 16 columns of K = 32 bytes further inside the swizzle span
-              v_mma_bf16(tmem_base + (uint32_t)j * 256u, v_smem_desc(sa + j * VT_A_BYTES + k4 * 32), v_smem_desc(sb + k4 * 32), idesc,
-                         (kb > 0 || k4 > 0) ? 1u : 0u);
-          v_mma_commit(bar_empty + 8 * s);               // frees the stage once these MMAs have read it
+            for (int k4 = 0; k4 < VT_BK / 16; ++k4)        // 16 columns of K = 32 bytes further inside the swizzle span
+              v_mma_bf16(tmem_base + (uint32_t)j * 256u, sa + j * (VT_A_BYTES >> 4) + k4 * 2, sb + k4 * 2, idesc, (kb > 0 || k4 > 0) ? 1u : 0u);
+          v_mma_commit(bar_empty + 8 * s);                 // frees the stage once these MMAs have read it
         }
-        if (ok) v_mma_commit(bar_acc_full);              // the pass's accumulators are complete
+        if (++s == VT_STAGES) { s = 0; ++u; }
       }
+      if (ok && v_elect()) v_mma_commit(bar_acc_full);     // the pass's accumulators are complete
     }
   } else {
     // ------------------------------------------------------------------ epilogue: one row per thread
