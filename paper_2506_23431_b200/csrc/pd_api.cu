@@ -1078,7 +1078,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
   // and blocks of up to 128 rows - 64 where those would leave SMs without one - (8-bit context: cross-attention runs on groups of up to 32)
   std::vector<int32_t> seq_row0, seq_rows;
   long long blocks128 = 0;
-  std::vector<int32_t> row_sub, row_tau, row_tok, row_tgt, g_row0, g_n, g_seq, g_ctx, b_row0, b_n, b_srow0, b_srows, b_seq, b_ctx;
+  std::vector<int32_t> row_sub, row_tau, row_tok, row_tgt, g_row0, g_n, g_seq, g_ctx, b_row0, b_n, b_srow0, b_srows, b_seq, b_ctx, b_tiles, row_key;
   std::vector<int32_t> ctx_len(h->batch), plan((size_t)h->batch * dm.SM);
   CU_TRY(h, cudaMemcpyAsync(ctx_len.data(), h->st.ctx_len, (size_t)h->batch * 4, cudaMemcpyDeviceToHost, h->stream));
   CU_TRY(h, cudaMemcpyAsync(plan.data(), h->st.plan, plan.size() * 4, cudaMemcpyDeviceToHost, h->stream));
@@ -1112,8 +1112,22 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
     for (int r = 0; r < seq_rows[b]; r += block_rows) {
       b_row0.push_back(seq_row0[b] + r); b_n.push_back(std::min(block_rows, seq_rows[b] - r));
       b_srow0.push_back(seq_row0[b]); b_srows.push_back(seq_rows[b]); b_seq.push_back(b); b_ctx.push_back(ctx_len[b]);
+      const auto first = row_sub.begin() + seq_row0[b], last = first + seq_rows[b];      // (sorted by subsequence)
+      b_tiles.push_back((int32_t)((std::upper_bound(first, last, *(first + std::min(r + block_rows, seq_rows[b]) - 1)) - first + 63) / 64));
     }
   const size_t R = row_sub.size(), G = g_row0.size(), NB = b_row0.size();
+  std::vector<int32_t> ranks;                           // timestamps beyond 23 bits: only their order matters to the dependency rule
+  if (dm.n_dist >= 1 << 23) {
+    ranks = row_tau;
+    std::sort(ranks.begin(), ranks.end());
+    ranks.erase(std::unique(ranks.begin(), ranks.end()), ranks.end());
+  }
+  row_key.reserve(2 * R);
+  for (size_t r = 0; r < R; ++r) {
+    const int tau = ranks.empty() ? row_tau[r] : (int)(std::lower_bound(ranks.begin(), ranks.end(), row_tau[r]) - ranks.begin());
+    row_key.push_back(row_sub[r] << 24 | tau);
+    row_key.push_back(4 * (row_tau[r] + row_sub[r]));
+  }
   if (rows_out) *rows_out = (int32_t)R;
   if (loss_out) *loss_out = 0.0;
   if (R == 0) return PD_OK;
@@ -1127,11 +1141,12 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
   int32_t *tab = reinterpret_cast<int32_t *>(base + L.tables);
   // all tables in one upload
   std::vector<int32_t> tables;
-  tables.reserve(4 * R + 4 * G + 6 * NB);
+  tables.reserve(6 * R + 4 * G + 7 * NB);
   auto put = [&](const std::vector<int32_t> &v) { int32_t *at = tab + tables.size(); tables.insert(tables.end(), v.begin(), v.end()); return at; };
+  const int2 *d_key = reinterpret_cast<const int2 *>(put(row_key));      // (first: 8-byte aligned)
   int32_t *d_sub = put(row_sub), *d_tau = put(row_tau), *d_tok = put(row_tok), *d_tgt = put(row_tgt);
   int32_t *d_grow0 = put(g_row0), *d_gn = put(g_n), *d_gseq = put(g_seq), *d_gctx = put(g_ctx);
-  int32_t *d_brow0 = put(b_row0), *d_bn = put(b_n), *d_bsrow0 = put(b_srow0), *d_bsrows = put(b_srows), *d_bseq = put(b_seq), *d_bctx = put(b_ctx);
+  int32_t *d_brow0 = put(b_row0), *d_bn = put(b_n), *d_bsrow0 = put(b_srow0), *d_bsrows = put(b_srows), *d_bseq = put(b_seq), *d_bctx = put(b_ctx), *d_btiles = put(b_tiles);
   CU_TRY(h, cudaMemcpyAsync(tab, tables.data(), tables.size() * 4, cudaMemcpyHostToDevice, s));
 
   float *x = reinterpret_cast<float *>(base + L.x);
@@ -1156,7 +1171,7 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
     memset(&da, 0, sizeof(da));
     da.H = dm.H; da.d = dm.d; da.n_groups = (int)NB; da.block_rows = block_rows; da.scale_log2e = dm.scale_log2e;
     da.q = reinterpret_cast<const __nv_bfloat16 *>(qkv_b); da.out = reinterpret_cast<__nv_bfloat16 *>(att);
-    da.row_sub = d_sub; da.row_tau = d_tau; da.grp_row0 = d_brow0; da.grp_n = d_bn; da.grp_key_row0 = d_bsrow0; da.grp_keys = d_bsrows;
+    da.row_key = d_key; da.grp_tiles = d_btiles; da.grp_row0 = d_brow0; da.grp_n = d_bn; da.grp_key_row0 = d_bsrow0; da.grp_keys = d_bsrows;
     da.bias_tab = rope ? nullptr : h->ptr<float>(h->lay.bias_tab); da.n_dist = dm.n_dist;
     OWN(h, PD_PROF_SELF_ATTN, launch_teacher_self(da, s));
     PD_TRY(gemm(h, false, M, dm.d, dm.d, att, lw[2], x, true, 1.f));

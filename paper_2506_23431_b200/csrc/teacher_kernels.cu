@@ -14,9 +14,11 @@ namespace {
 // P.V on mma.sync, online softmax in the log2 domain; a warp owns its rows, so nothing is merged.  The keys are the sequence's own
 // target rows, with the dependency rule and the T5 bias applied to the accumulator fragment; the key walk ends at the first tile of a
 // later subsequence.
+// A row's subsequence and timestamp share a word (8 and 24 bits) with a guard bit above each: one subtraction tells whether a query sees a
+// key - both guard bits stand - and the bias is read whatever it tells, at a place that is always in the table, so that no pair branches.
 // What bounds it: the mask and the bias, evaluated per pair.  11.5 k rows of 32 sequences, 16 heads, per layer: 203 us in groups of 32 rows
-// (every group reads its keys again), 157 us here with 16 rows per warp, 234 us with 32 (the mask needs the registers).  Where
-// 128-row blocks would leave SMs without one, 64-row blocks.
+// (every group reads its keys again), 160 us with 16 rows per warp, two comparisons and a branch per pair and the tiles to walk found by
+// search, 234 us with 32 (the mask needs the registers); 96 us here.  Where 128-row blocks would leave SMs without one, 64-row blocks.
 constexpr int TK = 64, TSLOTS = 3, TMAXD = 640;
 constexpr int TSLOT_BYTES = TK * 256;            // 64 key rows, then 64 value rows
 constexpr int TATTN_SMEM = TSLOTS * TSLOT_BYTES + 128;
@@ -25,17 +27,18 @@ __device__ __forceinline__ void t_cp_async16(uint32_t dst, const void *src, bool
   const int n = on ? 16 : 0;                     // 0 source bytes: the destination is zero-filled
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
 }
-__device__ __forceinline__ void t_cp_async4(uint32_t dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+__device__ __forceinline__ void t_cp_async8(uint32_t dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
+constexpr uint32_t kSees = 0x80800000u;          // guard bits above the timestamp (24 bits) and the subsequence (8 bits)
 
-template <int W>
+template <int W, bool BIAS>
 __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnArgs a) {
   using namespace mt;
   constexpr int TT = W * 32;
   extern __shared__ uint8_t t_raw[];
-  __shared__ int ki_s[TSLOTS][TK], kt_s[TSLOTS][TK];
-  __shared__ float bias_s[TMAXD];
+  __shared__ __align__(16) int2 key_s[TSLOTS][TK];      // (subsequence << 24 | timestamp, 4 x position)
+  __shared__ float bias_s[BIAS ? TMAXD : 1];
   const int grp = blockIdx.x, h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, tig = lane & 3;
   const int q0 = a.grp_row0[grp], nq = a.grp_n[grp];
@@ -43,8 +46,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
   const size_t ld = 3 * (size_t)a.d;
   const int k0 = a.grp_key_row0[grp], nk = a.grp_keys[grp];
   const __nv_bfloat16 *kp = a.q + (size_t)k0 * ld + a.d + (size_t)h * kDh, *vp = kp + a.d;      // row 0 of this head's keys and values
-  const bool use_bias = a.bias_tab != nullptr;
-  if (use_bias)
+  if (BIAS)
     for (int dd = tid; dd < a.n_dist; dd += TT) bias_s[dd] = a.bias_tab[(size_t)h * a.n_dist + dd];
 
   auto fetch = [&](int tile) {
@@ -57,22 +59,12 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
       const __nv_bfloat16 *src = (p < 8 ? kp : vp) + (on ? (size_t)(first + r) * ld : 0) + (p & 7) * 8;
       t_cp_async16(dst + (p >> 3) * (TK * 128) + swz(r, p & 7), src, on);
     }
-    for (int i = tid; i < TK && first + i < nk; i += TT) {
-      t_cp_async4(smem_u32(&ki_s[slot][i]), a.row_sub + k0 + first + i);
-      t_cp_async4(smem_u32(&kt_s[slot][i]), a.row_tau + k0 + first + i);
+    for (int i = tid; i < TK; i += TT) {
+      if (first + i < nk) t_cp_async8(smem_u32(&key_s[slot][i]), a.row_key + k0 + first + i);
+      else key_s[slot][i] = make_int2(0x7f << 24, 0);        // a subsequence no row reaches
     }
   };
-  // tiles to walk: keys are sorted by subsequence, and nothing of a later one than the block's last row's is visible
-  int n_tiles = (nk + TK - 1) / TK;
-  {
-    const int q_i_max = a.row_sub[q0 + nq - 1];
-    int lo = 0, hi = n_tiles;                    // first tile whose first key lies beyond
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (a.row_sub[k0 + mid * TK] > q_i_max) hi = mid; else lo = mid + 1;
-    }
-    n_tiles = lo;
-  }
+  const int n_tiles = a.grp_tiles[grp];          // keys are sorted by subsequence: nothing of a later one than the block's last row's is visible
 #pragma unroll
   for (int t = 0; t < TSLOTS - 1; ++t) {
     if (t < n_tiles) fetch(t);
@@ -90,10 +82,12 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
     qf[kk][2] = r_lo < nq ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8) : 0u;
     qf[kk][3] = r_hi < nq ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8) : 0u;
   }
-  // subsequence (-1: sees nothing) and timestamp of the rows
-  const int qi[2] = {r_lo < nq ? a.row_sub[q0 + r_lo] : -1, r_hi < nq ? a.row_sub[q0 + r_hi] : -1};
-  const int qt[2] = {r_lo < nq ? a.row_tau[q0 + r_lo] : 0, r_hi < nq ? a.row_tau[q0 + r_hi] : 0};
-  const int warp_i_max = w0 < nq ? a.row_sub[q0 + min(w0 + 15, nq - 1)] : -1;
+  // subsequence and timestamp of the rows under their guard bits (no row: sees nothing), 4 x position
+  const int2 none = make_int2((int)((0x7fu << 24) - kSees), 0);
+  const int2 k_lo = r_lo < nq ? a.row_key[q0 + r_lo] : none, k_hi = r_hi < nq ? a.row_key[q0 + r_hi] : none;
+  const uint32_t qk[2] = {(uint32_t)k_lo.x + kSees, (uint32_t)k_hi.x + kSees};
+  const int qp[2] = {k_lo.y, k_hi.y};
+  const int warp_i_max = w0 < nq ? a.row_key[q0 + min(w0 + 15, nq - 1)].x >> 24 : -1;
   TileAcc A;
   A.clear();
   const float sl2 = a.scale_log2e;
@@ -103,8 +97,8 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
     __syncthreads();                             // tile landed for everybody; everybody is through with the tile before
     if (tile + TSLOTS - 1 < n_tiles) fetch(tile + TSLOTS - 1);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    const int slot = tile % TSLOTS, nv = min(TK, nk - tile * TK);
-    if (w0 >= nq || ki_s[slot][0] > warp_i_max) continue;      // no row of this warp sees the tile
+    const int slot = tile % TSLOTS;
+    if (w0 >= nq || key_s[slot][0].x >> 24 > warp_i_max) continue;      // no row of this warp sees the tile
     const uint32_t kbase = base + slot * TSLOT_BYTES, vbase = kbase + TK * 128;
     float sc[8][4];
 #pragma unroll
@@ -118,21 +112,21 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
         mma_bf16(sc[nt], qf[2 * kq + 1][0], qf[2 * kq + 1][1], qf[2 * kq + 1][2], qf[2 * kq + 1][3], b2, b3);
       }
     }
-    // ---- scale, the dependency rule per pair (i' <= i and tau' <= tau), bias on the Manhattan distance (log2 domain)
+    // ---- scale, the dependency rule per pair (i' <= i and tau' <= tau), bias on the Manhattan distance (log2 domain).  A pair that is not
+    // visible may have any distance down to minus a position: it reads the table's start, and the value is dropped.
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
+    for (int nt = 0; nt < 8; ++nt) {
+      const int4 k2 = *reinterpret_cast<const int4 *>(&key_s[slot][nt * 8 + 2 * tig]);
 #pragma unroll
-      for (int kx = 0; kx < 2; ++kx) {
-        const int e = nt * 8 + 2 * tig + kx;
-        const int ki = ki_s[slot][e], ktau = kt_s[slot][e];
+      for (int kx = 0; kx < 2; ++kx)
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
+          const bool vis = ((qk[hh] - (uint32_t)(kx ? k2.z : k2.x)) & kSees) == kSees;
           float v = sc[nt][2 * hh + kx] * sl2;
-          const bool vis = e < nv && ki <= qi[hh] && ktau <= qt[hh];
-          if (use_bias && vis) v += bias_s[qt[hh] + qi[hh] - (ktau + ki)];
+          if (BIAS) v += *reinterpret_cast<const float *>(reinterpret_cast<const char *>(bias_s) + max(qp[hh] - (kx ? k2.w : k2.y), 0));
           sc[nt][2 * hh + kx] = vis ? v : -INFINITY;
         }
-      }
+    }
     uint32_t pf[4][4];
     float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
@@ -263,8 +257,10 @@ __global__ void __launch_bounds__(256) target_logprob_kernel(int V, const float 
 
 cudaError_t teacher_attn_prepare() {
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(teacher_self_kernel<8>, attr, TATTN_SMEM);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_self_kernel<4>, attr, TATTN_SMEM);
+  cudaError_t e = cudaFuncSetAttribute(teacher_self_kernel<8, true>, attr, TATTN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_self_kernel<4, true>, attr, TATTN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_self_kernel<8, false>, attr, TATTN_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(teacher_self_kernel<4, false>, attr, TATTN_SMEM);
   return e;
 }
 
@@ -272,8 +268,12 @@ cudaError_t launch_teacher_self(const DenseAttnArgs &a, cudaStream_t s) {
   if (a.n_groups < 1) return cudaSuccess;
   if (a.bias_tab != nullptr && a.n_dist > TMAXD) return cudaErrorInvalidValue;      // the head's bias row is held in shared memory
   const dim3 grid(a.n_groups, a.H);
-  if (a.block_rows == 128) teacher_self_kernel<8><<<grid, 256, TATTN_SMEM, s>>>(a);
-  else teacher_self_kernel<4><<<grid, 128, TATTN_SMEM, s>>>(a);
+  auto launch = [&](auto wide, auto narrow) {
+    if (a.block_rows == 128) wide<<<grid, 256, TATTN_SMEM, s>>>(a);
+    else narrow<<<grid, 128, TATTN_SMEM, s>>>(a);
+  };
+  if (a.bias_tab != nullptr) launch(teacher_self_kernel<8, true>, teacher_self_kernel<4, true>);
+  else launch(teacher_self_kernel<8, false>, teacher_self_kernel<4, false>);
   return cudaGetLastError();
 }
 
