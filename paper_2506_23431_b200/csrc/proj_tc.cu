@@ -90,6 +90,8 @@ __device__ __forceinline__ void t_tma_load(uint32_t dst, const CUtensorMap *tmap
       ::"r"(dst), "l"(tmap), "r"(bar), "r"(x), "r"(y)
       : "memory");
 }
+// The map itself on its way: a first copy with it would wait for a round trip more.
+__device__ __forceinline__ void t_map_prefetch(const CUtensorMap *tmap) { asm volatile("prefetch.tensormap [%0];" ::"l"(tmap) : "memory"); }
 __device__ __forceinline__ void t_tma_load3(uint32_t dst, const CUtensorMap *tmap, uint32_t bar, int x, int y, int z) {
   asm volatile(
       "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
@@ -173,6 +175,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
                  red_free = red_full + 8, acc_read = red_free + 8;
   int cnt = 0;
   for (int b = tid; b < a.batch; b += PT_THREADS) cnt += a.n_active[b];
+  if (tid < 2) t_map_prefetch(&wmaps.k[tid]);
   if (tid == 0) {
     for (int s = 0; s < PT_STAGES_MAX; ++s) { t_mbar_init(full + 8 * s, 1); t_mbar_init(empty + 8 * s, 1); }
     t_mbar_init(acc_full, 1);
@@ -186,6 +189,11 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
   if (lane == 0) rows_s[warp] = cnt;
+  if (warp == 1) {                                   // the product warp owns the tensor-memory allocation (of both CTAs together)
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(t_smem_u32(&tmem_base_s)), "r"(PT_TMEM) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  t_fence_before();
   __syncthreads();
   int rows = 0;
 #pragma unroll
@@ -197,6 +205,10 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
   const int row0 = (int)blockIdx.y * per, n_rows = min(per, rows - row0);
   if ((int)blockIdx.y >= gy || n_rows <= 0) {        // (the whole cluster)
     t_cluster_wait();
+    if (warp == 1) {
+      t_fence_after();
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_s), "r"(PT_TMEM) : "memory");
+    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
@@ -206,12 +218,6 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
   const int S = min(PT_STAGES_MAX, PT_RING / stage_bytes);
   const int kb_all = a.K / PT_BK, kb_per = (kb_all + ks - 1) / ks;
   const int kb0 = z * kb_per, nkb = min(kb_per, kb_all - kb0), nch = (nkb + CH - 1) / CH;    // (the launcher leaves no split without a block)
-  if (warp == 1) {                                   // the product warp owns the tensor-memory allocation (of both CTAs together)
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(t_smem_u32(&tmem_base_s)), "r"(PT_TMEM) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
-  t_fence_before();
-  __syncthreads();
   t_cluster_wait();                                  // every barrier of the cluster stands
   t_fence_after();
   const uint32_t tmem = tmem_base_s;
@@ -274,6 +280,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
       const CUtensorMap *map_a = &maps.box[R / 32 - 1];
       const int y = row0 + half * (R / 2);
       uint32_t dst = ring, bar = 0, parity = 1u;
+      t_map_prefetch(map_a);
       asm volatile("griddepcontrol.wait;" ::: "memory");
       for (int it = 0, kb = kb0; it < nch; ++it, kb += CH) {
         if (dst == ring_end) { dst = ring; bar = 0; parity ^= 1u; }
@@ -328,6 +335,15 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
       if (EPI == PROJ_QKV && t < R) meta_s[t] = row0 + t < lim ? __ldcg(a.row_meta + row0 + t) : make_int4(0, 0, 0, 0);
       t_epi_sync();
     }
+    // (cos, sin) of a chunk of eight rows, requested a chunk ahead: even lanes hold the even rows', odd lanes the odd rows'
+    const bool odd = lane & 1, rope = EPI == PROJ_QKV && a.rope_tab != nullptr && n0 < 2 * (a.N / 3);
+    float2 cs[4];
+    auto load_cs = [&](int jb) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        cs[k] = __ldg(a.rope_tab + (size_t)meta_s[EPI == PROJ_QKV ? (r0w + j0 + jb + 2 * k + odd) & (PT_R_MAX - 1) : 0].z * (kDh / 2) + c / 2);
+    };
+    if (rope) load_cs(0);
     ok = t_mbar_wait(acc_full, 0u);
     t_fence_after();
     const float *red = reinterpret_cast<const float *>(t_raw + (ring - t_smem_u32(t_raw)));
@@ -392,7 +408,6 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
       }
       const int rl = r0w + j0 + jb, r = row0 + rl;   // row of v[0] in the group, among the packed rows
       auto on = [&](int i) { return j0 + jb + i < j1 && r + i < lim; };
-      const bool odd = lane & 1;
       if (EPI == PROJ_RESID) {
         float f[8];
 #pragma unroll
@@ -433,13 +448,17 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
               else reinterpret_cast<__nv_bfloat16 *>(a.raw)[(size_t)(r + i) * a.N + col] = __float2bfloat16(v[i]);
             }
         }
-        if (a.rope_tab != nullptr && which < 2) {
+        if (rope) {
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            const float2 cs = a.rope_tab[(size_t)meta_s[(rl + i) & (PT_R_MAX - 1)].z * (kDh / 2) + c / 2];
+            const float2 mine = cs[i >> 1];
+            const float ox = __shfl_xor_sync(0xffffffffu, mine.x, 1), oy = __shfl_xor_sync(0xffffffffu, mine.y, 1);
+            const bool own_row = odd == (bool)(i & 1);
+            const float2 t = make_float2(own_row ? mine.x : ox, own_row ? mine.y : oy);
             const float other = __shfl_xor_sync(0xffffffffu, v[i], 1);
-            v[i] = odd ? other * cs.y + v[i] * cs.x : v[i] * cs.x - other * cs.y;
+            v[i] = odd ? other * t.y + v[i] * t.x : v[i] * t.x - other * t.y;
           }
+          if (jb + 8 < OWN_MAX && j0 + jb + 8 < j1) load_cs(jb + 8);
         }
 #pragma unroll
         for (int i = 0; i < 8; i += 2) {             // even lanes take row i, odd lanes row i + 1, two columns each
