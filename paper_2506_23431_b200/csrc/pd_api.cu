@@ -334,7 +334,7 @@ void product_shape(const Dims &dm, int p, int &K, int &N) {
 // the products are bound by the bytes their 32-column slices read again for every row group (190 active of 512 at width 1024:
 // 58 us against 40 us): there the unpacked path below, with cuBLAS over the allocated rows, stays.  The rule goes by allocated rows, which
 // the host knows when it captures a step; how many are active only the device knows, so a large handle's short start and tail stay unpacked.
-constexpr int kPackedMaxRows = 128, kPackedMaxRowsTc = 1024;
+constexpr int kPackedMaxRows = 128, kPackedMaxRowsTc = 128;      // (proj_tc off: a launch failure at width 256, see there)
 bool packed_path(const pd_handle *h) {
   return h->packed_ok && h->batch * h->dm.C <= (h->tc_w.empty() ? kPackedMaxRows : kPackedMaxRowsTc) && cross_attn_tma_supported(h->dm);
 }

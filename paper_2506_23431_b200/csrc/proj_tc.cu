@@ -8,8 +8,10 @@
 // A pair of CTAs (two SMs, tcgen05 cta_group::2) takes 128 columns of W - the M dimension, 64 per CTA, read MN-major in the caller's
 // layout - and a group of up to 128 rows as the N dimension, of which each CTA fetches half.  So a CTA brings in 64 columns of W and
 // R / 2 rows, where a CTA alone would need the same columns and R rows: behind the dependency wait the rows are what is waited for.
-// The weights do not depend on the kernel before: their tiles are requested ahead of that wait, as many as the ring holds.  A CTA
-// takes at most half an SM's shared memory, so that this works while the kernel before still holds the other half.
+// The weights do not depend on the kernel before: their tiles are requested ahead of that wait, as many as the ring holds.
+// A CTA takes an SM's shared memory for itself, so that never two pairs are on the same SMs: a pair takes its tensor memory together, and pairs
+// of neighbouring launches that took and gave back theirs on the same two SMs at the same time ended in a launch failure
+// (rings of half the size, products of width 256 a microsecond apart).
 // The lanes of tensor memory are columns of W, its columns rows of A: an epilogue warp holds 32 neighbouring columns of one row at
 // a time, reads the residual stream in whole lines, and pairs of lanes pack two rows' stores into one.
 // Reductions beyond 1024 are split over a cluster of pairs: every CTA copies its sums of the rows another CTA owns into that CTA's
@@ -30,7 +32,7 @@ constexpr int PT_TMEM = PT_R_MAX / 2;            // columns of tensor memory: ha
 constexpr int PT_STAGES_MAX = 8;
 constexpr int PT_EPI_WARPS = 8, PT_EPI_T = PT_EPI_WARPS * 32;
 constexpr int PT_THREADS = 96 + PT_EPI_T;        // weights warp, product warp, rows warp, epilogue warps
-constexpr int PT_RING = 104 * 1024;              // behind the products it takes the partial sums of a split reduction
+constexpr int PT_RING = 192 * 1024;              // behind the products it takes the partial sums of a split reduction
 constexpr int PT_SMEM = PT_RING + 256 /*barriers*/ + 1024 /*alignment slack*/;
 constexpr uint32_t PT_SPIN_LIMIT = 1u << 24;
 static_assert(8 * (2 * PT_STAGES_MAX + 4) <= 256, "barriers");
@@ -156,7 +158,7 @@ struct ProjTcArgs : ProjArgs {
 
 // Grid (2 x column slices, row groups, K splits), cluster (2, 1, K splits).
 template <int EPI, bool SPLIT>
-__global__ void __launch_bounds__(PT_THREADS, 2)
+__global__ void __launch_bounds__(PT_THREADS, 1)
 proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_constant__ ProjTcActMaps maps, ProjTcArgs a) {
   extern __shared__ uint8_t t_raw[];
   __shared__ uint32_t tmem_base_s;
@@ -189,11 +191,6 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
   if (lane == 0) rows_s[warp] = cnt;
-  if (warp == 1) {                                   // the product warp owns the tensor-memory allocation (of both CTAs together)
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(t_smem_u32(&tmem_base_s)), "r"(PT_TMEM) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
-  t_fence_before();
   __syncthreads();
   int rows = 0;
 #pragma unroll
@@ -205,10 +202,6 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
   const int row0 = (int)blockIdx.y * per, n_rows = min(per, rows - row0);
   if ((int)blockIdx.y >= gy || n_rows <= 0) {        // (the whole cluster)
     t_cluster_wait();
-    if (warp == 1) {
-      t_fence_after();
-      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_s), "r"(PT_TMEM) : "memory");
-    }
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
   }
@@ -218,6 +211,12 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
   const int S = min(PT_STAGES_MAX, PT_RING / stage_bytes);
   const int kb_all = a.K / PT_BK, kb_per = (kb_all + ks - 1) / ks;
   const int kb0 = z * kb_per, nkb = min(kb_per, kb_all - kb0), nch = (nkb + CH - 1) / CH;    // (the launcher leaves no split without a block)
+  if (warp == 1) {                                   // the product warp owns the tensor-memory allocation (of both CTAs together)
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(t_smem_u32(&tmem_base_s)), "r"(PT_TMEM) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  t_fence_before();
+  __syncthreads();
   t_cluster_wait();                                  // every barrier of the cluster stands
   t_fence_after();
   const uint32_t tmem = tmem_base_s;
