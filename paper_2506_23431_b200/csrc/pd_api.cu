@@ -327,14 +327,15 @@ void product_shape(const Dims &dm, int p, int &K, int &N) {
   N = p == P_QKV ? 3 * dm.d : p == P_UP ? dm.ff : dm.d;
 }
 
-// The packed decode path: every active row of a step in one packed row list, the layers' products on proj_mma.cu, every launch a
-// programmatic dependent of the one before it.  For few rows, where a step is a chain of launch and load latencies: the products
-// take less than cuBLAS with its norm kernels up to about 90 active rows (per layer, at width 768: 90 active of 128 allocated 30 us
-// against 31 us, 6 of 8 16 us against 31 us), and the dependent launches give the attentions a head start.  With more rows
-// the products are bound by the bytes their 32-column slices read again for every row group (190 active of 512 at width 1024:
-// 58 us against 40 us): there the unpacked path below, with cuBLAS over the allocated rows, stays.  The rule goes by allocated rows, which
-// the host knows when it captures a step; how many are active only the device knows, so a large handle's short start and tail stay unpacked.
-constexpr int kPackedMaxRows = 128, kPackedMaxRowsTc = 128;      // (proj_tc off: a launch failure at width 256, see there)
+// The packed decode path: every active row of a step in one packed row list, the layers' products on proj_mma.cu or proj_tc.cu, every launch
+// a programmatic dependent of the one before it.  For few rows, where a step is a chain of launch and load latencies, the register products
+// take less than cuBLAS with its norm kernels (per layer, at width 768: 90 active of 128 allocated 30 us against 31 us, 6 of 8 16 us against
+// 31 us), and the dependent launches give the attentions a head start; with more the products on tensor memory do (proj_tc_better).
+// Whole decodes of four layers with every allocated row active, against the unpacked path below, ms: width 1024, 130 rows 11.8 against
+// 13.0, 512 rows 15.2 against 15.9, 1024 rows 24.7 against 23.7; width 768, 1024 rows 20.0 against 20.8.  With fewer of them active
+// (204 of 512, twelve layers) 68.7 against 74.3.  The rule goes by allocated rows, which the host knows when it captures a step; how many are
+// active only the device knows, so a large handle's short start and tail stay unpacked.
+constexpr int kPackedMaxRows = 128, kPackedMaxRowsTc = 768;
 bool packed_path(const pd_handle *h) {
   return h->packed_ok && h->batch * h->dm.C <= (h->tc_w.empty() ? kPackedMaxRows : kPackedMaxRowsTc) && cross_attn_tma_supported(h->dm);
 }

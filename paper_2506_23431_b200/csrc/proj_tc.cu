@@ -8,14 +8,19 @@
 // A pair of CTAs (two SMs, tcgen05 cta_group::2) takes 128 columns of W - the M dimension, 64 per CTA, read MN-major in the caller's
 // layout - and a group of up to 128 rows as the N dimension, of which each CTA fetches half.  So a CTA brings in 64 columns of W and
 // R / 2 rows, where a CTA alone would need the same columns and R rows: behind the dependency wait the rows are what is waited for.
-// The weights do not depend on the kernel before: their tiles are requested ahead of that wait, as many as the ring holds.
-// A CTA takes an SM's shared memory for itself, so that never two pairs are on the same SMs: a pair takes its tensor memory together, and pairs
-// of neighbouring launches that took and gave back theirs on the same two SMs at the same time ended in a launch failure
-// (rings of half the size, products of width 256 a microsecond apart).
+// The weights do not depend on the kernel before: their tiles are requested ahead of that wait, as many as the ring holds.  A CTA
+// takes at most half an SM's shared memory, so that this works while the kernel before still holds the other half (with the whole of it,
+// decodes are slower by a tenth).  Tensor memory is taken ahead of the wait as well (behind it: 72.3 ms against 68.3 for the decode of 32 sequences
+// below), by pairs that have rows only, and the pair compares the two CTAs' addresses before the first product, which writes both CTAs'
+// tensor memory at one: pairs that took it before they knew their rows, and gave it back at once where they had none, ended in a launch failure.
 // The lanes of tensor memory are columns of W, its columns rows of A: an epilogue warp holds 32 neighbouring columns of one row at
 // a time, reads the residual stream in whole lines, and pairs of lanes pack two rows' stores into one.
 // Reductions beyond 1024 are split over a cluster of pairs: every CTA copies its sums of the rows another CTA owns into that CTA's
 // shared memory (one bulk copy per peer), which adds them in rank order (results do not depend on timing).
+// What bounds it: a launch is a chain of latencies - release of the launch before 1.2 us, first rows 0.5, products and the weights the
+// ring did not hold, accumulators out, 0.6 to the exit.  Per launch inside a decode of 32 sequences (204 rows active of 512, width 1024): 7.5 us
+// for queries, keys and values, 5.2-5.9 for the square products, 6.3 up, 9.4 down, where the library took 5.7, 4.3-4.5, 6.4 and 8.3 and
+// 2.4 for a norm in front of every other one, without overlap.  Fewer or more row groups, K splits of 1536 or 2048: slower or the same.
 // Every mbarrier wait is bounded: on expiry the kernel records PD_ERR_TIMEOUT, stops waiting, falls through to the
 // common exit and frees its tensor memory.
 #include <algorithm>
@@ -32,10 +37,10 @@ constexpr int PT_TMEM = PT_R_MAX / 2;            // columns of tensor memory: ha
 constexpr int PT_STAGES_MAX = 8;
 constexpr int PT_EPI_WARPS = 8, PT_EPI_T = PT_EPI_WARPS * 32;
 constexpr int PT_THREADS = 96 + PT_EPI_T;        // weights warp, product warp, rows warp, epilogue warps
-constexpr int PT_RING = 192 * 1024;              // behind the products it takes the partial sums of a split reduction
+constexpr int PT_RING = 104 * 1024;              // behind the products it takes the partial sums of a split reduction
 constexpr int PT_SMEM = PT_RING + 256 /*barriers*/ + 1024 /*alignment slack*/;
 constexpr uint32_t PT_SPIN_LIMIT = 1u << 24;
-static_assert(8 * (2 * PT_STAGES_MAX + 4) <= 256, "barriers");
+static_assert(8 * (2 * PT_STAGES_MAX + 5) <= 256, "barriers");
 // 64-wide blocks of K per stage and copy: a copy costs its issue and a round trip, so small boxes are taken several at a time
 __host__ __device__ constexpr int pt_blocks(int R) { return R <= 64 ? 4 : 2; }
 
@@ -143,6 +148,9 @@ __device__ __forceinline__ void t_tmem_ld8(uint32_t taddr, float (&v)[8]) {
 }
 __device__ __forceinline__ void t_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void t_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+// The product warp tells the epilogue warps where tensor memory is (they ask behind the products, and never wait here).
+__device__ __forceinline__ void t_tmem_told() { asm volatile("bar.arrive 2, %0;" ::"n"(PT_EPI_T + 32) : "memory"); }
+__device__ __forceinline__ void t_tmem_ask() { asm volatile("bar.sync 2, %0;" ::"n"(PT_EPI_T + 32) : "memory"); }
 __device__ __forceinline__ void t_epi_sync() { asm volatile("bar.sync 1, %0;" ::"n"(PT_EPI_T) : "memory"); }
 __device__ __forceinline__ void t_cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void t_cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
@@ -158,10 +166,10 @@ struct ProjTcArgs : ProjArgs {
 
 // Grid (2 x column slices, row groups, K splits), cluster (2, 1, K splits).
 template <int EPI, bool SPLIT>
-__global__ void __launch_bounds__(PT_THREADS, 1)
+__global__ void __launch_bounds__(PT_THREADS, 2)
 proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_constant__ ProjTcActMaps maps, ProjTcArgs a) {
   extern __shared__ uint8_t t_raw[];
-  __shared__ uint32_t tmem_base_s;
+  __shared__ uint32_t tmem_base_s, peer_base_s;
   __shared__ int rows_s[PT_THREADS / 32];
   __shared__ float inv_s[PT_R_MAX];
   __shared__ int4 meta_s[EPI == PROJ_QKV ? PT_R_MAX : 1];
@@ -174,7 +182,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
   // ---- ahead of the dependency wait: the number of rows (left by the previous step's scheduler), barriers, tensor memory, weights
   const uint32_t ring = (t_smem_u32(t_raw) + 1023u) & ~1023u;
   const uint32_t full = ring + PT_RING, empty = full + 8 * PT_STAGES_MAX, acc_full = empty + 8 * PT_STAGES_MAX, red_full = acc_full + 8,
-                 red_free = red_full + 8, acc_read = red_free + 8;
+                 red_free = red_full + 8, acc_read = red_free + 8, peer_has = acc_read + 8;
   int cnt = 0;
   for (int b = tid; b < a.batch; b += PT_THREADS) cnt += a.n_active[b];
   if (tid < 2) t_map_prefetch(&wmaps.k[tid]);
@@ -184,6 +192,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
     t_mbar_init(red_full, 1);
     t_mbar_init(red_free, (uint32_t)ks);
     t_mbar_init(acc_read, (uint32_t)(2 * PT_EPI_WARPS + (SPLIT ? ks : 0)));
+    t_mbar_init(peer_has, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
@@ -211,15 +220,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
   const int S = min(PT_STAGES_MAX, PT_RING / stage_bytes);
   const int kb_all = a.K / PT_BK, kb_per = (kb_all + ks - 1) / ks;
   const int kb0 = z * kb_per, nkb = min(kb_per, kb_all - kb0), nch = (nkb + CH - 1) / CH;    // (the launcher leaves no split without a block)
-  if (warp == 1) {                                   // the product warp owns the tensor-memory allocation (of both CTAs together)
-    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(t_smem_u32(&tmem_base_s)), "r"(PT_TMEM) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
-  }
-  t_fence_before();
-  __syncthreads();
   t_cluster_wait();                                  // every barrier of the cluster stands
-  t_fence_after();
-  const uint32_t tmem = tmem_base_s;
   const int n0 = (int)blockIdx.x * PT_COLS;
   bool ok = true;
 
@@ -248,12 +249,24 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
   } else if (warp == 1) {
     // ------------------------------------------------------------------ products (one lane of the pair).  The whole warp walks: a loop that
     // one lane walks keeps descriptors out of the uniform registers the products read, and a product then costs 128 cycles to issue
-    if (half == 0) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(t_smem_u32(&tmem_base_s)), "r"(PT_TMEM) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    __syncwarp();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(&tmem_base_s);
+    t_tmem_told();
+    if (half == 1) {                                 // the products write both CTAs' tensor memory, at one address
+      if (lane == 0) {
+        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(t_peer(t_smem_u32(&peer_base_s), leader)), "r"(tmem) : "memory");
+        t_mbar_arrive_peer(t_peer(peer_has, leader));
+      }
+    } else {
+      ok = t_mbar_wait<true>(peer_has, 0u);
+      if (ok && *reinterpret_cast<volatile uint32_t *>(&peer_base_s) != tmem) ok = false;
       const uint32_t idesc = t_idesc(R);
       const uint16_t mask = (uint16_t)(3u << leader);
       int s = 0;
       uint32_t u = 0, lo = t_desc_lo(ring);
-      for (int ch = 0; ch < nch; ++ch) {
+      for (int ch = 0; ch < nch && ok; ++ch) {
         if (!t_mbar_wait(full + 8 * s, u & 1u)) { ok = false; break; }
         t_fence_after();
         if (t_elect()) {
@@ -293,7 +306,6 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
     const int e = warp - 3, q = warp & 3;            // lanes 32 q .. of tensor memory
     const int RQ = R / 4;                            // rows per warp: column halves (q & 1) x row halves (q >> 1) x two warps each
     const int r0w = (q >> 1) * (R / 2) + (e >> 2) * RQ;      // first of this warp's rows in the group
-    const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((e >> 2) * RQ);
     const int c = (q & 1) * 32 + lane, col = n0 + c;
     const bool col_on = col < a.N;
     const int own = SPLIT ? ((RQ + ks - 1) / ks + 3) / 4 * 4 : RQ;      // rows of a warp a CTA of the cluster owns, in fours
@@ -344,7 +356,9 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
     };
     if (rope) load_cs(0);
     ok = t_mbar_wait(acc_full, 0u);
+    t_tmem_ask();
     t_fence_after();
+    const uint32_t taddr = tmem_base_s + ((uint32_t)(q * 32) << 16) + (uint32_t)((e >> 2) * RQ);
     const float *red = reinterpret_cast<const float *>(t_raw + (ring - t_smem_u32(t_raw)));
     const uint32_t blk = (uint32_t)own * (PT_EPI_WARPS * 128);      // bytes of one owner's rows: [warp][fours of rows][32 columns][4]
     auto read_done = [&]() {                         // this warp has read its accumulators
@@ -490,7 +504,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
     if (!t_mbar_wait<true>(acc_read, 0u)) atomicExch(a.status, (int)PD_ERR_TIMEOUT);
     __syncwarp();
     t_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(PT_TMEM) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_s), "r"(PT_TMEM) : "memory");
   }
 }
 
@@ -526,7 +540,10 @@ cudaError_t each_kernel(int epi, bool split, bool all, F f) {
 // Whole blocks of K, 16-byte tensor-map rows.
 bool proj_tc_supported(int K, int N) { return K >= PT_BK && K % PT_BK == 0 && N % 8 == 0; }
 
-bool proj_tc_better(int K, int N, int rows_cap) { return rows_cap > 128; }
+// Against the register products of proj_mma.cu, whole decodes of four layers, 512 keys, every row active, ms: width 1024, 130 rows
+// 11.8 against 12.2; width 768, 130 rows 10.8 against 10.6, 256 rows 11.8 against 13.9; width 256, 256 rows 9.1 against 7.7, 1024 rows
+// 11.5 against 12.1.  (K and N differ by the same factors at every width: the narrower side stands for it.)
+bool proj_tc_better(int K, int N, int rows_cap) { return rows_cap > 128 && (long long)rows_cap * std::min(K, N) > 110000; }
 
 cudaError_t proj_tc_prepare() {
   return each_kernel(0, false, true, [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PT_SMEM); });

@@ -437,11 +437,12 @@ def test_decodes_of_few_rows_repeat_bit_for_bit(batch, heads, ctx, kv8):
 
 PACKED = [
     # sequences, open rows per sequence, inner width, positions, longest subsequence, 8-bit context
-    (5, 26, 64, ROPE, 28, False),       # 130 rows allocated: the fewest that take the tensor-memory products; an inner width of one block
-    (9, 31, 1088, T5, 33, True),        # a reduction over two pairs of CTAs, the second one block shorter
-    (16, 32, 2112, ROPE, 34, False),    # 512 rows: three pairs; row groups grow past one per SM
-    (32, 32, 4160, T5, 36, False),      # 1024 rows, the most that run packed; four pairs, the last one block longer or shorter
-    (40, 7, 256, ROPE, 40, False),      # two pages per subsequence
+    (5, 26, 64, ROPE, 28, False),       # 130 rows allocated, register products beyond 128; an inner width of one block
+    (19, 31, 1088, T5, 33, True),       # 589 rows: tensor-memory products at this width; a reduction over two pairs of CTAs, the second one block shorter
+    (18, 32, 2112, ROPE, 34, False),    # 576 rows: three pairs
+    (24, 32, 4160, T5, 36, False),      # 768 rows, the most that run packed; four pairs, the last one shorter
+    (25, 31, 192, T5, 33, False),       # 775 rows: the kernels beyond
+    (90, 7, 256, ROPE, 40, False),      # 630 rows, two pages per subsequence
 ]
 
 
