@@ -343,7 +343,8 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
         for (int o = 4; o > 0; o >>= 1) sum[i] += __shfl_xor_sync(0xffffffffu, sum[i], o);
         if (l8 == 0) inv_s[i * 32 + (t >> 3)] = rsqrtf(sum[i] * a.inv_width + a.eps);
       }
-      if (EPI == PROJ_QKV && t < R) meta_s[t] = row0 + t < lim ? __ldcg(a.row_meta + row0 + t) : make_int4(0, 0, 0, 0);
+      // (all of it: a split's warp asks for the positions of whole chunks, which may end beyond the group's rows)
+      if (EPI == PROJ_QKV && t < PT_R_MAX) meta_s[t] = row0 + t < lim ? __ldcg(a.row_meta + row0 + t) : make_int4(0, 0, 0, 0);
       t_epi_sync();
     }
     // (cos, sin) of a chunk of eight rows, requested a chunk ahead: even lanes hold the even rows', odd lanes the odd rows'
@@ -354,7 +355,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
       for (int k = 0; k < 4; ++k)
         cs[k] = __ldg(a.rope_tab + (size_t)meta_s[EPI == PROJ_QKV ? (r0w + j0 + jb + 2 * k + odd) & (PT_R_MAX - 1) : 0].z * (kDh / 2) + c / 2);
     };
-    if (rope) load_cs(0);
+    if (rope && j0 < j1) load_cs(0);
     ok = t_mbar_wait(acc_full, 0u);
     t_tmem_ask();
     t_fence_after();

@@ -456,6 +456,20 @@ def test_decode_on_tensor_memory_products(batch, rows, d_ff, pos, length, kv8):
     assert s["max_err"] < parity.TOL["bf16"]
 
 
+@pytest.mark.parametrize("pos", [ROPE, T5])
+@pytest.mark.parametrize("heads", [17, 33, 49])
+def test_decode_on_split_tensor_memory_products(heads, pos):
+    """Widths whose every product is split over two, three and four pairs, the rows of a group (5 to 130) in all its sizes.  In rotary mode
+    the pairs ask for the positions of whole chunks of rows, of rows beyond the group's too.  A logit is a product of a normalised row, whose length
+    is sqrt(width), with a row of lm_head: at one weight scale its error grows with sqrt(width) (2.4e-2 at 2112).  The weights shrink by that factor, so that
+    logits and errors have the scale that the bar is for, that of width 1024."""
+    wl = W.CONFIGS["bart_base"].scaled(name="split", batch=5, sub_max=26, d_ff=192, pos_mode=pos, max_sub_len=28, time_max=32,
+                                       length_dist=("uniform", 24, 28), **dict(BASE, d_model=64 * heads, n_heads=heads, n_layers=1, ctx=40,
+                                                                            weight_std=0.02 * (1024 / (64 * heads)) ** 0.5))
+    s = check(wl, rows=[0, 4], ragged=True, free_run=False)
+    assert s["max_err"] < parity.TOL["bf16"]
+
+
 @pytest.mark.parametrize("kv8", [True, False])
 @pytest.mark.parametrize("batch,heads,ctx", [(24, 16, 512), (40, 12, 300)])
 def test_decodes_of_many_packed_rows_repeat_bit_for_bit(batch, heads, ctx, kv8):
