@@ -50,7 +50,8 @@ typedef enum {
   PD_ERR_POOL_EXHAUSTED = -4, /* the KV page pool ran out (set on the device)              */
   PD_ERR_CUDA = -5,           /* a CUDA or cuBLAS call failed                              */
   PD_ERR_TIMEOUT = -6,        /* a bounded device-side wait expired (set on the device)    */
-  PD_ERR_UNSUPPORTED = -7     /* valid request the build does not implement                */
+  PD_ERR_UNSUPPORTED = -7,    /* valid request the build does not implement                */
+  PD_ERR_DEVICE = -8          /* tensor memory of a pair of CTAs at two addresses (set on the device) */
 } pd_status;
 
 enum { PD_DTYPE_FP32 = 0, PD_DTYPE_BF16 = 1 };

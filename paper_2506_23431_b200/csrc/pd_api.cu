@@ -214,6 +214,14 @@ pd_status fail(pd_handle *h, pd_status s, const std::string &msg) {
   if (h) h->err = msg;
   return s;
 }
+// The error word a kernel left in the header.
+pd_status fail_device(pd_handle *h, int32_t status) {
+  const char *why = status == PD_ERR_POOL_EXHAUSTED ? ": the page pool is exhausted"
+                    : status == PD_ERR_TIMEOUT      ? ": a bounded wait expired"
+                    : status == PD_ERR_DEVICE       ? ": tensor memory of a pair of CTAs at two addresses"
+                                                    : "";
+  return fail(h, (pd_status)status, "device-side error " + std::to_string(status) + why);
+}
 #define CU_TRY(h, expr)                                                                                   \
   do {                                                                                                    \
     cudaError_t e__ = (expr);                                                                             \
@@ -618,7 +626,7 @@ pd_status device_status(pd_handle *h) {
   int32_t hdr[HDR_WORDS];
   CU_TRY(h, cudaMemcpyAsync(hdr, h->st.hdr, sizeof(hdr), cudaMemcpyDeviceToHost, h->stream));
   CU_TRY(h, cudaStreamSynchronize(h->stream));
-  if (hdr[HDR_STATUS] != 0) return fail(h, (pd_status)hdr[HDR_STATUS], "device-side error " + std::to_string(hdr[HDR_STATUS]));
+  if (hdr[HDR_STATUS] != 0) return fail_device(h, hdr[HDR_STATUS]);
   return PD_OK;
 }
 
@@ -920,7 +928,7 @@ pd_status pd_done(pd_handle *h, int32_t *all_done) {
   CU_TRY(h, cudaStreamSynchronize(h->stream));
   *all_done = h->pinned_flag[HDR_ALL_DONE];
   if (h->pinned_flag[HDR_STATUS] != 0)
-    return fail(h, (pd_status)h->pinned_flag[HDR_STATUS], "device-side error " + std::to_string(h->pinned_flag[HDR_STATUS]));
+    return fail_device(h, h->pinned_flag[HDR_STATUS]);
   return PD_OK;
 }
 
@@ -945,7 +953,7 @@ pd_status pd_run(pd_handle *h, int32_t poll_every, int32_t *steps_run) {
       const int old = (n - lag) % pd_handle::kRunSlots;
       CU_TRY(h, cudaEventSynchronize(h->ev_snap[old]));
       const int32_t *s_old = h->pinned_flag + 16 * (1 + old);
-      if (s_old[HDR_STATUS] != 0) return fail(h, (pd_status)s_old[HDR_STATUS], "device-side error " + std::to_string(s_old[HDR_STATUS]));
+      if (s_old[HDR_STATUS] != 0) return fail_device(h, s_old[HDR_STATUS]);
       done = s_old[HDR_ALL_DONE];
     }
   }

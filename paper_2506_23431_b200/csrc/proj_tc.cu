@@ -11,8 +11,14 @@
 // The weights do not depend on the kernel before: their tiles are requested ahead of that wait, as many as the ring holds.  A CTA
 // takes at most half an SM's shared memory, so that this works while the kernel before still holds the other half (with the whole of it,
 // decodes are slower by a tenth).  Tensor memory is taken ahead of the wait as well (behind it: 72.3 ms against 68.3 for the decode of 32 sequences
-// below), by pairs that have rows only, and the pair compares the two CTAs' addresses before the first product, which writes both CTAs'
-// tensor memory at one: pairs that took it before they knew their rows, and gave it back at once where they had none, ended in a launch failure.
+// below), by pairs that have rows only.
+// Tensor memory of a pair is taken and given back by instructions that belong to both CTAs, and nothing orders one CTA against the other by
+// itself.  A form that took it before it knew its rows, and gave it back at once where there were none, ended in a launch failure once; the cause was
+// never established.  By reading, a CTA of it could give back, and exit, while its peer was still taking.  So the CTAs meet behind the taking, and
+// compare addresses there (a product writes both CTAs' tensor memory at one), and meet again behind the giving back before either exits: 0.1 us
+// per launch.  Pairs of two launches, like pairs of one launch of more pairs than the chip has pairs of SMs, may take at the same time; shared
+// memory lets no third one onto their SMs, and columns never run out: two pairs take 128 of 512, the other kernels that fit beside one of them 256.
+// (With the next launch started only behind the taking a decode takes 1.9 % longer, and pairs of one launch still take at the same time.)
 // The lanes of tensor memory are columns of W, its columns rows of A: an epilogue warp holds 32 neighbouring columns of one row at
 // a time, reads the residual stream in whole lines, and pairs of lanes pack two rows' stores into one.
 // Reductions beyond 1024 are split over a cluster of pairs: every CTA copies its sums of the rows another CTA owns into that CTA's
@@ -40,7 +46,7 @@ constexpr int PT_THREADS = 96 + PT_EPI_T;        // weights warp, product warp, 
 constexpr int PT_RING = 104 * 1024;              // behind the products it takes the partial sums of a split reduction
 constexpr int PT_SMEM = PT_RING + 256 /*barriers*/ + 1024 /*alignment slack*/;
 constexpr uint32_t PT_SPIN_LIMIT = 1u << 24;
-static_assert(8 * (2 * PT_STAGES_MAX + 5) <= 256, "barriers");
+static_assert(8 * (2 * PT_STAGES_MAX + 6) <= 256, "barriers");
 // 64-wide blocks of K per stage and copy: a copy costs its issue and a round trip, so small boxes are taken several at a time
 __host__ __device__ constexpr int pt_blocks(int R) { return R <= 64 ? 4 : 2; }
 
@@ -170,19 +176,20 @@ __global__ void __launch_bounds__(PT_THREADS, 2)
 proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_constant__ ProjTcActMaps maps, ProjTcArgs a) {
   extern __shared__ uint8_t t_raw[];
   __shared__ uint32_t tmem_base_s, peer_base_s;
+  __shared__ int same_s;                             // the pair's tensor memory is at one address
   __shared__ int rows_s[PT_THREADS / 32];
   __shared__ float inv_s[PT_R_MAX];
   __shared__ int4 meta_s[EPI == PROJ_QKV ? PT_R_MAX : 1];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int half = (int)blockIdx.x & 1;              // this CTA's half of the pair's columns and rows
   const int ks = SPLIT ? (int)gridDim.z : 1, z = SPLIT ? (int)blockIdx.z : 0;
-  const uint32_t leader = 2u * z;                    // first CTA of this pair in the cluster
+  const uint32_t leader = 2u * z, peer = leader + (uint32_t)(half ^ 1);      // first CTA of this pair in the cluster, the other one of it
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   // ---- ahead of the dependency wait: the number of rows (left by the previous step's scheduler), barriers, tensor memory, weights
   const uint32_t ring = (t_smem_u32(t_raw) + 1023u) & ~1023u;
   const uint32_t full = ring + PT_RING, empty = full + 8 * PT_STAGES_MAX, acc_full = empty + 8 * PT_STAGES_MAX, red_full = acc_full + 8,
-                 red_free = red_full + 8, acc_read = red_free + 8, peer_has = acc_read + 8;
+                 red_free = red_full + 8, acc_read = red_free + 8, peer_has = acc_read + 8, peer_gave = peer_has + 8;
   int cnt = 0;
   for (int b = tid; b < a.batch; b += PT_THREADS) cnt += a.n_active[b];
   if (tid < 2) t_map_prefetch(&wmaps.k[tid]);
@@ -193,6 +200,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
     t_mbar_init(red_free, (uint32_t)ks);
     t_mbar_init(acc_read, (uint32_t)(2 * PT_EPI_WARPS + (SPLIT ? ks : 0)));
     t_mbar_init(peer_has, 1);
+    t_mbar_init(peer_gave, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
@@ -209,7 +217,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
   const int gy = max(1, min(min((int)gridDim.y, (rows + 15) / 16), max(a.groups, (rows + PT_R_MAX - 1) / PT_R_MAX)));
   const int per = ((rows + gy - 1) / gy + 7) / 8 * 8;
   const int row0 = (int)blockIdx.y * per, n_rows = min(per, rows - row0);
-  if ((int)blockIdx.y >= gy || n_rows <= 0) {        // (the whole cluster)
+  if ((int)blockIdx.y >= gy || n_rows <= 0) {        // (the whole cluster; it takes no tensor memory)
     t_cluster_wait();
     asm volatile("griddepcontrol.wait;" ::: "memory");
     return;
@@ -222,7 +230,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
   const int kb0 = z * kb_per, nkb = min(kb_per, kb_all - kb0), nch = (nkb + CH - 1) / CH;    // (the launcher leaves no split without a block)
   t_cluster_wait();                                  // every barrier of the cluster stands
   const int n0 = (int)blockIdx.x * PT_COLS;
-  bool ok = true;
+  bool ok = true, same = true;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ weights (one lane)
@@ -253,15 +261,17 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     __syncwarp();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t *>(&tmem_base_s);
+    // The two CTAs tell each other where: neither goes on before the pair's allocation is complete in both.
+    if (lane == 0) {
+      asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(t_peer(t_smem_u32(&peer_base_s), peer)), "r"(tmem) : "memory");
+      t_mbar_arrive_peer(t_peer(peer_has, peer));
+    }
+    ok = t_mbar_wait<true>(peer_has, 0u);
+    same = !ok || *reinterpret_cast<volatile uint32_t *>(&peer_base_s) == tmem;
+    if (lane == 0) *reinterpret_cast<volatile int *>(&same_s) = same;
+    __syncwarp();
     t_tmem_told();
-    if (half == 1) {                                 // the products write both CTAs' tensor memory, at one address
-      if (lane == 0) {
-        asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(t_peer(t_smem_u32(&peer_base_s), leader)), "r"(tmem) : "memory");
-        t_mbar_arrive_peer(t_peer(peer_has, leader));
-      }
-    } else {
-      ok = t_mbar_wait<true>(peer_has, 0u);
-      if (ok && *reinterpret_cast<volatile uint32_t *>(&peer_base_s) != tmem) ok = false;
+    if (half == 0) {
       const uint32_t idesc = t_idesc(R);
       const uint16_t mask = (uint16_t)(3u << leader);
       int s = 0;
@@ -270,7 +280,7 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
         if (!t_mbar_wait(full + 8 * s, u & 1u)) { ok = false; break; }
         t_fence_after();
         if (t_elect()) {
-          const int nb = min(CH, nkb - ch * CH);
+          const int nb = same ? min(CH, nkb - ch * CH) : 0;    // (a product writes both CTAs' tensor memory, at one address)
           for (int b = 0; b < nb; ++b) {
 #pragma unroll
             for (int k4 = 0; k4 < PT_BK / 16; ++k4)  // 16 of K: two groups of eight rows of W, 32 bytes of a row of A
@@ -358,6 +368,8 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
     if (rope && j0 < j1) load_cs(0);
     ok = t_mbar_wait(acc_full, 0u);
     t_tmem_ask();
+    same = *reinterpret_cast<volatile int *>(&same_s) != 0;
+    ok = ok && same;
     t_fence_after();
     const uint32_t taddr = tmem_base_s + ((uint32_t)(q * 32) << 16) + (uint32_t)((e >> 2) * RQ);
     const float *red = reinterpret_cast<const float *>(t_raw + (ring - t_smem_u32(t_raw)));
@@ -497,7 +509,8 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
       }
     }
   }
-  if (!ok) atomicExch(a.status, (int)PD_ERR_TIMEOUT);
+  if (!same) atomicExch(a.status, (int)PD_ERR_DEVICE);
+  else if (!ok) atomicExch(a.status, (int)PD_ERR_TIMEOUT);
   if (warp == 1) {
     // every warp of both CTAs is through with the accumulators, and the peers with this CTA's sums (nobody leaves while another
     // CTA reaches into it)
@@ -506,6 +519,9 @@ proj_tc_kernel(const __grid_constant__ ProjTcWeightMaps wmaps, const __grid_cons
     __syncwarp();
     t_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base_s), "r"(PT_TMEM) : "memory");
+    // neither CTA leaves while the other has a pair-wide instruction to finish
+    if (lane == 0) t_mbar_arrive_peer(t_peer(peer_gave, peer));
+    if (!t_mbar_wait<true>(peer_gave, 0u)) atomicExch(a.status, (int)PD_ERR_TIMEOUT);
   }
 }
 

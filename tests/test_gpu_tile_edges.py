@@ -474,3 +474,35 @@ def test_decode_on_split_tensor_memory_products(heads, pos):
 @pytest.mark.parametrize("batch,heads,ctx", [(24, 16, 512), (40, 12, 300)])
 def test_decodes_of_many_packed_rows_repeat_bit_for_bit(batch, heads, ctx, kv8):
     test_decodes_of_few_rows_repeat_bit_for_bit(batch, heads, ctx // 16 * 16, kv8)
+
+
+def test_two_handles_side_by_side_on_tensor_memory_products():
+    """Steps of two handles on streams of their own, whose pairs of CTAs share SMs and tensor memory: each gives what it gives alone."""
+    from paper_2506_23431_b200 import binding as B
+    runs = []
+    for batch, heads in ((24, 16), (40, 12)):
+        wl = W.CONFIGS["bart_base"].scaled(name="beside", batch=batch, n_layers=3, d_model=64 * heads, n_heads=heads, d_ff=256 * heads, vocab=2000, ctx=300,
+                                           sub_max=8, delta_t=4, max_sub_len=24, length_dist=("uniform", 10, 24), time_max=40, pos_mode=T5)
+        dec = B.PipelinedDecoder(wl.hyper(), W.make_weights(wl), wl.batch)
+        runs.append((dec, (dec.device_memory(W.make_encoder_memory(wl)), W.make_ctx_len(wl), W.make_forced_len(wl)), batch * dec.rows_per_seq * wl.d_model))
+
+    def result(dec, n):
+        return dec.debug_read(B.PD_BUF_X, np.float32, n).copy(), dec.get_chosen().copy()
+
+    alone = []
+    for dec, args, n in runs:
+        dec.encode_context(*args)
+        for _ in range(30):
+            dec.step()
+        alone.append(result(dec, n))
+    for _ in range(4):
+        for dec, args, _n in runs:
+            dec.encode_context(*args)
+        for _ in range(30):
+            for dec, _args, _n in runs:
+                dec.step()
+        for (dec, _args, n), want in zip(runs, alone):
+            got = result(dec, n)
+            assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+    for dec, _args, _n in runs:
+        dec.close()
