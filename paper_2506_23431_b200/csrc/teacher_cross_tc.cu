@@ -43,19 +43,27 @@ __device__ __forceinline__ void c_mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void c_mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ bool c_mbar_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // Bounded wait: false when the phase did not complete within the spin limit.
 __device__ __forceinline__ bool c_mbar_wait(uint32_t bar, uint32_t parity) {
-  for (uint32_t it = 0; it < XC_SPIN_LIMIT; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
+  for (uint32_t it = 0; it < XC_SPIN_LIMIT; ++it)
+    if (c_mbar_try(bar, parity)) return true;
+  return false;
+}
+// The same by a whole warp, whose lanes take every turn together: also where the limit runs out none goes on without the others.
+__device__ __forceinline__ bool c_mbar_wait_warp(uint32_t bar, uint32_t parity) {
+  for (uint32_t it = 0; it < XC_SPIN_LIMIT; ++it)
+    if (__all_sync(0xffffffffu, c_mbar_try(bar, parity))) return true;
   return false;
 }
 __device__ __forceinline__ void c_tma_load_2d(uint32_t dst, const CUtensorMap *tmap, uint32_t bar, int x, int y) {
@@ -222,7 +230,7 @@ __global__ void __launch_bounds__(XC_THREADS, 2) teacher_cross_kernel(const __gr
     const uint32_t q_lo = c_desc_lo(q_s), ring_lo = c_desc_lo(ring);
     auto scores = [&](int tile) {
       const int s = tile % XC_STAGES;
-      if (!c_mbar_wait(bar_full + 8 * s, (uint32_t)(tile / XC_STAGES) & 1u)) { ok = false; return; }
+      if (!c_mbar_wait_warp(bar_full + 8 * s, (uint32_t)(tile / XC_STAGES) & 1u)) { ok = false; return; }
       c_fence_after();
       if (c_elect()) {
 #pragma unroll
@@ -231,16 +239,16 @@ __global__ void __launch_bounds__(XC_THREADS, 2) teacher_cross_kernel(const __gr
         c_mma_commit(bar_s);
       }
     };
-    ok = c_mbar_wait(bar_q, 0);
+    ok = c_mbar_wait_warp(bar_q, 0);
     if (ok) scores(0);
     for (int j = 0; j < n_halves && ok; ++j) {
       const int tile = j >> 1, s = tile % XC_STAGES;
       if ((j & 1) != 0 && tile + 1 < n_tiles) {             // the tile's scores are all read: the next one's
-        if (!c_mbar_wait(bar_read, (uint32_t)tile & 1u)) { ok = false; break; }
+        if (!c_mbar_wait_warp(bar_read, (uint32_t)tile & 1u)) { ok = false; break; }
         c_fence_after();
         scores(tile + 1);
       }
-      if (!ok || !c_mbar_wait(bar_p + 8 * (j & 1), (uint32_t)(j >> 1) & 1u)) { ok = false; break; }
+      if (!ok || !c_mbar_wait_warp(bar_p + 8 * (j & 1), (uint32_t)(j >> 1) & 1u)) { ok = false; break; }
       c_fence_after();
       if (c_elect()) {
         const uint32_t v_lo = ring_lo + s * (XC_STAGE >> 4) + (XC_TILE >> 4) + (j & 1) * (XC_TILE / 2 >> 4);

@@ -71,19 +71,27 @@ __device__ __forceinline__ void v_mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void v_mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ bool v_mbar_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 // Bounded wait: false when the phase did not complete within the spin limit.
 __device__ __forceinline__ bool v_mbar_wait(uint32_t bar, uint32_t parity) {
-  for (uint32_t it = 0; it < VT_SPIN_LIMIT; ++it) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
-  }
+  for (uint32_t it = 0; it < VT_SPIN_LIMIT; ++it)
+    if (v_mbar_try(bar, parity)) return true;
+  return false;
+}
+// The same by a whole warp, whose lanes take every turn together: also where the limit runs out none goes on without the others.
+__device__ __forceinline__ bool v_mbar_wait_warp(uint32_t bar, uint32_t parity) {
+  for (uint32_t it = 0; it < VT_SPIN_LIMIT; ++it)
+    if (__all_sync(0xffffffffu, v_mbar_try(bar, parity))) return true;
   return false;
 }
 __device__ __forceinline__ void v_tma_load_2d(uint32_t dst, const CUtensorMap *tmap, uint32_t bar, int x, int y) {
@@ -254,10 +262,10 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     for (int p = 0; p < n_pass && ok; ++p) {
       const int tiles = min(TILES, n_tt - TILES * p);
       // the epilogue must be done with the previous pass's accumulators
-      if (!v_mbar_wait(bar_acc_empty, ((uint32_t)p & 1u) ^ 1u)) { ok = false; break; }
+      if (!v_mbar_wait_warp(bar_acc_empty, ((uint32_t)p & 1u) ^ 1u)) { ok = false; break; }
       v_fence_after();
       for (int kb = 0; kb < nkb; ++kb) {
-        if (!v_mbar_wait(bar_full + 8 * s, u & 1u)) { ok = false; break; }
+        if (!v_mbar_wait_warp(bar_full + 8 * s, u & 1u)) { ok = false; break; }
         v_fence_after();
         if (v_elect()) {
           const uint32_t sa = v_desc_lo(base + s * VT_STAGE_BYTES), sb = sa + (TILES * VT_A_BYTES >> 4);
@@ -290,7 +298,7 @@ vocab_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
         }
         inv_s[j * VT_M + quarter * 32 + lane] = rsqrtf((s0 + s1) * a.inv_width + a.eps);
       }
-      if (ok && !v_mbar_wait(bar_acc_full, (uint32_t)p & 1u)) ok = false;
+      if (ok && !v_mbar_wait_warp(bar_acc_full, (uint32_t)p & 1u)) ok = false;
       if (!ok) break;
       v_fence_after();
       for (int j = 0; j < tiles; ++j) {
