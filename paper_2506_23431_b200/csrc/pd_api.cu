@@ -339,13 +339,23 @@ void product_shape(const Dims &dm, int p, int &K, int &N) {
 // a programmatic dependent of the one before it.  For few rows, where a step is a chain of launch and load latencies, the register products
 // take less than cuBLAS with its norm kernels (per layer, at width 768: 90 active of 128 allocated 30 us against 31 us, 6 of 8 16 us against
 // 31 us), and the dependent launches give the attentions a head start; with more the products on tensor memory do (proj_tc_better).
-// Whole decodes of four layers with every allocated row active, against the unpacked path below, ms: width 1024, 130 rows 11.8 against
-// 13.0, 512 rows 15.2 against 15.9, 1024 rows 24.7 against 23.7; width 768, 1024 rows 20.0 against 20.8.  With fewer of them active
-// (204 of 512, twelve layers) 68.7 against 74.3.  The rule goes by allocated rows, which the host knows when it captures a step; how many are
-// active only the device knows, so a large handle's short start and tail stay unpacked.
-constexpr int kPackedMaxRows = 128, kPackedMaxRowsTc = 768;
+// Whole decodes of four layers (two beyond width 1024), 512 keys, inner sides of four widths, against the unpacked path below, "library / packed"
+// with about two thirds and with about 0.42 of the allocated rows active:
+//   width    130 rows       256           384           512           640           768
+//    256   1.300 1.356   1.262 1.327   1.212 1.315   1.191 1.290   1.127 1.203   1.111 1.192
+//    512   1.214 1.310   1.238 1.300   1.151 1.203   1.142 1.199   1.147 1.205   1.104 1.179
+//    768   1.215 1.315   1.147 1.224   1.110 1.151   1.091 1.164   1.088 1.158   1.075 1.139
+//   1024   1.179 1.264   1.122 1.164   1.095 1.184   1.080 1.139   1.074 1.182   1.059 1.161
+//   1536   1.034 1.140   0.992 1.081                 0.875 0.949                 0.747 0.869
+//   2048   1.021 1.108   0.944 1.014                 0.838 0.922                 0.761 0.879
+// With nearly every row active 768 rows of width 768 are even (0.999; 1.017 in fewer, larger groups), with an inner side of 8192 0.988.
+// Beyond width 1024 every product is split over clusters, and what the partial sums cost grows with the rows.  The rule goes by allocated
+// rows, which the host knows when it captures a step; how many are active only the device knows, so a large handle's short start and tail
+// stay unpacked.
+constexpr int kPackedMaxRows = 128, kPackedMaxRowsTc = 768, kPackedMaxWide = 230000;
+int packed_rows_tc(const Dims &dm) { return dm.d <= 1024 ? kPackedMaxRowsTc : std::max(kPackedMaxRows, kPackedMaxWide / dm.d); }
 bool packed_path(const pd_handle *h) {
-  return h->packed_ok && h->batch * h->dm.C <= (h->tc_w.empty() ? kPackedMaxRows : kPackedMaxRowsTc) && cross_attn_tma_supported(h->dm);
+  return h->packed_ok && h->batch * h->dm.C <= (h->tc_w.empty() ? kPackedMaxRows : packed_rows_tc(h->dm)) && cross_attn_tma_supported(h->dm);
 }
 
 // alone: not to overlap with the launch before (timing)

@@ -6,9 +6,9 @@
 // the product; the producer of A left x * gain in bf16 and the partial sums of x^2), ReLU, rotary positions and the
 // KV-append of the self-attention projection, or the residual add that leaves the next layer's A and sums.
 //
-// What bounds it: a step has a few to about a hundred rows and 1-8 MB of weights per product, so a product is a chain of
-// latencies.  The kernel keeps that chain short: everything that does not depend on the kernel before it happens ahead
-// of the programmatic-dependency wait - the CTA's whole slice of W (32 columns) travels through shared memory into mma
+// What bounds it: a step has a few to about a hundred rows (of narrow layers several hundred, see proj_tc_better) and
+// 1-8 MB of weights per product, so a product is a chain of latencies.  The kernel keeps that chain short: everything that
+// does not depend on the kernel before it happens ahead of the programmatic-dependency wait - the CTA's whole slice of W (32 columns) travels through shared memory into mma
 // fragments in REGISTERS, split along K over the warps.  Behind the wait there are left: one round of 16-byte loads of
 // the rows straight into fragment registers (the order of the 32 k of a unit is permuted alike on both sides, which
 // a contraction does not see), the mma chain, one sum over the warps through shared memory, the epilogue.
@@ -200,8 +200,8 @@ __global__ void __launch_bounds__(PJ_T, 2) proj_mma_kernel(ProjArgs a) {
   PjExtra ex;
   if (!CLUSTER && mine > 0) load_extra((int)blockIdx.y * 16 + (tid >> 4), ex);
   int buf = 0;
-  // (A step takes this path with at most 128 rows, one batch.  The loop keeps the kernel right for more, and costs nothing: without it the
-  // compiler spills at K = 1024, and decodes of that width are 1 % slower.)
+  // (128 rows are one batch.  With more, a wide layer of a short reduction - 300 rows of 64 by 4800 - leaves room for one row group, which takes
+  // three; a reduction over a cluster has no more rows than one batch, see proj_tc_better.)
   for (int t0 = 0; t0 < mine; t0 += PJ_BATCH) {
     const int tb = min(PJ_BATCH, mine - t0);
     if (t0 > 0) {                                     // the previous batch's scales and sums are read by now

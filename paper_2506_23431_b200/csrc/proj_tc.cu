@@ -562,10 +562,23 @@ cudaError_t each_kernel(int epi, bool split, bool all, F f) {
 // Whole blocks of K, 16-byte tensor-map rows.
 bool proj_tc_supported(int K, int N) { return K >= PT_BK && K % PT_BK == 0 && N % 8 == 0; }
 
-// Against the register products of proj_mma.cu, whole decodes of four layers, 512 keys, every row active, ms: width 1024, 130 rows
-// 11.8 against 12.2; width 768, 130 rows 10.8 against 10.6, 256 rows 11.8 against 13.9; width 256, 256 rows 9.1 against 7.7, 1024 rows
-// 11.5 against 12.1.  (K and N differ by the same factors at every width: the narrower side stands for it.)
-bool proj_tc_better(int K, int N, int rows_cap) { return rows_cap > 128 && (long long)rows_cap * std::min(K, N) > 110000; }
+// Against the register products of proj_mma.cu, whole decodes of four layers, 512 keys, every product on the one or the other, "register /
+// tensor memory" with about two thirds and with about 0.42 of the allocated rows active, inner sides of four widths:
+//   width    130 rows       256           384           512           640           768
+//    256   0.813 0.785   0.864 0.832   0.898 0.860   0.933 0.895   0.991 0.912   1.022 0.931
+//    512   0.901 0.861   0.982 0.935   1.075 0.997   1.146 1.057   1.206 1.111   1.237 1.151
+//    768   1.007 0.935   1.205 1.061   1.369 1.206   1.490 1.318   1.631 1.400   1.744 1.490
+//   1024   1.077 0.973   1.263 1.117   1.437 1.276   1.615 1.391   1.594 1.438   1.708 1.509
+// and with other inner sides:
+//   512 x 512    0.816 0.784 at 130 rows, 0.992 0.933 at 512, 1.054 1.000 at 768
+//   256 x 8192   0.996 0.910 at 130 rows, 1.413 1.220 at 512, 1.593 1.315 at 768
+//    64 x 8192   0.918 0.854 at 130 rows, 1.220 1.084 at 512, 1.359 1.165 at 768
+// A register product walks its rows at a rate that falls with its weights, one on tensor memory hardly notices either: the line where both
+// take the same is rows = 60 + 1.5e8 / weights.  (A side below 128 counts as 128: 64 x 4096, 1.081 at 512 rows, would seem alike only at 632.)
+// Whole decodes by this rule, each product by itself, are between 0.95 and 1.12 times as fast as with the better of the two for all products.
+bool proj_tc_better(int K, int N, int rows_cap) {
+  return rows_cap > 128 && (long long)(rows_cap - 60) * std::max(K, 128) * std::max(N, 128) > 150000000;
+}
 
 cudaError_t proj_tc_prepare() {
   return each_kernel(0, false, true, [](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PT_SMEM); });

@@ -456,6 +456,24 @@ def test_decode_on_tensor_memory_products(batch, rows, d_ff, pos, length, kv8):
     assert s["max_err"] < parity.TOL["bf16"]
 
 
+RULES = [
+    # sequences, open rows per sequence, heads, inner width -> products
+    (10, 30, 1, 4800),     # 300 rows: register products that take three batches of rows in one row group
+    (10, 31, 1, 4800),     # 310 rows: the wide ones on tensor memory, the others on registers
+    (24, 32, 4, 1024),     # 768 rows: queries, keys, values and the inner ones on tensor memory, the square ones on registers
+    (7, 30, 17, 192),      # 210 rows of width 1088: the most that run packed beyond width 1024 (211)
+    (8, 27, 17, 192),      # 216 rows: the library's
+]
+
+
+@pytest.mark.parametrize("batch,rows,heads,d_ff", RULES)
+def test_decode_where_the_products_change_kernels(batch, rows, heads, d_ff):
+    wl = W.CONFIGS["bart_base"].scaled(name="rules", batch=batch, sub_max=rows, d_ff=d_ff, pos_mode=ROPE, max_sub_len=rows + 2, time_max=rows + 6,
+                                       length_dist=("uniform", rows - 4, rows + 2), **dict(BASE, d_model=64 * heads, n_heads=heads, ctx=40))
+    s = check(wl, rows=[0, batch - 1], ragged=True, free_run=False)
+    assert s["max_err"] < parity.TOL["bf16"]
+
+
 @pytest.mark.parametrize("pos", [ROPE, T5])
 @pytest.mark.parametrize("heads", [17, 33, 49])
 def test_decode_on_split_tensor_memory_products(heads, pos):
