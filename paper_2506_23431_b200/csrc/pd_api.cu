@@ -174,9 +174,9 @@ struct pd_handle {
   bool kv8 = false;
   VocabMaps vmaps;                 // hidden rows and lm_head for the tcgen05 vocabulary projection
   bool vocab_tc = false;
-  bool packed_ok = false;          // bf16, and every kernel of the packed path takes this configuration
+  int packed_rows = 0;             // most allocated rows of a step on the packed path; 0: some kernel of it does not take this configuration
   bool f32_own = false;            // fp32: the layers' products on proj_f32 (at most 32 allocated rows)
-  std::vector<ProjTcWeightMaps> tc_w;   // per layer and product: the weights of proj_tc; empty: not usable
+  std::vector<ProjTcWeightMaps> tc_w;   // per layer and product: the weights of proj_tc; empty: no step of this handle is for it
   ProjTcActMaps tc_act[4];         // its activations: normalised input, self-attention output, cross-attention output, feed-forward rows
   bool rows_packed = false;        // the last step left the activation buffers packed (pd_debug_read)
   // pd_generate_host: host-to-device copies of the encoder memory run on a stream of their own, in
@@ -354,9 +354,7 @@ void product_shape(const Dims &dm, int p, int &K, int &N) {
 // stay unpacked.
 constexpr int kPackedMaxRows = 128, kPackedMaxRowsTc = 768, kPackedMaxWide = 230000;
 int packed_rows_tc(const Dims &dm) { return dm.d <= 1024 ? kPackedMaxRowsTc : std::max(kPackedMaxRows, kPackedMaxWide / dm.d); }
-bool packed_path(const pd_handle *h) {
-  return h->packed_ok && h->batch * h->dm.C <= (h->tc_w.empty() ? kPackedMaxRows : packed_rows_tc(h->dm)) && cross_attn_tma_supported(h->dm);
-}
+bool packed_path(const pd_handle *h) { return h->batch * h->dm.C <= h->packed_rows; }
 
 // alone: not to overlap with the launch before (timing)
 AttnArgs attn_args(pd_handle *h, int layer, bool self, bool alone) {
@@ -455,7 +453,7 @@ pd_status enqueue_step_packed(pd_handle *h) {
     const Product &pr = kProducts[which];
     product_shape(dm, which, a.K, a.N);
     a.w = bf(h->layer_w[(size_t)l * kLayerTensors + pr.weight]);
-    if (!h->tc_w.empty() && proj_tc_better(a.K, a.N, p.rows_cap))
+    if (proj_tc_better(a.K, a.N, p.rows_cap))
       OWN(h, PD_PROF_GEMM, launch_proj_tc(pr.epi, h->tc_w[(size_t)l * P_COUNT + which], h->tc_act[pr.act], a, h->st.hdr + HDR_STATUS, s));
     else
       OWN(h, PD_PROF_GEMM, launch_proj_mma(pr.epi, a, s));
@@ -761,21 +759,23 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
     if (vocab_tc_prepare(1, dm.V, cfg->store_logits != 0) != cudaSuccess || vocab_tc_prepare(dm.B * dm.C, dm.V, cfg->store_logits != 0) != cudaSuccess) return bail(PD_ERR_CUDA);   // (a smaller batch may take the other variant)
     h->vocab_tc = true;
   }
-  if (h->vocab_tc && h->have_tmap && self_attn_tc_supported(dm)) {
-    h->packed_ok = true;
-    bool tc = true;
+  if (h->vocab_tc && h->have_tmap && self_attn_tc_supported(dm) && cross_attn_tma_supported(dm)) {
+    const int most = dm.B * dm.C;                       // rows of this handle's largest step
+    bool mma = true, tc = true, need_tc = false;        // both kinds take every product; some product of some step is for tensor memory
     for (int l = 0; l < dm.L; ++l)
       for (int q = 0; q < P_COUNT; ++q) {
         int K, N;
         product_shape(dm, q, K, N);
-        h->packed_ok = h->packed_ok && proj_mma_supported(K, N, h->layer_w[(size_t)l * kLayerTensors + kProducts[q].weight]);
+        mma = mma && proj_mma_supported(K, N, h->layer_w[(size_t)l * kLayerTensors + kProducts[q].weight]);
         tc = tc && proj_tc_supported(K, N);
+        need_tc = need_tc || proj_tc_better(K, N, std::min(most, packed_rows_tc(dm)));
       }
-    if (h->packed_ok && tc) {
+    if (mma) h->packed_rows = tc ? packed_rows_tc(dm) : kPackedMaxRows;
+    if (mma && tc && need_tc) {
       const Region *act[4] = {&L.hbuf, &L.self_out, &L.cross_out, &L.ffn};
       bool good = proj_tc_prepare() == cudaSuccess;
       for (int i = 0; i < 4; ++i)
-        good = good && encode_proj_tc_act_maps(&h->tc_act[i], h->ptr<void>(*act[i]), (uint64_t)dm.B * dm.C, i == 3 ? dm.ff : dm.d) == cudaSuccess;
+        good = good && encode_proj_tc_act_maps(&h->tc_act[i], h->ptr<void>(*act[i]), (uint64_t)most, i == 3 ? dm.ff : dm.d) == cudaSuccess;
       h->tc_w.resize((size_t)dm.L * P_COUNT);
       for (size_t i = 0; i < h->tc_w.size(); ++i) {
         int K, N;
@@ -784,9 +784,9 @@ pd_status pd_init(const pd_config *cfg, const pd_weights *weights, void *workspa
       }
       if (!good) return bail(PD_ERR_CUDA);
     }
-    if (h->packed_ok && (proj_mma_prepare() != cudaSuccess ||
-                         cudaMemsetAsync(h->ptr<void>(L.row_at), 0xFF, L.row_at.bytes, h->stream) != cudaSuccess ||
-                         cudaStreamSynchronize(h->stream) != cudaSuccess))
+    if (mma && (proj_mma_prepare() != cudaSuccess ||
+                cudaMemsetAsync(h->ptr<void>(L.row_at), 0xFF, L.row_at.bytes, h->stream) != cudaSuccess ||
+                cudaStreamSynchronize(h->stream) != cudaSuccess))
       return bail(PD_ERR_CUDA);
   }
   if (cfg->dtype == PD_DTYPE_FP32) {
