@@ -1135,17 +1135,11 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
       b_tiles.push_back((int32_t)((std::upper_bound(first, last, *(first + std::min(r + block_rows, seq_rows[b]) - 1)) - first + 63) / 64));
     }
   const size_t R = row_sub.size(), G = g_row0.size(), NB = b_row0.size();
-  std::vector<int32_t> ranks;                           // timestamps beyond 23 bits: only their order matters to the dependency rule
-  if (dm.n_dist >= 1 << 23) {
-    ranks = row_tau;
-    std::sort(ranks.begin(), ranks.end());
-    ranks.erase(std::unique(ranks.begin(), ranks.end()), ranks.end());
-  }
+  const bool rope = dm.pos_mode == PD_POS_ROPE;
   row_key.reserve(2 * R);
-  for (size_t r = 0; r < R; ++r) {
-    const int tau = ranks.empty() ? row_tau[r] : (int)(std::lower_bound(ranks.begin(), ranks.end(), row_tau[r]) - ranks.begin());
-    row_key.push_back(row_sub[r] << 24 | tau);
-    row_key.push_back(4 * (row_tau[r] + row_sub[r]));
+  for (size_t r = 0; r < R; ++r) {                      // (with a bias timestamps are below 512)
+    row_key.push_back(rope ? row_sub[r] : row_sub[r] << 24 | row_tau[r]);
+    row_key.push_back(rope ? row_tau[r] : 4 * (row_tau[r] + row_sub[r]));
   }
   if (rows_out) *rows_out = (int32_t)R;
   if (loss_out) *loss_out = 0.0;
@@ -1171,7 +1165,6 @@ pd_status pd_teacher_forward(pd_handle *h, const int32_t *n_sub, const int32_t *
   float *x = reinterpret_cast<float *>(base + L.x);
   void *hb = base + L.hb, *qkv = base + L.qkv, *att = base + L.att, *cq = base + L.cq, *co = base + L.co, *ffn = base + L.ffn;
   const int M = (int)R;
-  const bool rope = dm.pos_mode == PD_POS_ROPE;
   OWN(h, PD_PROF_OTHER, launch_gather_rows(M, dm.d, d_tok, h->w.embed, x, s));
   CUtensorMap map_cq, map_ctx;
   if (!h->kv8)

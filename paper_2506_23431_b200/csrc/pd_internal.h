@@ -143,7 +143,7 @@ struct DenseAttnArgs {
   const int32_t *grp_row0, *grp_n;       // [groups] first row and number of rows (<= block_rows) of a query block
   const int32_t *grp_keys;               // [groups] self: row count of the block's sequence; cross: its context length
   // self
-  const int2 *row_key;                   // [rows] (subsequence i << 24 | timestamp tau, 4 x position tau + i) of every row; tau below 2^23 (or its rank)
+  const int2 *row_key;                   // [rows] with a bias (subsequence i << 24 | timestamp tau, 4 x position tau + i) of every row, else (i, tau)
   const int32_t *grp_tiles;              // [groups] 64-key tiles up to the first one of a later subsequence than the block's last row's
   const int32_t *grp_key_row0;           // [groups] first row of the block's sequence
   const float *bias_tab; int n_dist;     // T5 mode: [H][n_dist], log2(e)-scaled; else null

@@ -14,8 +14,9 @@ namespace {
 // P.V on mma.sync, online softmax in the log2 domain; a warp owns its rows, so nothing is merged.  The keys are the sequence's own
 // target rows, with the dependency rule and the T5 bias applied to the accumulator fragment; the key walk ends at the first tile of a
 // later subsequence.
-// A row's subsequence and timestamp share a word (8 and 24 bits) with a guard bit above each: one subtraction tells whether a query sees a
-// key - both guard bits stand - and the bias is read whatever it tells, at a place that is always in the table, so that no pair branches.
+// With a bias, whose table bounds the timestamps, a row's subsequence and timestamp share a word (8 and 24 bits) with a guard bit above each: one
+// subtraction tells whether a query sees a key - both guard bits stand - and the bias is read whatever it tells, at a place that is always in the
+// table, so that no pair branches.  Without one the two stand by themselves, and the signs of two differences tell.
 // What bounds it: the mask and the bias, evaluated per pair.  11.5 k rows of 32 sequences, 16 heads, per layer: 203 us in groups of 32 rows
 // (every group reads its keys again), 160 us with 16 rows per warp, two comparisons and a branch per pair and the tiles to walk found by
 // search, 234 us with 32 (the mask needs the registers); 96 us here.  Where 128-row blocks would leave SMs without one, 64-row blocks.
@@ -37,7 +38,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
   using namespace mt;
   constexpr int TT = W * 32;
   extern __shared__ uint8_t t_raw[];
-  __shared__ __align__(16) int2 key_s[TSLOTS][TK];      // (subsequence << 24 | timestamp, 4 x position)
+  __shared__ __align__(16) int2 key_s[TSLOTS][TK];      // BIAS: (subsequence << 24 | timestamp, 4 x position), else (subsequence, timestamp)
   __shared__ float bias_s[BIAS ? TMAXD : 1];
   const int grp = blockIdx.x, h = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, tig = lane & 3;
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
     }
     for (int i = tid; i < TK; i += TT) {
       if (first + i < nk) t_cp_async8(smem_u32(&key_s[slot][i]), a.row_key + k0 + first + i);
-      else key_s[slot][i] = make_int2(0x7f << 24, 0);        // a subsequence no row reaches
+      else key_s[slot][i] = make_int2(BIAS ? 0x7f << 24 : 0x7fffffff, 0);      // a subsequence no row reaches
     }
   };
   const int n_tiles = a.grp_tiles[grp];          // keys are sorted by subsequence: nothing of a later one than the block's last row's is visible
@@ -82,12 +83,13 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
     qf[kk][2] = r_lo < nq ? *reinterpret_cast<const uint32_t *>(q_lo + kk * 16 + 8) : 0u;
     qf[kk][3] = r_hi < nq ? *reinterpret_cast<const uint32_t *>(q_hi + kk * 16 + 8) : 0u;
   }
-  // subsequence and timestamp of the rows under their guard bits (no row: sees nothing), 4 x position
-  const int2 none = make_int2((int)((0x7fu << 24) - kSees), 0);
+  // BIAS: subsequence and timestamp of the rows under their guard bits (no row: sees nothing), 4 x position; else the two by themselves
+  const int2 none = make_int2(BIAS ? (int)((0x7fu << 24) - kSees) : -1, 0);
   const int2 k_lo = r_lo < nq ? a.row_key[q0 + r_lo] : none, k_hi = r_hi < nq ? a.row_key[q0 + r_hi] : none;
-  const uint32_t qk[2] = {(uint32_t)k_lo.x + kSees, (uint32_t)k_hi.x + kSees};
+  const uint32_t qk[2] = {(uint32_t)k_lo.x + (BIAS ? kSees : 0u), (uint32_t)k_hi.x + (BIAS ? kSees : 0u)};
   const int qp[2] = {k_lo.y, k_hi.y};
-  const int warp_i_max = w0 < nq ? a.row_key[q0 + min(w0 + 15, nq - 1)].x >> 24 : -1;
+  auto subsequence = [](int x) { return BIAS ? x >> 24 : x; };
+  const int warp_i_max = w0 < nq ? subsequence(a.row_key[q0 + min(w0 + 15, nq - 1)].x) : -1;
   TileAcc A;
   A.clear();
   const float sl2 = a.scale_log2e;
@@ -98,7 +100,7 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
     if (tile + TSLOTS - 1 < n_tiles) fetch(tile + TSLOTS - 1);
     asm volatile("cp.async.commit_group;" ::: "memory");
     const int slot = tile % TSLOTS;
-    if (w0 >= nq || key_s[slot][0].x >> 24 > warp_i_max) continue;      // no row of this warp sees the tile
+    if (w0 >= nq || subsequence(key_s[slot][0].x) > warp_i_max) continue;      // no row of this warp sees the tile
     const uint32_t kbase = base + slot * TSLOT_BYTES, vbase = kbase + TK * 128;
     float sc[8][4];
 #pragma unroll
@@ -121,7 +123,8 @@ __global__ void __launch_bounds__(W * 32, 16 / W) teacher_self_kernel(DenseAttnA
       for (int kx = 0; kx < 2; ++kx)
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
-          const bool vis = ((qk[hh] - (uint32_t)(kx ? k2.z : k2.x)) & kSees) == kSees;
+          const uint32_t di = qk[hh] - (uint32_t)(kx ? k2.z : k2.x);
+          const bool vis = BIAS ? (di & kSees) == kSees : ((int)di | (qp[hh] - (kx ? k2.w : k2.y))) >= 0;
           float v = sc[nt][2 * hh + kx] * sl2;
           if (BIAS) v += *reinterpret_cast<const float *>(reinterpret_cast<const char *>(bias_s) + max(qp[hh] - (kx ? k2.w : k2.y), 0));
           sc[nt][2 * hh + kx] = vis ? v : -INFINITY;

@@ -58,6 +58,13 @@ def test_teacher_forward_small(pos_mode):
     assert run_case(wl, 2e-2) < 2e-2
 
 
+def test_teacher_forward_subsequences_far_apart():
+    """Timestamps of subsequences far from one another: later than the other's last, whatever their distance."""
+    wl = W.CONFIGS["bart_base"].scaled(name="tf_apart", batch=2, ctx=100, sub_max=5, delta_t=20000, max_sub_len=90,
+                                       length_dist=("uniform", 0, 90), time_max=100000, pos_mode=W.POS_ROPE, **SMALL)
+    assert run_case(wl, 2e-2) < 2e-2
+
+
 def test_teacher_forward_8_bit_context_and_many_groups():
     """More than 256 row groups (several cross-attention launches) and the 8-bit context keys/values."""
     wl = W.CONFIGS["keyphrase"].scaled(name="tf_groups", batch=20, ctx=144, sub_max=24, delta_t=1, max_sub_len=30,
