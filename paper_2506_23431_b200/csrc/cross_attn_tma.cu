@@ -573,33 +573,49 @@ static int cross_cluster_size(const AttnArgs &a) {
 }
 static_assert(7 * XREC_FLOATS * 4 <= xring_bytes(1, true) && 7 * 2 * XREC_FLOATS * 4 <= xring_bytes(2, true), "the states of a cluster fit over the ring");
 
+// 8-bit launches begin under the kernel before from this many segments on, and with no more places on an SM than the launch needs if it is spread
+// evenly: their CTAs are small, and pile up, four on each of the SMs that the kernel before has left already.  Decodes of four layers, segments x
+// keys, ms: begun behind the kernel before / under it, piled up / under it, spread:
+//   8 x 96   4.10 / 4.32 / 4.43       16 x 4096  6.53 / 7.31 / 7.35     32 x 4096  6.89 / 7.66 / 6.76      48 x 784   6.68 / 7.12 / 6.52
+//   64 x 96  4.84 / 4.84 / 4.70       128 x 4096 10.89 / 14.25 / 10.59  144 x 2048 9.33 / 10.80 / 9.00     192 x 1024 9.87 / 10.32 / 9.52
+//   256 x 2048 12.58 / 13.39 / 12.15  384 x 2048 14.34 / 14.80 / 14.00  512 x 2048 16.31 / 15.84 / 15.81   768 x 1024 (another path) alike
+// Dynamic shared memory of such a launch of `ctas` CTAs:
+constexpr long long kX8EarlySegs = 48;
+constexpr int kSmSmem = 228 * 1024, kCtaSmem = 1024;      // shared memory of an SM; what a CTA takes beside its own
+static int x8_smem(int mt, long long ctas) {
+  const int places = (int)((ctas + kSms - 1) / kSms);
+  const int one_more = kSmSmem / (places + 1) - kCtaSmem + 16;      // places + 1 CTAs of this size do not fit
+  return places < xctas(mt, true) && one_more > xsmem(mt, true) ? one_more : xsmem(mt, true);
+}
+
 // rows_per_seq, fp8: the variant to prepare
 cudaError_t cross_attn_tma_prepare(int rows_per_seq, bool fp8) {
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if (rows_per_seq <= 16)
-    return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<1, true>, attr, xsmem(1, true)) : cudaFuncSetAttribute(cross_attn_tma_kernel<1, false>, attr, xsmem(1, false));
-  return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<2, true>, attr, xsmem(2, true)) : cudaFuncSetAttribute(cross_attn_tma_kernel<2, false>, attr, xsmem(2, false));
+    return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<1, true>, attr, x8_smem(1, 1)) : cudaFuncSetAttribute(cross_attn_tma_kernel<1, false>, attr, xsmem(1, false));
+  return fp8 ? cudaFuncSetAttribute(cross_attn_tma_kernel<2, true>, attr, x8_smem(2, 1)) : cudaFuncSetAttribute(cross_attn_tma_kernel<2, false>, attr, xsmem(2, false));
 }
 
 // 8-bit keys/values (a.kv_scale set): tmap = the keys' lines, tmap_v = the transposed values; else tmap alone.
 // a.pdl: launched as a programmatic dependent of the query projection before it, which writes none of the keys,
-// values, row counts and context lengths, so the first tiles travel while that kernel runs.
+// values, row counts and context lengths, so the first tiles travel while that kernel runs (8-bit: not with few segments).
 cudaError_t launch_cross_attn_tma(const AttnArgs &a, const CUtensorMap &tmap, const CUtensorMap &tmap_v, cudaStream_t s) {
   const int mt = (a.dm.C + 15) / 16;
   const bool fp8 = a.kv_scale != nullptr;
   if (mt < 1 || mt > 2 || a.batch > 65535) return cudaErrorInvalidValue;
   const int ns = cross_cluster_size(a);
+  const bool early = a.pdl && (!fp8 || (long long)a.batch * a.dm.H >= kX8EarlySegs);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ns, a.dm.H, a.batch);
   cfg.blockDim = dim3(XTHREADS, 1, 1);
-  cfg.dynamicSmemBytes = xsmem(mt, fp8);
+  cfg.dynamicSmemBytes = fp8 && early ? x8_smem(mt, (long long)ns * a.dm.H * a.batch) : xsmem(mt, fp8);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = ns; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = a.pdl ? 2 : 1;
+  cfg.attrs = attr; cfg.numAttrs = early ? 2 : 1;
   if (mt == 1) return fp8 ? cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, true>, tmap, tmap_v, a) : cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<1, false>, tmap, tmap_v, a);
   return fp8 ? cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, true>, tmap, tmap_v, a) : cudaLaunchKernelEx(&cfg, cross_attn_tma_kernel<2, false>, tmap, tmap_v, a);
 }
