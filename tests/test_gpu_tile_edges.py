@@ -438,8 +438,8 @@ def test_decodes_of_few_rows_repeat_bit_for_bit(batch, heads, ctx, kv8):
 PACKED = [
     # sequences, open rows per sequence, inner width, positions, longest subsequence, 8-bit context
     (5, 26, 64, ROPE, 28, False),       # 130 rows allocated, register products beyond 128; an inner width of one block
-    (19, 31, 1088, T5, 33, True),       # 589 rows: tensor-memory products at this width; a reduction over two pairs of CTAs, the second one block shorter
-    (18, 32, 2112, ROPE, 34, False),    # 576 rows: three pairs
+    (19, 31, 1088, T5, 33, True),       # 589 rows: register products still; a reduction over two CTAs
+    (18, 32, 2112, ROPE, 34, False),    # 576 rows: the inner products on tensor memory; a reduction over three pairs of CTAs
     (24, 32, 4160, T5, 36, False),      # 768 rows, the most that run packed; four pairs, the last one shorter
     (25, 31, 192, T5, 33, False),       # 775 rows: the kernels beyond
     (90, 7, 256, ROPE, 40, False),      # 630 rows, two pages per subsequence
@@ -456,11 +456,29 @@ def test_decode_on_tensor_memory_products(batch, rows, d_ff, pos, length, kv8):
     assert s["max_err"] < parity.TOL["bf16"]
 
 
+WHOLE = [
+    # sequences, open rows per sequence, heads, inner width, positions, 8-bit context; weights and rows that put every product on tensor memory
+    (18, 32, 9, 1088, ROPE, False),     # 576 rows of width 576, which ends inside a pair's columns; a reduction over two pairs, the second one block shorter
+    (18, 32, 9, 1088, T5, True),
+    (8, 26, 16, 2112, ROPE, False),     # 208 rows of width 1024, the longest reduction that is not split; an inner one over three pairs
+    (8, 27, 16, 4160, T5, False),       # 216 rows; four pairs
+]
+
+
+@pytest.mark.parametrize("batch,rows,heads,d_ff,pos,kv8", WHOLE)
+def test_decode_with_every_product_on_tensor_memory(batch, rows, heads, d_ff, pos, kv8):
+    wl = W.CONFIGS["bart_base"].scaled(name="whole", batch=batch, sub_max=rows, d_ff=d_ff, pos_mode=pos, max_sub_len=rows + 2, time_max=rows + 6,
+                                       length_dist=("uniform", rows - 4, rows + 2), kv_c_dtype="e4m3" if kv8 else "same",
+                                       **dict(BASE, d_model=64 * heads, n_heads=heads, ctx=48))
+    s = check(wl, rows=[0, batch - 1], ragged=True, free_run=False)
+    assert s["max_err"] < parity.TOL["bf16"]
+
+
 RULES = [
     # sequences, open rows per sequence, heads, inner width -> products
     (10, 30, 1, 4800),     # 300 rows: register products that take three batches of rows in one row group
     (10, 31, 1, 4800),     # 310 rows: the wide ones on tensor memory, the others on registers
-    (24, 32, 4, 1024),     # 768 rows: queries, keys, values and the inner ones on tensor memory, the square ones on registers
+    (24, 32, 4, 1024),     # 768 rows: the inner products on tensor memory, the others on registers
     (7, 30, 17, 192),      # 210 rows of width 1088: the most that run packed beyond width 1024 (211)
     (8, 27, 17, 192),      # 216 rows: the library's
 ]
@@ -524,3 +542,13 @@ def test_two_handles_side_by_side_on_tensor_memory_products():
             assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
     for dec, _args, _n in runs:
         dec.close()
+
+
+@pytest.mark.parametrize("batch,rows", [(15, 3), (16, 3), (16, 20), (49, 3), (50, 3), (98, 3), (99, 3), (148, 3), (149, 3)])
+def test_decode_where_8_bit_launches_change_their_spread(batch, rows):
+    """45, 48, 147, 150, 294, 297, 444 and 447 segments over 8-bit context: launches behind the kernel before, and under it with one to four CTAs per SM
+    (20 rows per sequence: the form of two row tiles)."""
+    wl = W.CONFIGS["bart_base"].scaled(name="spread", batch=batch, sub_max=rows, d_ff=192, pos_mode=T5, max_sub_len=rows + 3, time_max=rows + 6,
+                                       length_dist=("uniform", 2, rows + 3), kv_c_dtype="e4m3", **dict(BASE, n_layers=1, ctx=272))
+    s = check(wl, rows=[0, batch - 1], ragged=True, free_run=False)
+    assert s["max_err"] < parity.TOL["bf16"]
