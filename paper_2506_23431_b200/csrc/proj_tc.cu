@@ -24,8 +24,8 @@
 // Reductions beyond 1024 are split over a cluster of pairs: every CTA copies its sums of the rows another CTA owns into that CTA's
 // shared memory (one bulk copy per peer), which adds them in rank order (results do not depend on timing).
 // What bounds it: a launch is a chain of latencies - release of the launch before 1.2 us, first rows 0.5, products and the weights the
-// ring did not hold, accumulators out, 0.6 to the exit.  Per launch inside a decode of 32 sequences (204 rows active of 512, width 1024): 7.5 us
-// for queries, keys and values, 5.2-5.9 for the square products, 6.3 up, 9.4 down, where the library took 5.7, 4.3-4.5, 6.4 and 8.3 and
+// ring did not hold, accumulators out, 0.6 to the exit.  What a launch advances a decode of 32 sequences by (204 rows active of 512, width 1024): 7.1 us
+// for queries, keys and values, 5.2-5.7 for the square products, 6.7 up, 9.2 down, where the library took 5.6, 4.3-4.6, 6.3 and 8.3 and
 // 2.4 for a norm in front of every other one, without overlap.  Fewer or more row groups, K splits of 1536 or 2048: slower or the same.
 // Every mbarrier wait is bounded: on expiry the kernel records PD_ERR_TIMEOUT, stops waiting, falls through to the
 // common exit and frees its tensor memory.
